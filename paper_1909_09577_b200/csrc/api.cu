@@ -81,6 +81,26 @@ int desc_dims(const sc_block_desc* d, Dims* o) {
     return SC_OK;
 }
 
+// Blocks that the tensor-core kernels can only take in packed form (kernels.h): a row length that is not a multiple of 8
+// frames, or taps two frames apart.  The batch-norm kernels convert between the dense tensors of the call and the packed
+// operands on the way; only the input, its gradient and u need a copy of their own.
+struct Packed { int phases = 0, Tq = 0; Dims m; };     // m: the block on the packed operands
+Packed plan_packed(const sc_block_desc* d, const Dims& m) {
+    Packed k;
+    if (d->io_dtype == SC_F32 || m.full || !d->has_bn || !d->has_relu || !d->res_before_relu) return k;
+    const bool dilated = m.dil == 2 && (m.K & 1) && m.s == 1;
+    if (m.dil != 1 && !dilated) return k;
+    if (!dilated && m.T % 8 == 0 && m.Tp % 8 == 0) return k;
+    if (m.Cin % 8 || (d->residual == SC_RES_PROJ && m.Cres % 8)) return k;
+    const int ph = dilated ? 2 : 1;
+    const int Tq = dilated ? ((m.T + 1) / 2 + 7) / 8 * 8 : (m.T + 8 * m.s - 1) / (8 * m.s) * (8 * m.s);
+    const long long most = (long long)m.B * ph * std::max(std::max(m.Cin, m.Cout), m.Cres) * Tq;
+    if (most >= (1ll << 31)) return k;                      // the copies index with 32 bits
+    k.phases = ph; k.Tq = Tq; k.m = m;
+    k.m.B = m.B * ph; k.m.T = Tq; k.m.Tp = Tq / m.s; k.m.dil = 1; k.m.plain = (m.K & 1) != 0;
+    return k;
+}
+
 int check_tensor(const sc_tensor* t, int dtype, int64_t B, int64_t C, int64_t T) {
     if (!t || !t->ptr) return SC_ERR_NULL;
     if (t->dtype != dtype || t->rank != 3) return SC_ERR_INCOMPATIBLE;
@@ -107,6 +127,10 @@ struct BlockIO {                 // raw pointers after validation
     bool lengths_ready;          // len_out / nvalid already computed
     void* w16_keep;              // optional: where to leave the float16 copy of wp for the backward pass
     bool w16_ready;              // w16_keep already holds the copy
+    int T_valid;                 // largest legal length when that is not m.T (an encoder input padded to a longer row)
+    // packed block: x (and a projected xres) are packed, y and an identity xres are dense [., ., Td] with lengths
+    // len_dense, and u, v, vr are also written to the dense tensors of `dense` (nullable members)
+    int phases, Td; const int* len_dense; sc_block_saved dense;
 };
 
 // Type of the library-internal contraction operands (u, gv, gu) of this layer.
@@ -180,7 +204,7 @@ int block_fwd_impl(sc_ctx* ctx, const Launch& L, const sc_block_desc* d, const D
                    const sc_block_params* p, sc_block_saved* sv, float* rmean, float* rvar,
                    const FwdScratch& f, const InferStats* inf = nullptr) {
     const int dt = d->io_dtype;
-    if (!io.lengths_ready) lengths(L, io.len_in, m.B, m.T, m.s, io.len_out, io.nvalid, io.blk_off);
+    if (!io.lengths_ready) lengths(L, io.len_in, m.B, io.T_valid ? io.T_valid : m.T, m.s, io.len_out, io.nvalid, io.blk_off);
     const int odt = op_dtype(d);
     if (d->has_bn && d->residual == SC_RES_PROJ) {
         // the residual projection does not depend on the main branch: its contraction and statistics go to the
@@ -258,8 +282,47 @@ int block_fwd_impl(sc_ctx* ctx, const Launch& L, const sc_block_desc* d, const D
         a.vr = sv->vr; a.mean_r = inf ? inf->mean_r : sv->mean_r; a.invstd_r = sv->invstd_r; a.gamma_r = p->gamma_r; a.beta_r = p->beta_r;
         wait_side(ctx, L, ctx->ev[5]);      // the projection branch (enqueued above on the side stream) is complete
     }
+    if (io.phases) {
+        a.phases = io.phases; a.B = m.B / io.phases; a.T = io.Td; a.len_out = io.len_dense;
+        a.v_out = io.dense.v; a.vr_out = io.dense.vr; a.u = u; a.u_out = io.dense.u; a.Cu = m.Cin;
+    }
     bn_apply(L, dt, a);
     return SC_OK;
+}
+
+// Operands of a packed forward pass.
+struct FwdPack { void *x, *xres; int* len_dense; sc_block_saved sv; };
+void plan_fwd_pack(const sc_block_desc* d, const Packed& k, Bump& ws, FwdPack* f) {
+    const size_t e = esize(d->io_dtype), in = e * k.m.B * k.m.T;
+    memset(f, 0, sizeof(*f));
+    f->len_dense = (int*)ws.take(sizeof(int) * k.m.B / k.phases);
+    f->x = ws.take(in * k.m.Cin);
+    if (d->residual == SC_RES_PROJ) f->xres = ws.take(e * k.m.B * k.m.Cres * k.m.Tp);
+    f->sv.u = ws.take(e * k.m.B * k.m.Cin * k.m.Tp);
+    f->sv.v = ws.take((size_t)2 * k.m.B * k.m.Cout * k.m.Tp);
+    if (d->residual == SC_RES_PROJ) f->sv.vr = ws.take((size_t)2 * k.m.B * k.m.Cout * k.m.Tp);
+}
+// Packs the inputs and points io / sv (the caller's, dense) at the packed operands.
+void enter_packed(const Launch& L, const sc_block_desc* d, const Dims& m, const Packed& k, const FwdPack& f, BlockIO& io,
+                  sc_block_saved& sv) {
+    lengths(L, io.len_in, m.B, m.T, m.s, io.len_out, io.nvalid, io.blk_off, k.phases, k.phases > 1 ? f.len_dense : nullptr);
+    PackList pl{};
+    auto add = [&](const void* src, void* dst, int C, const int* len) { pl.src[pl.count] = src; pl.dst[pl.count] = dst; pl.C[pl.count] = C; pl.len[pl.count] = len; ++pl.count; };
+    add(io.x, f.x, m.Cin, io.len_in);
+    const bool own = d->residual == SC_RES_PROJ && io.xres == io.x && m.s == 1;       // the residual source is the input itself
+    if (d->residual == SC_RES_PROJ && !own && m.s == 1) add(io.xres, f.xres, m.Cres, io.len_in);
+    pack_frames(L, pl, m.B, m.T, k.Tq, k.phases);
+    if (d->residual == SC_RES_PROJ && m.s != 1) {
+        PackList pr{}; pr.count = 1; pr.src[0] = io.xres; pr.dst[0] = f.xres; pr.C[0] = m.Cres; pr.len[0] = io.len_out;
+        pack_frames(L, pr, m.B, m.Tp, k.m.Tp, 1);
+    }
+    io.x = f.x;
+    if (d->residual == SC_RES_PROJ) io.xres = own ? f.x : f.xres;
+    io.x_clean = io.res_clean = io.lengths_ready = true;
+    io.phases = k.phases; io.Td = m.Tp; io.len_dense = k.phases > 1 ? f.len_dense : io.len_out;
+    if (k.phases > 1) io.len_in = io.len_out;
+    io.dense.u = sv.u; io.dense.v = sv.v; io.dense.vr = sv.vr;
+    sv.u = f.sv.u; sv.v = f.sv.v; sv.vr = f.sv.vr;
 }
 
 // ---- backward scratch --------------------------------------------------------------------------
@@ -329,6 +392,7 @@ struct BwdIO {
     bool x_clean, res_clean;
     const void* w16_kept;        // float16 copy of wp left by the forward pass (optional)
     cudaEvent_t done;            // recorded on the side stream after this layer's last side-stream kernel
+    int phases, Td; uint32_t total_dense;      // packed block: dy, y and the saved v, vr are dense [., ., Td]; the rest is packed
     float* gmax_zeroed;          // optional: a float the caller has already set to zero, used for the |gv| bound
                                  // (a memset between two kernels would end the programmatic overlap of that pair)
 };
@@ -368,6 +432,7 @@ int block_bwd_impl(sc_ctx* ctx, const Launch& L, const sc_block_desc* d, const D
     a.gv = s.gv; a.gvr = s.gvr;
     // identity residual: its gradient is the gated upstream gradient itself
     a.gres = (d->residual == SC_RES_IDENTITY) ? (io.dx_res ? io.dx_res : s.gres) : nullptr;
+    a.phases = io.phases; a.T = io.Td; a.total_dense = io.total_dense;
     bn_bwd_reduce_finalize(L, dt, a, p->gamma, p->gamma_r, g->dgamma, g->dbeta, g->dgamma_r, g->dbeta_r,
                            d->has_bias ? g->dbias : nullptr, acc);
     bn_bwd_apply(L, dt, a);
@@ -452,6 +517,17 @@ int block_bwd_impl(sc_ctx* ctx, const Launch& L, const sc_block_desc* d, const D
     // the caller joins: it waits for io.done on its stream before it reuses this scratch or returns
     if (io.done) record_side(ctx, io.done);
     return SC_OK;
+}
+
+// Packed operands of a backward pass.
+struct BwdPack { void *x, *xres, *u, *dx, *dx_res, *dx_add; int* len_dense; };
+void plan_bwd_pack(const sc_block_desc* d, const Packed& k, Bump& ws, BwdPack* b) {
+    const size_t e = esize(d->io_dtype), in = e * k.m.B * k.m.Cin * k.m.T;
+    memset(b, 0, sizeof(*b));
+    b->len_dense = (int*)ws.take(sizeof(int) * k.m.B / k.phases);
+    b->x = ws.take(in); b->dx = ws.take(in); b->dx_add = ws.take(in);
+    b->u = ws.take(e * k.m.B * k.m.Cin * k.m.Tp);
+    if (d->residual != SC_RES_NONE) { b->xres = ws.take(e * k.m.B * k.m.Cres * k.m.Tp); b->dx_res = ws.take(e * k.m.B * k.m.Cres * k.m.Tp); }
 }
 
 int check_params(const sc_block_desc* d, const sc_block_params* p) {
@@ -618,8 +694,15 @@ const char* sepconv_kernel_class_name(int c) { return kclass_name(c); }
 int sepconv_workspace_bytes(const sc_block_desc* desc, size_t* fwd, size_t* bwd) {
     Dims m;
     SC_TRY(desc_dims(desc, &m));
-    if (fwd) { Bump b(nullptr, 0); FwdScratch f; plan_fwd(desc, m, b, &f, nullptr); *fwd = b.off + 256; }
-    if (bwd) { Bump b(nullptr, 0); BwdScratch s; plan_bwd(desc, m, b, &s, nullptr); *bwd = b.off + 256; }
+    const Packed k = plan_packed(desc, m);
+    if (fwd) {
+        Bump b(nullptr, 0); FwdScratch f; plan_fwd(desc, m, b, &f, nullptr); *fwd = b.off + 256;
+        if (k.phases) { Bump q(nullptr, 0); FwdPack fp; plan_fwd(desc, k.m, q, &f, nullptr); plan_fwd_pack(desc, k, q, &fp); *fwd = std::max(*fwd, q.off + 256); }
+    }
+    if (bwd) {
+        Bump b(nullptr, 0); BwdScratch s; plan_bwd(desc, m, b, &s, nullptr); *bwd = b.off + 256;
+        if (k.phases) { Bump q(nullptr, 0); BwdPack bp; plan_bwd(desc, k.m, q, &s, nullptr); plan_bwd_pack(desc, k, q, &bp); *bwd = std::max(*bwd, q.off + 256); }
+    }
     return SC_OK;
 }
 
@@ -640,18 +723,23 @@ int sepconv_fwd(sc_ctx* ctx, const sc_block_desc* desc, const sc_tensor* x, cons
     SC_TRY(check_params(desc, params));
     SC_TRY(check_saved(desc, saved, false));
     if (!workspace) return SC_ERR_WORKSPACE;
+    Packed pk;
+    if (ctx->gemm_mode == 0) pk = plan_packed(desc, m);
     Bump ws(workspace, workspace_bytes);
-    FwdScratch f;
-    plan_fwd(desc, m, ws, &f, &ctx->tc);
+    FwdScratch f; FwdPack fp;
+    plan_fwd(desc, pk.phases ? pk.m : m, ws, &f, &ctx->tc);
+    if (pk.phases) plan_fwd_pack(desc, pk, ws, &fp);
     if (!ws.ok()) return SC_ERR_WORKSPACE;
     Launch L{(cudaStream_t)cuda_stream, ctx->status_dev, &ctx->launches, &ctx->prof, ctx->gemm_mode, ctx->pdl};
     BlockIO io{};
     io.x = x->ptr; io.xres = desc->residual != SC_RES_NONE ? (x_res ? x_res->ptr : x->ptr) : nullptr;
     io.y = y->ptr; io.len_in = lengths_dev; io.len_out = f.len_out; io.nvalid = f.nvalid; io.blk_off = f.blk_off;
     io.x_clean = false; io.res_clean = false; io.lengths_ready = false;
-    SC_TRY(block_fwd_impl(ctx, L, desc, m, io, params, saved, running_mean, running_var, f));
+    sc_block_saved sv = *saved;
+    if (pk.phases) enter_packed(L, desc, m, pk, fp, io, sv);
+    SC_TRY(block_fwd_impl(ctx, L, desc, pk.phases ? pk.m : m, io, params, &sv, running_mean, running_var, f));
     if (out_lengths_dev)
-        cudaMemcpyAsync(out_lengths_dev, f.len_out, sizeof(int) * m.B, cudaMemcpyDeviceToDevice, L.stream);
+        cudaMemcpyAsync(out_lengths_dev, io.phases ? io.len_dense : f.len_out, sizeof(int) * m.B, cudaMemcpyDeviceToDevice, L.stream);
     return finish(ctx);
 }
 
@@ -674,6 +762,11 @@ int sepconv_infer_workspace_bytes(const sc_block_desc* desc, size_t* bytes) {
     SC_TRY(desc_dims(desc, &m));
     Bump b(nullptr, 0); InferScratch q; plan_infer(desc, m, b, &q, nullptr);
     *bytes = b.off + 256;
+    const Packed k = plan_packed(desc, m);
+    if (k.phases) {
+        Bump c(nullptr, 0); FwdPack fp; plan_infer(desc, k.m, c, &q, nullptr); plan_fwd_pack(desc, k, c, &fp);
+        *bytes = std::max(*bytes, c.off + 256);
+    }
     return SC_OK;
 }
 
@@ -695,18 +788,22 @@ int sepconv_infer(sc_ctx* ctx, const sc_block_desc* desc, const sc_tensor* x, co
     if (desc->has_bn && (!running_mean || !running_var)) return SC_ERR_NULL;
     if (desc->residual == SC_RES_PROJ && (!running_mean_r || !running_var_r)) return SC_ERR_NULL;
     if (!workspace) return SC_ERR_WORKSPACE;
+    Packed pk;
+    if (ctx->gemm_mode == 0) pk = plan_packed(desc, m);
     Bump ws(workspace, workspace_bytes);
-    InferScratch q;
-    plan_infer(desc, m, ws, &q, &ctx->tc);
+    InferScratch q; FwdPack fp;
+    plan_infer(desc, pk.phases ? pk.m : m, ws, &q, &ctx->tc);
+    if (pk.phases) plan_fwd_pack(desc, pk, ws, &fp);
     if (!ws.ok()) return SC_ERR_WORKSPACE;
     Launch L{(cudaStream_t)cuda_stream, ctx->status_dev, &ctx->launches, &ctx->prof, ctx->gemm_mode, ctx->pdl};
     BlockIO io{};
     io.x = x->ptr; io.xres = desc->residual != SC_RES_NONE ? (x_res ? x_res->ptr : x->ptr) : nullptr;
     io.y = y->ptr; io.len_in = lengths_dev; io.len_out = q.f.len_out; io.nvalid = q.f.nvalid; io.blk_off = q.f.blk_off;
     InferStats inf{running_mean, running_var, running_mean_r, running_var_r};
-    SC_TRY(block_fwd_impl(ctx, L, desc, m, io, params, &q.sv, nullptr, nullptr, q.f, &inf));
+    if (pk.phases) { enter_packed(L, desc, m, pk, fp, io, q.sv); memset(&io.dense, 0, sizeof(io.dense)); }
+    SC_TRY(block_fwd_impl(ctx, L, desc, pk.phases ? pk.m : m, io, params, &q.sv, nullptr, nullptr, q.f, &inf));
     if (out_lengths_dev)
-        cudaMemcpyAsync(out_lengths_dev, q.f.len_out, sizeof(int) * m.B, cudaMemcpyDeviceToDevice, L.stream);
+        cudaMemcpyAsync(out_lengths_dev, io.phases ? io.len_dense : q.f.len_out, sizeof(int) * m.B, cudaMemcpyDeviceToDevice, L.stream);
     return finish(ctx);
 }
 
@@ -736,12 +833,17 @@ int sepconv_bwd(sc_ctx* ctx, const sc_block_desc* desc, const sc_tensor* dy, con
     SC_TRY(check_saved(desc, saved, false));
     SC_TRY(check_grads(desc, grads));
     if (!workspace) return SC_ERR_WORKSPACE;
+    Packed pk;
+    if (ctx->gemm_mode == 0) pk = plan_packed(desc, m);
+    const Dims& mq = pk.phases ? pk.m : m;
     Bump ws(workspace, workspace_bytes);
-    BwdScratch s;
-    plan_bwd(desc, m, ws, &s, &ctx->tc);
+    BwdScratch s; BwdPack bp;
+    plan_bwd(desc, mq, ws, &s, &ctx->tc);
+    if (pk.phases) plan_bwd_pack(desc, pk, ws, &bp);
     if (!ws.ok()) return SC_ERR_WORKSPACE;
     Launch L{(cudaStream_t)cuda_stream, ctx->status_dev, &ctx->launches, &ctx->prof, ctx->gemm_mode, ctx->pdl};
-    lengths(L, lengths_dev, m.B, m.T, m.s, s.len_out, s.nvalid, s.blk_off);
+    const bool two = pk.phases > 1;
+    lengths(L, lengths_dev, m.B, m.T, m.s, s.len_out, s.nvalid, s.blk_off, two ? pk.phases : 1, two ? bp.len_dense : nullptr);
     BwdIO io{};
     io.dy = dy->ptr; io.x = x->ptr; io.y = y->ptr;
     io.xres = desc->residual != SC_RES_NONE ? (x_res ? x_res->ptr : x->ptr) : nullptr;
@@ -750,7 +852,37 @@ int sepconv_bwd(sc_ctx* ctx, const sc_block_desc* desc, const sc_tensor* dy, con
     io.len_in = lengths_dev; io.len_out = s.len_out; io.nvalid = s.nvalid; io.blk_off = s.blk_off;
     io.x_clean = false; io.res_clean = false;
     io.done = ctx->ev[2];
-    SC_TRY(block_bwd_impl(ctx, L, desc, m, io, params, saved, grads, accumulate, s));
+    sc_block_saved sv = *saved;
+    if (pk.phases) {
+        // packs what the contractions read; the batch-norm kernels read dy, y, v and vr as they are
+        PackList in{}, out{};
+        auto add = [&](PackList& l, const void* src, void* dst, int C, const int* len) { l.src[l.count] = src; l.dst[l.count] = dst; l.C[l.count] = C; l.len[l.count] = len; ++l.count; };
+        const bool proj = desc->residual == SC_RES_PROJ, own = proj && io.xres == io.x && m.s == 1;
+        add(in, io.x, bp.x, m.Cin, lengths_dev);
+        if (io.dx_add) { add(in, io.dx_add, bp.dx_add, m.Cin, lengths_dev); io.dx_add = bp.dx_add; }
+        const int* len_o = two ? bp.len_dense : s.len_out;
+        PackList& o = m.s == 1 ? in : out;               // tensors with output frames share the launch when the frames agree
+        if (desc->has_dw) { add(o, sv.u, bp.u, m.Cin, len_o); sv.u = bp.u; }
+        if (proj && !own) add(o, io.xres, bp.xres, m.Cres, len_o);
+        pack_frames(L, in, m.B, m.T, pk.Tq, pk.phases);
+        if (m.s != 1) pack_frames(L, out, m.B, m.Tp, mq.Tp, 1);
+        if (proj) io.xres = own ? bp.x : bp.xres;
+        io.x = bp.x; io.dx = bp.dx;
+        if (io.dx_res) io.dx_res = bp.dx_res;
+        io.x_clean = io.res_clean = true;
+        if (two) io.len_in = s.len_out;
+        io.phases = pk.phases; io.Td = m.Tp; io.total_dense = (uint32_t)m.B * m.Cout * m.Tp;
+    }
+    SC_TRY(block_bwd_impl(ctx, L, desc, mq, io, params, &sv, grads, accumulate, s));
+    if (pk.phases) {
+        PackList l{}; l.count = 1; l.src[0] = bp.dx; l.dst[0] = dx->ptr; l.C[0] = m.Cin; l.len[0] = lengths_dev;
+        if (io.dx_res && m.s == 1) { l.count = 2; l.src[1] = bp.dx_res; l.dst[1] = dx_res->ptr; l.C[1] = m.Cres; l.len[1] = lengths_dev; }
+        unpack_frames(L, l, m.B, m.T, pk.Tq, pk.phases);
+        if (io.dx_res && m.s != 1) {
+            PackList r{}; r.count = 1; r.src[0] = bp.dx_res; r.dst[0] = dx_res->ptr; r.C[0] = m.Cres; r.len[0] = s.len_out;
+            unpack_frames(L, r, m.B, m.Tp, mq.Tp, 1);
+        }
+    }
     wait_side(ctx, L, ctx->ev[2]);
     return finish(ctx);
 }
@@ -776,13 +908,45 @@ struct EncPlan {
     size_t bytes;
     size_t scratch_mark;           // offset where the shared per-layer scratch starts
     size_t scratch_size;           // its size; kScratchRegions regions of that size in all (backward layers rotate)
+    // An input whose row lengths the tensor-core kernels cannot take runs on rows padded to T_pad frames: the frames past a
+    // sample's length are masked anyway, so only the call's own tensors are copied (x and dlogits in, logits and dx out).
+    int T_pad = 0, T_out = 0;      // 0: not padded; frames of the last layer's dense output
+    void *x_pad, *dlogits_pad, *logits_pad, *dx_pad;
 };
 
-int plan_encoder(const sc_encoder_desc* e, void* base, size_t cap, EncPlan* P, const TcState* tc) {
+// Row length for a padded pass (0: none needed): the stride product times 8, so that every layer's rows are whole vectors.
+int encoder_pad(const sc_encoder_desc* e) {
+    if (e->layers[0].io_dtype == SC_F32) return 0;
+    int t = e->layers[0].T_in, div = 8;
+    if (t < 1) return 0;
+    bool fits = t % 8 == 0;
+    for (int i = 0; i < e->n_layers; ++i) {
+        const sc_block_desc& d = e->layers[i];
+        const int s = (d.has_dw || d.full_conv) ? d.stride : 1;
+        if (s != 1 && s != 2) return 0;
+        t = (t - 1) / s + 1;
+        fits &= t % 8 == 0;
+        if (div > (1 << 16)) return 0;
+        div *= s;
+    }
+    if (fits) return 0;
+    const int T = e->layers[0].T_in, Tq = (T + div - 1) / div * div;
+    const sc_block_desc &f = e->layers[0], &l = e->layers[e->n_layers - 1];
+    return (long long)f.B * std::max(f.C_in, l.C_out) * Tq < (1ll << 31) ? Tq : 0;      // the copies index with 32 bits
+}
+
+int plan_encoder(const sc_encoder_desc* e, void* base, size_t cap, EncPlan* P, const TcState* tc, bool pad) {
     if (!e || !e->layers || e->n_layers < 1) return SC_ERR_NULL;
     Bump ws(base, cap);
     P->L.resize(e->n_layers);
     int B = e->layers[0].B, T = e->layers[0].T_in, C = e->layers[0].C_in;
+    P->T_pad = pad ? encoder_pad(e) : 0;
+    if (P->T_pad) {
+        P->T_out = T;
+        for (int i = 0; i < e->n_layers; ++i)
+            P->T_out = (P->T_out - 1) / ((e->layers[i].has_dw || e->layers[i].full_conv) ? e->layers[i].stride : 1) + 1;
+        T = P->T_pad;
+    }
     size_t max_act = 0, max_res = 0;
     // Residual spans [source, layer]: the residual path's gradient waits in a pending buffer from the backward step of
     // `layer` down to that of `source`.  Spans that do not overlap share a buffer (the five blocks of the QuartzNet
@@ -872,6 +1036,11 @@ int plan_encoder(const sc_encoder_desc* e, void* base, size_t cap, EncPlan* P, c
         P->pend_tmp = need_tmp ? ws.take(max_res) : nullptr;
     }
     P->gmax_all = (float*)ws.take(sizeof(float) * e->n_layers);
+    if (P->T_pad) {
+        const LayerPlan &f = P->L[0], &l = P->L[nl - 1];
+        const size_t es = esize(f.d.io_dtype), in = es * f.m.B * f.m.Cin * f.m.T, out = es * l.m.B * l.m.Cout * l.m.Tp;
+        P->x_pad = ws.take(in); P->dx_pad = ws.take(in); P->logits_pad = ws.take(out); P->dlogits_pad = ws.take(out);
+    }
     P->bytes = ws.off + 256;
     if (!ws.ok()) return SC_ERR_WORKSPACE;
     P->scratch_mark = mark;
@@ -892,13 +1061,19 @@ sc_block_grads layer_grads(void* blob, const int64_t* off) {
     g.dwr = at(5); g.dgamma_r = at(6); g.dbeta_r = at(7);
     return g;
 }
+// one tensor in (pack) or out (unpack) of padded rows
+void copy_frames(const Launch& L, bool in, const void* src, void* dst, int C, const int* len, int B, int T, int Tq) {
+    PackList l{}; l.count = 1; l.src[0] = src; l.dst[0] = dst; l.C[0] = C; l.len[0] = len;
+    if (in) pack_frames(L, l, B, T, Tq, 1); else unpack_frames(L, l, B, T, Tq, 1);
+}
 }  // namespace
 
 int encoder_workspace_bytes(const sc_encoder_desc* desc, size_t* bytes) {
     if (!bytes) return SC_ERR_NULL;
     EncPlan P;
-    SC_TRY(plan_encoder(desc, nullptr, 0, &P, nullptr));
+    SC_TRY(plan_encoder(desc, nullptr, 0, &P, nullptr, true));
     *bytes = P.bytes;
+    if (P.T_pad) { SC_TRY(plan_encoder(desc, nullptr, 0, &P, nullptr, false)); *bytes = std::max(*bytes, P.bytes); }
     return SC_OK;
 }
 
@@ -913,14 +1088,18 @@ int encoder_infer(sc_ctx* ctx, const sc_encoder_desc* e, const sc_tensor* x, con
     if (!ctx || !lengths_dev || !params_blob || !param_offsets || !running_blob || !running_offsets) return SC_ERR_NULL;
     if (!workspace) return SC_ERR_WORKSPACE;
     EncPlan P;
-    SC_TRY(plan_encoder(e, workspace, workspace_bytes, &P, &ctx->tc));
+    SC_TRY(plan_encoder(e, workspace, workspace_bytes, &P, &ctx->tc, ctx->gemm_mode == 0));
     const int n = e->n_layers;
     const Dims& m0 = P.L[0].m; const Dims& ml = P.L[n - 1].m;
     const int dt = P.L[0].d.io_dtype;
-    SC_TRY(check_tensor(x, dt, m0.B, m0.Cin, m0.T));
-    SC_TRY(check_tensor(out, dt, ml.B, ml.Cout, ml.Tp));
+    const int T_in = e->layers[0].T_in;
+    SC_TRY(check_tensor(x, dt, m0.B, m0.Cin, T_in));
+    SC_TRY(check_tensor(out, dt, ml.B, ml.Cout, P.T_pad ? P.T_out : ml.Tp));
     Launch L{(cudaStream_t)cuda_stream, ctx->status_dev, &ctx->launches, &ctx->prof, ctx->gemm_mode, ctx->pdl};
-    auto input_of = [&](int i) -> const void* { return i == 0 ? x->ptr : P.L[i - 1].y; };
+    const void* x_in = x->ptr;
+    void* y_out = out->ptr;
+    if (P.T_pad) { copy_frames(L, true, x->ptr, P.x_pad, m0.Cin, lengths_dev, m0.B, T_in, m0.T); x_in = P.x_pad; y_out = P.logits_pad; }
+    auto input_of = [&](int i) -> const void* { return i == 0 ? x_in : P.L[i - 1].y; };
     auto res_src = [&](int i) -> int { return (e->res_from && e->res_from[i] >= 0) ? e->res_from[i] : i; };
     auto stat = [&](int i, int j) -> const float* {
         const int64_t o = running_offsets[4 * i + j];
@@ -938,13 +1117,16 @@ int encoder_infer(sc_ctx* ctx, const sc_encoder_desc* e, const sc_tensor* x, con
         BlockIO io{};
         io.x = input_of(i);
         io.xres = lp.d.residual != SC_RES_NONE ? input_of(res_src(i)) : nullptr;
-        io.y = (i + 1 < n) ? lp.y : out->ptr;
+        io.y = (i + 1 < n) ? lp.y : y_out;
+        if (i == 0) io.T_valid = T_in;
         io.len_in = i == 0 ? lengths_dev : P.L[i - 1].len_out; io.len_out = lp.len_out; io.nvalid = lp.nvalid; io.blk_off = lp.blk_off;
         io.x_clean = i > 0; io.res_clean = lp.d.residual != SC_RES_NONE && res_src(i) > 0;
         io.lengths_ready = !lp.own_lengths;
         io.w16_keep = lp.w16; io.w16_ready = false;
+        if (P.T_pad) io.x_clean = true;
         SC_TRY(block_fwd_impl(ctx, L, &lp.d, lp.m, io, &prm, &lp.sv, nullptr, nullptr, f, &inf));
     }
+    if (P.T_pad) copy_frames(L, false, P.logits_pad, out->ptr, ml.Cout, P.L[n - 1].len_out, ml.B, P.T_out, ml.Tp);
     if (out_lengths_dev)
         cudaMemcpyAsync(out_lengths_dev, P.L[n - 1].len_out, sizeof(int) * m0.B, cudaMemcpyDeviceToDevice, L.stream);
     return finish(ctx);
@@ -958,15 +1140,16 @@ int encoder_fwd_bwd(sc_ctx* ctx, const sc_encoder_desc* e, const sc_tensor* x, c
     if (!ctx || !lengths_dev || !params_blob || !param_offsets || !grads_blob || !grad_offsets) return SC_ERR_NULL;
     if (!workspace) return SC_ERR_WORKSPACE;
     EncPlan P;
-    SC_TRY(plan_encoder(e, workspace, workspace_bytes, &P, &ctx->tc));
+    SC_TRY(plan_encoder(e, workspace, workspace_bytes, &P, &ctx->tc, ctx->gemm_mode == 0));
     const int n = e->n_layers;
     const size_t mark = P.scratch_mark;
     const Dims& m0 = P.L[0].m; const Dims& ml = P.L[n - 1].m;
     const int dt = P.L[0].d.io_dtype;
-    SC_TRY(check_tensor(x, dt, m0.B, m0.Cin, m0.T));
-    SC_TRY(check_tensor(logits, dt, ml.B, ml.Cout, ml.Tp));
-    SC_TRY(check_tensor(dlogits, dt, ml.B, ml.Cout, ml.Tp));
-    if (dx) SC_TRY(check_tensor(dx, dt, m0.B, m0.Cin, m0.T));
+    const int T_in = e->layers[0].T_in, T_out = P.T_pad ? P.T_out : ml.Tp;
+    SC_TRY(check_tensor(x, dt, m0.B, m0.Cin, T_in));
+    SC_TRY(check_tensor(logits, dt, ml.B, ml.Cout, T_out));
+    SC_TRY(check_tensor(dlogits, dt, ml.B, ml.Cout, T_out));
+    if (dx) SC_TRY(check_tensor(dx, dt, m0.B, m0.Cin, T_in));
     std::vector<sc_block_params> prm(n);
     std::vector<sc_block_grads> grd(n);
     for (int i = 0; i < n; ++i) {
@@ -976,7 +1159,14 @@ int encoder_fwd_bwd(sc_ctx* ctx, const sc_encoder_desc* e, const sc_tensor* x, c
         SC_TRY(check_grads(&P.L[i].d, &grd[i]));
     }
     Launch L{(cudaStream_t)cuda_stream, ctx->status_dev, &ctx->launches, &ctx->prof, ctx->gemm_mode, ctx->pdl};
-    auto input_of = [&](int i) -> const void* { return i == 0 ? x->ptr : P.L[i - 1].y; };
+    const void *x_in = x->ptr, *dl = dlogits->ptr;
+    void *lg = logits->ptr, *dx_out = dx ? dx->ptr : nullptr;
+    if (P.T_pad) {
+        copy_frames(L, true, x->ptr, P.x_pad, m0.Cin, lengths_dev, m0.B, T_in, m0.T);
+        copy_frames(L, true, dlogits->ptr, P.dlogits_pad, ml.Cout, nullptr, ml.B, T_out, ml.Tp);
+        x_in = P.x_pad; dl = P.dlogits_pad; lg = P.logits_pad; if (dx) dx_out = P.dx_pad;
+    }
+    auto input_of = [&](int i) -> const void* { return i == 0 ? x_in : P.L[i - 1].y; };
     auto len_in_of = [&](int i) -> const int* { return i == 0 ? lengths_dev : P.L[i - 1].len_out; };
     auto res_src = [&](int i) -> int { return (e->res_from && e->res_from[i] >= 0) ? e->res_from[i] : i; };
 
@@ -1000,9 +1190,10 @@ int encoder_fwd_bwd(sc_ctx* ctx, const sc_encoder_desc* e, const sc_tensor* x, c
         BlockIO io{};
         io.x = input_of(i);
         io.xres = lp.d.residual != SC_RES_NONE ? input_of(res_src(i)) : nullptr;
-        io.y = (i + 1 < n) ? lp.y : logits->ptr;
+        io.y = (i + 1 < n) ? lp.y : lg;
         io.len_in = len_in_of(i); io.len_out = lp.len_out; io.nvalid = lp.nvalid; io.blk_off = lp.blk_off;
-        io.x_clean = i > 0; io.res_clean = lp.d.residual != SC_RES_NONE && res_src(i) > 0;
+        io.x_clean = i > 0 || P.T_pad; io.res_clean = lp.d.residual != SC_RES_NONE && res_src(i) > 0;
+        if (i == 0) io.T_valid = T_in;
         io.lengths_ready = !lp.own_lengths;
         io.w16_keep = lp.w16; io.w16_ready = true;
         SC_TRY(block_fwd_impl(ctx, L, &lp.d, lp.m, io, &prm[i], &lp.sv, nullptr, nullptr, f));
@@ -1010,8 +1201,10 @@ int encoder_fwd_bwd(sc_ctx* ctx, const sc_encoder_desc* e, const sc_tensor* x, c
     if (out_lengths_dev)
         cudaMemcpyAsync(out_lengths_dev, P.L[n - 1].len_out, sizeof(int) * m0.B, cudaMemcpyDeviceToDevice, L.stream);
 
+    if (P.T_pad) copy_frames(L, false, lg, logits->ptr, ml.Cout, P.L[n - 1].len_out, ml.B, T_out, ml.Tp);
+
     // backward
-    const void* g = dlogits->ptr;
+    const void* g = dl;
     std::vector<char> has_pending(n, 0);
     bool side_busy[kScratchRegions] = {};
     cudaEvent_t done_ev[3] = {ctx->ev[2], ctx->ev[3], ctx->ev[6]};
@@ -1024,9 +1217,9 @@ int encoder_fwd_bwd(sc_ctx* ctx, const sc_encoder_desc* e, const sc_tensor* x, c
         BwdScratch s; plan_bwd(&lp.d, lp.m, b, &s, &ctx->tc);
         BwdIO io{};
         io.done = done_ev[region]; side_busy[region] = true;
-        io.dy = g; io.x = input_of(i); io.y = (i + 1 < n) ? lp.y : logits->ptr;
+        io.dy = g; io.x = input_of(i); io.y = (i + 1 < n) ? lp.y : lg;
         io.xres = lp.d.residual != SC_RES_NONE ? input_of(res_src(i)) : nullptr;
-        io.dx = (i == 0) ? (dx ? dx->ptr : nullptr) : P.gbuf[i & 1];
+        io.dx = (i == 0) ? dx_out : P.gbuf[i & 1];
         io.dx_res = nullptr;
         const int src = res_src(i);
         const bool to_pending = lp.d.residual != SC_RES_NONE && src != i;
@@ -1034,7 +1227,7 @@ int encoder_fwd_bwd(sc_ctx* ctx, const sc_encoder_desc* e, const sc_tensor* x, c
         if (to_pending) { io.dx_res = second ? P.pend_tmp : P.pend[src]; has_pending[src] = 1; }
         io.dx_add = has_pending[i] ? P.pend[i] : nullptr;
         io.len_in = len_in_of(i); io.len_out = lp.len_out; io.nvalid = lp.nvalid; io.blk_off = lp.blk_off;
-        io.x_clean = i > 0; io.res_clean = lp.d.residual != SC_RES_NONE && res_src(i) > 0;
+        io.x_clean = i > 0 || P.T_pad; io.res_clean = lp.d.residual != SC_RES_NONE && res_src(i) > 0;
         io.w16_kept = lp.w16;
         io.gmax_zeroed = P.gmax_all + i;
         SC_TRY(block_bwd_impl(ctx, L, &lp.d, lp.m, io, &prm[i], &lp.sv, &grd[i], accumulate, s));
@@ -1042,6 +1235,7 @@ int encoder_fwd_bwd(sc_ctx* ctx, const sc_encoder_desc* e, const sc_tensor* x, c
             ew_add_masked(L, dt, P.pend[src], P.pend[src], P.pend_tmp, nullptr, len_in_of(src), P.L[src].m.B, P.L[src].m.Cin, P.L[src].m.T);
         g = io.dx;
     }
+    if (P.T_pad && dx) copy_frames(L, false, dx_out, dx->ptr, m0.Cin, lengths_dev, m0.B, T_in, m0.T);
     for (int q = 0; q < kScratchRegions; ++q) if (side_busy[q]) wait_side(ctx, L, done_ev[q]);     // join before returning
     return finish(ctx);
 }

@@ -157,6 +157,50 @@ template <> __device__ __forceinline__ void st8<__nv_bfloat16>(__nv_bfloat16* p,
     *reinterpret_cast<uint4*>(p) = r;
 }
 
+// Eight consecutive 16-bit elements that start at any element index of a 16-byte aligned dense array: two aligned
+// vectors and a funnel shift.  idx < total; elements at and beyond `total` come back unspecified.  (The second vector
+// is read only when it holds at least one element of the array, so no 16-byte line outside it is touched.)
+__device__ __forceinline__ uint4 ld8_any(const void* base, uint32_t idx, uint32_t total) {
+    const uint4* p = reinterpret_cast<const uint4*>(base) + (idx >> 3);
+    const uint32_t sh = idx & 7;
+    const uint4 lo = p[0];
+    if (sh == 0) return lo;
+    uint4 hi = make_uint4(0, 0, 0, 0);
+    if ((idx | 7u) + 1 < total) hi = p[1];
+    uint32_t w[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+    if (sh & 4) {
+#pragma unroll
+        for (int i = 0; i < 6; ++i) w[i] = w[i + 2];
+    }
+    if (sh & 2) {
+#pragma unroll
+        for (int i = 0; i < 5; ++i) w[i] = w[i + 1];
+    }
+    if (sh & 1) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) w[i] = __funnelshift_r(w[i], w[i + 1], 16);
+    }
+    return make_uint4(w[0], w[1], w[2], w[3]);
+}
+// Eight elements idx, idx + 2, ..., idx + 14 of the same kind of array.
+__device__ __forceinline__ uint4 ld8_even(const void* base, uint32_t idx, uint32_t total) {
+    const uint4 a = ld8_any(base, idx, total);
+    uint4 b = make_uint4(0, 0, 0, 0);
+    if (idx + 8 < total) b = ld8_any(base, idx + 8, total);
+    return make_uint4(__byte_perm(a.x, a.y, 0x5410), __byte_perm(a.z, a.w, 0x5410), __byte_perm(b.x, b.y, 0x5410),
+                      __byte_perm(b.z, b.w, 0x5410));
+}
+// zeroes the elements n, n + 1, ... (n < 8) of a vector of eight 16-bit elements
+__device__ __forceinline__ uint4 keep_first(const uint4& r, int n) {
+    uint32_t w[4] = {r.x, r.y, r.z, r.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        if (2 * i >= n) w[i] = 0u;
+        else if (2 * i + 1 >= n) w[i] &= 0x0000FFFFu;
+    }
+    return make_uint4(w[0], w[1], w[2], w[3]);
+}
+
 __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);

@@ -40,31 +40,47 @@ __device__ __forceinline__ void block_sum(float (&v)[N]) {
 
 __device__ __forceinline__ float block_max(float v) { return warp_max(v); }
 
-__global__ void lengths_kernel(const int* __restrict__ len_in, int B, int T_in, int stride,
-                               int* __restrict__ len_out, int* __restrict__ nvalid, int* __restrict__ blk_off,
-                               int* status) {
+// One CTA.  The block offsets are an exclusive scan over the samples: each thread sums a contiguous run of samples, the
+// runs are scanned through shared memory.  (A scan by one thread is a chain of dependent loads: 10 us at 32 samples.)
+constexpr int kLenThreads = 256;
+__global__ void __launch_bounds__(kLenThreads)
+lengths_kernel(const int* __restrict__ len_in, int B, int T_in, int stride, int phases, int* __restrict__ len_out,
+               int* __restrict__ nvalid, int* __restrict__ blk_off, int* __restrict__ len_dense, int* status) {
     pdl_sync();
-    // single CTA; B is small (<= a few thousand)
-    __shared__ int total;
-    if (threadIdx.x == 0) total = 0;
-    __syncthreads();
-    int local = 0;
-    for (int b = threadIdx.x; b < B; b += blockDim.x) {
+    __shared__ int s_frames[kLenThreads / 32], s_blocks[kLenThreads / 32];
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const int n = B * phases, per = (n + kLenThreads - 1) / kLenThreads, i0 = min(n, tid * per), i1 = min(n, i0 + per);
+    auto out_len = [&](int i) -> int {
+        const int b = i / phases, p = i - b * phases;
         int l = len_in[b];
         if (l < 1 || l > T_in) { raise_status(status, kErrLengths); l = min(max(l, 0), T_in); }
-        int lo = (l + stride - 1) / stride;
-        len_out[b] = lo;
-        local += lo;
+        if (len_dense && p == 0) len_dense[b] = l;
+        return phases > 1 ? (l - p + phases - 1) / phases : (l + stride - 1) / stride;
+    };
+    int frames = 0, blocks = 0;
+    for (int i = i0; i < i1; ++i) {
+        const int lo = out_len(i);
+        len_out[i] = lo;
+        frames += lo; blocks += (lo + 63) / 64;
     }
-    atomicAdd(&total, local);   // integer: order-independent
+    int incl = blocks;                                   // inclusive scan over the warp
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) { const int q = __shfl_up_sync(0xffffffffu, incl, o); if (lane >= o) incl += q; }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) frames += __shfl_xor_sync(0xffffffffu, frames, o);
+    if (lane == 31) s_blocks[w] = incl;
+    if (lane == 0) s_frames[w] = frames;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        *nvalid = total;
-        if (blk_off) {              // B is small: a serial scan by one thread
-            int acc = 0;
-            for (int b = 0; b < B; ++b) { blk_off[b] = acc; acc += (len_out[b] + 63) / 64; }
-            blk_off[B] = acc;
-        }
+    int base = incl - blocks;
+    for (int q = 0; q < w; ++q) base += s_blocks[q];
+    if (blk_off) {
+        for (int i = i0; i < i1; ++i) { blk_off[i] = base; base += (len_out[i] + 63) / 64; }
+        if (tid == kLenThreads - 1) blk_off[n] = base;   // the last thread's runs end the list
+    }
+    if (tid == 0) {
+        int t = 0;
+        for (int q = 0; q < kLenThreads / 32; ++q) t += s_frames[q];
+        *nvalid = t;
     }
 }
 
@@ -736,7 +752,99 @@ __global__ void __launch_bounds__(256) bn_apply_fast_kernel(ApplyArgs a, int vpr
     }
 }
 
-template <typename T, typename NT, typename GT, int RES, int V>
+// The same step from packed v / vr to dense y: a thread takes V aligned 8-element vectors of the dense tensor and gathers
+// the packed operands (for one phase a vector that starts anywhere in its row; for two, four elements of each phase).
+// A vector that runs over the end of a row is done element by element.  Blocks past the tensor's own copy u out.
+// What it replaces: four extra passes (v, vr, y and u copied to dense form one after the other) and their launches.
+template <int D>
+__device__ __forceinline__ uint32_t packed_index(const ApplyArgs& a, int b, int c, int C, int t) {
+    return D == 1 ? ((uint32_t)b * C + c) * a.Tp + t : (((uint32_t)b * 2 + (t & 1)) * C + c) * a.Tp + (t >> 1);
+}
+template <int D>
+__device__ __forceinline__ uint4 gather_packed(const ApplyArgs& a, const void* src, int b, int c, int C, int t, uint32_t total) {
+    if (D == 1) return ld8_any(src, packed_index<1>(a, b, c, C, t), total);
+    const unsigned short* s = reinterpret_cast<const unsigned short*>(src);
+    const unsigned short* e0 = s + packed_index<2>(a, b, c, C, t);
+    const unsigned short* e1 = s + packed_index<2>(a, b, c, C, t + 1);
+    uint4 r;
+    r.x = e0[0] | ((uint32_t)e1[0] << 16); r.y = e0[1] | ((uint32_t)e1[1] << 16);
+    r.z = e0[2] | ((uint32_t)e1[2] << 16); r.w = e0[3] | ((uint32_t)e1[3] << 16);
+    return r;
+}
+template <typename T, typename NT, int RES, int D>
+__global__ void __launch_bounds__(256) bn_apply_unpack_kernel(ApplyArgs a, uint32_t total, int nblk_apply, uint32_t total_u) {
+    pdl_sync();
+    const bool copy = (int)blockIdx.x >= nblk_apply;
+    const int C = copy ? a.Cu : a.C;
+    const uint32_t tot = copy ? total_u : total;
+    const uint32_t tot_packed = (uint32_t)a.B * D * C * a.Tp;
+    constexpr int V = 2;
+    const uint32_t tid = (blockIdx.x - (copy ? nblk_apply : 0)) * 256u + threadIdx.x;
+    const uint32_t base = ((tid >> 5) * (32u * V) + (threadIdx.x & 31)) * 8u;
+    uint4 rv[V], rr[V]; int ch[V], n[V]; bool whole[V];
+#pragma unroll
+    for (int j = 0; j < V; ++j) {
+        const uint32_t f = base + 256u * j;
+        whole[j] = false; n[j] = 0; ch[j] = 0;
+        rv[j] = rr[j] = make_uint4(0, 0, 0, 0);
+        if (f >= tot) continue;
+        const int row = (int)a.dT.div(f), t = (int)(f - (uint32_t)row * a.T);
+        const int b = row / C;
+        ch[j] = row - b * C;
+        if (t + 8 > a.T || f + 8 > tot) continue;
+        whole[j] = true;
+        n[j] = min(a.len_out[b], a.T) - t;
+        if (n[j] > 0) {
+            rv[j] = gather_packed<D>(a, copy ? a.u : a.v, b, ch[j], C, t, tot_packed);
+            if (!copy && RES == 1) rr[j] = *reinterpret_cast<const uint4*>((const T*)a.xres + f);
+            if (!copy && RES == 2) rr[j] = gather_packed<D>(a, a.vr, b, ch[j], C, t, tot_packed);
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < V; ++j) {
+        const uint32_t f = base + 256u * j;
+        if (f >= tot) continue;
+        if (whole[j]) {
+            if (copy) { *reinterpret_cast<uint4*>((NT*)a.u_out + f) = n[j] >= 8 ? rv[j] : keep_first(rv[j], n[j]); continue; }
+            apply_vec<T, NT, RES>(a, ch[j], n[j], f, rv[j], rr[j]);
+            if (a.v_out) *reinterpret_cast<uint4*>((NT*)a.v_out + f) = rv[j];
+            if (RES == 2 && a.vr_out) *reinterpret_cast<uint4*>((NT*)a.vr_out + f) = rr[j];
+            continue;
+        }
+        for (uint32_t e = f; e < min(f + 8, tot); ++e) {
+            const int row = (int)a.dT.div(e), t = (int)(e - (uint32_t)row * a.T);
+            const int b = row / C, o = row - b * C;
+            const bool in = t < min(a.len_out[b], a.T);
+            const uint32_t q = packed_index<D>(a, b, o, C, t);
+            if (copy) { ((unsigned short*)a.u_out)[e] = in ? ((const unsigned short*)a.u)[q] : (unsigned short)0; continue; }
+            const NT vq = in ? ((const NT*)a.v)[q] : NT(0.f);
+            float r = 0.f;
+            if (RES == 1 && in) r = ldf((const T*)a.xres + e);
+            if (RES == 2) {
+                const NT vrq = in ? ((const NT*)a.vr)[q] : NT(0.f);
+                r = fmaf(a.gamma_r[o], bn_norm(ldf(&vrq), a.mean_r[o], a.invstd_r[o]), a.beta_r[o]);
+                if (a.vr_out) ((NT*)a.vr_out)[e] = vrq;
+            }
+            const float y = fmaxf(fmaf(a.gamma[o], bn_norm(ldf(&vq), a.mean[o], a.invstd[o]), a.beta[o]) + r, 0.f);
+            stf((T*)a.y + e, in ? y : 0.f);
+            if (a.v_out) ((NT*)a.v_out)[e] = vq;
+        }
+    }
+}
+
+// Operand of the backward kernels: eight frames of packed row `row`, position t0 of it, from a tensor that has the same
+// (packed) layout (G = 0, element offset off) or is dense with one or two phases per sample (G = 1, 2).  n > 0 frames
+// are inside the sample; a dense tensor's frames past them are unspecified and come back as zero (a masked gradient times
+// a NaN would not be zero).
+template <int G>
+__device__ __forceinline__ uint4 bwd_load(const BnBwdArgs& a, const void* src, size_t off, int b, int o, int t0, int n) {
+    if (G == 0) return *reinterpret_cast<const uint4*>(reinterpret_cast<const unsigned short*>(src) + off);
+    const uint4 r = G == 1 ? ld8_any(src, ((uint32_t)b * a.C + o) * a.T + t0, a.total_dense)
+                           : ld8_even(src, ((uint32_t)(b >> 1) * a.C + o) * a.T + 2 * t0 + (b & 1), a.total_dense);
+    return n < 8 ? keep_first(r, n) : r;
+}
+
+template <typename T, typename NT, typename GT, int RES, int V, int G>
 __global__ void __launch_bounds__(256) bn_bwd_apply_fast_kernel(BnBwdArgs a, int vpr, long long total) {
     pdl_sync();
     const uint32_t tid = blockIdx.x * 256u + threadIdx.x;        // the launcher guarantees total < 2^31
@@ -757,10 +865,10 @@ __global__ void __launch_bounds__(256) bn_bwd_apply_fast_kernel(BnBwdArgs a, int
             nin[j] = max(0, min(a.len_out[b], a.Tp) - t0);        // frames of this vector inside the sample
             off[j] = (size_t)row * a.Tp + t0;
             if (nin[j] > 0) {
-                rg[j] = *reinterpret_cast<const uint4*>((const T*)a.g + off[j]);
-                rv[j] = *reinterpret_cast<const uint4*>((const NT*)a.v + off[j]);
-                if (RES == 2) rr[j] = *reinterpret_cast<const uint4*>((const NT*)a.vr + off[j]);
-                if (RES != 0) ry[j] = *reinterpret_cast<const uint4*>((const T*)a.y + off[j]);
+                rg[j] = bwd_load<G>(a, a.g, off[j], b, ch[j], t0, nin[j]);
+                rv[j] = bwd_load<G>(a, a.v, off[j], b, ch[j], t0, nin[j]);
+                if (RES == 2) rr[j] = bwd_load<G>(a, a.vr, off[j], b, ch[j], t0, nin[j]);
+                if (RES != 0) ry[j] = bwd_load<G>(a, a.y, off[j], b, ch[j], t0, nin[j]);
             }
         }
     }
@@ -846,7 +954,7 @@ constexpr int kChThreads = 512;
 
 // Backward reduction of channel o over every sample, then the channel's coefficients, parameter gradients and its
 // term of the bound on |gv| (what bn_bwd_finalize_kernel does for the row-mapped reduction).
-template <typename T, typename NT, int RES>
+template <typename T, typename NT, int RES, int G>
 __global__ void __launch_bounds__(kChThreads, 2)
 bn_bwd_reduce_ch_kernel(BnBwdArgs a, int vpr, const float* gamma_r, float* dgamma, float* dbeta, float* dgamma_r,
                         float* dbeta_r, int accumulate) {
@@ -874,10 +982,10 @@ bn_bwd_reduce_ch_kernel(BnBwdArgs a, int vpr, const float* gamma_r, float* dgamm
                 nin[u] = max(0, min(a.len_out[b], a.Tp) - t0);
                 if (nin[u] > 0) {
                     const size_t off = ((size_t)b * a.C + o) * a.Tp + t0;
-                    rg[u] = *reinterpret_cast<const uint4*>((const T*)a.g + off);
-                    rv[u] = *reinterpret_cast<const uint4*>((const NT*)a.v + off);
-                    if (RES == 2) rr[u] = *reinterpret_cast<const uint4*>((const NT*)a.vr + off);
-                    if (RES != 0) ry[u] = *reinterpret_cast<const uint4*>((const T*)a.y + off);
+                    rg[u] = bwd_load<G>(a, a.g, off, b, o, t0, nin[u]);
+                    rv[u] = bwd_load<G>(a, a.v, off, b, o, t0, nin[u]);
+                    if (RES == 2) rr[u] = bwd_load<G>(a, a.vr, off, b, o, t0, nin[u]);
+                    if (RES != 0) ry[u] = bwd_load<G>(a, a.y, off, b, o, t0, nin[u]);
                 }
             }
         }
@@ -969,9 +1077,10 @@ ew_add_masked_kernel(T* out, const T* a, const T* b, const T* c, const int* len,
         default:  { using T = __nv_bfloat16; __VA_ARGS__; break; }          \
     }
 
-void lengths(const Launch& L, const int* len_in, int B, int T_in, int stride, int* len_out, int* nvalid, int* blk_off) {
-    KScope ks_(L, KC_LENGTHS, 8.0 * B, 0.0);
-    launch_k(L, lengths_kernel, 1, 256, 0, len_in, B, T_in, stride, len_out, nvalid, blk_off, L.status);
+void lengths(const Launch& L, const int* len_in, int B, int T_in, int stride, int* len_out, int* nvalid, int* blk_off, int phases,
+             int* len_dense) {
+    KScope ks_(L, KC_LENGTHS, 8.0 * B * phases, 0.0);
+    launch_k(L, lengths_kernel, 1, kLenThreads, 0, len_in, B, T_in, stride, phases, len_out, nvalid, blk_off, len_dense, L.status);
     L.count();
 }
 
@@ -1013,7 +1122,20 @@ static bool channel_mapped(int B, int C, int Tp) { return C >= 32 && (long long)
 void bn_apply(const Launch& L, int dtype, const ApplyArgs& a_in) {
     ApplyArgs a = a_in;
     const double e = (double)dtype_size(dtype), en = (double)dtype_size(ntype_of(dtype));
-    KScope ks_(L, KC_BN_APPLY, (double)a.B * a.C * a.Tp * (en + e + (a.residual == 1 ? e : 0) + (a.residual == 2 ? en : 0)), 0.0);
+    KScope ks_(L, KC_BN_APPLY, (double)a.B * a.C * (a.phases ? a.T : a.Tp) * (en + e + (a.residual == 1 ? e : 0) + (a.residual == 2 ? en : 0)), 0.0);
+    if (a.phases) {
+        a.dT = FastDiv((uint32_t)a.T);
+        const uint32_t total = (uint32_t)a.B * a.C * a.T, total_u = a.u_out ? (uint32_t)a.B * a.Cu * a.T : 0;
+        const int nba = (int)fast_grid((total + 7) / 8, 2);
+        const unsigned grid = nba + (a.u_out ? fast_grid((total_u + 7) / 8, 2) : 0);
+#define SC_APPLY_UNPACK(RES)                                                                                                  \
+        if (a.phases == 2) { SC_DISPATCH16(dtype, (launch_k(L, bn_apply_unpack_kernel<T, NT, RES, 2>, grid, 256, 0, a, total, nba, total_u))) } \
+        else { SC_DISPATCH16(dtype, (launch_k(L, bn_apply_unpack_kernel<T, NT, RES, 1>, grid, 256, 0, a, total, nba, total_u))) }
+        if (a.residual == 0) { SC_APPLY_UNPACK(0) } else if (a.residual == 1) { SC_APPLY_UNPACK(1) } else { SC_APPLY_UNPACK(2) }
+#undef SC_APPLY_UNPACK
+        L.count();
+        return;
+    }
     if (dtype != F32 && a.Tp % 8 == 0 && a.has_relu && a.res_before_relu && fits32(a.B, a.C, a.Tp)) {
         const int vpr = a.Tp / 8;
         a.dvpr = FastDiv((uint32_t)vpr); a.dC = FastDiv((uint32_t)a.C);
@@ -1066,15 +1188,17 @@ void bn_bwd_finalize(const Launch& L, const BnBwdArgs& a, const float* gamma, co
 void bn_bwd_reduce_finalize(const Launch& L, int dtype, BnBwdArgs& a, const float* gamma, const float* gamma_r,
                             float* dgamma, float* dbeta, float* dgamma_r, float* dbeta_r, float* dbias, int accumulate) {
     const bool fast = dtype != F32 && a.Tp % 8 == 0 && a.has_bn && a.has_relu && a.res_before_relu && fits32(a.B, a.C, a.Tp);
-    if (fast && channel_mapped(a.B, a.C, a.Tp)) {
+    if (a.phases || (fast && channel_mapped(a.B, a.C, a.Tp))) {
         a.nslots = 1; a.vpw = 32; a.vpw_shift = 5;
         const double e = (double)dtype_size(dtype), en = (double)dtype_size(ntype_of(dtype));
         KScope ks_(L, KC_BN_BWD_REDUCE, (double)a.B * a.C * a.Tp * (e * (a.residual == 0 ? 1 : 2) + en * (a.residual == 2 ? 2 : 1)), 0.0);
         const int vpr = a.Tp / 8;
         a.dvpr = FastDiv((uint32_t)vpr);
-#define SC_RED_CH(RES) SC_DISPATCH16(dtype, (launch_k(L, bn_bwd_reduce_ch_kernel<T, NT, RES>, (unsigned)a.C, kChThreads, 0, a, vpr, \
-                                                       gamma_r, dgamma, dbeta, dgamma_r, dbeta_r, accumulate)))
-        if (a.residual == 2) { SC_RED_CH(2); } else if (a.residual == 1) { SC_RED_CH(1); } else { SC_RED_CH(0); }
+#define SC_RED_CH_G(RES, G) SC_DISPATCH16(dtype, (launch_k(L, bn_bwd_reduce_ch_kernel<T, NT, RES, G>, (unsigned)a.C, kChThreads, 0, a, vpr, \
+                                                          gamma_r, dgamma, dbeta, dgamma_r, dbeta_r, accumulate)))
+#define SC_RED_CH(RES) if (a.phases == 2) { SC_RED_CH_G(RES, 2) } else if (a.phases == 1) { SC_RED_CH_G(RES, 1) } else { SC_RED_CH_G(RES, 0) }
+        if (a.residual == 2) { SC_RED_CH(2) } else if (a.residual == 1) { SC_RED_CH(1) } else { SC_RED_CH(0) }
+#undef SC_RED_CH_G
 #undef SC_RED_CH
         L.count();
         return;
@@ -1093,12 +1217,14 @@ void bn_bwd_apply(const Launch& L, int dtype, const BnBwdArgs& a_in) {
         a.dvpr = FastDiv((uint32_t)vpr); a.dC = FastDiv((uint32_t)a.C);
         const long long total = (long long)a.B * a.C * vpr;
         const unsigned grid = fast_grid(total, 2);
-#define SC_BWD_FAST(RES)                                                                                             \
+#define SC_BWD_FAST_G(RES, G)                                                                                        \
         if (dtype == BF16 && a.gv_dtype == F16)                                                                      \
-            launch_k(L, bn_bwd_apply_fast_kernel<__nv_bfloat16, __half, __half, RES, 2>, grid, 256, 0, a, vpr, total); \
-        else { SC_DISPATCH16(dtype, (launch_k(L, bn_bwd_apply_fast_kernel<T, NT, T, RES, 2>, grid, 256, 0, a, vpr, total))); }
-        if (a.residual == 0) { SC_BWD_FAST(0); } else if (a.residual == 1) { SC_BWD_FAST(1); } else { SC_BWD_FAST(2); }
+            launch_k(L, bn_bwd_apply_fast_kernel<__nv_bfloat16, __half, __half, RES, 2, G>, grid, 256, 0, a, vpr, total); \
+        else { SC_DISPATCH16(dtype, (launch_k(L, bn_bwd_apply_fast_kernel<T, NT, T, RES, 2, G>, grid, 256, 0, a, vpr, total))); }
+#define SC_BWD_FAST(RES) if (a.phases == 2) { SC_BWD_FAST_G(RES, 2) } else if (a.phases == 1) { SC_BWD_FAST_G(RES, 1) } else { SC_BWD_FAST_G(RES, 0) }
+        if (a.residual == 0) { SC_BWD_FAST(0) } else if (a.residual == 1) { SC_BWD_FAST(1) } else { SC_BWD_FAST(2) }
 #undef SC_BWD_FAST
+#undef SC_BWD_FAST_G
         L.count();
         return;
     }

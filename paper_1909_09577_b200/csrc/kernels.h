@@ -88,8 +88,23 @@ template <auto Kern> inline void set_max_smem_once(int smem) {
 // len_out[b] = ceil(len_in[b]/stride); *nvalid = sum_b len_out[b]; flags lengths outside [1,T_in].
 // blk_off (nullable, int [B+1]): exclusive prefix sum of ceil(len_out[b] / 64), the number of 64-frame blocks
 // of each sample that hold at least one valid frame; blk_off[B] is their total.
+// phases > 1 (stride 1): sample b becomes `phases` samples b * phases + p that hold the frames p, p + phases, ... of it;
+// len_out and blk_off then have B * phases (+ 1) entries and len_dense (int [B]) receives the clamped lengths themselves.
 void lengths(const Launch& L, const int* len_in, int B, int T_in, int stride, int* len_out, int* nvalid,
-             int* blk_off = nullptr);
+             int* blk_off = nullptr, int phases = 1, int* len_dense = nullptr);
+
+// ---- packed tensors (k_pack.cu) ---------------------------------------------------------------
+// The tensor-core kernels move rows with 16-byte copies, so they need a row length that is a multiple of 8 frames, and
+// taps that are neighbours in memory.  A dense 16-bit [B, C, T] tensor of any T is brought into that form by packing:
+// row pitch Tq (a multiple of 8, >= ceil(T / phases)), and for taps `phases` frames apart (phases 1 or 2) sample b is
+// split into the samples b * phases + p of the frames p, p + phases, ..., on which the dilated taps are adjacent.
+// Frames at and beyond a sample's length are written as zero.
+constexpr int kMaxPack = 4;
+struct PackList { const void* src[kMaxPack]; void* dst[kMaxPack]; int C[kMaxPack]; const int* len[kMaxPack]; int count; };
+// src dense [B, C, T] -> dst packed [B * phases, C, Tq]; len[i]: valid frames [B] of the dense tensor (nullable: T)
+void pack_frames(const Launch& L, const PackList& list, int B, int T, int Tq, int phases);
+// src packed -> dst dense; values at and beyond len (nullable: T) are written as zero
+void unpack_frames(const Launch& L, const PackList& list, int B, int T, int Tq, int phases);
 
 // ---- depthwise ------------------------------------------------------------------------------
 // u[b,c,t] = sum_k wd[c,k] * x[b,c,t*s+k*dil-P] (x masked by len_in), written as 0 for t >= len_out[b];
@@ -228,6 +243,11 @@ struct ApplyArgs {
     void* y; const int* len_out;
     int B, C, Tp, has_relu, res_before_relu;
     FastDiv dvpr, dC;                              // by Tp / 8 and by C (set by bn_apply)
+    // Packed operands (phases > 0): v and vr are packed [B * phases, C, Tp] while y and xres are dense [B, C, T]; B and
+    // len_out are then the dense tensor's.  v_out / vr_out (nullable): dense copies of v and vr.  u / u_out (nullable):
+    // a packed [B * phases, Cu, Tp] tensor that the same launch copies out to dense form.
+    int phases, T; void *v_out, *vr_out; const void* u; void* u_out; int Cu;
+    FastDiv dT;
 };
 void bn_apply(const Launch& L, int dtype, const ApplyArgs& a);
 
@@ -251,6 +271,9 @@ struct BnBwdArgs {
     // bf16 (8 significand bits): multiplied by pow2_scale(*gmax), rounded with error diffusion.
     void* gv16; void* gvr16;
     FastDiv dvpr, dC;                              // by Tp / 8 and by C (set by the launchers)
+    // Packed results (phases > 0): g, y, v and vr are dense [B / phases, C, T] while everything that is written is packed
+    // [B, C, Tp] with the lengths len_out [B].
+    int phases, T; uint32_t total_dense;
 };
 void bn_bwd_reduce(const Launch& L, int dtype, BnBwdArgs& a);
 // partial slots per row that bn_bwd_reduce may use for rows of Tp frames (for scratch sizing)

@@ -1,0 +1,68 @@
+"""Blocks and encoders whose row length is not a multiple of 8 frames, or whose taps are two frames apart: these run on
+packed copies through the tensor-core kernels.  Sizes at the edges: one frame, rows shorter than a vector, a row that ends
+one frame short of or past a vector, batches on both sides of the 16-sample kernels."""
+import pytest
+import torch
+
+import synth_inputs as si
+from tests import parity_util as U
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def api():
+    import paper_1909_09577_b200 as api
+    return api
+
+
+@pytest.fixture(scope="module")
+def ctx(api):
+    c = api.Context(0)
+    yield c
+    c.close()
+
+
+CASES = [
+    # (layer kwargs, B, T, shortest length)
+    (dict(C_in=16, C_out=24, K=5, residual="proj"), 3, 9, 5),
+    (dict(C_in=64, C_out=72, K=33, residual="proj"), 17, 271, 60),
+    (dict(C_in=72, C_out=64, K=39), 16, 129, 1),
+    (dict(C_in=32, C_out=32, K=11, residual="identity"), 18, 257, 100),
+    (dict(C_in=40, C_out=136, K=15, stride=2), 5, 333, 90),
+    (dict(C_in=16, C_out=16, K=9, stride=2), 33, 136, 30),                      # T a multiple of 8, T / 2 not
+    (dict(C_in=64, C_out=48, K=1, has_dw=False), 4, 203, 50),
+    (dict(C_in=64, C_out=64, K=87, dilation=2), 17, 400, 60),
+    (dict(C_in=24, C_out=40, K=11, dilation=2, residual="proj"), 8, 161, 1),    # a length of one: an empty second phase
+    (dict(C_in=32, C_out=32, K=7, dilation=2, residual="identity"), 20, 262, 31),
+]
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f16"])
+@pytest.mark.parametrize("case", range(len(CASES)))
+def test_packed_blocks(api, ctx, dtype, case):
+    kw, B, T, lo = CASES[case]
+    L = si.LayerCfg(**kw)
+    d = si.draw(si.Workload("packed", dtype, B, T, [L], 500 + case, len_lo=lo, len_hi=T, affine="random"))
+    d.lengths[0], d.lengths[-1] = T, lo
+    rep = U.run_block(ctx, api, L, dtype, d.x, d.lengths, d.params[0], d.g)
+    print(f"\npacked case {case} {dtype}: {rep}")
+    rep.check()
+
+
+@pytest.mark.parametrize("T", [497, 500])
+def test_padded_encoder_equals_chain(api, ctx, T):
+    """A whole encoder on rows that are no multiple of 8 frames against the chain of (packed) block calls."""
+    w = si.tiny_encoder(dtype="bf16", B=18, T=T, ragged=True, width=32)
+    d = si.draw(w)
+    d.lengths[3] = T
+    reports, chain = U.run_chain(ctx, api, w, d)
+    spec = api.EncoderSpec(w.layers, w.B, w.T, w.dtype)
+    blob = spec.pack_params(d.params, "cuda")
+    logits, out_len, grads, dx = api.encoder_fwd_bwd(ctx, spec, U.dev(d.x, w.dtype), torch.from_numpy(d.lengths).cuda(), blob,
+                                                     U.dev(d.g, w.dtype), want_dx=True)
+    assert ctx.last_status() == 0
+    scale = torch.as_tensor(chain["logits"]).float().pow(2).mean().sqrt()
+    assert (logits.float() - chain["logits"].float()).abs().max() <= 0.1 * scale
+    assert logits.shape[2] == spec.T_out and (out_len.cpu().numpy() == chain["out_len"]).all()
+    assert (dx.float() - chain["dx"].float()).norm() <= 0.05 * chain["dx"].float().norm()
