@@ -39,7 +39,10 @@
  *     SC_ERR_RANGE; backward, those gradients carry a per-layer power-of-two scale chosen on the
  *     device from the gradient's magnitude, so any upstream scale (e.g. a loss scale) is safe.
  *   - Calls enqueue work on `cuda_stream` and return without synchronising.  The library never
- *     allocates or frees device memory inside these calls and keeps no pointer past the call.
+ *     allocates or frees device memory inside these calls and keeps no pointer past the call, except that a
+ *     call made for the third time with the same arguments is instantiated as a CUDA graph, which the
+ *     context keeps (at most 64; what the runtime sets aside for them is freed with the context) and
+ *     replays for further calls with those arguments.  sepconv_fwd_static never does that.
  *   - Return value: SC_OK or a negative sc_status.  Nothing throws across the boundary.  Errors
  *     that only the device can see (a length outside [1, T], a bounded wait that ran out) are
  *     written to a status word that sepconv_last_status() returns.

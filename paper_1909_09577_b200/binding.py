@@ -141,25 +141,53 @@ def _check(code: int, where: str):
         raise SepconvError(code, where)
 
 
+def _raw_stream(device: int) -> int:
+    return torch._C._cuda_getCurrentRawStream(device)      # the current stream's handle without building a Stream object
+
+
 def _stream_ptr(stream) -> int:
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return int(s.cuda_stream)
+    return int(stream.cuda_stream) if stream is not None else _raw_stream(torch.cuda.current_device())
+
+
+# A call marshals up to eight tensors, and filling an sc_tensor field by field costs about as much as enqueueing a kernel:
+# the descriptor of a dense tensor differs from that of any other of its type and shape in the address alone.
+_DTYPES = {torch.float32: SC_F32, torch.float16: SC_F16, torch.bfloat16: SC_BF16}
+_templates: Dict[tuple, bytes] = {}
+
+
+def _describe(t: torch.Tensor, tags) -> sc_tensor:
+    st = sc_tensor()
+    st.dtype = _DTYPES.get(t.dtype, -1)
+    st.rank = t.dim()
+    for i in range(min(3, t.dim())):
+        st.size[i] = t.shape[i]
+        st.stride[i] = t.stride(i)
+        st.tag[i] = tags[i]
+    return st
 
 
 def tensor_arg(t: Optional[torch.Tensor], tags=(0, 1, 2)):
     """torch [B,C,T] tensor -> sc_tensor (by reference); None -> NULL."""
     if t is None:
         return None
-    code = {torch.float32: SC_F32, torch.float16: SC_F16, torch.bfloat16: SC_BF16}.get(t.dtype, -1)
-    st = sc_tensor()
+    if tags == (0, 1, 2) and t.is_contiguous():
+        key = (t.dtype, t.shape)
+        tmpl = _templates.get(key)
+        if tmpl is None:
+            if len(_templates) >= 1024:
+                _templates.clear()
+            tmpl = _templates[key] = bytes(_describe(t, tags))
+        st = sc_tensor.from_buffer_copy(tmpl)
+    else:
+        st = _describe(t, tags)
     st.ptr = t.data_ptr()
-    st.dtype = code
-    st.rank = t.dim()
-    for i in range(min(3, t.dim())):
-        st.size[i] = t.shape[i]
-        st.stride[i] = t.stride(i)
-        st.tag[i] = tags[i]
     return C.byref(st)
+
+
+def _pointers(struct, tensors: Dict[str, torch.Tensor]):
+    """A struct of device pointers from the tensors of its field names (absent ones null)."""
+    get = tensors.get
+    return struct(*[None if (t := get(n)) is None else t.data_ptr() for n, _ in struct._fields_])
 
 
 def block_desc(L, B: int, T: int, dtype: str) -> sc_block_desc:
@@ -249,10 +277,7 @@ def _workspace(nbytes: int, device) -> torch.Tensor:
 
 
 def _params_struct(params: Dict[str, torch.Tensor]) -> sc_block_params:
-    p = sc_block_params()
-    for n in PARAM_ORDER:
-        setattr(p, n, params[n].data_ptr() if n in params and params[n] is not None else None)
-    return p
+    return _pointers(sc_block_params, params)
 
 
 def sepconv_fwd(ctx: Context, desc: sc_block_desc, x: torch.Tensor, lengths: torch.Tensor,
@@ -270,17 +295,16 @@ def sepconv_fwd(ctx: Context, desc: sc_block_desc, x: torch.Tensor, lengths: tor
         ut = torch.float16 if (desc.has_dw and desc.has_bn and desc.io_dtype != SC_F32) else td
         saved = {"u": torch.empty((B, Ci, Tp), dtype=ut, device=dev)}
         nt = torch.float32 if desc.io_dtype == SC_F32 else torch.float16   # type of the saved pointwise results
+        stats = ()                               # the saved statistics share one allocation
         if desc.has_bn:
             saved["v"] = torch.empty((B, Co, Tp), dtype=nt, device=dev)
-            saved["mean"] = torch.empty((Co,), dtype=torch.float32, device=dev)
-            saved["invstd"] = torch.empty((Co,), dtype=torch.float32, device=dev)
+            stats = ("mean", "invstd")
         if desc.residual == 2:
             saved["vr"] = torch.empty((B, Co, Tp), dtype=nt, device=dev)
-            saved["mean_r"] = torch.empty((Co,), dtype=torch.float32, device=dev)
-            saved["invstd_r"] = torch.empty((Co,), dtype=torch.float32, device=dev)
-    sv = sc_block_saved()
-    for n, _ in sc_block_saved._fields_:
-        setattr(sv, n, saved[n].data_ptr() if n in saved else None)
+            stats += ("mean_r", "invstd_r")
+        if stats:
+            saved.update(zip(stats, torch.empty((len(stats), Co), dtype=torch.float32, device=dev).unbind()))
+    sv = _pointers(sc_block_saved, saved)
     if workspace is None:
         workspace = _workspace(sepconv_workspace_bytes(desc)[0], dev)
     p = _params_struct(params)
@@ -321,9 +345,7 @@ def sepconv_fwd_static(ctx: Context, desc: sc_block_desc, x: torch.Tensor, lengt
                        saved: Dict[str, torch.Tensor], x_res: Optional[torch.Tensor] = None, stream=None):
     """sepconv_fwd for callers that cannot allocate: every buffer (y, out_lengths, saved) is passed in
     and the scratch is the library's built-in fixed array.  This wrapper allocates nothing either."""
-    sv = sc_block_saved()
-    for n, _ in sc_block_saved._fields_:
-        setattr(sv, n, saved[n].data_ptr() if n in saved else None)
+    sv = _pointers(sc_block_saved, saved)
     p = _params_struct(params)
     rc = ctx.lib.sepconv_fwd_static(ctx.h, C.byref(desc), tensor_arg(x), tensor_arg(x_res), lengths.data_ptr(),
                                     C.byref(p), tensor_arg(y), out_lengths.data_ptr(), C.byref(sv),
@@ -347,12 +369,8 @@ def sepconv_bwd(ctx: Context, desc: sc_block_desc, dy: torch.Tensor, x: torch.Te
     if grads is None:
         grads = {"d" + n: torch.zeros(params[n].shape, dtype=torch.float32, device=dev)
                  for n in PARAM_ORDER if n in params and params[n] is not None}
-    g = sc_block_grads()
-    for n, _ in sc_block_grads._fields_:
-        setattr(g, n, grads[n].data_ptr() if n in grads else None)
-    sv = sc_block_saved()
-    for n, _ in sc_block_saved._fields_:
-        setattr(sv, n, saved[n].data_ptr() if n in saved else None)
+    g = _pointers(sc_block_grads, grads)
+    sv = _pointers(sc_block_saved, saved)
     if workspace is None:
         workspace = _workspace(sepconv_workspace_bytes(desc)[1], dev)
     p = _params_struct(params)

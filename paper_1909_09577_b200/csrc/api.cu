@@ -6,7 +6,9 @@
 #include <vector>
 
 #include "../../include/sepconv.h"
+#include "api_internal.h"
 #include "common.cuh"
+#include "graph_cache.h"
 #include "kernels.h"
 #include "tc_gemm.h"
 
@@ -27,6 +29,8 @@ struct sc_ctx {
     cudaEvent_t ev[8] = {};     // backward fork, (unused), done[0], done[1], forward fork, forward join, done[2], (unused)
     int overlap = 1;
     int pdl = 1;          // launch kernels with programmatic stream serialization
+    GraphCache graphs;
+    CallKey key;
 };
 
 namespace sc {
@@ -561,6 +565,25 @@ int finish(sc_ctx* ctx) {
     return SC_OK;
 }
 
+// ---- calls through the graph cache -----------------------------------------------------------------
+enum CallTag : uint32_t { CALL_FWD = 1, CALL_BWD, CALL_INFER, CALL_ENC, CALL_ENC_INFER };
+void key_tensor(CallKey& k, const sc_tensor* t) { k.add(t, offsetof(sc_tensor, tag) + sizeof(t->tag)); }
+void key_begin(sc_ctx* ctx, CallTag tag, void* ws, size_t ws_bytes) {
+    CallKey& k = ctx->key;
+    k.reset(tag);
+    k.val(ws); k.val(ws_bytes);
+    k.val(ctx->gemm_mode); k.val(ctx->overlap); k.val(ctx->pdl); k.val(ctx->tc.flat_shape);
+}
+// The key holds every argument, so a replayed call is one that has passed validation before.  Calls that are being
+// timed launch by launch are never replayed.
+template <typename F> int run_call(sc_ctx* ctx, void* stream, F&& body) {
+    auto go = [&](cudaStream_t s) -> int {
+        return body(Launch{s, ctx->status_dev, &ctx->launches, &ctx->prof, ctx->gemm_mode, ctx->pdl});
+    };
+    if (ctx->prof.filter != -2) return go((cudaStream_t)stream);
+    return ctx->graphs.run(ctx->key, (cudaStream_t)stream, &ctx->launches, SC_ERR_CUDA, go);
+}
+
 #define SC_TRY(expr) do { int _r = (expr); if (_r != SC_OK) return _r; } while (0)
 
 }  // namespace
@@ -591,6 +614,7 @@ int sepconv_ctx_create(sc_ctx** out, int device) {
 
 void sepconv_ctx_destroy(sc_ctx* ctx) {
     if (!ctx) return;
+    ctx->graphs.clear();
     for (cudaEvent_t e : ctx->prof.events) cudaEventDestroy(e);
     for (cudaEvent_t e : ctx->ev) if (e) cudaEventDestroy(e);
     if (ctx->side) cudaStreamDestroy(ctx->side);
@@ -706,11 +730,10 @@ int sepconv_workspace_bytes(const sc_block_desc* desc, size_t* fwd, size_t* bwd)
     return SC_OK;
 }
 
-int sepconv_fwd(sc_ctx* ctx, const sc_block_desc* desc, const sc_tensor* x, const sc_tensor* x_res,
-                const int32_t* lengths_dev, const sc_block_params* params, sc_tensor* y,
-                int32_t* out_lengths_dev, sc_block_saved* saved, float* running_mean, float* running_var,
-                void* workspace, size_t workspace_bytes, void* cuda_stream) {
-    if (!ctx || !lengths_dev) return SC_ERR_NULL;
+namespace {
+int fwd_call(sc_ctx* ctx, const Launch& L, const sc_block_desc* desc, const sc_tensor* x, const sc_tensor* x_res,
+             const int32_t* lengths_dev, const sc_block_params* params, sc_tensor* y, int32_t* out_lengths_dev,
+             sc_block_saved* saved, float* running_mean, float* running_var, void* workspace, size_t workspace_bytes) {
     Dims m;
     SC_TRY(desc_dims(desc, &m));
     const int dt = desc->io_dtype;
@@ -730,7 +753,6 @@ int sepconv_fwd(sc_ctx* ctx, const sc_block_desc* desc, const sc_tensor* x, cons
     plan_fwd(desc, pk.phases ? pk.m : m, ws, &f, &ctx->tc);
     if (pk.phases) plan_fwd_pack(desc, pk, ws, &fp);
     if (!ws.ok()) return SC_ERR_WORKSPACE;
-    Launch L{(cudaStream_t)cuda_stream, ctx->status_dev, &ctx->launches, &ctx->prof, ctx->gemm_mode, ctx->pdl};
     BlockIO io{};
     io.x = x->ptr; io.xres = desc->residual != SC_RES_NONE ? (x_res ? x_res->ptr : x->ptr) : nullptr;
     io.y = y->ptr; io.len_in = lengths_dev; io.len_out = f.len_out; io.nvalid = f.nvalid; io.blk_off = f.blk_off;
@@ -741,6 +763,22 @@ int sepconv_fwd(sc_ctx* ctx, const sc_block_desc* desc, const sc_tensor* x, cons
     if (out_lengths_dev)
         cudaMemcpyAsync(out_lengths_dev, io.phases ? io.len_dense : f.len_out, sizeof(int) * m.B, cudaMemcpyDeviceToDevice, L.stream);
     return finish(ctx);
+}
+}  // namespace
+
+int sepconv_fwd(sc_ctx* ctx, const sc_block_desc* desc, const sc_tensor* x, const sc_tensor* x_res,
+                const int32_t* lengths_dev, const sc_block_params* params, sc_tensor* y,
+                int32_t* out_lengths_dev, sc_block_saved* saved, float* running_mean, float* running_var,
+                void* workspace, size_t workspace_bytes, void* cuda_stream) {
+    if (!ctx || !lengths_dev || !desc) return SC_ERR_NULL;
+    CallKey& k = ctx->key;
+    key_begin(ctx, CALL_FWD, workspace, workspace_bytes);
+    k.add(desc, sizeof(*desc)); key_tensor(k, x); key_tensor(k, x_res); k.val(lengths_dev); k.add(params, sizeof(*params));
+    key_tensor(k, y); k.val(out_lengths_dev); k.add(saved, sizeof(*saved)); k.val(running_mean); k.val(running_var);
+    return run_call(ctx, cuda_stream, [&](const Launch& L) {
+        return fwd_call(ctx, L, desc, x, x_res, lengths_dev, params, y, out_lengths_dev, saved, running_mean, running_var, workspace,
+                        workspace_bytes);
+    });
 }
 
 namespace {
@@ -770,11 +808,11 @@ int sepconv_infer_workspace_bytes(const sc_block_desc* desc, size_t* bytes) {
     return SC_OK;
 }
 
-int sepconv_infer(sc_ctx* ctx, const sc_block_desc* desc, const sc_tensor* x, const sc_tensor* x_res,
-                  const int32_t* lengths_dev, const sc_block_params* params, const float* running_mean,
-                  const float* running_var, const float* running_mean_r, const float* running_var_r, sc_tensor* y,
-                  int32_t* out_lengths_dev, void* workspace, size_t workspace_bytes, void* cuda_stream) {
-    if (!ctx || !lengths_dev) return SC_ERR_NULL;
+namespace {
+int infer_call(sc_ctx* ctx, const Launch& L, const sc_block_desc* desc, const sc_tensor* x, const sc_tensor* x_res,
+               const int32_t* lengths_dev, const sc_block_params* params, const float* running_mean,
+               const float* running_var, const float* running_mean_r, const float* running_var_r, sc_tensor* y,
+               int32_t* out_lengths_dev, void* workspace, size_t workspace_bytes) {
     Dims m;
     SC_TRY(desc_dims(desc, &m));
     const int dt = desc->io_dtype;
@@ -795,7 +833,6 @@ int sepconv_infer(sc_ctx* ctx, const sc_block_desc* desc, const sc_tensor* x, co
     plan_infer(desc, pk.phases ? pk.m : m, ws, &q, &ctx->tc);
     if (pk.phases) plan_fwd_pack(desc, pk, ws, &fp);
     if (!ws.ok()) return SC_ERR_WORKSPACE;
-    Launch L{(cudaStream_t)cuda_stream, ctx->status_dev, &ctx->launches, &ctx->prof, ctx->gemm_mode, ctx->pdl};
     BlockIO io{};
     io.x = x->ptr; io.xres = desc->residual != SC_RES_NONE ? (x_res ? x_res->ptr : x->ptr) : nullptr;
     io.y = y->ptr; io.len_in = lengths_dev; io.len_out = q.f.len_out; io.nvalid = q.f.nvalid; io.blk_off = q.f.blk_off;
@@ -806,13 +843,27 @@ int sepconv_infer(sc_ctx* ctx, const sc_block_desc* desc, const sc_tensor* x, co
         cudaMemcpyAsync(out_lengths_dev, io.phases ? io.len_dense : q.f.len_out, sizeof(int) * m.B, cudaMemcpyDeviceToDevice, L.stream);
     return finish(ctx);
 }
+}  // namespace
 
-int sepconv_bwd(sc_ctx* ctx, const sc_block_desc* desc, const sc_tensor* dy, const sc_tensor* x,
-                const sc_tensor* x_res, const sc_tensor* y, const int32_t* lengths_dev,
-                const sc_block_params* params, const sc_block_saved* saved, sc_tensor* dx,
-                sc_tensor* dx_res, const sc_tensor* dx_add, sc_block_grads* grads, int accumulate,
-                void* workspace, size_t workspace_bytes, void* cuda_stream) {
-    if (!ctx || !lengths_dev) return SC_ERR_NULL;
+int sepconv_infer(sc_ctx* ctx, const sc_block_desc* desc, const sc_tensor* x, const sc_tensor* x_res,
+                  const int32_t* lengths_dev, const sc_block_params* params, const float* running_mean,
+                  const float* running_var, const float* running_mean_r, const float* running_var_r, sc_tensor* y,
+                  int32_t* out_lengths_dev, void* workspace, size_t workspace_bytes, void* cuda_stream) {
+    if (!ctx || !lengths_dev || !desc) return SC_ERR_NULL;
+    CallKey& k = ctx->key;
+    key_begin(ctx, CALL_INFER, workspace, workspace_bytes);
+    k.add(desc, sizeof(*desc)); key_tensor(k, x); key_tensor(k, x_res); k.val(lengths_dev); k.add(params, sizeof(*params));
+    k.val(running_mean); k.val(running_var); k.val(running_mean_r); k.val(running_var_r);
+    key_tensor(k, y); k.val(out_lengths_dev);
+    return run_call(ctx, cuda_stream, [&](const Launch& L) { return infer_call(ctx, L, desc, x, x_res, lengths_dev, params, running_mean, running_var, running_mean_r,
+                          running_var_r, y, out_lengths_dev, workspace, workspace_bytes); });
+}
+
+namespace {
+int bwd_call(sc_ctx* ctx, const Launch& L, const sc_block_desc* desc, const sc_tensor* dy, const sc_tensor* x, const sc_tensor* x_res,
+             const sc_tensor* y, const int32_t* lengths_dev, const sc_block_params* params, const sc_block_saved* saved,
+             sc_tensor* dx, sc_tensor* dx_res, const sc_tensor* dx_add, sc_block_grads* grads, int accumulate,
+             void* workspace, size_t workspace_bytes) {
     Dims m;
     SC_TRY(desc_dims(desc, &m));
     const int dt = desc->io_dtype;
@@ -841,7 +892,6 @@ int sepconv_bwd(sc_ctx* ctx, const sc_block_desc* desc, const sc_tensor* dy, con
     plan_bwd(desc, mq, ws, &s, &ctx->tc);
     if (pk.phases) plan_bwd_pack(desc, pk, ws, &bp);
     if (!ws.ok()) return SC_ERR_WORKSPACE;
-    Launch L{(cudaStream_t)cuda_stream, ctx->status_dev, &ctx->launches, &ctx->prof, ctx->gemm_mode, ctx->pdl};
     const bool two = pk.phases > 1;
     lengths(L, lengths_dev, m.B, m.T, m.s, s.len_out, s.nvalid, s.blk_off, two ? pk.phases : 1, two ? bp.len_dense : nullptr);
     BwdIO io{};
@@ -885,6 +935,22 @@ int sepconv_bwd(sc_ctx* ctx, const sc_block_desc* desc, const sc_tensor* dy, con
     }
     wait_side(ctx, L, ctx->ev[2]);
     return finish(ctx);
+}
+}  // namespace
+
+int sepconv_bwd(sc_ctx* ctx, const sc_block_desc* desc, const sc_tensor* dy, const sc_tensor* x,
+                const sc_tensor* x_res, const sc_tensor* y, const int32_t* lengths_dev,
+                const sc_block_params* params, const sc_block_saved* saved, sc_tensor* dx,
+                sc_tensor* dx_res, const sc_tensor* dx_add, sc_block_grads* grads, int accumulate,
+                void* workspace, size_t workspace_bytes, void* cuda_stream) {
+    if (!ctx || !lengths_dev || !desc) return SC_ERR_NULL;
+    CallKey& k = ctx->key;
+    key_begin(ctx, CALL_BWD, workspace, workspace_bytes);
+    k.add(desc, sizeof(*desc)); key_tensor(k, dy); key_tensor(k, x); key_tensor(k, x_res); key_tensor(k, y); k.val(lengths_dev);
+    k.add(params, sizeof(*params)); k.add(saved, sizeof(*saved)); key_tensor(k, dx); key_tensor(k, dx_res); key_tensor(k, dx_add);
+    k.add(grads, sizeof(*grads)); k.val(accumulate);
+    return run_call(ctx, cuda_stream, [&](const Launch& L) { return bwd_call(ctx, L, desc, dy, x, x_res, y, lengths_dev, params, saved, dx, dx_res, dx_add,
+                        grads, accumulate, workspace, workspace_bytes); });
 }
 
 // ---- encoder ---------------------------------------------------------------------------------
@@ -1081,11 +1147,11 @@ int encoder_infer_workspace_bytes(const sc_encoder_desc* desc, size_t* bytes) {
     return encoder_workspace_bytes(desc, bytes);      // the same plan: per-layer buffers double as scratch
 }
 
-int encoder_infer(sc_ctx* ctx, const sc_encoder_desc* e, const sc_tensor* x, const int32_t* lengths_dev,
-                  const void* params_blob, const int64_t* param_offsets, const void* running_blob,
-                  const int64_t* running_offsets, sc_tensor* out, int32_t* out_lengths_dev, void* workspace,
-                  size_t workspace_bytes, void* cuda_stream) {
-    if (!ctx || !lengths_dev || !params_blob || !param_offsets || !running_blob || !running_offsets) return SC_ERR_NULL;
+namespace {
+int encoder_infer_call(sc_ctx* ctx, const Launch& L, const sc_encoder_desc* e, const sc_tensor* x, const int32_t* lengths_dev,
+                       const void* params_blob, const int64_t* param_offsets, const void* running_blob,
+                       const int64_t* running_offsets, sc_tensor* out, int32_t* out_lengths_dev, void* workspace,
+                       size_t workspace_bytes) {
     if (!workspace) return SC_ERR_WORKSPACE;
     EncPlan P;
     SC_TRY(plan_encoder(e, workspace, workspace_bytes, &P, &ctx->tc, ctx->gemm_mode == 0));
@@ -1095,7 +1161,6 @@ int encoder_infer(sc_ctx* ctx, const sc_encoder_desc* e, const sc_tensor* x, con
     const int T_in = e->layers[0].T_in;
     SC_TRY(check_tensor(x, dt, m0.B, m0.Cin, T_in));
     SC_TRY(check_tensor(out, dt, ml.B, ml.Cout, P.T_pad ? P.T_out : ml.Tp));
-    Launch L{(cudaStream_t)cuda_stream, ctx->status_dev, &ctx->launches, &ctx->prof, ctx->gemm_mode, ctx->pdl};
     const void* x_in = x->ptr;
     void* y_out = out->ptr;
     if (P.T_pad) { copy_frames(L, true, x->ptr, P.x_pad, m0.Cin, lengths_dev, m0.B, T_in, m0.T); x_in = P.x_pad; y_out = P.logits_pad; }
@@ -1131,13 +1196,29 @@ int encoder_infer(sc_ctx* ctx, const sc_encoder_desc* e, const sc_tensor* x, con
         cudaMemcpyAsync(out_lengths_dev, P.L[n - 1].len_out, sizeof(int) * m0.B, cudaMemcpyDeviceToDevice, L.stream);
     return finish(ctx);
 }
+}  // namespace
 
-int encoder_fwd_bwd(sc_ctx* ctx, const sc_encoder_desc* e, const sc_tensor* x, const int32_t* lengths_dev,
-                    const void* params_blob, const int64_t* param_offsets, const sc_tensor* dlogits,
-                    sc_tensor* logits, int32_t* out_lengths_dev, void* grads_blob,
-                    const int64_t* grad_offsets, sc_tensor* dx, int accumulate, void* workspace,
-                    size_t workspace_bytes, void* cuda_stream) {
-    if (!ctx || !lengths_dev || !params_blob || !param_offsets || !grads_blob || !grad_offsets) return SC_ERR_NULL;
+int encoder_infer(sc_ctx* ctx, const sc_encoder_desc* e, const sc_tensor* x, const int32_t* lengths_dev,
+                  const void* params_blob, const int64_t* param_offsets, const void* running_blob,
+                  const int64_t* running_offsets, sc_tensor* out, int32_t* out_lengths_dev, void* workspace,
+                  size_t workspace_bytes, void* cuda_stream) {
+    if (!ctx || !lengths_dev || !params_blob || !param_offsets || !running_blob || !running_offsets) return SC_ERR_NULL;
+    if (!e || !e->layers || e->n_layers < 1) return SC_ERR_NULL;
+    CallKey& k = ctx->key;
+    key_begin(ctx, CALL_ENC_INFER, workspace, workspace_bytes);
+    k.val(e->n_layers); k.add(e->layers, sizeof(sc_block_desc) * e->n_layers); k.add(e->res_from, e->res_from ? sizeof(int32_t) * e->n_layers : 0);
+    key_tensor(k, x); k.val(lengths_dev); k.val(params_blob); k.add(param_offsets, sizeof(int64_t) * 8 * e->n_layers);
+    k.val(running_blob); k.add(running_offsets, sizeof(int64_t) * 4 * e->n_layers); key_tensor(k, out); k.val(out_lengths_dev);
+    return run_call(ctx, cuda_stream, [&](const Launch& L) { return encoder_infer_call(ctx, L, e, x, lengths_dev, params_blob, param_offsets, running_blob,
+                                  running_offsets, out, out_lengths_dev, workspace, workspace_bytes); });
+}
+
+namespace {
+int encoder_call(sc_ctx* ctx, const Launch& L, const sc_encoder_desc* e, const sc_tensor* x, const int32_t* lengths_dev,
+                         const void* params_blob, const int64_t* param_offsets, const sc_tensor* dlogits,
+                         sc_tensor* logits, int32_t* out_lengths_dev, void* grads_blob,
+                         const int64_t* grad_offsets, sc_tensor* dx, int accumulate, void* workspace,
+                         size_t workspace_bytes) {
     if (!workspace) return SC_ERR_WORKSPACE;
     EncPlan P;
     SC_TRY(plan_encoder(e, workspace, workspace_bytes, &P, &ctx->tc, ctx->gemm_mode == 0));
@@ -1158,7 +1239,6 @@ int encoder_fwd_bwd(sc_ctx* ctx, const sc_encoder_desc* e, const sc_tensor* x, c
         SC_TRY(check_params(&P.L[i].d, &prm[i]));
         SC_TRY(check_grads(&P.L[i].d, &grd[i]));
     }
-    Launch L{(cudaStream_t)cuda_stream, ctx->status_dev, &ctx->launches, &ctx->prof, ctx->gemm_mode, ctx->pdl};
     const void *x_in = x->ptr, *dl = dlogits->ptr;
     void *lg = logits->ptr, *dx_out = dx ? dx->ptr : nullptr;
     if (P.T_pad) {
@@ -1239,5 +1319,31 @@ int encoder_fwd_bwd(sc_ctx* ctx, const sc_encoder_desc* e, const sc_tensor* x, c
     for (int q = 0; q < kScratchRegions; ++q) if (side_busy[q]) wait_side(ctx, L, done_ev[q]);     // join before returning
     return finish(ctx);
 }
+}  // namespace
+
+int encoder_fwd_bwd(sc_ctx* ctx, const sc_encoder_desc* e, const sc_tensor* x, const int32_t* lengths_dev,
+                    const void* params_blob, const int64_t* param_offsets, const sc_tensor* dlogits,
+                    sc_tensor* logits, int32_t* out_lengths_dev, void* grads_blob,
+                    const int64_t* grad_offsets, sc_tensor* dx, int accumulate, void* workspace,
+                    size_t workspace_bytes, void* cuda_stream) {
+    if (!ctx || !lengths_dev || !params_blob || !param_offsets || !grads_blob || !grad_offsets) return SC_ERR_NULL;
+    if (!e || !e->layers || e->n_layers < 1) return SC_ERR_NULL;
+    CallKey& k = ctx->key;
+    key_begin(ctx, CALL_ENC, workspace, workspace_bytes);
+    k.val(e->n_layers); k.add(e->layers, sizeof(sc_block_desc) * e->n_layers); k.add(e->res_from, e->res_from ? sizeof(int32_t) * e->n_layers : 0);
+    key_tensor(k, x); k.val(lengths_dev); k.val(params_blob); k.add(param_offsets, sizeof(int64_t) * 8 * e->n_layers);
+    key_tensor(k, dlogits); key_tensor(k, logits); k.val(out_lengths_dev); k.val(grads_blob);
+    k.add(grad_offsets, sizeof(int64_t) * 8 * e->n_layers); key_tensor(k, dx); k.val(accumulate);
+    return run_call(ctx, cuda_stream, [&](const Launch& L) { return encoder_call(ctx, L, e, x, lengths_dev, params_blob, param_offsets, dlogits, logits,
+                                    out_lengths_dev, grads_blob, grad_offsets, dx, accumulate, workspace, workspace_bytes); });
+}
 
 }  // extern "C"
+
+int sc::fwd_direct(sc_ctx* ctx, const sc_block_desc* desc, const sc_tensor* x, const sc_tensor* x_res, const int32_t* lengths_dev,
+                   const sc_block_params* params, sc_tensor* y, int32_t* out_lengths_dev, sc_block_saved* saved, void* workspace,
+                   size_t workspace_bytes, void* cuda_stream) {
+    if (!ctx || !lengths_dev) return SC_ERR_NULL;
+    return fwd_call(ctx, Launch{(cudaStream_t)cuda_stream, ctx->status_dev, &ctx->launches, &ctx->prof, ctx->gemm_mode, ctx->pdl}, desc, x,
+                    x_res, lengths_dev, params, y, out_lengths_dev, saved, nullptr, nullptr, workspace, workspace_bytes);
+}

@@ -5,7 +5,7 @@
 #include <cuda_runtime.h>
 #include <cstdio>
 
-#include "../../include/sepconv.h"
+#include "api_internal.h"
 #include "kernels.h"
 
 // One array per GPU that loads the library, held until the process exits.
@@ -54,6 +54,6 @@ extern "C" int sepconv_fwd_static(sc_ctx* ctx, const sc_block_desc* desc, const 
     // The array keeps whatever the previous call left.  Every scratch word the forward kernels read
     // they write first in the same call (lengths, frame count, statistics partials, masked copies), so
     // nothing has to start at zero and nothing is enqueued before sepconv_fwd has validated its arguments.
-    return sepconv_fwd(ctx, desc, x, x_res, lengths_dev, params, y, out_lengths_dev, saved, nullptr, nullptr,
-                       ws, (size_t)SEPCONV_STATIC_SCRATCH_BYTES, cuda_stream);
+    return sc::fwd_direct(ctx, desc, x, x_res, lengths_dev, params, y, out_lengths_dev, saved, ws,
+                          (size_t)SEPCONV_STATIC_SCRATCH_BYTES, cuda_stream);
 }
