@@ -91,9 +91,10 @@ int desc_dims(const sc_block_desc* d, Dims* o) {
 struct Packed { int phases = 0, Tq = 0; Dims m; };     // m: the block on the packed operands
 Packed plan_packed(const sc_block_desc* d, const Dims& m) {
     Packed k;
-    if (d->io_dtype == SC_F32 || m.full || !d->has_bn || !d->has_relu || !d->res_before_relu) return k;
-    const bool dilated = m.dil == 2 && (m.K & 1) && m.s == 1;
-    if (m.dil != 1 && !dilated) return k;
+    if (d->io_dtype == SC_F32 || !d->has_bn || !d->has_relu || !d->res_before_relu) return k;
+    if (m.full && (m.s != 1 || m.Cout % 8)) return k;       // the non-separable convolution takes any dilation as it is
+    const bool dilated = !m.full && m.dil == 2 && (m.K & 1) && m.s == 1;
+    if (m.dil != 1 && !dilated && !m.full) return k;
     if (!dilated && m.T % 8 == 0 && m.Tp % 8 == 0) return k;
     if (m.Cin % 8 || (d->residual == SC_RES_PROJ && m.Cres % 8)) return k;
     const int ph = dilated ? 2 : 1;
@@ -101,7 +102,7 @@ Packed plan_packed(const sc_block_desc* d, const Dims& m) {
     const long long most = (long long)m.B * ph * std::max(std::max(m.Cin, m.Cout), m.Cres) * Tq;
     if (most >= (1ll << 31)) return k;                      // the copies index with 32 bits
     k.phases = ph; k.Tq = Tq; k.m = m;
-    k.m.B = m.B * ph; k.m.T = Tq; k.m.Tp = Tq / m.s; k.m.dil = 1; k.m.plain = (m.K & 1) != 0;
+    k.m.B = m.B * ph; k.m.T = Tq; k.m.Tp = Tq / m.s; if (dilated) k.m.dil = 1; k.m.plain = (m.K & 1) != 0;
     return k;
 }
 
@@ -141,7 +142,11 @@ struct BlockIO {                 // raw pointers after validation
 int op_dtype(const sc_block_desc* d) { return otype_of(d->io_dtype, d->has_dw && d->has_bn); }
 
 // ---- forward scratch ---------------------------------------------------------------------------
-struct FwdScratch { void* partials; void* partials_r; void *xr, *w16; float* zf32; int* len_out; int* nvalid; int* blk_off; };
+struct FwdScratch { void* partials; void* partials_r; void *xr, *w16, *x_tm, *taps; float* zf32; int* len_out; int* nvalid; int* blk_off; };
+
+bool conv_on_tc(const TcState* tc, const sc_block_desc* d, const Dims& m) {
+    return m.full && tc_conv_supported(tc, d->io_dtype, m.B, m.Cin, m.Cout, m.T, m.s);
+}
 
 void plan_fwd(const sc_block_desc* d, const Dims& m, Bump& ws, FwdScratch* f, const TcState* tc) {
     f->len_out = (int*)ws.take(sizeof(int) * m.B);
@@ -151,7 +156,23 @@ void plan_fwd(const sc_block_desc* d, const Dims& m, Bump& ws, FwdScratch* f, co
     f->partials_r = (d->residual == SC_RES_PROJ) ? ws.take(tc_stats_bytes(m.B, m.Cout, m.Tp)) : nullptr;
     f->zf32 = d->log_softmax ? (float*)ws.take(sizeof(float) * m.B * m.Cout * m.Tp) : nullptr;
     f->xr = (d->residual == SC_RES_PROJ) ? ws.take(esize(d->io_dtype) * m.B * m.Cres * m.Tp) : nullptr;
+    const bool conv = conv_on_tc(tc, d, m);
+    f->x_tm = conv ? ws.take((size_t)2 * m.B * m.Cin * m.T) : nullptr;
+    f->taps = conv ? ws.take((size_t)2 * m.Cin * m.Cout * m.K) : nullptr;
     f->w16 = (op_dtype(d) != d->io_dtype) ? ws.take((size_t)2 * m.Cout * m.Cin) : nullptr;
+}
+
+// Batch statistics of v from what the contraction left behind (or from v itself).
+void finalize_stats(const Launch& L, const sc_block_desc* d, const Dims& m, StatsLayout sl, const void* v, int vdt, const int* len_out,
+                    const int* nvalid, const int* blk_off, void* partials, float* mean, float* invstd, float* rmean, float* rvar) {
+    if (sl.kind == 2) {
+        bn_finalize_flat(L, (const float4*)partials, sl.grid, sl.tiles_m, sl.rows_per_tile, blk_off, nvalid, m.B, m.Cout,
+                         d->bn_eps, d->bn_momentum, mean, invstd, rmean, rvar);
+        return;
+    }
+    if (sl.kind == 0) { bn_stats(L, vdt, v, len_out, m.B, m.Cout, m.Tp, (float2*)partials); sl.parts_per_b = 1; sl.tile_w = m.Tp; }
+    bn_finalize(L, (const float2*)partials, sl.parts_per_b, sl.tile_w, len_out, nvalid, m.B, m.Cout, d->bn_eps, d->bn_momentum,
+                mean, invstd, rmean, rvar);
 }
 
 // v = w * u for every sample (stored once, in the type it is kept in for the backward pass), plus masked
@@ -165,14 +186,7 @@ void pointwise_bn(sc_ctx* ctx, const Launch& L, const sc_block_desc* d, const Di
         tc_gemm_fwd(&ctx->tc, L, opdt, w, u, nullptr, v, vdt, len_out, blk_off, m.B, Cin, m.Cout, m.Tp, partials, &sl);
     else
         gemm_fwd_simt(L, opdt, w, u, nullptr, v, vdt, len_out, m.B, Cin, m.Cout, m.Tp);
-    if (sl.kind == 2) {
-        bn_finalize_flat(L, (const float4*)partials, sl.grid, sl.tiles_m, sl.rows_per_tile, blk_off, nvalid, m.B, m.Cout,
-                         d->bn_eps, d->bn_momentum, mean, invstd, rmean, rvar);
-        return;
-    }
-    if (sl.kind == 0) { bn_stats(L, vdt, v, len_out, m.B, m.Cout, m.Tp, (float2*)partials); sl.parts_per_b = 1; sl.tile_w = m.Tp; }
-    bn_finalize(L, (const float2*)partials, sl.parts_per_b, sl.tile_w, len_out, nvalid, m.B, m.Cout, d->bn_eps, d->bn_momentum,
-                mean, invstd, rmean, rvar);
+    finalize_stats(L, d, m, sl, v, vdt, len_out, nvalid, blk_off, partials, mean, invstd, rmean, rvar);
 }
 
 // The launch context of the side stream (same status word, counters and profile), or L itself when overlap is off.
@@ -224,20 +238,22 @@ int block_fwd_impl(sc_ctx* ctx, const Launch& L, const sc_block_desc* d, const D
     }
     if (m.full) {
         // block variant: one K-tap convolution over all input channels (it masks its input by len_in itself)
-        if (!d->has_bn) {
-            conv_fwd_simt(L, dt, p->wp, io.x, d->has_bias ? p->bias : nullptr, io.y, dt, io.len_in, io.len_out, m.B, m.Cin, m.Cout,
-                          m.T, m.Tp, m.K, m.s, m.dil);
-            return SC_OK;
-        }
-        const int vdt = ntype_of(dt);
-        conv_fwd_simt(L, dt, p->wp, io.x, nullptr, sv->v, vdt, io.len_in, io.len_out, m.B, m.Cin, m.Cout, m.T, m.Tp, m.K, m.s, m.dil);
-        if (inf) {
-            invstd_from_var(L, inf->var, d->bn_eps, sv->invstd, m.Cout);
+        const int vdt = d->has_bn ? ntype_of(dt) : dt;
+        void* v = d->has_bn ? sv->v : io.y;
+        const float* bias = !d->has_bn && d->has_bias ? p->bias : nullptr;
+        const bool stats = d->has_bn && !inf;
+        StatsLayout sl;
+        if (ctx->gemm_mode == 0 && conv_on_tc(&ctx->tc, d, m)) {
+            to_time_major(L, io.x, f.x_tm, io.len_in, m.B, m.Cin, m.T);
+            split_taps(L, p->wp, f.taps, m.Cout, m.Cin, m.K, 0);
+            tc_conv_fwd(&ctx->tc, L, dt, f.taps, f.x_tm, bias, v, vdt, io.len_out, io.blk_off, m.B, m.Cin, m.Cout, m.T, m.K, m.dil,
+                        stats ? f.partials : nullptr, stats ? &sl : nullptr);
         } else {
-            bn_stats(L, vdt, sv->v, io.len_out, m.B, m.Cout, m.Tp, (float2*)f.partials);
-            bn_finalize(L, (const float2*)f.partials, 1, m.Tp, io.len_out, io.nvalid, m.B, m.Cout, d->bn_eps, d->bn_momentum, sv->mean,
-                        sv->invstd, rmean, rvar);
+            conv_fwd_simt(L, dt, p->wp, io.x, bias, v, vdt, io.len_in, io.len_out, m.B, m.Cin, m.Cout, m.T, m.Tp, m.K, m.s, m.dil);
         }
+        if (!d->has_bn) return SC_OK;
+        if (stats) finalize_stats(L, d, m, sl, v, vdt, io.len_out, io.nvalid, io.blk_off, f.partials, sv->mean, sv->invstd, rmean, rvar);
+        else invstd_from_var(L, inf->var, d->bn_eps, sv->invstd, m.Cout);
     }
     const void* u = nullptr;
     if (m.full) {
@@ -288,7 +304,7 @@ int block_fwd_impl(sc_ctx* ctx, const Launch& L, const sc_block_desc* d, const D
     }
     if (io.phases) {
         a.phases = io.phases; a.B = m.B / io.phases; a.T = io.Td; a.len_out = io.len_dense;
-        a.v_out = io.dense.v; a.vr_out = io.dense.vr; a.u = u; a.u_out = io.dense.u; a.Cu = m.Cin;
+        a.v_out = io.dense.v; a.vr_out = io.dense.vr; a.u = u; a.u_out = u ? io.dense.u : nullptr; a.Cu = m.Cin;
     }
     bn_apply(L, dt, a);
     return SC_OK;
@@ -335,6 +351,7 @@ struct BwdScratch {
     float4 *partials, *coef, *coef_r;
     float *amax_part, *gmax;
     void *gv, *gvr, *gres, *gu, *gxr, *xr, *w16, *dz;
+    void *x_tm, *gv_tm, *taps;           // operand copies of the non-separable convolution's tensor-core form
     void *gv16, *gvr16, *x16, *xr16;     // half copies for the weight gradients of bf16 layers (see block_bwd_impl)
     float* wpart; size_t wpart_bytes;
 };
@@ -369,6 +386,11 @@ void plan_bwd(const sc_block_desc* d, const Dims& m, Bump& ws, BwdScratch* s, co
     wb = std::max(wb, tc_wgrad_scratch_bytes(tc, std::max(m.Cin, m.Cres), m.Cout));
     wb = std::max(wb, dw_wgrad_scratch_bytes(m.B, m.Cin, m.K));
     if (m.full) wb = std::max(wb, conv_wgrad_scratch_bytes(m.B, m.Cin, m.Cout, m.K));
+    const bool conv = conv_on_tc(tc, d, m);
+    if (conv) wb = std::max(wb, tc_conv_wgrad_scratch_bytes(m.B, m.Cin, m.Cout, m.T, m.K));
+    s->x_tm = conv ? ws.take((size_t)2 * m.B * m.Cin * m.T) : nullptr;
+    s->gv_tm = conv ? ws.take((size_t)2 * m.B * m.Cout * m.T) : nullptr;
+    s->taps = conv ? ws.take((size_t)2 * m.Cin * m.Cout * m.K) : nullptr;
     s->wpart = (float*)ws.take(wb);
     s->wpart_bytes = wb;
 }
@@ -440,6 +462,8 @@ int block_bwd_impl(sc_ctx* ctx, const Launch& L, const sc_block_desc* d, const D
     bn_bwd_reduce_finalize(L, dt, a, p->gamma, p->gamma_r, g->dgamma, g->dbeta, g->dgamma_r, g->dbeta_r,
                            d->has_bias ? g->dbias : nullptr, acc);
     bn_bwd_apply(L, dt, a);
+    const bool conv_tc = tc_ok && conv_on_tc(&ctx->tc, d, m);
+    if (conv_tc) to_time_major(L, s.gv, s.gv_tm, io.len_out, m.B, m.Cout, m.T);
 
     // The weight gradients are off the critical path (nothing later in the backward pass reads them): they run on the
     // side stream.  They are enqueued after the input-gradient kernels of this stream: the host issues launches in
@@ -451,7 +475,10 @@ int block_bwd_impl(sc_ctx* ctx, const Launch& L, const sc_block_desc* d, const D
     auto weight_gradients = [&]() {
         fork_to_side(ctx, L, ctx->ev[0]);               // gv, gvr, gu and the half copies are complete
         const void* u = d->has_dw ? sv->u : (io.x_clean ? io.x : sv->u);
-        if (m.full) {
+        if (conv_tc) {
+            to_time_major(Ls, io.x, s.x_tm, io.len_in, m.B, m.Cin, m.T);
+            tc_conv_wgrad(&ctx->tc, Ls, dt, s.gv_tm, s.x_tm, g->dwp, s.wpart, acc, io.len_out, m.B, m.Cin, m.Cout, m.T, m.K, m.dil);
+        } else if (m.full) {
             conv_wgrad_simt(Ls, dt, s.gv, io.x, g->dwp, s.wpart, acc, io.len_in, io.len_out, m.B, m.Cin, m.Cout, m.T, m.Tp, m.K, m.s, m.dil);
         } else if (half_gv) {
             mask_convert_f16(Ls, s.x16, io.x, io.len_in, m.B, m.Cin, m.T);
@@ -496,7 +523,12 @@ int block_bwd_impl(sc_ctx* ctx, const Launch& L, const sc_block_desc* d, const D
     if (m.full) {
         if (io.dx) {
             void* tgt = (!io.dx_add && !extra) ? io.dx : s.gu;
-            conv_dgrad_simt(L, dt, p->wp, s.gv, tgt, io.len_in, io.len_out, m.B, m.Cin, m.Cout, m.T, m.Tp, m.K, m.s, m.dil);
+            if (conv_tc) {
+                split_taps(L, p->wp, s.taps, m.Cout, m.Cin, m.K, 1);
+                tc_conv_dgrad(&ctx->tc, L, dt, s.taps, s.gv_tm, tgt, io.len_in, io.blk_off, m.B, m.Cin, m.Cout, m.T, m.K, m.dil);
+            } else {
+                conv_dgrad_simt(L, dt, p->wp, s.gv, tgt, io.len_in, io.len_out, m.B, m.Cin, m.Cout, m.T, m.Tp, m.K, m.s, m.dil);
+            }
             if (tgt != io.dx) ew_add_masked(L, dt, io.dx, s.gu, io.dx_add, extra, io.len_in, m.B, m.Cin, m.T);
         }
     } else if (d->has_dw) {

@@ -183,6 +183,13 @@ size_t conv_wgrad_scratch_bytes(int B, int Cin, int Cout, int K);
 void conv_wgrad_simt(const Launch& L, int dtype, const void* gv, const void* x, float* dw, float* partials, int accumulate,
                      const int* len_in, const int* len_out, int B, int Cin, int Cout, int T, int Tp, int K, int stride, int dil);
 
+// Operand copies of its tensor-core form (k_conv_tc.cu), 16-bit: in [B, C, T] -> out [B, T, C], zero from len[b] on (C and T
+// multiples of 8); w [C_out, C_in, K] -> [K][C_out][C_in], or [K][C_in][C_out] with swap; out[n, K] (+)= the sum of
+// partials [nsplit][K][n].
+void to_time_major(const Launch& L, const void* in, void* out, const int* len, int B, int C, int T);
+void split_taps(const Launch& L, const void* w, void* out, int Cout, int Cin, int K, int swap);
+void conv_reduce_taps(const Launch& L, const float* partials, int nsplit, int n, int K, float* out, int accumulate);
+
 // ---- batch norm -----------------------------------------------------------------------------
 // Per-(b,channel) row moments over t < len_out[b]: partials[(b*C+o)] = (sum, M2 about the row mean).
 void bn_stats(const Launch& L, int vdtype, const void* v, const int* len_out, int B, int C, int Tp,

@@ -27,7 +27,14 @@
 namespace sc {
 namespace {
 
-enum { MODE_FWD = 0, MODE_DGRAD = 1, MODE_WGRAD = 2 };
+// The CONV modes are the same contractions of the non-separable convolution, with the tap as an outer part of the
+// contraction index (forward, input gradient) or of the output (weight gradient).  Their activations are time-major
+// [B, T, C], so that a tap's shift is a shift of the row coordinate, which a TMA copy may take anywhere (the innermost
+// coordinate must stay on 16-byte boundaries); rows outside [0, T) are zero-filled, which is the "same" padding.
+enum { MODE_FWD = 0, MODE_DGRAD = 1, MODE_WGRAD = 2, MODE_CONV_FWD = 3, MODE_CONV_DGRAD = 4, MODE_CONV_WGRAD = 5 };
+__host__ __device__ constexpr bool is_fwd(int m) { return m == MODE_FWD || m == MODE_CONV_FWD; }
+__host__ __device__ constexpr bool is_conv(int m) { return m >= MODE_CONV_FWD; }
+__host__ __device__ constexpr bool is_wgrad(int m) { return m == MODE_WGRAD || m == MODE_CONV_WGRAD; }
 constexpr int BK = 64;            // contraction elements per stage (one 128-byte swizzle row)
 constexpr int kThreads = 128;
 
@@ -41,6 +48,7 @@ struct TcParams {
     int out_kind;   // forward: type of the result tensor: 0 = the operand type, 1 = float32, 2 = float16
     int nkb_t;      // weight gradient: 64-frame blocks per sample
     int kb_per_split, nkb_total;
+    int nsplit, tap_row0, tap_step;   // convolution weight gradient: z = tap * nsplit + slice; x row = frame + tap_row0 + tap * tap_step
 };
 
 template <typename T> struct Fmt;
@@ -106,7 +114,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
     constexpr int STAGE = A_BYTES + B_BYTES;
     constexpr uint32_t TMEM_COLS = MT * BN;
     static_assert(TMEM_COLS == 64 || TMEM_COLS == 128 || TMEM_COLS == 256 || TMEM_COLS == 512, "tmem columns");
-    constexpr uint32_t IDESC = ptx::instr_desc(Fmt<T>::v, MODE == MODE_DGRAD ? 1u : 0u, MODE == MODE_WGRAD ? 0u : 1u, 128, BN);
+    constexpr uint32_t IDESC = ptx::instr_desc(Fmt<T>::v, (MODE == MODE_DGRAD || MODE == MODE_CONV_WGRAD) ? 1u : 0u, MODE == MODE_WGRAD ? 0u : 1u, 128, BN);
 
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
@@ -119,10 +127,12 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int n0 = blockIdx.x * BN;
     const int m0 = blockIdx.y * (128 * MT);
-    const int z = blockIdx.z;                      // sample (forward / input gradient) or k-split (weight gradient)
+    const int z = MODE == MODE_CONV_WGRAD ? blockIdx.z % p.nsplit : blockIdx.z;    // sample, or k-split (weight gradients)
+    const int tap = MODE == MODE_CONV_WGRAD ? blockIdx.z / p.nsplit : 0;
+    const int tap_row = p.tap_row0 + tap * p.tap_step;
 
     int len = p.Tp;
-    if (MODE != MODE_WGRAD) {
+    if (!is_wgrad(MODE)) {
         if (p.len_out) len = min(p.len_out[z], p.Tp);
         if (n0 >= len) {                           // whole tile in padding
             if (p.zero_fill) {
@@ -155,10 +165,10 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
 
     // k-block range of this CTA
     int kb_begin = 0, kb_end = (p.Kdim + BK - 1) / BK;
-    if (MODE == MODE_WGRAD) { kb_begin = z * p.kb_per_split; kb_end = min(p.nkb_total, kb_begin + p.kb_per_split); }
+    if (is_wgrad(MODE)) { kb_begin = z * p.kb_per_split; kb_end = min(p.nkb_total, kb_begin + p.kb_per_split); }
     // weight gradient: blocks that start in a sample's padding are skipped (by every role alike)
     auto kb_valid = [&](int kb, int& b, int& t0) -> bool {
-        if (MODE != MODE_WGRAD) return true;
+        if (!is_wgrad(MODE)) return true;
         b = kb / p.nkb_t; t0 = (kb % p.nkb_t) * BK;
         const int l = p.len_out ? min(p.len_out[b], p.Tp) : p.Tp;
         return t0 < l;
@@ -189,10 +199,15 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
                             ptx::tma_load_2d(sA + mt * 16384 + j * 8192, &mapA, &full[s], m0 + mt * 128 + 64 * j, k0);
 #pragma unroll
                     for (int j = 0; j < BN / 64; ++j) ptx::tma_load_3d(sB + j * 8192, &mapB, &full[s], n0 + 64 * j, k0, z);
-                } else {
+                } else if (MODE == MODE_WGRAD) {
 #pragma unroll
                     for (int mt = 0; mt < MT; ++mt) ptx::tma_load_3d(sA + mt * 16384, &mapA, &full[s], t0, m0 + mt * 128, b);
                     ptx::tma_load_3d(sB, &mapB, &full[s], t0, n0, b);
+                } else {
+#pragma unroll
+                    for (int j = 0; j < 2 * MT; ++j) ptx::tma_load_3d(sA + j * 8192, &mapA, &full[s], m0 + 64 * j, t0, b);
+#pragma unroll
+                    for (int j = 0; j < BN / 64; ++j) ptx::tma_load_3d(sB + j * 8192, &mapB, &full[s], n0 + 64 * j, t0 + tap_row, b);
                 }
                 ++it;
             }
@@ -214,7 +229,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
                                                                 : ptx::smem_desc(aB + ks * 2048, 8192, 1024);
 #pragma unroll
                     for (int mt = 0; mt < MT; ++mt) {
-                        const uint64_t adesc = (MODE == MODE_DGRAD) ? ptx::smem_desc(aA + mt * 16384 + ks * 2048, 8192, 1024)
+                        const uint64_t adesc = (MODE == MODE_DGRAD || MODE == MODE_CONV_WGRAD) ? ptx::smem_desc(aA + mt * 16384 + ks * 2048, 8192, 1024)
                                                                     : ptx::smem_desc(aA + mt * 16384 + ks * 32, 16, 1024);
                         ptx::mma_f16(tmem + mt * BN, adesc, bdesc, IDESC, (it > 0 || ks > 0) ? 1u : 0u);
                     }
@@ -229,7 +244,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
 
     // did this CTA accumulate anything? (weight gradient with every block in padding: no)
     bool any = true;
-    if (MODE == MODE_WGRAD) {
+    if (is_wgrad(MODE)) {
         any = false;
         for (int kb = kb_begin; kb < kb_end && !any; ++kb) { int b, t0; any = kb_valid(kb, b, t0); }
     }
@@ -276,10 +291,12 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
                 }
                 {
                     const int row_w = m0 + mt * 128 + warp * 32;             // first row of this warp's block
-                    const size_t base = ((size_t)z * p.M + row_w) * p.Ncols + n0 + c0;
+                    // weight gradients: one [M, Ncols] matrix per (slice, tap)
+                    const size_t zz = MODE == MODE_CONV_WGRAD ? (size_t)z * (gridDim.z / p.nsplit) + tap : (size_t)z;
+                    const size_t base = (zz * p.M + row_w) * p.Ncols + n0 + c0;
                     float* stg = stg_all + warp * kStgFloatsPerWarp;
                     const int rl = p.M - row_w, cl = p.Ncols - (n0 + c0);
-                    if ((MODE == MODE_FWD && p.out_kind == 1) || MODE == MODE_WGRAD)
+                    if ((MODE == MODE_FWD && p.out_kind == 1) || is_wgrad(MODE))
                         store_block_staged<float>(stg, f, reinterpret_cast<float*>(p.out) + base, p.Ncols, rl, cl, lane);
                     else if (MODE == MODE_FWD && p.out_kind == 2)
                         store_block_staged<__half>(stg, f, reinterpret_cast<__half*>(p.out) + base, p.Ncols, rl, cl, lane);
@@ -530,6 +547,8 @@ struct FlatParams {
     int B, Tp, nbT; // nbT = ceil(Tp / 64)
     int tiles_m;
     int zero_fill;  // blocks wholly in padding must be written as zeros
+    int tap_row0, tap_step, tap_blocks;    // CONV modes: operand row = frame + tap_row0 + tap * tap_step; 64-channel blocks per tap
+    int ntaps;
     int out_half;   // the result is float16 although the operands are bfloat16
     int out_f32;    // the result is float32 (one M sub-tile per CTA only: narrow heads such as the class scores)
     int tma_out;    // 16-bit result leaves through TMA stores (third tensor map: 32 frames x 32 rows, 64-byte swizzle)
@@ -606,7 +625,7 @@ __device__ __forceinline__ bool flat_next_tile(uint32_t& pos, uint32_t end, uint
 template <int MT, int NB, int OCC, int EPI = 1> struct FlatCfg {
     static constexpr int A_BYTES = MT * 128 * 128;
     static constexpr int STAGE = A_BYTES + NB * 8192;
-    static constexpr int STAGES = OCC == 2 ? 2 : (STAGE <= 49152 ? 4 : 3);
+    static constexpr int STAGES = OCC == 2 ? 2 : (STAGE <= 32768 ? 6 : (STAGE <= 49152 ? 4 : 3));
     // per-warp staging: 32 x 32 16-bit values, or (one M sub-tile, one CTA per SM only) 32 x 32 floats for a float32 result
     static constexpr int STG = EPI >= 2 ? 2048 : ((MT == 1 && OCC == 1) ? kStgFloatsPerWarp * 4 : kOutStageBytes);
     static constexpr int MAXB = (OCC == 2 || EPI >= 2) ? 256 : kFlatMaxB;
@@ -618,7 +637,7 @@ __global__ void __launch_bounds__(32 * (4 * MT * EPI + 2), OCC)
 tc_gemm_flat_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
                     const __grid_constant__ CUtensorMap mapO, FlatParams p) {
     pdl_launch_dependents();
-    static_assert(MODE == MODE_FWD || MODE == MODE_DGRAD, "forward / input gradient only");
+    static_assert(!is_wgrad(MODE), "forward / input gradient only");
     constexpr int A_BYTES = FlatCfg<MT, NB, OCC, EPI>::A_BYTES;
     constexpr int STAGE = FlatCfg<MT, NB, OCC, EPI>::STAGE;
     constexpr int STAGES = FlatCfg<MT, NB, OCC, EPI>::STAGES;
@@ -658,7 +677,7 @@ tc_gemm_flat_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
     __syncthreads();
     ptx::tc_fence_after();
     const uint32_t tmem = *tmem_slot;
-    const int nkb = (p.Kdim + BK - 1) / BK;
+    const int nkb = is_conv(MODE) ? p.ntaps * p.tap_blocks : (p.Kdim + BK - 1) / BK;
     const int nblk = s_off[p.B];
     // 32-bit arithmetic throughout (the launcher bounds the unit count): 64-bit divisions in front of the first copy
     // cost every CTA about a microsecond.  floor(U * c / G) = (U / G) * c + ((U % G) * c) / G, every product below 2^32
@@ -683,6 +702,7 @@ tc_gemm_flat_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
                     } else { bb[i] = 0; tt[i] = 0; }
                 }
                 const int m0 = m * (128 * MT);
+                int tap = 0, cb = 0;
                 for (int kb = 0; kb < nkb; ++kb, ++it) {
                     const int s = it % STAGES, ph = (it / STAGES) & 1;
                     if (!ptx::mbar_wait(&empty[s], ph ^ 1)) { raise_status(p.status, kErrTimeout); dead = true; break; }
@@ -690,6 +710,16 @@ tc_gemm_flat_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
                     uint8_t* sA = smem + s * STAGE;
                     uint8_t* sB = sA + A_BYTES;
                     const int k0 = kb * BK;
+                    if (is_conv(MODE)) {
+                        const int c0 = cb * BK, dt = p.tap_row0 + tap * p.tap_step;
+#pragma unroll
+                        for (int mt = 0; mt < MT; ++mt) ptx::tma_load_3d(sA + mt * 16384, &mapA, &full[s], c0, m0 + mt * 128, tap);
+#pragma unroll
+                        for (int i = 0; i < NB; ++i)
+                            if (i < nb) ptx::tma_load_3d(sB + i * 8192, &mapB, &full[s], c0, tt[i] + dt, bb[i]);
+                        if (++cb == p.tap_blocks) { cb = 0; ++tap; }
+                        continue;
+                    }
                     if (MODE == MODE_FWD) {
 #pragma unroll
                         for (int mt = 0; mt < MT; ++mt) ptx::tma_load_2d(sA + mt * 16384, &mapA, &full[s], k0, m0 + mt * 128);
@@ -724,7 +754,7 @@ tc_gemm_flat_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
                 }
                 if (!whole_later && !ptx::mbar_wait(&acc_empty[buf], par_prev)) { raise_status(p.status, kErrTimeout); break; }
                 ptx::tc_fence_after();
-                const uint32_t idesc = ptx::instr_desc(Fmt<T>::v, MODE == MODE_DGRAD ? 1u : 0u, 1u, 128, 64u * nb);
+                const uint32_t idesc = ptx::instr_desc(Fmt<T>::v, MODE == MODE_DGRAD ? 1u : 0u, is_conv(MODE) ? 0u : 1u, 128, 64u * nb);
                 for (int kb = 0; kb < nkb; ++kb, ++it) {
                     const int s = it % STAGES, ph = (it / STAGES) & 1;
                     if (!ptx::mbar_wait(&full[s], ph)) { raise_status(p.status, kErrTimeout); dead = true; break; }
@@ -732,7 +762,7 @@ tc_gemm_flat_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
                     const uint32_t aA = ptx::smem_u32(smem + s * STAGE), aB = aA + A_BYTES;
 #pragma unroll
                     for (int ks = 0; ks < BK / 16; ++ks) {
-                        const uint64_t bdesc = ptx::smem_desc(aB + ks * 2048, 8192, 1024);
+                        const uint64_t bdesc = is_conv(MODE) ? ptx::smem_desc(aB + ks * 32, 16, 1024) : ptx::smem_desc(aB + ks * 2048, 8192, 1024);
 #pragma unroll
                         for (int mt = 0; mt < MT; ++mt) {
                             const uint64_t adesc = (MODE == MODE_DGRAD) ? ptx::smem_desc(aA + mt * 16384 + ks * 2048, 8192, 1024)
@@ -786,7 +816,7 @@ tc_gemm_flat_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
         float sn = 0.f, sd = 0.f, sq = 0.f, pivot = 0.f;     // statistics of this thread's channel over the CTA's range of one M tile
         bool dead = false;            // a wait ran out: no further accumulator is touched, but every pair barrier below is still met
         auto flush_stats = [&]() {
-            if (MODE != MODE_FWD || !p.stats || cur_m < 0) return;
+            if (!is_fwd(MODE) || !p.stats || cur_m < 0) return;
             float n = sn, sum = fmaf(pivot, sn, sd), m2 = sn > 0.f ? sq - sd * sd / sn : 0.f;
             if (EPI > 1) {
                 // the EPI warps of a row hold the statistics of its column chunks: the others hand their triples
@@ -826,7 +856,7 @@ tc_gemm_flat_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
             ptx::tc_fence_after();
             const int row_w = m * (128 * MT) + mt * 128 + wq * 32;
             const int row = row_w + lane;
-            const float bias = (MODE == MODE_FWD && p.bias && row < p.M) ? p.bias[row] : 0.f;
+            const float bias = (is_fwd(MODE) && p.bias && row < p.M) ? p.bias[row] : 0.f;
             int b = flat_find_sample(s_off, p.B, j);
             for (int i = 0; i < nb; ++i) {
                 while (j + i >= s_off[b + 1]) ++b;
@@ -845,7 +875,14 @@ tc_gemm_flat_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
 #pragma unroll
                         for (int q = 0; q < 32; ++q) f[q] = __uint_as_float(r[q]);
                     }
-                    if (MODE == MODE_FWD) {
+                    if (MODE == MODE_CONV_DGRAD) {        // the taps reach past the sample's end: no gradient there
+                        const int nv = len - c0;
+                        if (nv < 32) {
+#pragma unroll
+                            for (int q = 0; q < 32; ++q) if (q >= nv) f[q] = 0.f;
+                        }
+                    }
+                    if (is_fwd(MODE)) {
                         if (p.bias) {
 #pragma unroll
                             for (int q = 0; q < 32; ++q) f[q] += bias;
@@ -885,7 +922,7 @@ tc_gemm_flat_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
                         uint8_t* sb = stg + ((p.stg_nbuf == 2 && (nstore & 1)) ? 2048 : 0);
                         if (lane == 0) { if (p.stg_nbuf == 2) ptx::bulk_wait_read1(); else ptx::bulk_wait_read(); }
                         __syncwarp();
-                        if (MODE == MODE_FWD && p.out_half) stage_block16_swz<__half>(sb, f, lane);
+                        if (is_fwd(MODE) && p.out_half) stage_block16_swz<__half>(sb, f, lane);
                         else stage_block16_swz<T>(sb, f, lane);
                         ptx::fence_proxy_async();
                         __syncwarp();
@@ -893,9 +930,9 @@ tc_gemm_flat_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
                             if (lane == 0) { ptx::tma_store_3d(&mapO, sb, c0, row_w, b); ptx::bulk_commit(); }
                             ++nstore;
                         }
-                    } else if (MT == 1 && OCC == 1 && MODE == MODE_FWD && p.out_f32)
+                    } else if (MT == 1 && OCC == 1 && is_fwd(MODE) && p.out_f32)
                         store_block_staged<float>(reinterpret_cast<float*>(stg), f, reinterpret_cast<float*>(p.out) + base, p.Tp, rl, cl, lane);
-                    else if (MODE == MODE_FWD && p.out_half)
+                    else if (is_fwd(MODE) && p.out_half)
                         store_block16<__half>(stg, f, reinterpret_cast<__half*>(p.out) + base, p.Tp, rl, cl, lane);
                     else
                         store_block16<T>(stg, f, reinterpret_cast<T*>(p.out) + base, p.Tp, rl, cl, lane);
@@ -1243,6 +1280,113 @@ void tc_gemm_wgrad(const TcState* st, const Launch& L, int dtype, const void* gv
         }
     }
     reduce_partials(L, partials, w.nsplit, (int64_t)Cin * Cout, dw, accumulate, gmax);
+}
+
+// ---- non-separable convolution -----------------------------------------------------------------------
+bool tc_conv_supported(const TcState* st, int dtype, int B, int Cin, int Cout, int T, int stride) {
+    return (!st || (st->ready && st->flat)) && dtype != F32 && stride == 1 && Cin % 8 == 0 && Cout % 8 == 0 && T % 8 == 0 &&
+           B <= kFlatMaxB && flat_units_fit(B, T, std::max(Cin, Cout));
+}
+
+// 256-row tiles halve the activation traffic, 128-row tiles make twice the units: the larger tile only where its units
+// still fill the SMs.
+static int conv_mt(const TcState* st, int rows, int B, int T) {
+    return rows > 128 && (long long)((rows + 255) / 256) * B * ((T + 63) / 64) >= st->sm_count ? 2 : 1;
+}
+template <int MODE>
+static void launch_flat_conv(int dtype, int mt, const Launch& L, int sm_count, const CUtensorMap& a, const CUtensorMap& b,
+                             const CUtensorMap& o, const FlatParams& p, int* grid_out) {
+    const bool wide = p.B <= FlatCfg<2, 4, 1, 2>::MAXB;      // sixteen epilogue warps (see launch_flat_shape)
+    auto go = [&](auto t) {
+        using T = decltype(t);
+        // few units per CTA: tiles of at most two blocks, so that six stages (not four half-empty ones) are in flight
+        if (mt == 1 && (long long)p.tiles_m * p.B * p.nbT <= 2ll * sm_count) launch_flat<T, MODE, 1, 2, 2>(L, sm_count, a, b, o, p, grid_out);
+        else if (mt == 1) launch_flat<T, MODE, 1, 4, 2>(L, sm_count, a, b, o, p, grid_out);
+        else if (wide) launch_flat<T, MODE, 2, 4, 1, 1, 2>(L, sm_count, a, b, o, p, grid_out);
+        else launch_flat<T, MODE, 2, 4, 1>(L, sm_count, a, b, o, p, grid_out);
+    };
+    if (dtype == F16) go(__half{}); else go(__nv_bfloat16{});
+}
+
+// A = taps [K][rows][Kc] (K-major), B = activations [B, T, Kc] time-major (K-major)
+static bool conv_maps(const TcState* st, int dtype, const void* w, const void* act, int rows, int Kc, int K, int B, int T,
+                      CUtensorMap* ma, CUtensorMap* mb) {
+    const uint64_t da[3] = {(uint64_t)Kc, (uint64_t)rows, (uint64_t)K};
+    const uint32_t ba[3] = {64, 128, 1};
+    const uint64_t db[3] = {(uint64_t)Kc, (uint64_t)T, (uint64_t)B};
+    const uint32_t bb[3] = {64, 64, 1};
+    return make_map(st, ma, dtype, w, 3, da, ba) && make_map(st, mb, dtype, act, 3, db, bb);
+}
+
+void tc_conv_fwd(const TcState* st, const Launch& L, int dtype, const void* w_taps, const void* x_tm, const float* bias, void* v,
+                 int out_dtype, const int* len_out, const int* blk_off, int B, int Cin, int Cout, int T, int K, int dil,
+                 void* partials, StatsLayout* layout) {
+    KScope ks_(L, KC_PW_FWD, 2.0 * B * T * (Cin + Cout) + 2.0 * Cin * Cout * K, 2.0 * B * T * Cin * Cout * K);
+    CUtensorMap ma, mb, mo;
+    if (layout) *layout = StatsLayout{};
+    if (!conv_maps(st, dtype, w_taps, x_tm, Cout, Cin, K, B, T, &ma, &mb) || !make_out_map(st, &mo, v, B, Cout, T)) return;
+    const int mt = conv_mt(st, Cout, B, T);
+    FlatParams p{};
+    p.out = v; p.bias = bias; p.len_out = len_out; p.blk_off = blk_off; p.stats = (float4*)partials; p.status = L.status;
+    p.M = Cout; p.Kdim = Cin; p.B = B; p.Tp = T; p.nbT = (T + 63) / 64;
+    p.tiles_m = (Cout + 128 * mt - 1) / (128 * mt);
+    p.zero_fill = partials ? 0 : 1;
+    p.out_half = (out_dtype == F16 && dtype != F16) ? 1 : 0;
+    p.tma_out = 1;
+    p.tap_row0 = -(dil * (K - 1)) / 2; p.tap_step = dil; p.tap_blocks = (Cin + BK - 1) / BK; p.ntaps = K;
+    int grid = 0;
+    launch_flat_conv<MODE_CONV_FWD>(dtype, mt, L, st->sm_count, ma, mb, mo, p, &grid);
+    if (layout && partials) { layout->kind = 2; layout->grid = grid; layout->tiles_m = p.tiles_m; layout->rows_per_tile = 128 * mt; }
+}
+
+void tc_conv_dgrad(const TcState* st, const Launch& L, int dtype, const void* w_taps, const void* gv_tm, void* dx, const int* len,
+                   const int* blk_off, int B, int Cin, int Cout, int T, int K, int dil) {
+    KScope ks_(L, KC_PW_DGRAD, 2.0 * B * T * (Cin + Cout) + 2.0 * Cin * Cout * K, 2.0 * B * T * Cin * Cout * K);
+    CUtensorMap ma, mb, mo;
+    if (!conv_maps(st, dtype, w_taps, gv_tm, Cin, Cout, K, B, T, &ma, &mb) || !make_out_map(st, &mo, dx, B, Cin, T)) return;
+    const int mt = conv_mt(st, Cin, B, T);
+    FlatParams p{};
+    p.out = dx; p.len_out = len; p.blk_off = blk_off; p.status = L.status;
+    p.M = Cin; p.Kdim = Cout; p.B = B; p.Tp = T; p.nbT = (T + 63) / 64;
+    p.tiles_m = (Cin + 128 * mt - 1) / (128 * mt);
+    p.zero_fill = 1; p.tma_out = 1;
+    p.tap_row0 = (dil * (K - 1)) / 2; p.tap_step = -dil; p.tap_blocks = (Cout + BK - 1) / BK; p.ntaps = K;
+    launch_flat_conv<MODE_CONV_DGRAD>(dtype, mt, L, st->sm_count, ma, mb, mo, p, nullptr);
+}
+
+// One (output tile, tap, slice) per CTA: slices enough to fill the SMs once.
+static WgradPlan plan_conv_wgrad(int B, int Cin, int Cout, int T, int K) {
+    WgradPlan w = plan_wgrad(B, Cin, Cout, T);
+    w.bn = Cin > 128 ? 256 : (Cin > 64 ? 128 : 64);
+    w.tiles = ((Cout + 127) / 128) * ((Cin + w.bn - 1) / w.bn) * K;
+    const int ns = std::min(std::max(1, 148 / w.tiles), w.nkb_total);
+    w.kb_per_split = (w.nkb_total + ns - 1) / ns;
+    w.nsplit = (w.nkb_total + w.kb_per_split - 1) / w.kb_per_split;
+    return w;
+}
+size_t tc_conv_wgrad_scratch_bytes(int B, int Cin, int Cout, int T, int K) {
+    return (size_t)plan_conv_wgrad(B, Cin, Cout, T, K).nsplit * Cin * Cout * K * sizeof(float);
+}
+void tc_conv_wgrad(const TcState* st, const Launch& L, int dtype, const void* gv_tm, const void* x_tm, float* dw, float* partials,
+                   int accumulate, const int* len_out, int B, int Cin, int Cout, int T, int K, int dil) {
+    const WgradPlan w = plan_conv_wgrad(B, Cin, Cout, T, K);
+    {
+        KScope ks_(L, KC_PW_WGRAD, 2.0 * B * T * (Cin + Cout), 2.0 * B * T * Cin * Cout * K);
+        CUtensorMap ma, mb;
+        const uint64_t da[3] = {(uint64_t)Cout, (uint64_t)T, (uint64_t)B}, db[3] = {(uint64_t)Cin, (uint64_t)T, (uint64_t)B};
+        const uint32_t box[3] = {64, 64, 1};
+        if (!make_map(st, &ma, dtype, gv_tm, 3, da, box) || !make_map(st, &mb, dtype, x_tm, 3, db, box)) return;
+        TcParams p{};
+        p.out = partials; p.len_out = len_out; p.status = L.status;
+        p.M = Cout; p.Ncols = Cin; p.B = B; p.Tp = T;
+        p.nkb_t = w.nkb_t; p.kb_per_split = w.kb_per_split; p.nkb_total = w.nkb_total;
+        p.nsplit = w.nsplit; p.tap_row0 = -(dil * (K - 1)) / 2; p.tap_step = dil;
+        const dim3 grid((Cin + w.bn - 1) / w.bn, (Cout + 127) / 128, K * w.nsplit);
+        if (w.bn == 256) launch_dt<MODE_CONV_WGRAD, 1, 256, 3>(dtype, L, grid, ma, mb, p);
+        else if (w.bn == 128) launch_dt<MODE_CONV_WGRAD, 1, 128, 4>(dtype, L, grid, ma, mb, p);
+        else launch_dt<MODE_CONV_WGRAD, 1, 64, 4>(dtype, L, grid, ma, mb, p);
+    }
+    conv_reduce_taps(L, partials, w.nsplit, Cin * Cout, K, dw, accumulate);
 }
 
 }  // namespace sc

@@ -61,4 +61,17 @@ void tc_gemm_wgrad(const TcState* st, const Launch& L, int dtype, const void* gv
                    float* partials, int accumulate, int B, int Cin, int Cout, int Tp, const int* len_out,
                    const float* gmax = nullptr);
 
+// The same three contractions for the non-separable convolution (stride 1, "same" padding, dilation dil).  x_tm / gv_tm are
+// time-major [B, T, C] copies that are zero at and beyond the sample's length (k_conv_tc.cu); w_taps is the weight as
+// [K][C_out][C_in] (forward) or [K][C_in][C_out] (input gradient).
+bool tc_conv_supported(const TcState* st, int dtype, int B, int Cin, int Cout, int T, int stride);
+void tc_conv_fwd(const TcState* st, const Launch& L, int dtype, const void* w_taps, const void* x_tm, const float* bias, void* v,
+                 int out_dtype, const int* len_out, const int* blk_off, int B, int Cin, int Cout, int T, int K, int dil,
+                 void* partials, StatsLayout* layout);
+void tc_conv_dgrad(const TcState* st, const Launch& L, int dtype, const void* w_taps, const void* gv_tm, void* dx, const int* len,
+                   const int* blk_off, int B, int Cin, int Cout, int T, int K, int dil);
+size_t tc_conv_wgrad_scratch_bytes(int B, int Cin, int Cout, int T, int K);
+void tc_conv_wgrad(const TcState* st, const Launch& L, int dtype, const void* gv_tm, const void* x_tm, float* dw, float* partials,
+                   int accumulate, const int* len_out, int B, int Cin, int Cout, int T, int K, int dil);
+
 }  // namespace sc
