@@ -660,6 +660,10 @@ void dw_fwd(const Launch& L, int dtype, int odt, const void* x, const void* wd, 
         dw_tc_fwd(L, dtype, odt, x, wd, u, len_in, len_out, B, C, Tt, K);
         return;
     }
+    if (s == 2 && plain && dw_s2_supported(dtype, Tt, Tp, K)) {
+        dw_s2_fwd(L, dtype, odt, x, wd, u, len_in, len_out, B, C, Tt, Tp, K);
+        return;
+    }
     if (s == 1 && plain) {
         const int Kp = kpad(K);
         const size_t smem = (size_t)CH * (host_phys(TT + Kp) + 4 + Kp) * sizeof(float);
@@ -684,6 +688,10 @@ void dw_dgrad(const Launch& L, int dtype, int odt, const void* gu, const void* w
                2.0 * B * C * Tp * K);
     if (!L.simt_only && plain && dw_tc_supported(dtype, Tt, K, s)) {
         dw_tc_dgrad(L, dtype, odt, gu, wd, dx, add1, add2, gmax, len_in, len_out, B, C, Tt, K);
+        return;
+    }
+    if (s == 2 && plain && dw_s2_supported(dtype, Tt, Tp, K)) {
+        dw_s2_dgrad(L, dtype, odt, gu, wd, dx, add1, add2, gmax, len_in, len_out, B, C, Tt, Tp, K);
         return;
     }
     if (s == 1 && plain) {
@@ -717,7 +725,9 @@ void dw_wgrad(const Launch& L, int dtype, int odt, const void* gu, const void* x
     // the register kernels stage whole rows: one row (double-buffered) must fit their shared-memory limit
     const bool reg_fits = (dtype == F32) ? (size_t)2 * ((host_phys(Tt + 8 * nch + 8) + 4 + 3) / 4 * 4) * sizeof(float) <= 64 * 1024
                                          : (size_t)2 * 2 * ((Tt + 8 * nch + 8 + 7) / 8 * 8) * 2 <= 96 * 1024;
-    if (plain && s == 1 && Tt % 8 == 0 && nch >= 2 && nch <= 12 && reg_fits) {
+    if (s == 2 && plain && dw_s2_supported(dtype, Tt, Tp, K)) {
+        nsplit = dw_s2_wgrad(L, dtype, odt, gu, x, partials, len_in, len_out, B, C, Tt, Tp, K);
+    } else if (plain && s == 1 && Tt % 8 == 0 && nch >= 2 && nch <= 12 && reg_fits) {
         // rows staged per pass: the count whose (rows x chunks) best fills the 128 threads
         const int cpr = Tt / 8;
         const int NST = (dtype == F32) ? 2 : 4;

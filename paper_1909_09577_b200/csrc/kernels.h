@@ -146,6 +146,15 @@ void dw_tc_fwd(const Launch& L, int dtype, int odt, const void* x, const void* w
 void dw_tc_dgrad(const Launch& L, int dtype, int odt, const void* gu, const void* wd, void* dx, const void* add1,
                  const void* add2, const float* gmax, const int* len_in, const int* len_out, int B, int C, int T,
                  int K);
+// Stride-2 forms (16-bit types, odd K up to 95, T = 2 T' with T' a multiple of 8); dw_s2_wgrad returns how many [C, K]
+// partial rows (at most B) it wrote.
+bool dw_s2_supported(int dtype, int Tt, int Tp, int K);
+void dw_s2_fwd(const Launch& L, int dtype, int odt, const void* x, const void* wd, void* u, const int* len_in, const int* len_out,
+               int B, int C, int Tt, int Tp, int K);
+void dw_s2_dgrad(const Launch& L, int dtype, int odt, const void* gu, const void* wd, void* dx, const void* add1, const void* add2,
+                 const float* gmax, const int* len_in, const int* len_out, int B, int C, int Tt, int Tp, int K);
+int dw_s2_wgrad(const Launch& L, int dtype, int odt, const void* gu, const void* x, float* partials, const int* len_in,
+                const int* len_out, int B, int C, int Tt, int Tp, int K);
 // out = [t < len[b]] * (a + b + c)   (b, c nullable)
 void ew_add_masked(const Launch& L, int dtype, void* out, const void* a, const void* b, const void* c,
                    const int* len, int B, int C, int T);

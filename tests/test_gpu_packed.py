@@ -66,3 +66,14 @@ def test_padded_encoder_equals_chain(api, ctx, T):
     assert (logits.float() - chain["logits"].float()).abs().max() <= 0.1 * scale
     assert logits.shape[2] == spec.T_out and (out_len.cpu().numpy() == chain["out_len"]).all()
     assert (dx.float() - chain["dx"].float()).norm() <= 0.05 * chain["dx"].float().norm()
+
+
+@pytest.mark.parametrize("K,B,T", [(1, 3, 16), (3, 2, 1040), (7, 9, 528), (35, 4, 512), (87, 2, 4112), (95, 5, 304)])
+def test_stride_two_depthwise(api, ctx, K, B, T):
+    """The stride-2 depthwise kernels: both parities of the padding, one tap to the most they take, rows around their tiles."""
+    L = si.LayerCfg(C_in=24, C_out=16, K=K, stride=2)
+    d = si.draw(si.Workload("s2", "bf16", B, T, [L], 700 + K, len_lo=max(1, T // 5), len_hi=T, affine="random"))
+    d.lengths[0], d.lengths[-1] = T, T // 5
+    rep = U.run_block(ctx, api, L, "bf16", d.x, d.lengths, d.params[0], d.g)
+    print(f"\nstride 2 K={K}: {rep}")
+    rep.check()
