@@ -224,6 +224,10 @@ int block_fwd_impl(sc_ctx* ctx, const Launch& L, const sc_block_desc* d, const D
     const int dt = d->io_dtype;
     if (!io.lengths_ready) lengths(L, io.len_in, m.B, io.T_valid ? io.T_valid : m.T, m.s, io.len_out, io.nvalid, io.blk_off);
     const int odt = op_dtype(d);
+    // evaluation mode on whole rows: batch norm, residual and ReLU end the contraction, v is never stored
+    const bool fused = inf && d->has_bn && !m.full && !io.phases && ctx->gemm_mode == 0 &&
+                       tc_affine_supported(&ctx->tc, odt, m.B, m.Cin, m.Cout, m.Tp) &&
+                       (d->residual != SC_RES_PROJ || tc_affine_supported(&ctx->tc, dt, m.B, m.Cres, m.Cout, m.Tp));
     if (d->has_bn && d->residual == SC_RES_PROJ) {
         // the residual projection does not depend on the main branch: its contraction and statistics go to the
         // side stream and are joined just before the apply step
@@ -231,7 +235,9 @@ int block_fwd_impl(sc_ctx* ctx, const Launch& L, const sc_block_desc* d, const D
         const Launch Ls = side_launch(ctx, L);
         const void* xr = io.xres;
         if (!io.res_clean) { mask_copy(Ls, dt, f.xr, io.xres, io.len_out, m.B, m.Cres, m.Tp); xr = f.xr; }
-        if (inf) pointwise_fixed(ctx, Ls, d, m, m.Cres, dt, p->wr, xr, sv->vr, io.len_out, io.blk_off, inf->var_r, sv->invstd_r);
+        if (fused) tc_gemm_affine(&ctx->tc, Ls, dt, p->wr, xr, sv->vr, SC_F16, AffineTail{inf->mean_r, inf->var_r, p->gamma_r, p->beta_r, d->bn_eps},
+                                  io.len_out, io.blk_off, m.B, m.Cres, m.Cout, m.Tp);
+        else if (inf) pointwise_fixed(ctx, Ls, d, m, m.Cres, dt, p->wr, xr, sv->vr, io.len_out, io.blk_off, inf->var_r, sv->invstd_r);
         else pointwise_bn(ctx, Ls, d, m, m.Cres, dt, p->wr, xr, sv->vr, io.len_out, io.nvalid, io.blk_off, sv->mean_r,
                           sv->invstd_r, f.partials_r, nullptr, nullptr);
         record_side(ctx, ctx->ev[5]);
@@ -288,6 +294,14 @@ int block_fwd_impl(sc_ctx* ctx, const Launch& L, const sc_block_desc* d, const D
         void* dst = io.w16_keep ? io.w16_keep : f.w16;
         if (!(io.w16_keep && io.w16_ready)) convert_bf16_to_f16(L, p->wp, dst, (int64_t)m.Cout * m.Cin);
         wp_op = dst;
+    }
+    if (fused) {
+        AffineTail aff{inf->mean, inf->var, p->gamma, p->beta, d->bn_eps};
+        aff.relu = d->has_relu; aff.res_before_relu = d->res_before_relu;
+        if (d->residual == SC_RES_PROJ) { aff.add = sv->vr; aff.add_dtype = SC_F16; wait_side(ctx, L, ctx->ev[5]); }
+        if (d->residual == SC_RES_IDENTITY) { aff.add = io.xres; aff.add_dtype = dt; }
+        tc_gemm_affine(&ctx->tc, L, odt, wp_op, u, io.y, dt, aff, io.len_out, io.blk_off, m.B, m.Cin, m.Cout, m.Tp);
+        return SC_OK;
     }
     if (m.full) {}
     else if (inf) pointwise_fixed(ctx, L, d, m, m.Cin, odt, wp_op, u, sv->v, io.len_out, io.blk_off, inf->var, sv->invstd);

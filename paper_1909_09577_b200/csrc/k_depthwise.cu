@@ -639,6 +639,9 @@ dw_wgrad_reg16_kernel(const TG* __restrict__ gu, const T* __restrict__ x, float*
     }
 }
 
+// Below this many multiply-adds the register-blocked kernel is done before a tensor-core CTA has built its Toeplitz blocks.
+inline bool small_corr(int B, int C, int Tt, int K) { return (double)B * C * Tt * K <= 1.0e8; }
+
 inline int kpad(int K) { return (K + R - 1) / R * R; }
 inline int host_phys(int i) { return i + ((i >> 5) << 2); }
 
@@ -656,7 +659,7 @@ void dw_fwd(const Launch& L, int dtype, int odt, const void* x, const void* wd, 
             const int* len_out, int B, int C, int Tt, int Tp, int K, int s, int dil) {
     KScope ks_(L, KC_DW_FWD, (double)B * C * (dtype_size(dtype) * Tt + dtype_size(odt) * Tp), 2.0 * B * C * Tp * K);
     const bool plain = dil == 1 && (K & 1);      // odd K, adjacent taps: the forms the specialised kernels are written for
-    if (!L.simt_only && plain && dw_tc_supported(dtype, Tt, K, s)) {
+    if (!L.simt_only && plain && !small_corr(B, C, Tt, K) && dw_tc_supported(dtype, Tt, K, s)) {
         dw_tc_fwd(L, dtype, odt, x, wd, u, len_in, len_out, B, C, Tt, K);
         return;
     }
@@ -686,7 +689,7 @@ void dw_dgrad(const Launch& L, int dtype, int odt, const void* gu, const void* w
     const bool plain = dil == 1 && (K & 1);
     KScope ks_(L, KC_DW_DGRAD, (double)B * C * (dtype_size(dtype) * Tt * (1 + (add1 ? 1 : 0) + (add2 ? 1 : 0)) + dtype_size(odt) * Tp),
                2.0 * B * C * Tp * K);
-    if (!L.simt_only && plain && dw_tc_supported(dtype, Tt, K, s)) {
+    if (!L.simt_only && plain && !small_corr(B, C, Tt, K) && dw_tc_supported(dtype, Tt, K, s)) {
         dw_tc_dgrad(L, dtype, odt, gu, wd, dx, add1, add2, gmax, len_in, len_out, B, C, Tt, K);
         return;
     }

@@ -31,9 +31,10 @@ namespace {
 // contraction index (forward, input gradient) or of the output (weight gradient).  Their activations are time-major
 // [B, T, C], so that a tap's shift is a shift of the row coordinate, which a TMA copy may take anywhere (the innermost
 // coordinate must stay on 16-byte boundaries); rows outside [0, T) are zero-filled, which is the "same" padding.
-enum { MODE_FWD = 0, MODE_DGRAD = 1, MODE_WGRAD = 2, MODE_CONV_FWD = 3, MODE_CONV_DGRAD = 4, MODE_CONV_WGRAD = 5 };
-__host__ __device__ constexpr bool is_fwd(int m) { return m == MODE_FWD || m == MODE_CONV_FWD; }
-__host__ __device__ constexpr bool is_conv(int m) { return m >= MODE_CONV_FWD; }
+enum { MODE_FWD = 0, MODE_DGRAD = 1, MODE_WGRAD = 2, MODE_CONV_FWD = 3, MODE_CONV_DGRAD = 4, MODE_CONV_WGRAD = 5,
+       MODE_AFFINE = 6 };   // forward whose epilogue ends with the evaluation-mode batch norm, residual and ReLU
+__host__ __device__ constexpr bool is_fwd(int m) { return m == MODE_FWD || m == MODE_CONV_FWD || m == MODE_AFFINE; }
+__host__ __device__ constexpr bool is_conv(int m) { return m >= MODE_CONV_FWD && m <= MODE_CONV_WGRAD; }
 __host__ __device__ constexpr bool is_wgrad(int m) { return m == MODE_WGRAD || m == MODE_CONV_WGRAD; }
 constexpr int BK = 64;            // contraction elements per stage (one 128-byte swizzle row)
 constexpr int kThreads = 128;
@@ -549,7 +550,9 @@ struct FlatParams {
     int zero_fill;  // blocks wholly in padding must be written as zeros
     int tap_row0, tap_step, tap_blocks;    // CONV modes: operand row = frame + tap_row0 + tap * tap_step; 64-channel blocks per tap
     int ntaps;
+    AffineTail aff; // MODE_AFFINE
     int out_half;   // the result is float16 although the operands are bfloat16
+    int out_bf16;   // the result is bfloat16 although the operands are float16 (MODE_AFFINE)
     int out_f32;    // the result is float32 (one M sub-tile per CTA only: narrow heads such as the class scores)
     int tma_out;    // 16-bit result leaves through TMA stores (third tensor map: 32 frames x 32 rows, 64-byte swizzle)
     int stg_stride; // bytes of staging per epilogue warp (a multiple of 512)
@@ -625,7 +628,7 @@ __device__ __forceinline__ bool flat_next_tile(uint32_t& pos, uint32_t end, uint
 template <int MT, int NB, int OCC, int EPI = 1> struct FlatCfg {
     static constexpr int A_BYTES = MT * 128 * 128;
     static constexpr int STAGE = A_BYTES + NB * 8192;
-    static constexpr int STAGES = OCC == 2 ? 2 : (STAGE <= 32768 ? 6 : (STAGE <= 49152 ? 4 : 3));
+    static constexpr int STAGES = OCC == 2 ? 2 : (STAGE <= 24576 ? 8 : STAGE <= 32768 ? 6 : (STAGE <= 49152 ? 4 : 3));
     // per-warp staging: 32 x 32 16-bit values, or (one M sub-tile, one CTA per SM only) 32 x 32 floats for a float32 result
     static constexpr int STG = EPI >= 2 ? 2048 : ((MT == 1 && OCC == 1) ? kStgFloatsPerWarp * 4 : kOutStageBytes);
     static constexpr int MAXB = (OCC == 2 || EPI >= 2) ? 256 : kFlatMaxB;
@@ -720,7 +723,7 @@ tc_gemm_flat_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
                         if (++cb == p.tap_blocks) { cb = 0; ++tap; }
                         continue;
                     }
-                    if (MODE == MODE_FWD) {
+                    if (is_fwd(MODE)) {
 #pragma unroll
                         for (int mt = 0; mt < MT; ++mt) ptx::tma_load_2d(sA + mt * 16384, &mapA, &full[s], k0, m0 + mt * 128);
                     } else {
@@ -857,6 +860,10 @@ tc_gemm_flat_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
             const int row_w = m * (128 * MT) + mt * 128 + wq * 32;
             const int row = row_w + lane;
             const float bias = (is_fwd(MODE) && p.bias && row < p.M) ? p.bias[row] : 0.f;
+            float mu = 0.f, is = 0.f, ga = 0.f, be = 0.f;
+            if (MODE == MODE_AFFINE && row < p.M) {
+                mu = p.aff.mean[row]; is = 1.f / sqrtf(p.aff.var[row] + p.aff.eps); ga = p.aff.gamma[row]; be = p.aff.beta[row];
+            }
             int b = flat_find_sample(s_off, p.B, j);
             for (int i = 0; i < nb; ++i) {
                 while (j + i >= s_off[b + 1]) ++b;
@@ -888,6 +895,31 @@ tc_gemm_flat_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
                             for (int q = 0; q < 32; ++q) f[q] += bias;
                         }
                         const int nv = max(0, min(32, len - c0));
+                        if (MODE == MODE_AFFINE) {
+                            const bool relu_first = p.aff.relu && !p.aff.res_before_relu;
+#pragma unroll
+                            for (int q = 0; q < 32; ++q) {
+                                f[q] = fmaf(ga, bn_norm(f[q], mu, is), be);
+                                if (relu_first) f[q] = fmaxf(f[q], 0.f);
+                            }
+                            if (p.aff.add && row < p.M) {
+                                const size_t at = ((size_t)b * p.M + row) * p.Tp + c0;
+#pragma unroll
+                                for (int q = 0; q < 4; ++q) {
+                                    float r[8];
+                                    if (c0 + 8 * q < p.Tp) {                // rows are whole vectors
+                                        if (p.aff.add_dtype == F16) ld8<__half>((const __half*)p.aff.add + at + 8 * q, r);
+                                        else ld8<__nv_bfloat16>((const __nv_bfloat16*)p.aff.add + at + 8 * q, r);
+#pragma unroll
+                                        for (int e = 0; e < 8; ++e) f[8 * q + e] += r[e];
+                                    }
+                                }
+                            }
+                            if (p.aff.relu && p.aff.res_before_relu) {
+#pragma unroll
+                                for (int q = 0; q < 32; ++q) f[q] = fmaxf(f[q], 0.f);
+                            }
+                        }
                         if (p.stats && nv > 0) {
                             if (sn == 0.f) pivot = f[0];
                             if (nv == 32) {
@@ -913,7 +945,7 @@ tc_gemm_flat_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
 #pragma unroll
                             for (int q = 0; q < 32; ++q) if (q >= nv) f[q] = 0.f;
                         }
-                        if (!p.out_f32 && (p.out_half || Fmt<T>::v == 0)) clamp_half32(f, p.status);
+                        if (!p.out_f32 && !p.out_bf16 && (p.out_half || Fmt<T>::v == 0)) clamp_half32(f, p.status);
                     }
                     const size_t base = ((size_t)b * p.M + row_w) * p.Tp + c0;
                     const int rl = p.M - row_w, cl = p.Tp - c0;
@@ -923,6 +955,7 @@ tc_gemm_flat_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
                         if (lane == 0) { if (p.stg_nbuf == 2) ptx::bulk_wait_read1(); else ptx::bulk_wait_read(); }
                         __syncwarp();
                         if (is_fwd(MODE) && p.out_half) stage_block16_swz<__half>(sb, f, lane);
+                        else if (MODE == MODE_AFFINE && p.out_bf16) stage_block16_swz<__nv_bfloat16>(sb, f, lane);
                         else stage_block16_swz<T>(sb, f, lane);
                         ptx::fence_proxy_async();
                         __syncwarp();
@@ -1280,6 +1313,43 @@ void tc_gemm_wgrad(const TcState* st, const Launch& L, int dtype, const void* gv
         }
     }
     reduce_partials(L, partials, w.nsplit, (int64_t)Cin * Cout, dw, accumulate, gmax);
+}
+
+// ---- evaluation mode --------------------------------------------------------------------------------
+void tc_gemm_affine(const TcState* st, const Launch& L, int dtype, const void* w, const void* u, void* y, int out_dtype,
+                    const AffineTail& aff, const int* len_out, const int* blk_off, int B, int Cin, int Cout, int Tp) {
+    KScope ks_(L, KC_PW_FWD, 2.0 * B * Tp * (Cin + Cout) + 2.0 * Cin * Cout + (aff.add ? 2.0 * B * Tp * Cout : 0.0), 2.0 * B * Tp * Cin * Cout);
+    CUtensorMap ma, mb, mo;
+    const uint64_t da[2] = {(uint64_t)Cin, (uint64_t)Cout};
+    const uint32_t ba[2] = {64, 128};
+    const uint64_t db[3] = {(uint64_t)Tp, (uint64_t)Cin, (uint64_t)B};
+    const uint32_t bb[3] = {64, 64, 1};
+    if (!make_map(st, &ma, dtype, w, 2, da, ba) || !make_map(st, &mb, dtype, u, 3, db, bb) || !make_out_map(st, &mo, y, B, Cout, Tp)) return;
+    // Few units (a unit is 128 or 256 rows of one 64-frame block): the smallest tile spreads them over the most SMs and has
+    // its whole contraction (up to 512 channels) in flight in eight stages; its weight traffic per flop only matters once
+    // every SM has several units.
+    const long long units = (long long)((Cout + 127) / 128) * B * ((Tp + 63) / 64);
+    const bool small = units <= 2ll * st->sm_count && B <= FlatCfg<1, 1, 1, 2>::MAXB;
+    const bool wide = B <= FlatCfg<2, 4, 1, 2>::MAXB;
+    const int mt = small || Cout <= 128 ? 1 : 2;
+    FlatParams p{};
+    p.out = y; p.len_out = len_out; p.blk_off = blk_off; p.status = L.status; p.aff = aff;
+    p.M = Cout; p.Kdim = Cin; p.B = B; p.Tp = Tp; p.nbT = (Tp + 63) / 64;
+    p.tiles_m = (Cout + 128 * mt - 1) / (128 * mt);
+    p.zero_fill = 1; p.tma_out = 1;
+    p.out_half = (out_dtype == F16 && dtype != F16) ? 1 : 0;
+    p.out_bf16 = (out_dtype == BF16 && dtype != BF16) ? 1 : 0;
+    auto go = [&](auto t) {
+        using T = decltype(t);
+        if (small) launch_flat<T, MODE_AFFINE, 1, 1, 2, 1, 2>(L, st->sm_count, ma, mb, mo, p, nullptr);
+        else if (mt == 1) launch_flat<T, MODE_AFFINE, 1, 4, 2>(L, st->sm_count, ma, mb, mo, p, nullptr);
+        else if (wide) launch_flat<T, MODE_AFFINE, 2, 4, 1, 1, 2>(L, st->sm_count, ma, mb, mo, p, nullptr);
+        else launch_flat<T, MODE_AFFINE, 2, 4, 1>(L, st->sm_count, ma, mb, mo, p, nullptr);
+    };
+    if (dtype == F16) go(__half{}); else go(__nv_bfloat16{});
+}
+bool tc_affine_supported(const TcState* st, int dtype, int B, int Cin, int Cout, int Tp) {
+    return shape_ok(st, dtype, Cin, Cout, Tp) && st->flat && B <= kFlatMaxB && flat_units_fit(B, Tp, Cout);
 }
 
 // ---- non-separable convolution -----------------------------------------------------------------------

@@ -61,6 +61,14 @@ void tc_gemm_wgrad(const TcState* st, const Launch& L, int dtype, const void* gv
                    float* partials, int accumulate, int B, int Cin, int Cout, int Tp, const int* len_out,
                    const float* gmax = nullptr);
 
+// Evaluation mode: y = [t < len_out[b]] relu(gamma (v - mean) / sqrt(var + eps) + beta + add) with v = w u (the fp32
+// accumulators, never stored), in out_dtype.  add (nullable) is [B, C_out, T'] in add_dtype (F16 or BF16);
+// with res_before_relu = 0 it is added after the ReLU.
+struct AffineTail { const float *mean, *var, *gamma, *beta; float eps; const void* add; int add_dtype, relu, res_before_relu; };
+bool tc_affine_supported(const TcState* st, int dtype, int B, int Cin, int Cout, int Tp);
+void tc_gemm_affine(const TcState* st, const Launch& L, int dtype, const void* w, const void* u, void* y, int out_dtype,
+                    const AffineTail& aff, const int* len_out, const int* blk_off, int B, int Cin, int Cout, int Tp);
+
 // The same three contractions for the non-separable convolution (stride 1, "same" padding, dilation dil).  x_tm / gv_tm are
 // time-major [B, T, C] copies that are zero at and beyond the sample's length (k_conv_tc.cu); w_taps is the weight as
 // [K][C_out][C_in] (forward) or [K][C_in][C_out] (input gradient).
