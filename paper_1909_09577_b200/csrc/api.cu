@@ -130,9 +130,7 @@ struct BlockIO {                 // raw pointers after validation
     const int* len_in; int* len_out; int* nvalid; int* blk_off;
     bool x_clean, res_clean;     // inputs known to be zero in padded frames
     bool lengths_ready;          // len_out / nvalid already computed
-    void* w16_keep;              // optional: where to leave the float16 copy of wp for the backward pass
-    bool w16_ready;              // w16_keep already holds the copy
-    int T_valid;                 // largest legal length when that is not m.T (an encoder input padded to a longer row)
+    const void* w16;             // float16 copy of wp, where the layer's operands are float16 and wp is not
     // packed block: x (and a projected xres) are packed, y and an identity xres are dense [., ., Td] with lengths
     // len_dense, and u, v, vr are also written to the dense tensors of `dense` (nullable members)
     int phases, Td; const int* len_dense; sc_block_saved dense;
@@ -218,11 +216,21 @@ void pointwise_fixed(sc_ctx* ctx, const Launch& L, const sc_block_desc* d, const
     invstd_from_var(L, var, d->bn_eps, invstd, m.Cout);
 }
 
+Prologue length_prologue(const Dims& m, const int* len_in, int* len_out, int* nvalid, int* blk_off) {
+    Prologue p;
+    p.len_in = len_in; p.B = m.B; p.T_in = m.T; p.stride = m.s; p.len_out = len_out; p.nvalid = nvalid; p.blk_off = blk_off;
+    return p;
+}
+bool needs_w16(const sc_block_desc* d, const Dims& m) { return op_dtype(d) != d->io_dtype && !m.full; }
+
 int block_fwd_impl(sc_ctx* ctx, const Launch& L, const sc_block_desc* d, const Dims& m, BlockIO io,
                    const sc_block_params* p, sc_block_saved* sv, float* rmean, float* rvar,
                    const FwdScratch& f, const InferStats* inf = nullptr) {
     const int dt = d->io_dtype;
-    if (!io.lengths_ready) lengths(L, io.len_in, m.B, io.T_valid ? io.T_valid : m.T, m.s, io.len_out, io.nvalid, io.blk_off);
+    if (!io.lengths_ready) {                                  // a later striding layer of an encoder
+        Prologue pr = length_prologue(m, io.len_in, io.len_out, io.nvalid, io.blk_off);
+        prologue(L, pr);
+    }
     const int odt = op_dtype(d);
     // evaluation mode on whole rows: batch norm, residual and ReLU end the contraction, v is never stored
     const bool fused = inf && d->has_bn && !m.full && !io.phases && ctx->gemm_mode == 0 &&
@@ -290,11 +298,7 @@ int block_fwd_impl(sc_ctx* ctx, const Launch& L, const sc_block_desc* d, const D
         return SC_OK;
     }
     const void* wp_op = p->wp;
-    if (odt != dt && !m.full) {
-        void* dst = io.w16_keep ? io.w16_keep : f.w16;
-        if (!(io.w16_keep && io.w16_ready)) convert_bf16_to_f16(L, p->wp, dst, (int64_t)m.Cout * m.Cin);
-        wp_op = dst;
-    }
+    if (needs_w16(d, m)) wp_op = io.w16;
     if (fused) {
         AffineTail aff{inf->mean, inf->var, p->gamma, p->beta, d->bn_eps};
         aff.relu = d->has_relu; aff.res_before_relu = d->res_before_relu;
@@ -336,10 +340,19 @@ void plan_fwd_pack(const sc_block_desc* d, const Packed& k, Bump& ws, FwdPack* f
     f->sv.v = ws.take((size_t)2 * k.m.B * k.m.Cout * k.m.Tp);
     if (d->residual == SC_RES_PROJ) f->sv.vr = ws.take((size_t)2 * k.m.B * k.m.Cout * k.m.Tp);
 }
+// The prologue of a single block's forward pass.
+void enter(const Launch& L, const sc_block_desc* d, const Dims& m, const Packed& k, const FwdPack& fp, const FwdScratch& f,
+           const sc_block_params* p, BlockIO& io, int* out_lengths) {
+    Prologue pr = length_prologue(m, io.len_in, io.len_out, io.nvalid, io.blk_off);
+    pr.len_user = out_lengths;
+    if (k.phases > 1) { pr.phases = k.phases; pr.len_dense = fp.len_dense; }
+    if (needs_w16(d, m)) { pr.convert(p->wp, f.w16, m.Cout * m.Cin); io.w16 = f.w16; }
+    prologue(L, pr);
+    io.lengths_ready = true;
+}
 // Packs the inputs and points io / sv (the caller's, dense) at the packed operands.
 void enter_packed(const Launch& L, const sc_block_desc* d, const Dims& m, const Packed& k, const FwdPack& f, BlockIO& io,
                   sc_block_saved& sv) {
-    lengths(L, io.len_in, m.B, m.T, m.s, io.len_out, io.nvalid, io.blk_off, k.phases, k.phases > 1 ? f.len_dense : nullptr);
     PackList pl{};
     auto add = [&](const void* src, void* dst, int C, const int* len) { pl.src[pl.count] = src; pl.dst[pl.count] = dst; pl.C[pl.count] = C; pl.len[pl.count] = len; ++pl.count; };
     add(io.x, f.x, m.Cin, io.len_in);
@@ -352,7 +365,7 @@ void enter_packed(const Launch& L, const sc_block_desc* d, const Dims& m, const 
     }
     io.x = f.x;
     if (d->residual == SC_RES_PROJ) io.xres = own ? f.x : f.xres;
-    io.x_clean = io.res_clean = io.lengths_ready = true;
+    io.x_clean = io.res_clean = true;
     io.phases = k.phases; io.Td = m.Tp; io.len_dense = k.phases > 1 ? f.len_dense : io.len_out;
     if (k.phases > 1) io.len_in = io.len_out;
     io.dense.u = sv.u; io.dense.v = sv.v; io.dense.vr = sv.vr;
@@ -430,11 +443,10 @@ struct BwdIO {
     void *dx, *dx_res; const void* dx_add;
     const int* len_in; const int* len_out; const int* nvalid; const int* blk_off;
     bool x_clean, res_clean;
-    const void* w16_kept;        // float16 copy of wp left by the forward pass (optional)
+    const void* w16;             // float16 copy of wp (see BlockIO)
     cudaEvent_t done;            // recorded on the side stream after this layer's last side-stream kernel
     int phases, Td; uint32_t total_dense;      // packed block: dy, y and the saved v, vr are dense [., ., Td]; the rest is packed
-    float* gmax_zeroed;          // optional: a float the caller has already set to zero, used for the |gv| bound
-                                 // (a memset between two kernels would end the programmatic overlap of that pair)
+    float* gmax;                 // where the bound on |gv| collects; already zero
 };
 
 int block_bwd_impl(sc_ctx* ctx, const Launch& L, const sc_block_desc* d, const Dims& m, BwdIO io,
@@ -452,8 +464,7 @@ int block_bwd_impl(sc_ctx* ctx, const Launch& L, const sc_block_desc* d, const D
                          tc_wgrad_supported(&ctx->tc, SC_F16, m.Cin, m.Cout, m.Tp);
     const bool half_gvr = dt == SC_BF16 && d->has_bn && d->residual == SC_RES_PROJ && s.gvr16 && tc_ok &&
                           tc_wgrad_supported(&ctx->tc, SC_F16, m.Cres, m.Cout, m.Tp);
-    float* gmax = (dt != SC_F32 && d->has_bn && (d->has_dw || half_gv || half_gvr)) ? (io.gmax_zeroed ? io.gmax_zeroed : s.gmax) : nullptr;
-    if (gmax && !io.gmax_zeroed) cudaMemsetAsync(gmax, 0, sizeof(float), L.stream);
+    float* gmax = (dt != SC_F32 && d->has_bn && (d->has_dw || half_gv || half_gvr)) ? io.gmax : nullptr;
     const void* dy = io.dy;
     if (d->log_softmax) {      // upstream gradient is w.r.t. the log-probabilities: back through the log-softmax first
         log_softmax_bwd(L, dt, s.dz, io.dy, io.y, io.len_out, m.B, m.Cout, m.Tp);
@@ -521,10 +532,7 @@ int block_bwd_impl(sc_ctx* ctx, const Launch& L, const sc_block_desc* d, const D
     };
 
     const void* wp_op = p->wp;
-    if (odt != dt && !m.full) {
-        if (io.w16_kept) wp_op = io.w16_kept;
-        else { convert_bf16_to_f16(L, p->wp, s.w16, (int64_t)m.Cout * m.Cin); wp_op = s.w16; }
-    }
+    if (needs_w16(d, m)) wp_op = io.w16;
     const void* extra = nullptr;    // residual-path gradient to fold into dx
     if (d->residual == SC_RES_PROJ) {
         void* tgt = io.dx_res ? io.dx_res : s.gxr;
@@ -804,10 +812,9 @@ int fwd_call(sc_ctx* ctx, const Launch& L, const sc_block_desc* desc, const sc_t
     io.y = y->ptr; io.len_in = lengths_dev; io.len_out = f.len_out; io.nvalid = f.nvalid; io.blk_off = f.blk_off;
     io.x_clean = false; io.res_clean = false; io.lengths_ready = false;
     sc_block_saved sv = *saved;
+    enter(L, desc, m, pk, fp, f, params, io, out_lengths_dev);
     if (pk.phases) enter_packed(L, desc, m, pk, fp, io, sv);
     SC_TRY(block_fwd_impl(ctx, L, desc, pk.phases ? pk.m : m, io, params, &sv, running_mean, running_var, f));
-    if (out_lengths_dev)
-        cudaMemcpyAsync(out_lengths_dev, io.phases ? io.len_dense : f.len_out, sizeof(int) * m.B, cudaMemcpyDeviceToDevice, L.stream);
     return finish(ctx);
 }
 }  // namespace
@@ -883,10 +890,9 @@ int infer_call(sc_ctx* ctx, const Launch& L, const sc_block_desc* desc, const sc
     io.x = x->ptr; io.xres = desc->residual != SC_RES_NONE ? (x_res ? x_res->ptr : x->ptr) : nullptr;
     io.y = y->ptr; io.len_in = lengths_dev; io.len_out = q.f.len_out; io.nvalid = q.f.nvalid; io.blk_off = q.f.blk_off;
     InferStats inf{running_mean, running_var, running_mean_r, running_var_r};
+    enter(L, desc, m, pk, fp, q.f, params, io, out_lengths_dev);
     if (pk.phases) { enter_packed(L, desc, m, pk, fp, io, q.sv); memset(&io.dense, 0, sizeof(io.dense)); }
     SC_TRY(block_fwd_impl(ctx, L, desc, pk.phases ? pk.m : m, io, params, &q.sv, nullptr, nullptr, q.f, &inf));
-    if (out_lengths_dev)
-        cudaMemcpyAsync(out_lengths_dev, io.phases ? io.len_dense : q.f.len_out, sizeof(int) * m.B, cudaMemcpyDeviceToDevice, L.stream);
     return finish(ctx);
 }
 }  // namespace
@@ -939,8 +945,13 @@ int bwd_call(sc_ctx* ctx, const Launch& L, const sc_block_desc* desc, const sc_t
     if (pk.phases) plan_bwd_pack(desc, pk, ws, &bp);
     if (!ws.ok()) return SC_ERR_WORKSPACE;
     const bool two = pk.phases > 1;
-    lengths(L, lengths_dev, m.B, m.T, m.s, s.len_out, s.nvalid, s.blk_off, two ? pk.phases : 1, two ? bp.len_dense : nullptr);
+    Prologue pr = length_prologue(m, lengths_dev, s.len_out, s.nvalid, s.blk_off);
+    if (two) { pr.phases = pk.phases; pr.len_dense = bp.len_dense; }
+    pr.zero = s.gmax; pr.nzero = 1;
+    if (needs_w16(desc, m)) pr.convert(params->wp, s.w16, m.Cout * m.Cin);
+    prologue(L, pr);
     BwdIO io{};
+    io.gmax = s.gmax; io.w16 = s.w16;
     io.dy = dy->ptr; io.x = x->ptr; io.y = y->ptr;
     io.xres = desc->residual != SC_RES_NONE ? (x_res ? x_res->ptr : x->ptr) : nullptr;
     io.dx = dx->ptr; io.dx_res = (desc->residual != SC_RES_NONE && dx_res) ? dx_res->ptr : nullptr;
@@ -1178,6 +1189,28 @@ void copy_frames(const Launch& L, bool in, const void* src, void* dst, int C, co
     PackList l{}; l.count = 1; l.src[0] = src; l.dst[0] = dst; l.C[0] = C; l.len[0] = len;
     if (in) pack_frames(L, l, B, T, Tq, 1); else unpack_frames(L, l, B, T, Tq, 1);
 }
+// whether a layer after the first changes the lengths again
+bool strided_later(const EncPlan& P) {
+    for (size_t i = 1; i < P.L.size(); ++i) if (P.L[i].own_lengths) return true;
+    return false;
+}
+// Lengths of the first layer (the encoder's, unless a later layer strides too), float16 copies of the pointwise weights of
+// every layer that needs one and, for a training pass, the zeroed |gv| bounds.
+void encoder_prologue(const Launch& L, const sc_encoder_desc* e, const EncPlan& P, const int* lengths, int* out_lengths,
+                      const void* blob, const int64_t* offs, bool train) {
+    const LayerPlan& f = P.L[0];
+    Prologue pr = length_prologue(f.m, lengths, f.len_out, f.nvalid, f.blk_off);
+    pr.T_in = e->layers[0].T_in;                  // the legal range, whatever the rows are padded to
+    if (!strided_later(P)) pr.len_user = out_lengths;
+    if (train) { pr.zero = P.gmax_all; pr.nzero = e->n_layers; }
+    for (int i = 0; i < e->n_layers; ++i) {
+        const LayerPlan& l = P.L[i];
+        if (!l.w16) continue;
+        if (pr.conv.count == kMaxConvert) { Prologue more; std::swap(more.conv, pr.conv); prologue(L, more); }
+        pr.convert(layer_params(blob, offs + 8 * i).wp, l.w16, l.m.Cout * l.m.Cin);
+    }
+    prologue(L, pr);
+}
 }  // namespace
 
 int encoder_workspace_bytes(const sc_encoder_desc* desc, size_t* bytes) {
@@ -1207,38 +1240,41 @@ int encoder_infer_call(sc_ctx* ctx, const Launch& L, const sc_encoder_desc* e, c
     const int T_in = e->layers[0].T_in;
     SC_TRY(check_tensor(x, dt, m0.B, m0.Cin, T_in));
     SC_TRY(check_tensor(out, dt, ml.B, ml.Cout, P.T_pad ? P.T_out : ml.Tp));
-    const void* x_in = x->ptr;
-    void* y_out = out->ptr;
-    if (P.T_pad) { copy_frames(L, true, x->ptr, P.x_pad, m0.Cin, lengths_dev, m0.B, T_in, m0.T); x_in = P.x_pad; y_out = P.logits_pad; }
-    auto input_of = [&](int i) -> const void* { return i == 0 ? x_in : P.L[i - 1].y; };
-    auto res_src = [&](int i) -> int { return (e->res_from && e->res_from[i] >= 0) ? e->res_from[i] : i; };
     auto stat = [&](int i, int j) -> const float* {
         const int64_t o = running_offsets[4 * i + j];
         return o < 0 ? nullptr : (const float*)((const char*)running_blob + o);
     };
     for (int i = 0; i < n; ++i) {
+        const sc_block_params prm = layer_params(params_blob, param_offsets + 8 * i);
+        SC_TRY(check_params(&P.L[i].d, &prm));
+        if (P.L[i].d.has_bn && (!stat(i, 0) || !stat(i, 1))) return SC_ERR_NULL;
+        if (P.L[i].d.residual == SC_RES_PROJ && (!stat(i, 2) || !stat(i, 3))) return SC_ERR_NULL;
+    }
+    encoder_prologue(L, e, P, lengths_dev, out_lengths_dev, params_blob, param_offsets, false);
+    const void* x_in = x->ptr;
+    void* y_out = out->ptr;
+    if (P.T_pad) { copy_frames(L, true, x->ptr, P.x_pad, m0.Cin, lengths_dev, m0.B, T_in, m0.T); x_in = P.x_pad; y_out = P.logits_pad; }
+    auto input_of = [&](int i) -> const void* { return i == 0 ? x_in : P.L[i - 1].y; };
+    auto res_src = [&](int i) -> int { return (e->res_from && e->res_from[i] >= 0) ? e->res_from[i] : i; };
+    for (int i = 0; i < n; ++i) {
         LayerPlan& lp = P.L[i];
         sc_block_params prm = layer_params(params_blob, param_offsets + 8 * i);
-        SC_TRY(check_params(&lp.d, &prm));
         InferStats inf{stat(i, 0), stat(i, 1), stat(i, 2), stat(i, 3)};
-        if (lp.d.has_bn && (!inf.mean || !inf.var)) return SC_ERR_NULL;
-        if (lp.d.residual == SC_RES_PROJ && (!inf.mean_r || !inf.var_r)) return SC_ERR_NULL;
         Bump b(workspace, workspace_bytes); b.off = P.scratch_mark;
         FwdScratch f; plan_fwd(&lp.d, lp.m, b, &f, &ctx->tc);
         BlockIO io{};
         io.x = input_of(i);
         io.xres = lp.d.residual != SC_RES_NONE ? input_of(res_src(i)) : nullptr;
         io.y = (i + 1 < n) ? lp.y : y_out;
-        if (i == 0) io.T_valid = T_in;
         io.len_in = i == 0 ? lengths_dev : P.L[i - 1].len_out; io.len_out = lp.len_out; io.nvalid = lp.nvalid; io.blk_off = lp.blk_off;
         io.x_clean = i > 0; io.res_clean = lp.d.residual != SC_RES_NONE && res_src(i) > 0;
-        io.lengths_ready = !lp.own_lengths;
-        io.w16_keep = lp.w16; io.w16_ready = false;
+        io.lengths_ready = i == 0 || !lp.own_lengths;
+        io.w16 = lp.w16;
         if (P.T_pad) io.x_clean = true;
         SC_TRY(block_fwd_impl(ctx, L, &lp.d, lp.m, io, &prm, &lp.sv, nullptr, nullptr, f, &inf));
     }
     if (P.T_pad) copy_frames(L, false, P.logits_pad, out->ptr, ml.Cout, P.L[n - 1].len_out, ml.B, P.T_out, ml.Tp);
-    if (out_lengths_dev)
+    if (out_lengths_dev && strided_later(P))
         cudaMemcpyAsync(out_lengths_dev, P.L[n - 1].len_out, sizeof(int) * m0.B, cudaMemcpyDeviceToDevice, L.stream);
     return finish(ctx);
 }
@@ -1296,18 +1332,7 @@ int encoder_call(sc_ctx* ctx, const Launch& L, const sc_encoder_desc* e, const s
     auto len_in_of = [&](int i) -> const int* { return i == 0 ? lengths_dev : P.L[i - 1].len_out; };
     auto res_src = [&](int i) -> int { return (e->res_from && e->res_from[i] >= 0) ? e->res_from[i] : i; };
 
-    cudaMemsetAsync(P.gmax_all, 0, sizeof(float) * n, L.stream);
-    // float16 copies of the pointwise weights of every layer that needs one: one launch
-    {
-        ConvertList cl; cl.count = 0;
-        for (int i = 0; i < n; ++i) {
-            if (!P.L[i].w16) continue;
-            if (cl.count == 48) { convert_bf16_to_f16_many(L, cl); cl.count = 0; }
-            cl.src[cl.count] = prm[i].wp; cl.dst[cl.count] = P.L[i].w16; cl.n[cl.count] = P.L[i].m.Cout * P.L[i].m.Cin;
-            ++cl.count;
-        }
-        convert_bf16_to_f16_many(L, cl);
-    }
+    encoder_prologue(L, e, P, lengths_dev, out_lengths_dev, params_blob, param_offsets, true);
     // forward
     for (int i = 0; i < n; ++i) {
         LayerPlan& lp = P.L[i];
@@ -1319,12 +1344,11 @@ int encoder_call(sc_ctx* ctx, const Launch& L, const sc_encoder_desc* e, const s
         io.y = (i + 1 < n) ? lp.y : lg;
         io.len_in = len_in_of(i); io.len_out = lp.len_out; io.nvalid = lp.nvalid; io.blk_off = lp.blk_off;
         io.x_clean = i > 0 || P.T_pad; io.res_clean = lp.d.residual != SC_RES_NONE && res_src(i) > 0;
-        if (i == 0) io.T_valid = T_in;
-        io.lengths_ready = !lp.own_lengths;
-        io.w16_keep = lp.w16; io.w16_ready = true;
+        io.lengths_ready = i == 0 || !lp.own_lengths;
+        io.w16 = lp.w16;
         SC_TRY(block_fwd_impl(ctx, L, &lp.d, lp.m, io, &prm[i], &lp.sv, nullptr, nullptr, f));
     }
-    if (out_lengths_dev)
+    if (out_lengths_dev && strided_later(P))
         cudaMemcpyAsync(out_lengths_dev, P.L[n - 1].len_out, sizeof(int) * m0.B, cudaMemcpyDeviceToDevice, L.stream);
 
     if (P.T_pad) copy_frames(L, false, lg, logits->ptr, ml.Cout, P.L[n - 1].len_out, ml.B, T_out, ml.Tp);
@@ -1354,8 +1378,8 @@ int encoder_call(sc_ctx* ctx, const Launch& L, const sc_encoder_desc* e, const s
         io.dx_add = has_pending[i] ? P.pend[i] : nullptr;
         io.len_in = len_in_of(i); io.len_out = lp.len_out; io.nvalid = lp.nvalid; io.blk_off = lp.blk_off;
         io.x_clean = i > 0 || P.T_pad; io.res_clean = lp.d.residual != SC_RES_NONE && res_src(i) > 0;
-        io.w16_kept = lp.w16;
-        io.gmax_zeroed = P.gmax_all + i;
+        io.w16 = lp.w16;
+        io.gmax = P.gmax_all + i;
         SC_TRY(block_bwd_impl(ctx, L, &lp.d, lp.m, io, &prm[i], &lp.sv, &grd[i], accumulate, s));
         if (second)
             ew_add_masked(L, dt, P.pend[src], P.pend[src], P.pend_tmp, nullptr, len_in_of(src), P.L[src].m.B, P.L[src].m.Cin, P.L[src].m.T);

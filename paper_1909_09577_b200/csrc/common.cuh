@@ -218,15 +218,16 @@ __device__ __forceinline__ void chan_merge(float& n, float& mean, float& m2, flo
 }
 
 // Programmatic dependent launch.  Every kernel of the library is launched so that it may start while the
-// kernel before it on the stream is still draining; it therefore (1) tells the runtime right away that its own
-// dependents may be launched -- the trigger fires once every CTA has said so, i.e. when the last wave is on
-// the SMs -- and (2) waits for the kernels before it to complete, with their writes visible, before it reads
-// or writes global memory.  Work placed before pdl_wait() (barrier set-up, tensor-memory allocation,
-// descriptor prefetch) overlaps the previous kernel's tail.  Both are no-ops in a kernel launched without
-// the attribute.
+// kernel before it on the stream is still running.  It (1) waits for the kernels before it to complete, with their writes
+// visible, before it reads or writes global memory, and (2) tells the runtime after that wait that its own dependents may
+// be launched.  Work placed before pdl_wait() (barrier set-up, tensor-memory allocation, descriptor prefetch) overlaps the
+// previous kernel.  Because the trigger comes after the wait, a kernel starts only once everything up to the kernel before
+// the previous one has completed; so it may also read, ahead of its wait, what was settled that early: the caller's
+// parameters (from the second kernel of a call on) and the lengths and weight copies (when another kernel lies between it
+// and the prologue that wrote them).  Both are no-ops in a kernel launched without the attribute.
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void pdl_sync() { pdl_launch_dependents(); pdl_wait(); }
+__device__ __forceinline__ void pdl_sync() { pdl_wait(); pdl_launch_dependents(); }
 
 __device__ __forceinline__ void raise_status(int* status, int code) {
     if (status) atomicCAS(status, 0, code);

@@ -40,27 +40,48 @@ __device__ __forceinline__ void block_sum(float (&v)[N]) {
 
 __device__ __forceinline__ float block_max(float v) { return warp_max(v); }
 
-// One CTA.  The block offsets are an exclusive scan over the samples: each thread sums a contiguous run of samples, the
-// runs are scanned through shared memory.  (A scan by one thread is a chain of dependent loads: 10 us at 32 samples.)
-constexpr int kLenThreads = 256;
-__global__ void __launch_bounds__(kLenThreads)
-lengths_kernel(const int* __restrict__ len_in, int B, int T_in, int stride, int phases, int* __restrict__ len_out,
-               int* __restrict__ nvalid, int* __restrict__ blk_off, int* __restrict__ len_dense, int* status) {
+// Block 0: lengths.  The block offsets are an exclusive scan over the samples: each thread sums a contiguous run of
+// samples, the runs are scanned through shared memory.  (A scan by one thread is a chain of dependent loads: 10 us at 32
+// samples.)  The other blocks convert 2048 elements each, one 16-byte vector per thread; as a launch of its own with scalar
+// accesses the conversion of an encoder's weights cost 12 us in front of every training step.
+constexpr int kLenThreads = 256, kConvertChunk = 2048;
+__global__ void __launch_bounds__(kLenThreads) prologue_kernel(const __grid_constant__ Prologue p, int* status) {
     pdl_sync();
+    const int tid = threadIdx.x;
+    if (blockIdx.x > 0) {
+        const ConvertList& l = p.conv;
+        const int blk = blockIdx.x - 1;
+        int k = 0;
+        while (k + 1 < l.count && blk >= l.first[k + 1]) ++k;
+        const int i = (blk - l.first[k]) * kConvertChunk + 8 * tid, n = l.n[k];
+        const __nv_bfloat16* src = (const __nv_bfloat16*)l.src[k];
+        __half* dst = (__half*)l.dst[k];
+        if (i + 8 <= n && ((reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst)) & 15) == 0) {
+            float f[8];
+            ld8<__nv_bfloat16>(src + i, f);
+            st8<__half>(dst + i, f);
+        } else {
+            for (int e = i; e < min(i + 8, n); ++e) dst[e] = __float2half_rn(__bfloat162float(src[e]));
+        }
+        return;
+    }
+    for (int i = tid; i < p.nzero; i += kLenThreads) p.zero[i] = 0.f;
+    if (!p.len_in) return;
     __shared__ int s_frames[kLenThreads / 32], s_blocks[kLenThreads / 32];
-    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-    const int n = B * phases, per = (n + kLenThreads - 1) / kLenThreads, i0 = min(n, tid * per), i1 = min(n, i0 + per);
-    auto out_len = [&](int i) -> int {
-        const int b = i / phases, p = i - b * phases;
-        int l = len_in[b];
-        if (l < 1 || l > T_in) { raise_status(status, kErrLengths); l = min(max(l, 0), T_in); }
-        if (len_dense && p == 0) len_dense[b] = l;
-        return phases > 1 ? (l - p + phases - 1) / phases : (l + stride - 1) / stride;
-    };
+    const int lane = tid & 31, w = tid >> 5;
+    const int n = p.B * p.phases, per = (n + kLenThreads - 1) / kLenThreads, i0 = min(n, tid * per), i1 = min(n, i0 + per);
     int frames = 0, blocks = 0;
     for (int i = i0; i < i1; ++i) {
-        const int lo = out_len(i);
-        len_out[i] = lo;
+        const int b = i / p.phases, ph = i - b * p.phases;
+        int l = p.len_in[b];
+        if (l < 1 || l > p.T_in) { raise_status(status, kErrLengths); l = min(max(l, 0), p.T_in); }
+        const int lo = p.phases > 1 ? (l - ph + p.phases - 1) / p.phases : (l + p.stride - 1) / p.stride;
+        if (ph == 0) {
+            const int dense = p.phases > 1 ? l : lo;
+            if (p.len_dense) p.len_dense[b] = dense;
+            if (p.len_user) p.len_user[b] = dense;
+        }
+        p.len_out[i] = lo;
         frames += lo; blocks += (lo + 63) / 64;
     }
     int incl = blocks;                                   // inclusive scan over the warp
@@ -73,14 +94,14 @@ lengths_kernel(const int* __restrict__ len_in, int B, int T_in, int stride, int 
     __syncthreads();
     int base = incl - blocks;
     for (int q = 0; q < w; ++q) base += s_blocks[q];
-    if (blk_off) {
-        for (int i = i0; i < i1; ++i) { blk_off[i] = base; base += (len_out[i] + 63) / 64; }
-        if (tid == kLenThreads - 1) blk_off[n] = base;   // the last thread's runs end the list
+    if (p.blk_off) {
+        for (int i = i0; i < i1; ++i) { p.blk_off[i] = base; base += (p.len_out[i] + 63) / 64; }
+        if (tid == kLenThreads - 1) p.blk_off[n] = base; // the last thread's runs end the list
     }
     if (tid == 0) {
         int t = 0;
         for (int q = 0; q < kLenThreads / 32; ++q) t += s_frames[q];
-        *nvalid = t;
+        *p.nvalid = t;
     }
 }
 
@@ -1077,10 +1098,15 @@ ew_add_masked_kernel(T* out, const T* a, const T* b, const T* c, const int* len,
         default:  { using T = __nv_bfloat16; __VA_ARGS__; break; }          \
     }
 
-void lengths(const Launch& L, const int* len_in, int B, int T_in, int stride, int* len_out, int* nvalid, int* blk_off, int phases,
-             int* len_dense) {
-    KScope ks_(L, KC_LENGTHS, 8.0 * B * phases, 0.0);
-    launch_k(L, lengths_kernel, 1, kLenThreads, 0, len_in, B, T_in, stride, phases, len_out, nvalid, blk_off, len_dense, L.status);
+void prologue(const Launch& L, Prologue& p) {
+    double bytes = 8.0 * p.B * p.phases;
+    int blocks = 0;
+    for (int k = 0; k < p.conv.count; ++k) {
+        p.conv.first[k] = blocks;
+        blocks += (p.conv.n[k] + kConvertChunk - 1) / kConvertChunk; bytes += 4.0 * p.conv.n[k];
+    }
+    KScope ks_(L, KC_LENGTHS, bytes, 0.0);
+    launch_k(L, prologue_kernel, 1 + blocks, kLenThreads, 0, p, L.status);
     L.count();
 }
 
@@ -1240,35 +1266,6 @@ void ew_add_masked(const Launch& L, int dtype, void* out, const void* a, const v
     KScope ks_(L, KC_EW, (double)dtype_size(dtype) * B * C * Tt * (2 + (b ? 1 : 0) + (c ? 1 : 0)), 0.0);
     SC_DISPATCH(dtype, (launch_k(L, ew_add_masked_kernel<T>, (B * C + kRowsPerCta - 1) / kRowsPerCta, kRowThreads, 0, (T*)out, (const T*)a, (const T*)b,
                                                                                       (const T*)c, len, B * C, C, Tt)));
-    L.count();
-}
-
-__global__ void convert_bf16_to_f16_kernel(const __nv_bfloat16* __restrict__ src, __half* __restrict__ dst, long long n) {
-    pdl_sync();
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) dst[i] = __float2half_rn(__bfloat162float(src[i]));
-}
-void convert_bf16_to_f16(const Launch& L, const void* src, void* dst, int64_t n) {
-    KScope ks_(L, KC_EW, 4.0 * n, 0.0);
-    launch_k(L, convert_bf16_to_f16_kernel, (unsigned)((n + 255) / 256), 256, 0, (const __nv_bfloat16*)src, (__half*)dst, n);
-    L.count();
-}
-
-__global__ void convert_many_kernel(ConvertList list) {
-    pdl_sync();
-    const int item = blockIdx.y;
-    const __nv_bfloat16* src = (const __nv_bfloat16*)list.src[item];
-    __half* dst = (__half*)list.dst[item];
-    const int n = list.n[item];
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-        dst[i] = __float2half_rn(__bfloat162float(src[i]));
-}
-void convert_bf16_to_f16_many(const Launch& L, const ConvertList& list) {
-    if (list.count == 0) return;
-    double total = 0;
-    for (int i = 0; i < list.count; ++i) total += list.n[i];
-    KScope ks_(L, KC_EW, 4.0 * total, 0.0);
-    launch_k(L, convert_many_kernel, dim3(64, list.count), 256, 0, list);
     L.count();
 }
 

@@ -39,7 +39,6 @@ dw_corr_s1_kernel(const TI* __restrict__ in, const TW* __restrict__ w, TO* __res
                   const TO* __restrict__ add1, const TO* __restrict__ add2, const float* __restrict__ gmax,
                   const int* __restrict__ len_src, const int* __restrict__ len_dst,
                   int C, int Tt, int K, int Kpad, int flip, int* status) {
-    pdl_sync();
     using T = TO;
     extern __shared__ float smem[];
     const int lane = threadIdx.x, wrp = threadIdx.y;
@@ -49,6 +48,10 @@ dw_corr_s1_kernel(const TI* __restrict__ in, const TW* __restrict__ w, TO* __res
     const int XW = TT + Kpad;                 // logical tile width
     float* xs = smem + (size_t)wrp * (phys(XW) + 4 + Kpad);
     float* ws = xs + phys(XW) + 4;
+    // the taps are the caller's parameters: read ahead of the wait (zero padded to Kpad)
+    for (int k = lane; k < Kpad; k += 32)
+        ws[k] = (k < K) ? ldf(w + (size_t)c * K + (flip ? K - 1 - k : k)) : 0.f;
+    pdl_sync();
     const int ls = min(len_src[b], Tt), ld = min(len_dst[b], Tt);
     const size_t row = ((size_t)b * C + c) * Tt;
     T* orow = out + row;
@@ -61,9 +64,6 @@ dw_corr_s1_kernel(const TI* __restrict__ in, const TW* __restrict__ w, TO* __res
         else { for (int r = 0; r < R; ++r) if (t + r < Tt) stf(orow + t + r, 0.f); }
         return;
     }
-    // taps (zero padded to Kpad)
-    for (int k = lane; k < Kpad; k += 32)
-        ws[k] = (k < K) ? ldf(w + (size_t)c * K + (flip ? K - 1 - k : k)) : 0.f;
     // input tile: logical index i <-> frame tau = t0 - P + i, zero outside [0, ls)
     const TI* irow = in + row;
     const int tau0 = t0 - P;
@@ -73,7 +73,7 @@ dw_corr_s1_kernel(const TI* __restrict__ in, const TW* __restrict__ w, TO* __res
         for (int j = lane; j < nchunk; j += 32) {
             const int ta = a0 + 8 * j;
             float f[8];
-            if (ta >= 0 && ta < ls) ld8<TI>(irow + ta, f);
+            if (ta >= 0 && ta < Tt) ld8<TI>(irow + ta, f);      // not bounded by ls: the load need not wait for the length
             else {
 #pragma unroll
                 for (int e = 0; e < 8; ++e) f[e] = 0.f;

@@ -86,7 +86,6 @@ __device__ __forceinline__ void named_bar(int id, int nthreads) {
 template <typename TI, typename TW, typename TO>
 __global__ void __launch_bounds__(DT_THREADS, 1)
 dw_tma_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CUtensorMap mapO, DtParams p) {
-    pdl_launch_dependents();
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
     uint8_t* sB = smem + p.nstages * p.stage_bytes;                         // [2][b_stride], 1024-byte aligned
@@ -112,7 +111,8 @@ dw_tma_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ 
         ptx::prefetch_tensormap(&mapO);
     }
     if (warp == 0) { ptx::tmem_alloc(tmem_slot, DT_NACC * DT_ACC_COLS); ptx::tmem_relinquish(); }
-    pdl_wait();                                        // everything above overlaps the previous kernel's tail
+    // No wait for the previous kernel here: the Toeplitz builders need only the taps, which no kernel of the call writes, so
+    // the first block is built under that kernel's tail.  The roles that touch the tensors wait for it themselves.
     ptx::tc_fence_before();
     __syncthreads();
     ptx::tc_fence_after();
@@ -126,6 +126,8 @@ dw_tma_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ 
         const bool active = lane < nbox;
         const int dst_off = q * 16384 + tbl * box_bytes;
         int s = 0, ph = 0; bool dead = false;
+        pdl_wait();
+        pdl_launch_dependents();
         for (int c = blockIdx.x; c < p.C && !dead; c += gridDim.x) {
             for (int chunk = 0; chunk < p.nchunks && !dead; ++chunk) {
                 for (int g = 0; g < p.ngrp; ++g) {
@@ -218,6 +220,7 @@ dw_tma_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ 
     } else if (warp == 8) {                            // ---- input masking (warp 8): rows mt, mt + 32, mt + 64, mt + 96 ----
         if (p.mask) {
             const int mt = tid - 256;                  // 0 .. 31
+            pdl_wait();
             int s = 0, ph = 0; bool dead = false;
             for (int c = blockIdx.x; c < p.C && !dead; c += gridDim.x) {
                 for (int chunk = 0; chunk < p.nchunks && !dead; ++chunk) {
@@ -262,6 +265,7 @@ dw_tma_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ 
     } else {                                           // ---- epilogue (warps 0-7) ----
         const int wq = warp & 3, half = warp >> 2;
         uint8_t* stg = stg_all + warp * DT_STG_BYTES;
+        pdl_wait();
         const float inv = p.gmax ? 1.f / pow2_scale(*p.gmax) : 1.f;
         const bool has_add = p.add1 != nullptr || p.add2 != nullptr;
         TO* out = reinterpret_cast<TO*>(p.out);
@@ -411,7 +415,7 @@ dw_tma_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ 
             }
         }
     done:
-        ptx::bulk_wait_all();                              // this thread's output stores have completed
+        ptx::bulk_wait_read();                             // the stores have read their source; the end of the grid orders their writes
         if (amax > 65504.f) raise_status(p.status, kErrRange);
     }
     ptx::tc_fence_before();

@@ -116,7 +116,6 @@ struct Ring {
 template <typename TG, typename TX>
 __global__ void __launch_bounds__(WT_THREADS, 1)
 dw_wgrad_tc_kernel(const __grid_constant__ CUtensorMap mapG, const __grid_constant__ CUtensorMap mapX, WtParams p) {
-    pdl_launch_dependents();
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
     uint64_t* full = reinterpret_cast<uint64_t*>(smem + WT_RING_BYTES);
@@ -144,7 +143,8 @@ dw_wgrad_tc_kernel(const __grid_constant__ CUtensorMap mapG, const __grid_consta
         ptx::prefetch_tensormap(&mapG);
         ptx::prefetch_tensormap(&mapX);
     }
-    pdl_wait();                                        // the barrier set-up above overlaps the previous kernel's tail
+    // the set-up below reads the lengths only, which were settled well before the previous kernel; the roles that read or
+    // write the tensors wait for it themselves
     // longest output length in every sample chunk: time blocks past it hold only zeros of gu
     for (int ch = tid; ch < p.nchunks && ch < WT_MAX_CHUNKS; ch += WT_THREADS) {
         int m = 0;
@@ -171,6 +171,8 @@ dw_wgrad_tc_kernel(const __grid_constant__ CUtensorMap mapG, const __grid_consta
         const void* map = is_g ? (const void*)&mapG : (const void*)&mapX;
         const int dst_off = is_g ? hb * g_bytes + bx * box_bytes : 2 * g_bytes + hb * x_bytes + q * box_bytes;
         const int t_off = 128 * hb + (is_g ? 64 * bx : 64 * q - p.Pa);
+        pdl_wait();
+        pdl_launch_dependents();
         for (int unit = blockIdx.x; unit < p.units && !dead; unit += gridDim.x) {
             const int c = unit / p.S, sp = unit - c * p.S;
             StepWalk w; w.begin(sp, p.ks_per_split, ks_total, p.ntb, chunk_len);
@@ -292,6 +294,7 @@ dw_wgrad_tc_kernel(const __grid_constant__ CUtensorMap mapG, const __grid_consta
         // k = lane + 1 - delta + 32 n with n = q - 1 and n = q.
         float* stg = stg_all + warp * WT_STG_FLOATS;
         const int nq = (62 + p.delta + p.K) / 32;          // 32-column chunks this warp reads (<= 6)
+        pdl_wait();
         int j = 0;
         for (int unit = blockIdx.x; unit < p.units; unit += gridDim.x, ++j) {
             const int c = unit / p.S, sp = unit - c * p.S;

@@ -84,14 +84,26 @@ template <auto Kern> inline void set_max_smem_once(int smem) {
     if (dev >= 0 && dev < 64) done |= 1ull << dev;
 }
 
-// ---- lengths -------------------------------------------------------------------------------
-// len_out[b] = ceil(len_in[b]/stride); *nvalid = sum_b len_out[b]; flags lengths outside [1,T_in].
-// blk_off (nullable, int [B+1]): exclusive prefix sum of ceil(len_out[b] / 64), the number of 64-frame blocks
-// of each sample that hold at least one valid frame; blk_off[B] is their total.
-// phases > 1 (stride 1): sample b becomes `phases` samples b * phases + p that hold the frames p, p + phases, ... of it;
-// len_out and blk_off then have B * phases (+ 1) entries and len_dense (int [B]) receives the clamped lengths themselves.
-void lengths(const Launch& L, const int* len_in, int B, int T_in, int stride, int* len_out, int* nvalid,
-             int* blk_off = nullptr, int phases = 1, int* len_dense = nullptr);
+// ---- prologue ------------------------------------------------------------------------------
+// What a call needs before its first layer, in one launch:
+//   lengths      len_out[b] = ceil(len_in[b]/stride); *nvalid = sum_b len_out[b]; flags lengths outside [1,T_in].
+//                blk_off (nullable, int [B+1]): exclusive prefix sum of ceil(len_out[b] / 64), the number of 64-frame
+//                blocks of each sample that hold at least one valid frame; blk_off[B] is their total.
+//                phases > 1 (stride 1): sample b becomes the samples b * phases + p that hold the frames p, p + phases, ...
+//                of it; len_out and blk_off then have B * phases (+ 1) entries, and len_dense (int [B]) receives the
+//                clamped lengths themselves.  len_user (nullable, int [B]): another copy of the dense output lengths.
+//   zero         nzero floats set to zero
+//   conv         float16 copies of bfloat16 arrays (the pointwise weights of layers whose operands are float16)
+constexpr int kMaxConvert = 48;
+struct ConvertList { const void* src[kMaxConvert]; void* dst[kMaxConvert]; int n[kMaxConvert]; int first[kMaxConvert + 1]; int count; };
+struct Prologue {
+    const int* len_in = nullptr; int B = 0, T_in = 0, stride = 1, phases = 1;
+    int *len_out = nullptr, *nvalid = nullptr, *blk_off = nullptr, *len_dense = nullptr, *len_user = nullptr;
+    float* zero = nullptr; int nzero = 0;
+    ConvertList conv{};
+    void convert(const void* src, void* dst, int n) { conv.src[conv.count] = src; conv.dst[conv.count] = dst; conv.n[conv.count++] = n; }
+};
+void prologue(const Launch& L, Prologue& p);
 
 // ---- packed tensors (k_pack.cu) ---------------------------------------------------------------
 // The tensor-core kernels move rows with 16-byte copies, so they need a row length that is a multiple of 8 frames, and
@@ -174,11 +186,6 @@ size_t gemm_wgrad_simt_scratch_bytes(int B, int Cin, int Cout);
 // out[i] (+)= (sum_s partials[s*n + i]) / pow2_scale(*gmax), fixed order (gmax nullable: no scaling)
 void reduce_partials(const Launch& L, const float* partials, int nsplit, int64_t n, float* out, int accumulate,
                      const float* gmax = nullptr);
-// dst (half) = src (bf16), n elements
-void convert_bf16_to_f16(const Launch& L, const void* src, void* dst, int64_t n);
-// the same for up to 48 arrays in one launch
-struct ConvertList { const void* src[48]; void* dst[48]; int n[48]; int count; };
-void convert_bf16_to_f16_many(const Launch& L, const ConvertList& list);
 
 // ---- non-separable convolution (block variant; k_conv_simt.cu) ---------------------------------
 // w [Cout, Cin, K] and x [B, Cin, T] in `dtype`; v [B, Cout, Tp] in out_dtype (dtype, or F16 for BF16 operands).

@@ -109,7 +109,6 @@ __device__ __forceinline__ void store_block_staged(float* stg, const float (&f)[
 template <typename T, int MODE, int MT, int BN, int STAGES>
 __global__ void __launch_bounds__(kThreads, 1)
 tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, TcParams p) {
-    pdl_sync();
     constexpr int A_BYTES = MT * 128 * 128;        // MT sub-tiles of 128 rows x 128 bytes
     constexpr int B_BYTES = BN * 128;
     constexpr int STAGE = A_BYTES + B_BYTES;
@@ -136,6 +135,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
     if (!is_wgrad(MODE)) {
         if (p.len_out) len = min(p.len_out[z], p.Tp);
         if (n0 >= len) {                           // whole tile in padding
+            pdl_wait();
             if (p.zero_fill) {
                 const int esz = (MODE == MODE_FWD && p.out_kind == 1) ? 4 : (int)sizeof(T);
                 const int vec_per_row = BN * esz / 16;
@@ -175,6 +175,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
         return t0 < l;
     };
 
+    pdl_wait();                                        // the set-up above overlaps the previous kernel's tail
+    pdl_launch_dependents();
     if (warp == 0) {
         if (lane == 0) {                           // ---- TMA producer ----
             int it = 0;
@@ -639,7 +641,6 @@ template <typename T, int MODE, int MT, int NB, int NBUF, int OCC, int EPI>
 __global__ void __launch_bounds__(32 * (4 * MT * EPI + 2), OCC)
 tc_gemm_flat_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
                     const __grid_constant__ CUtensorMap mapO, FlatParams p) {
-    pdl_launch_dependents();
     static_assert(!is_wgrad(MODE), "forward / input gradient only");
     constexpr int A_BYTES = FlatCfg<MT, NB, OCC, EPI>::A_BYTES;
     constexpr int STAGE = FlatCfg<MT, NB, OCC, EPI>::STAGE;
@@ -674,7 +675,8 @@ tc_gemm_flat_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
         if (p.tma_out) ptx::prefetch_tensormap(&mapO);
     }
     if (warp == 0) { ptx::tmem_alloc(tmem_slot, TMEM_COLS); ptx::tmem_relinquish(); }
-    pdl_wait();                                   // everything above overlaps the previous kernel's tail
+    // Ahead of the wait for the previous kernel: the block offsets (the lengths were settled at least two kernels ago), and
+    // in the producer the first stages' weights.  Both latencies then overlap that kernel's last wave.
     for (int i = tid; i <= p.B; i += blockDim.x) s_off[i] = p.blk_off[i];
     ptx::tc_fence_before();
     __syncthreads();
@@ -694,6 +696,36 @@ tc_gemm_flat_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
             int it = 0, m, j, nb;
             bool dead = false;
             uint32_t pos = u_begin;
+            auto load_weights = [&](int s, int kb, int tap, int cb, int m0) {
+                uint8_t* sA = smem + s * STAGE;
+                if (is_conv(MODE)) {
+#pragma unroll
+                    for (int mt = 0; mt < MT; ++mt) ptx::tma_load_3d(sA + mt * 16384, &mapA, &full[s], cb * BK, m0 + mt * 128, tap);
+                } else if (is_fwd(MODE)) {
+#pragma unroll
+                    for (int mt = 0; mt < MT; ++mt) ptx::tma_load_2d(sA + mt * 16384, &mapA, &full[s], kb * BK, m0 + mt * 128);
+                } else {
+#pragma unroll
+                    for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+                        for (int h = 0; h < 2; ++h)
+                            ptx::tma_load_2d(sA + mt * 16384 + h * 8192, &mapA, &full[s], m0 + mt * 128 + 64 * h, kb * BK);
+                }
+            };
+            // the convolution's tap matrices may come from the kernel just before this one
+            int early = 0;
+            if (!is_conv(MODE)) {
+                uint32_t pos0 = u_begin;
+                if (flat_next_tile<NB>(pos0, u_end, nblk, m, j, nb)) {
+                    early = min(STAGES, nkb);
+                    for (int kb = 0; kb < early; ++kb) {
+                        ptx::mbar_arrive_expect_tx(&full[kb], A_BYTES + nb * 8192);
+                        load_weights(kb, kb, 0, 0, m * (128 * MT));
+                    }
+                }
+            }
+            pdl_wait();
+            pdl_launch_dependents();
             while (!dead && flat_next_tile<NB>(pos, u_end, nblk, m, j, nb)) {
                 int bb[NB], tt[NB];
                 int b = flat_find_sample(s_off, p.B, j);
@@ -708,34 +740,23 @@ tc_gemm_flat_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
                 int tap = 0, cb = 0;
                 for (int kb = 0; kb < nkb; ++kb, ++it) {
                     const int s = it % STAGES, ph = (it / STAGES) & 1;
-                    if (!ptx::mbar_wait(&empty[s], ph ^ 1)) { raise_status(p.status, kErrTimeout); dead = true; break; }
-                    ptx::mbar_arrive_expect_tx(&full[s], A_BYTES + nb * 8192);
-                    uint8_t* sA = smem + s * STAGE;
-                    uint8_t* sB = sA + A_BYTES;
-                    const int k0 = kb * BK;
+                    uint8_t* sB = smem + s * STAGE + A_BYTES;
+                    if (it >= early) {
+                        if (!ptx::mbar_wait(&empty[s], ph ^ 1)) { raise_status(p.status, kErrTimeout); dead = true; break; }
+                        ptx::mbar_arrive_expect_tx(&full[s], A_BYTES + nb * 8192);
+                        load_weights(s, kb, tap, cb, m0);
+                    }
                     if (is_conv(MODE)) {
-                        const int c0 = cb * BK, dt = p.tap_row0 + tap * p.tap_step;
-#pragma unroll
-                        for (int mt = 0; mt < MT; ++mt) ptx::tma_load_3d(sA + mt * 16384, &mapA, &full[s], c0, m0 + mt * 128, tap);
+                        const int dt = p.tap_row0 + tap * p.tap_step;
 #pragma unroll
                         for (int i = 0; i < NB; ++i)
-                            if (i < nb) ptx::tma_load_3d(sB + i * 8192, &mapB, &full[s], c0, tt[i] + dt, bb[i]);
+                            if (i < nb) ptx::tma_load_3d(sB + i * 8192, &mapB, &full[s], cb * BK, tt[i] + dt, bb[i]);
                         if (++cb == p.tap_blocks) { cb = 0; ++tap; }
-                        continue;
-                    }
-                    if (is_fwd(MODE)) {
-#pragma unroll
-                        for (int mt = 0; mt < MT; ++mt) ptx::tma_load_2d(sA + mt * 16384, &mapA, &full[s], k0, m0 + mt * 128);
                     } else {
 #pragma unroll
-                        for (int mt = 0; mt < MT; ++mt)
-#pragma unroll
-                            for (int h = 0; h < 2; ++h)
-                                ptx::tma_load_2d(sA + mt * 16384 + h * 8192, &mapA, &full[s], m0 + mt * 128 + 64 * h, k0);
+                        for (int i = 0; i < NB; ++i)
+                            if (i < nb) ptx::tma_load_3d(sB + i * 8192, &mapB, &full[s], tt[i], kb * BK, bb[i]);
                     }
-#pragma unroll
-                    for (int i = 0; i < NB; ++i)
-                        if (i < nb) ptx::tma_load_3d(sB + i * 8192, &mapB, &full[s], tt[i], k0, bb[i]);
                 }
             }
         }
@@ -787,6 +808,7 @@ tc_gemm_flat_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
                                                       // 2 * block + half belongs to the warp with hsel == chunk % EPI
         uint8_t* stg = stg_all + warp * p.stg_stride;
         uint32_t nstore = 0;                          // TMA stores issued by this warp
+        pdl_wait();
         if (p.zero_fill) {
             // blocks wholly in padding: sample b's blocks [off[b+1]-off[b], nbT); CTAs share them round-robin
             const int inv_per_m = p.B * p.nbT - nblk;
@@ -855,8 +877,6 @@ tc_gemm_flat_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
             if (m != cur_m) { flush_stats(); cur_m = m; sn = sd = sq = 0.f; }
             const int buf = jt % NBUF;
             if (dead) { ++jt; continue; }
-            if (!ptx::mbar_wait_warp(&acc_full[buf], (jt / NBUF) & 1)) { if (lane == 0) raise_status(p.status, kErrTimeout); dead = true; ++jt; continue; }
-            ptx::tc_fence_after();
             const int row_w = m * (128 * MT) + mt * 128 + wq * 32;
             const int row = row_w + lane;
             const float bias = (is_fwd(MODE) && p.bias && row < p.M) ? p.bias[row] : 0.f;
@@ -864,6 +884,8 @@ tc_gemm_flat_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
             if (MODE == MODE_AFFINE && row < p.M) {
                 mu = p.aff.mean[row]; is = 1.f / sqrtf(p.aff.var[row] + p.aff.eps); ga = p.aff.gamma[row]; be = p.aff.beta[row];
             }
+            if (!ptx::mbar_wait_warp(&acc_full[buf], (jt / NBUF) & 1)) { if (lane == 0) raise_status(p.status, kErrTimeout); dead = true; ++jt; continue; }
+            ptx::tc_fence_after();
             int b = flat_find_sample(s_off, p.B, j);
             for (int i = 0; i < nb; ++i) {
                 while (j + i >= s_off[b + 1]) ++b;
@@ -981,7 +1003,7 @@ tc_gemm_flat_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
             ++jt;
         }
         flush_stats();
-        if (p.tma_out && lane == 0) ptx::bulk_wait_all();     // this thread's stores have completed
+        if (p.tma_out && lane == 0) ptx::bulk_wait_read();    // the stores have read their staging buffers; the end of the grid orders their writes
     }
     ptx::tc_fence_before();
     __syncthreads();
