@@ -12,8 +12,11 @@
 // 128-byte swizzle; frames outside [0, T) are zero-filled by the TMA unit, which is the "same" padding.
 // Each input element is read from HBM once (window overlaps hit L2).  Rows of a tile are
 // (time block within a group of 128/BB, sample within a chunk of BB).
-// Warps: 0-7 epilogue (TMEM lane quarter w%4, column half w/4), 8 input masking (only when the input
-// may be non-zero beyond a sample's length), 10-13 Toeplitz builders, 14 TMA producer (one box per lane),
+// Warps: 0-7 epilogue (TMEM lane quarter w%4, column half w/4), 8 idle, 10-13 Toeplitz builders, which also
+// mask the input when it may be non-zero beyond a sample's length (they walk the rows that need it, one 16-byte vector per
+// lane, and build the next channel's block after a channel's tiles; with one warp and a row per lane a masked tile took
+// 12 k cycles, several times its loads and MMAs: a ragged fp16 block of 32 x 400 frames 102.2 -> 100.0 us, the projected
+// bf16 one 176.9 -> 171.6), 14 TMA producer (one box per lane),
 // 15 and 9 MMA issuers for the even and odd tiles (a tile costs its issuer about twenty barrier, MMA and
 // commit instructions of a hundred cycles or more each, so two issuers alternate; their tiles use
 // different accumulators and stages).  Accumulators are quadruple-buffered in tensor memory.  In the epilogue a
@@ -58,7 +61,6 @@ struct DtParams {
     int ntb, ngrp, nchunks, tpc;   // time blocks, groups, sample chunks, tiles per channel
     int nstages, stage_bytes;
     int b_stride;         // bytes per Toeplitz buffer: 64 rows x 128 bytes per 64-element chunk of NK2
-    int mask;             // 1: zero input frames at or beyond len_src
     int flip;             // 1: taps reversed (input gradient)
 };
 
@@ -82,8 +84,9 @@ __device__ __forceinline__ void named_bar(int id, int nthreads) {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
 }
 
-// TI: type of the input tensor and of both MMA operands; TW: stored tap type; TO: output / addend type.
-template <typename TI, typename TW, typename TO>
+// TI: type of the input tensor and of both MMA operands; TW: stored tap type; TO: output / addend type; MASK: the
+// input may be non-zero at and beyond a sample's length.
+template <typename TI, typename TW, typename TO, bool MASK>
 __global__ void __launch_bounds__(DT_THREADS, 1)
 dw_tma_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CUtensorMap mapO, DtParams p) {
     extern __shared__ uint8_t smem_raw[];
@@ -103,7 +106,7 @@ dw_tma_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ 
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     if (tid == 0) {
-        for (int s = 0; s < DT_MAX_STAGES; ++s) { ptx::mbar_init(&full[s], 1); ptx::mbar_init(&prep[s], 1); ptx::mbar_init(&empty[s], 1); }
+        for (int s = 0; s < DT_MAX_STAGES; ++s) { ptx::mbar_init(&full[s], 1); ptx::mbar_init(&prep[s], 4); ptx::mbar_init(&empty[s], 1); }
         for (int i = 0; i < DT_NACC; ++i) { ptx::mbar_init(&acc_full[i], 1); ptx::mbar_init(&acc_empty[i], 256); }
         for (int i = 0; i < 2; ++i) { ptx::mbar_init(&b_full[i], 4); ptx::mbar_init(&b_empty[i], 2); }
         ptx::fence_barrier_init();
@@ -160,7 +163,7 @@ dw_tma_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ 
                     if ((j & 1) != mine) { if (++s == p.nstages) { s = 0; ph ^= 1; } continue; }
                     const int buf = j & (DT_NACC - 1);
                     if (!ptx::mbar_wait(&acc_empty[buf], ((j / DT_NACC) & 1) ^ 1)) { raise_status(p.status, kErrTimeout); dead = true; break; }
-                    if (!ptx::mbar_wait(p.mask ? &prep[s] : &full[s], ph)) { raise_status(p.status, kErrTimeout); dead = true; break; }
+                    if (!ptx::mbar_wait(MASK ? &prep[s] : &full[s], ph)) { raise_status(p.status, kErrTimeout); dead = true; break; }
                     ptx::tc_fence_after();
                     const uint32_t aA = smem_a + s * p.stage_bytes, aB = smem_b + bb * p.b_stride;
                     const uint64_t dB0 = dk | (uint64_t)((aB & 0x3FFFFu) >> 4);
@@ -191,8 +194,8 @@ dw_tma_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ 
         // index, so rows with an odd base read the copy that is shifted by one element
         const int base = DT_WOFF - j - p.delta;
         const uint32_t* src0 = reinterpret_cast<const uint32_t*>((base & 1) ? (wpadO + base - 1) : (wpadE + base));
-        int ci = 0; bool dead = false;
-        for (int c = blockIdx.x; c < p.C && !dead; c += gridDim.x, ++ci) {
+        // `ok` is false once a wait of this warp has run out: it then only meets the named barriers
+        auto build = [&](int c, int ci, bool ok) -> bool {
             const int bb = ci & 1;
             named_bar(2, 128);                         // everyone is done reading the previous channel's taps
             for (int i = bt; i < DT_WLEN; i += 128) {
@@ -205,8 +208,8 @@ dw_tma_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ 
                 if (i == DT_WLEN - 1) wpadO[i] = 0;
             }
             named_bar(2, 128);
-            const bool ok = ptx::mbar_wait_warp(&b_empty[bb], ((ci >> 1) & 1) ^ 1, 32);
-            if (!ok) { if (lane == 0) raise_status(p.status, kErrTimeout); dead = true; break; }
+            if (!ok) return false;
+            if (!ptx::mbar_wait_warp(&b_empty[bb], ((ci >> 1) & 1) ^ 1, 32)) { if (lane == 0) raise_status(p.status, kErrTimeout); return false; }
             uint4* rowbase = reinterpret_cast<uint4*>(sB + bb * p.b_stride + j * 128);
             for (int v = hv; v < nvec; v += 2) {       // vector v holds j' = 8 v .. 8 v + 7
                 const uint32_t* src = src0 + 4 * v;
@@ -216,42 +219,32 @@ dw_tma_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ 
             ptx::fence_proxy_async();
             __syncwarp();
             if (lane == 0) ptx::mbar_arrive(&b_full[bb]);
-        }
-    } else if (warp == 8) {                            // ---- input masking (warp 8): rows mt, mt + 32, mt + 64, mt + 96 ----
-        if (p.mask) {
-            const int mt = tid - 256;                  // 0 .. 31
-            pdl_wait();
-            int s = 0, ph = 0; bool dead = false;
-            for (int c = blockIdx.x; c < p.C && !dead; c += gridDim.x) {
-                for (int chunk = 0; chunk < p.nchunks && !dead; ++chunk) {
-                    for (int g = 0; g < p.ngrp; ++g) {
-                        const bool ok = ptx::mbar_wait_warp(&full[s], ph);
-                        if (!ok) { if (lane == 0) raise_status(p.status, kErrTimeout); dead = true; break; }
-                        bool wrote = false;
-#pragma unroll 1
-                        for (int rsel = 0; rsel < 4; ++rsel) {
-                            const int r = mt + 32 * rsel;
-                            const int tbl = r / p.BB, bi = r - tbl * p.BB;
-                            const int b = chunk * p.BB + bi;
-                            const int len = b < p.B ? min(p.len_src[b], p.T) : 0;
-                            const int t0 = 128 * (g * p.TBL + tbl) - p.Pa;      // first frame of this row's window
-                            if (t0 + 64 * p.nxb <= len) continue;
-                            uint8_t* row = smem + s * p.stage_bytes + r * 128;
-                            for (int v = 0; v < 8 * p.nxb; ++v) {
-                                const int t = t0 + 8 * v;                    // logical vector v: frames t .. t + 7
-                                if (t + 8 <= len) continue;
-                                uint4* pv = reinterpret_cast<uint4*>(row + (v >> 3) * 16384) + ((v & 7) ^ (r & 7));
-                                wrote = true;
-                                if (t >= len) { *pv = make_uint4(0, 0, 0, 0); continue; }
-                                uint4 x = *pv;
-                                uint32_t wv[4] = {x.x, x.y, x.z, x.w};
-                                const int nv = len - t;
-#pragma unroll
-                                for (int i = 0; i < 4; ++i) {
-                                    if (2 * i >= nv) wv[i] = 0u;
-                                    else if (2 * i + 1 >= nv) wv[i] &= 0x0000FFFFu;
-                                }
-                                *pv = make_uint4(wv[0], wv[1], wv[2], wv[3]);
+            return true;
+        };
+        const int r0 = 32 * (warp - 10), lb = p.BB == 32 ? 5 : 4;      // masking: this warp's 32 tile rows
+        const int tbl0 = (r0 + lane) >> lb, bi = (r0 + lane) & (p.BB - 1);
+        int ci = 0, s = 0, ph = 0;
+        bool ok = true;
+        for (int c = blockIdx.x; c < p.C; c += gridDim.x, ++ci) {
+            if (!MASK || ci == 0) ok = build(c, ci, ok);
+            if (MASK) {
+                if (ci == 0) pdl_wait();
+                for (int chunk = 0; chunk < p.nchunks && ok; ++chunk) {
+                    const int b = chunk * p.BB + bi;
+                    const int len = b < p.B ? min(p.len_src[b], p.T) : 0;               // of this lane's row
+                    for (int g = 0; g < p.ngrp && ok; ++g) {
+                        const int left = len - (128 * (g * p.TBL + tbl0) - p.Pa);       // valid frames from the window's start
+                        uint32_t todo = __ballot_sync(0xffffffffu, left < 64 * p.nxb);
+                        const bool wrote = todo != 0;
+                        ok = ptx::mbar_wait_warp(&full[s], ph);
+                        if (!ok) { if (lane == 0) raise_status(p.status, kErrTimeout); break; }
+                        uint8_t* tile = smem + s * p.stage_bytes + (lane >> 3) * 16384;
+                        for (; todo; todo &= todo - 1) {
+                            const int rr = __ffs(todo) - 1, r = r0 + rr;
+                            const int n = __shfl_sync(0xffffffffu, left, rr) - 8 * lane;   // valid frames of vector `lane`
+                            if (lane < 8 * p.nxb && n < 8) {
+                                uint4* pv = reinterpret_cast<uint4*>(tile + r * 128) + ((lane & 7) ^ (r & 7));
+                                *pv = n <= 0 ? make_uint4(0, 0, 0, 0) : keep_first(*pv, n);
                             }
                         }
                         if (wrote) ptx::fence_proxy_async();
@@ -261,8 +254,9 @@ dw_tma_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ 
                     }
                 }
             }
+            if (MASK && c + gridDim.x < p.C) ok = build(c + gridDim.x, ci + 1, ok);
         }
-    } else {                                           // ---- epilogue (warps 0-7) ----
+    } else if (warp < 8) {                                           // ---- epilogue (warps 0-7) ----
         const int wq = warp & 3, half = warp >> 2;
         uint8_t* stg = stg_all + warp * DT_STG_BYTES;
         pdl_wait();
@@ -427,10 +421,14 @@ constexpr int kDtSmem = 1024 + DT_AB_BYTES + 8 * DT_STG_BYTES + 2 * DT_WLEN * 2 
 static_assert(kDtSmem <= 232448, "shared memory per CTA");
 
 template <typename TI, typename TW, typename TO>
-void launch_dt(const Launch& L, int grid, const CUtensorMap& mx, const CUtensorMap& mo, const DtParams& p) {
-    auto kern = dw_tma_kernel<TI, TW, TO>;
-    set_max_smem_once<dw_tma_kernel<TI, TW, TO>>(kDtSmem);
-    launch_k(L, kern, grid, DT_THREADS, kDtSmem, mx, mo, p);
+void launch_dt(const Launch& L, int grid, const CUtensorMap& mx, const CUtensorMap& mo, const DtParams& p, bool mask) {
+    if (mask) {
+        set_max_smem_once<dw_tma_kernel<TI, TW, TO, true>>(kDtSmem);
+        launch_k(L, dw_tma_kernel<TI, TW, TO, true>, grid, DT_THREADS, kDtSmem, mx, mo, p);
+    } else {
+        set_max_smem_once<dw_tma_kernel<TI, TW, TO, false>>(kDtSmem);
+        launch_k(L, dw_tma_kernel<TI, TW, TO, false>, grid, DT_THREADS, kDtSmem, mx, mo, p);
+    }
     L.count();
 }
 
@@ -452,17 +450,17 @@ void run(const TcState* st, const Launch& L, int in_dtype, int w_dtype, int out_
     p.stage_bytes = p.nxb * 16384;
     p.b_stride = ((p.NK2 + 63) / 64) * 8192;
     p.nstages = std::min(DT_MAX_STAGES, (DT_AB_BYTES - 2 * p.b_stride) / p.stage_bytes);
-    p.mask = mask; p.flip = flip;
+    p.flip = flip;
     CUtensorMap mx;
     const uint64_t dims[3] = {(uint64_t)T, (uint64_t)C, (uint64_t)B};
     const uint32_t box[3] = {64, 1, (uint32_t)p.BB};
     CUtensorMap mo;
     if (!tc_make_map(st, &mx, in_dtype, in, 3, dims, box) || !tc_make_map(st, &mo, out_dtype, out, 3, dims, box)) return;
     const int grid = std::min(std::max(1, st->sm_count), C);
-    if (in_dtype == F16 && w_dtype == F16) launch_dt<__half, __half, __half>(L, grid, mx, mo, p);
-    else if (in_dtype == F16 && out_dtype == BF16) launch_dt<__half, __nv_bfloat16, __nv_bfloat16>(L, grid, mx, mo, p);
-    else if (out_dtype == F16) launch_dt<__nv_bfloat16, __nv_bfloat16, __half>(L, grid, mx, mo, p);
-    else launch_dt<__nv_bfloat16, __nv_bfloat16, __nv_bfloat16>(L, grid, mx, mo, p);
+    if (in_dtype == F16 && w_dtype == F16) launch_dt<__half, __half, __half>(L, grid, mx, mo, p, mask != 0);
+    else if (in_dtype == F16 && out_dtype == BF16) launch_dt<__half, __nv_bfloat16, __nv_bfloat16>(L, grid, mx, mo, p, mask != 0);
+    else if (out_dtype == F16) launch_dt<__nv_bfloat16, __nv_bfloat16, __half>(L, grid, mx, mo, p, mask != 0);
+    else launch_dt<__nv_bfloat16, __nv_bfloat16, __nv_bfloat16>(L, grid, mx, mo, p, mask != 0);
 }
 
 }  // namespace
