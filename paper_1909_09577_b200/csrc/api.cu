@@ -26,7 +26,7 @@ struct sc_ctx {
     // residual projection's contraction) run there, forked from and joined back into the caller's stream with
     // events, so that they fill the SMs a latency-bound kernel of the critical path leaves idle.
     cudaStream_t side = nullptr;
-    cudaEvent_t ev[8] = {};     // backward fork, (unused), done[0], done[1], forward fork, forward join, done[2], (unused)
+    cudaEvent_t ev[8] = {};     // backward fork (and the tap gradients' of a block call), done[0], done[1], forward fork, forward join, done[2], (unused)
     int overlap = 1;
     int pdl = 1;          // launch kernels with programmatic stream serialization
     GraphCache graphs;
@@ -444,6 +444,7 @@ struct BwdIO {
     const int* len_in; const int* len_out; const int* nvalid; const int* blk_off;
     bool x_clean, res_clean;
     const void* w16;             // float16 copy of wp (see BlockIO)
+    bool fork_early;             // a single block: nothing follows that the weight gradients could overlap
     cudaEvent_t done;            // recorded on the side stream after this layer's last side-stream kernel
     int phases, Td; uint32_t total_dense;      // packed block: dy, y and the saved v, vr are dense [., ., Td]; the rest is packed
     float* gmax;                 // where the bound on |gv| collects; already zero
@@ -495,10 +496,10 @@ int block_bwd_impl(sc_ctx* ctx, const Launch& L, const sc_block_desc* d, const D
     // program order, and kernels of the critical path that sit behind side-stream launches in that order start late
     // whenever the GPU is ahead of the host.  One event, recorded behind this layer's last main-stream kernel, releases
     // them (an event between two kernels ends the programmatic overlap of that pair, so there is only one per layer);
-    // they then overlap the next layer's main-stream kernels.
+    // they then overlap the next layer's main-stream kernels.  A block call has no next layer: there they are released as
+    // soon as their operands are complete and overlap this block's own input-gradient kernels.
     const Launch Ls = side_launch(ctx, L);
-    auto weight_gradients = [&]() {
-        fork_to_side(ctx, L, ctx->ev[0]);               // gv, gvr, gu and the half copies are complete
+    auto pointwise_weight_gradients = [&]() {
         const void* u = d->has_dw ? sv->u : (io.x_clean ? io.x : sv->u);
         if (conv_tc) {
             to_time_major(Ls, io.x, s.x_tm, io.len_in, m.B, m.Cin, m.T);
@@ -522,6 +523,8 @@ int block_bwd_impl(sc_ctx* ctx, const Launch& L, const sc_block_desc* d, const D
                 pointwise_wgrad(ctx, Ls, dt, s.gvr, xr, g->dwr, s.wpart, acc, m.B, m.Cres, m.Cout, m.Tp, io.len_out, nullptr);
             }
         }
+    };
+    auto tap_gradients = [&]() {
         if (d->has_dw && !m.full) {
             if (ctx->gemm_mode == 0 && m.plain && dw_wgrad_tc_supported(&ctx->tc, dt, m.B, m.T, m.K, m.s))
                 dw_wgrad_tc(&ctx->tc, Ls, dt, odt, s.gu, io.x, g->dwd, s.wpart, acc, gmax, io.len_in, io.len_out, m.B, m.Cin,
@@ -531,6 +534,10 @@ int block_bwd_impl(sc_ctx* ctx, const Launch& L, const sc_block_desc* d, const D
         }
     };
 
+    if (io.fork_early) {
+        fork_to_side(ctx, L, ctx->ev[0]);               // gv, gvr and the half copies are complete
+        pointwise_weight_gradients();
+    }
     const void* wp_op = p->wp;
     if (needs_w16(d, m)) wp_op = io.w16;
     const void* extra = nullptr;    // residual-path gradient to fold into dx
@@ -555,6 +562,10 @@ int block_bwd_impl(sc_ctx* ctx, const Launch& L, const sc_block_desc* d, const D
         }
     } else if (d->has_dw) {
         pointwise_dgrad(ctx, L, odt, wp_op, s.gv, s.gu, m.B, m.Cin, m.Cout, m.Tp, io.len_out, io.blk_off);
+        if (io.fork_early) {
+            fork_to_side(ctx, L, ctx->ev[1]);           // gu is complete
+            tap_gradients();
+        }
         if (io.dx) {
             if (ctx->gemm_mode == 0 && m.plain && dw_tma_supported(&ctx->tc, dt, m.B, m.T, m.K, m.s))
                 dw_tma_dgrad(&ctx->tc, L, dt, odt, s.gu, p->wd, io.dx, io.dx_add, extra, gmax, io.len_in, io.len_out, m.B,
@@ -571,7 +582,11 @@ int block_bwd_impl(sc_ctx* ctx, const Launch& L, const sc_block_desc* d, const D
             ew_add_masked(L, dt, io.dx, s.gu, io.dx_add, extra, io.len_in, m.B, m.Cin, m.T);
         }
     }
-    weight_gradients();
+    if (!io.fork_early) {
+        fork_to_side(ctx, L, ctx->ev[0]);               // gv, gvr, gu and the half copies are complete
+        pointwise_weight_gradients();
+        tap_gradients();
+    }
     // the caller joins: it waits for io.done on its stream before it reuses this scratch or returns
     if (io.done) record_side(ctx, io.done);
     return SC_OK;
@@ -958,7 +973,7 @@ int bwd_call(sc_ctx* ctx, const Launch& L, const sc_block_desc* desc, const sc_t
     io.dx_add = dx_add ? dx_add->ptr : nullptr;
     io.len_in = lengths_dev; io.len_out = s.len_out; io.nvalid = s.nvalid; io.blk_off = s.blk_off;
     io.x_clean = false; io.res_clean = false;
-    io.done = ctx->ev[2];
+    io.done = ctx->ev[2]; io.fork_early = true;
     sc_block_saved sv = *saved;
     if (pk.phases) {
         // packs what the contractions read; the batch-norm kernels read dy, y, v and vr as they are

@@ -206,12 +206,12 @@ bn_finalize_kernel(const float2* __restrict__ partials, int parts_per_b, int til
 // The same merge for the per-(CTA, channel) partials (count, sum, M2) of the flattened-block contraction.
 // CTA c of the contraction contributed to M tile m iff its unit range [c U / G, (c+1) U / G) meets
 // [m nblk, (m+1) nblk); the pivot is the mean of the first contributing CTA's partial.
+constexpr int kFlatParts = 10;        // partials per lane: the contraction has at most 320 CTAs
 __global__ void __launch_bounds__(32 * kFinWarps)
 bn_finalize_flat_kernel(const float4* __restrict__ partials, int G, int tiles_m, int rows_per_tile,
                         const int* __restrict__ blk_off, const int* __restrict__ nvalid, int B, int C, float eps,
                         float momentum, float* __restrict__ mean_out, float* __restrict__ invstd_out,
                         float* running_mean, float* running_var) {
-    pdl_sync();
     __shared__ float2 s_red[kFinWarps][32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int o = blockIdx.x * 32 + lane;
@@ -229,31 +229,34 @@ bn_finalize_flat_kernel(const float4* __restrict__ partials, int G, int tiles_m,
     };
     int c_first = U > 0 ? (small ? (int)((uint32_t)lo * (uint32_t)G / (uint32_t)U) : (int)(lo * G / U)) : 0;
     while (c_first < G - 1 && !takes_part(c_first)) ++c_first;
-    float pivot = 0.f;
-    if (act && U > 0) { const float4 pv = partials[(size_t)c_first * C + o]; pivot = pv.x > 0.f ? pv.y / pv.x : 0.f; }
+    // everything above works on the lengths alone and runs ahead of the wait for the contraction; after it the pivot and
+    // the partials are one round of independent loads
+    uint32_t part = 0;
+#pragma unroll
+    for (int i = 0; i < kFlatParts; ++i) {
+        const int c = w + i * kFinWarps;
+        if (act && U > 0 && c < G && takes_part(c)) part |= 1u << i;
+    }
+    const float N = (float)(*nvalid);
+    pdl_sync();
+    float4 pv = make_float4(0.f, 0.f, 0.f, 0.f), v[kFlatParts];
+    if (act && U > 0) pv = partials[(size_t)c_first * C + o];
+#pragma unroll
+    for (int i = 0; i < kFlatParts; ++i)
+        v[i] = (part >> i) & 1 ? partials[(size_t)(w + i * kFinWarps) * C + o] : make_float4(0.f, 0.f, 0.f, 0.f);
+    const float pivot = pv.x > 0.f ? pv.y / pv.x : 0.f;
     float s1 = 0.f, q = 0.f;
-    if (act && U > 0) {
-        for (int c0 = w; c0 < G; c0 += 8 * kFinWarps) {
-            float4 v[8];
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {        // issue every load before the first use
-                const int c = c0 + i * kFinWarps;
-                v[i] = (c < G && takes_part(c)) ? partials[(size_t)c * C + o] : make_float4(0.f, 0.f, 0.f, 0.f);
-            }
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                if (v[i].x > 0.f) {
-                    const float d = v[i].y / v[i].x - pivot;
-                    s1 += v[i].y;
-                    q += fmaf(v[i].x * d, d, v[i].z);
-                }
-            }
+    for (int i = 0; i < kFlatParts; ++i) {
+        if (v[i].x > 0.f) {
+            const float d = v[i].y / v[i].x - pivot;
+            s1 += v[i].y;
+            q += fmaf(v[i].x * d, d, v[i].z);
         }
     }
     s_red[w][lane] = make_float2(s1, q);
     __syncthreads();
     if (w != 0 || !act) return;
-    const float N = (float)(*nvalid);
     float t = 0.f, m2 = 0.f;
 #pragma unroll
     for (int i = 0; i < kFinWarps; ++i) { t += s_red[i][lane].x; m2 += s_red[i][lane].y; }
@@ -743,7 +746,6 @@ __device__ __forceinline__ void reduce_vec(const BnBwdArgs& a, int o, int n, con
 // l, l + 32, ...: no row tails, and V independent 16-byte loads per tensor in flight per thread.
 template <typename T, typename NT, int RES, int V>
 __global__ void __launch_bounds__(256) bn_apply_fast_kernel(ApplyArgs a, int vpr, long long total) {
-    pdl_sync();
     const uint32_t tid = blockIdx.x * 256u + threadIdx.x;        // the launcher guarantees total < 2^31
     const uint32_t base = (tid >> 5) * (32u * V) + (threadIdx.x & 31), tot = (uint32_t)total;
     size_t off[V]; int nin[V], ch[V];
@@ -759,11 +761,15 @@ __global__ void __launch_bounds__(256) bn_apply_fast_kernel(ApplyArgs a, int vpr
             ch[j] = row - b * a.C;
             nin[j] = max(0, min(a.len_out[b], a.Tp) - t0);
             off[j] = (size_t)row * a.Tp + t0;
-            if (nin[j] > 0) {
-                rv[j] = *reinterpret_cast<const uint4*>((const NT*)a.v + off[j]);
-                if (RES == 1) rr[j] = *reinterpret_cast<const uint4*>((const T*)a.xres + off[j]);
-                if (RES == 2) rr[j] = *reinterpret_cast<const uint4*>((const NT*)a.vr + off[j]);
-            }
+        }
+    }
+    pdl_sync();              // indices and lengths (settled well before the previous kernel) are worked out ahead of the wait
+#pragma unroll
+    for (int j = 0; j < V; ++j) {
+        if (nin[j] > 0) {
+            rv[j] = *reinterpret_cast<const uint4*>((const NT*)a.v + off[j]);
+            if (RES == 1) rr[j] = *reinterpret_cast<const uint4*>((const T*)a.xres + off[j]);
+            if (RES == 2) rr[j] = *reinterpret_cast<const uint4*>((const NT*)a.vr + off[j]);
         }
     }
 #pragma unroll
@@ -867,30 +873,35 @@ __device__ __forceinline__ uint4 bwd_load(const BnBwdArgs& a, const void* src, s
 
 template <typename T, typename NT, typename GT, int RES, int V, int G>
 __global__ void __launch_bounds__(256) bn_bwd_apply_fast_kernel(BnBwdArgs a, int vpr, long long total) {
-    pdl_sync();
     const uint32_t tid = blockIdx.x * 256u + threadIdx.x;        // the launcher guarantees total < 2^31
     const uint32_t base = (tid >> 5) * (32u * V) + (threadIdx.x & 31), tot = (uint32_t)total;
-    const float sc = a.gmax ? pow2_scale(*a.gmax) : 1.f;          // multiplying by it is exact: a power of two
     const bool fold = !a.gv16 && a.gv_scaled;
-    size_t off[V]; int nin[V], ch[V];
+    size_t off[V]; int nin[V], ch[V], bs[V], t0s[V];
     uint4 rg[V], rv[V], rr[V], ry[V];
 #pragma unroll
     for (int j = 0; j < V; ++j) {
         const uint32_t idx = base + 32u * j;
-        nin[j] = -1; ch[j] = 0; off[j] = 0;
+        nin[j] = -1; ch[j] = 0; off[j] = 0; bs[j] = 0; t0s[j] = 0;
         rg[j] = rv[j] = rr[j] = ry[j] = make_uint4(0, 0, 0, 0);
         if (idx < tot) {
-            const int row = (int)a.dvpr.div(idx), t0 = ((int)idx - row * vpr) * 8;
-            const int b = (int)a.dC.div((uint32_t)row);
-            ch[j] = row - b * a.C;
-            nin[j] = max(0, min(a.len_out[b], a.Tp) - t0);        // frames of this vector inside the sample
-            off[j] = (size_t)row * a.Tp + t0;
-            if (nin[j] > 0) {
-                rg[j] = bwd_load<G>(a, a.g, off[j], b, ch[j], t0, nin[j]);
-                rv[j] = bwd_load<G>(a, a.v, off[j], b, ch[j], t0, nin[j]);
-                if (RES == 2) rr[j] = bwd_load<G>(a, a.vr, off[j], b, ch[j], t0, nin[j]);
-                if (RES != 0) ry[j] = bwd_load<G>(a, a.y, off[j], b, ch[j], t0, nin[j]);
-            }
+            const int row = (int)a.dvpr.div(idx);
+            t0s[j] = ((int)idx - row * vpr) * 8;
+            bs[j] = (int)a.dC.div((uint32_t)row);
+            ch[j] = row - bs[j] * a.C;
+            nin[j] = max(0, min(a.len_out[bs[j]], a.Tp) - t0s[j]);        // frames of this vector inside the sample
+            off[j] = (size_t)row * a.Tp + t0s[j];
+        }
+    }
+    pdl_sync();              // as in the forward apply step
+    const float sc = a.gmax ? pow2_scale(*a.gmax) : 1.f;          // multiplying by it is exact: a power of two
+#pragma unroll
+    for (int j = 0; j < V; ++j) {
+        if (nin[j] > 0) {
+            const int b = bs[j], t0 = t0s[j];
+            rg[j] = bwd_load<G>(a, a.g, off[j], b, ch[j], t0, nin[j]);
+            rv[j] = bwd_load<G>(a, a.v, off[j], b, ch[j], t0, nin[j]);
+            if (RES == 2) rr[j] = bwd_load<G>(a, a.vr, off[j], b, ch[j], t0, nin[j]);
+            if (RES != 0) ry[j] = bwd_load<G>(a, a.y, off[j], b, ch[j], t0, nin[j]);
         }
     }
 #pragma unroll
@@ -979,7 +990,6 @@ template <typename T, typename NT, int RES, int G>
 __global__ void __launch_bounds__(kChThreads, 2)
 bn_bwd_reduce_ch_kernel(BnBwdArgs a, int vpr, const float* gamma_r, float* dgamma, float* dbeta, float* dgamma_r,
                         float* dbeta_r, int accumulate) {
-    pdl_sync();
     constexpr int NT_ = kChThreads;
     constexpr int U = RES == 2 ? 2 : 4;            // 16-byte loads in flight per thread: U * (2 or 4 tensors)
     __shared__ float4 s_sum[NT_ / 32];
@@ -988,6 +998,7 @@ bn_bwd_reduce_ch_kernel(BnBwdArgs a, int vpr, const float* gamma_r, float* dgamm
     c.mu = a.mean[o]; c.is = a.invstd[o];
     if (RES == 0) { c.ga = a.gamma[o]; c.be = a.beta[o]; }
     if (RES == 2) { c.mur = a.mean_r[o]; c.isr = a.invstd_r[o]; }
+    pdl_sync();              // the coefficients above come from the forward pass and the caller's parameters
     const int nvec = a.B * vpr;
     float s0 = 0.f, s1 = 0.f, s3 = 0.f, amax = 0.f;
     for (int jb = tid; jb < nvec; jb += U * NT_) {

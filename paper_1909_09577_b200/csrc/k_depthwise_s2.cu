@@ -37,7 +37,6 @@ template <typename T, typename TO>
 __global__ void __launch_bounds__(32 * CH)
 dw_s2_fwd_kernel(const T* __restrict__ x, const T* __restrict__ w, TO* __restrict__ u, const int* __restrict__ len_in,
                  const int* __restrict__ len_out, int C, int Tt, int Tp, int K, int Kh, int* status) {
-    pdl_sync();
     extern __shared__ float smem[];
     const int lane = threadIdx.x, wrp = threadIdx.y;
     const int b = blockIdx.z, c = blockIdx.y * CH + wrp, t0 = blockIdx.x * TT;
@@ -47,6 +46,11 @@ dw_s2_fwd_kernel(const T* __restrict__ x, const T* __restrict__ w, TO* __restric
     float* xo = xe + XP;                                     // frames 2 t0 - P + 2 i + 1
     float* we = xo + XP;                                     // even taps, then odd taps, zero padded to Kh each
     float* wo = we + Kh;
+    for (int j = lane; j < Kh; j += 32) {
+        we[j] = 2 * j < K ? ldf(w + (size_t)c * K + 2 * j) : 0.f;
+        wo[j] = 2 * j + 1 < K ? ldf(w + (size_t)c * K + 2 * j + 1) : 0.f;
+    }
+    pdl_sync();                               // the taps are the caller's parameters
     const int li = min(len_in[b], Tt), lo = min(len_out[b], Tp);
     TO* urow = u + ((size_t)b * C + c) * Tp;
     const int t = t0 + lane * R;
@@ -55,15 +59,11 @@ dw_s2_fwd_kernel(const T* __restrict__ x, const T* __restrict__ w, TO* __restric
         if (t < Tp) st8<TO>(urow + t, z);
         return;
     }
-    for (int j = lane; j < Kh; j += 32) {
-        we[j] = 2 * j < K ? ldf(w + (size_t)c * K + 2 * j) : 0.f;
-        wo[j] = 2 * j + 1 < K ? ldf(w + (size_t)c * K + 2 * j + 1) : 0.f;
-    }
     const T* xrow = x + ((size_t)b * C + c) * Tt;
     const int tau0 = 2 * t0 - P, a0 = tau0 & ~7;             // arithmetic: rounds towards minus infinity
     for (int ta = a0 + 8 * lane; ta < tau0 + 2 * XW; ta += 256) {
         float f[8] = {};
-        if (ta >= 0 && ta < li) ld8<T>(xrow + ta, f);
+        if (ta >= 0 && ta < Tt) ld8<T>(xrow + ta, f);          // not bounded by li: need not wait for it
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
             const int i = ta + e - tau0;
@@ -107,7 +107,6 @@ __global__ void __launch_bounds__(32 * CH)
 dw_s2_dgrad_kernel(const TG* __restrict__ gu, const T* __restrict__ w, T* __restrict__ dx, const T* __restrict__ add1,
                    const T* __restrict__ add2, const float* __restrict__ gmax, const int* __restrict__ len_in,
                    const int* __restrict__ len_out, int C, int Tt, int Tp, int K, int Kh) {
-    pdl_sync();
     extern __shared__ float smem[];
     const int lane = threadIdx.x, wrp = threadIdx.y;
     const int b = blockIdx.z, c = blockIdx.y * CH + wrp, i0 = blockIdx.x * TT;     // output pairs i0 ..: frames 2 i, 2 i + 1
@@ -116,6 +115,12 @@ dw_s2_dgrad_kernel(const TG* __restrict__ gu, const T* __restrict__ w, T* __rest
     float* g = smem + (size_t)wrp * (GP + 2 * Kh);           // frame g0 + i
     float* we = g + GP;                                      // taps 2 (Kh - 1 - j), then 2 (Kh - 1 - j) + 1
     float* wo = we + Kh;
+    for (int j = lane; j < Kh; j += 32) {
+        const int k = 2 * (Kh - 1 - j);
+        we[j] = k < K ? ldf(w + (size_t)c * K + k) : 0.f;
+        wo[j] = k + 1 < K ? ldf(w + (size_t)c * K + k + 1) : 0.f;
+    }
+    pdl_sync();
     const int li = min(len_in[b], Tt), lo = min(len_out[b], Tp);
     const size_t row = ((size_t)b * C + c) * Tt;
     const int tau = 2 * i0 + 16 * lane;
@@ -123,11 +128,6 @@ dw_s2_dgrad_kernel(const TG* __restrict__ gu, const T* __restrict__ w, T* __rest
         const float z[8] = {};
         if (tau < Tt) { st8<T>(dx + row + tau, z); st8<T>(dx + row + tau + 8, z); }
         return;
-    }
-    for (int j = lane; j < Kh; j += 32) {
-        const int k = 2 * (Kh - 1 - j);
-        we[j] = k < K ? ldf(w + (size_t)c * K + k) : 0.f;
-        wo[j] = k + 1 < K ? ldf(w + (size_t)c * K + k + 1) : 0.f;
     }
     // odd-tap outputs of pair i: a = i + P / 2; even-tap ones: a + OP; the first frame met is a - (Kh - 1)
     const int g0 = i0 + P / 2 - (Kh - 1), a0 = g0 & ~7;

@@ -1,13 +1,13 @@
 // Pointwise (1x1) convolution as plain SIMT tiled GEMMs with fp32 accumulation.
 // These serve the fp32 path (whose tolerance rules out reduced-precision tensor-core formats) and
-// any shape the tensor-core kernels do not tile.  64x64 output tile, 16-deep k-steps, 4x4 per thread.
+// any shape the tensor-core kernels do not tile.
+#include <algorithm>
+
 #include "common.cuh"
 #include "kernels.h"
 
 namespace sc {
 namespace {
-
-constexpr int BM = 64, BN = 64, BK = 16, NT = 256;
 
 // D[m,n] = sum_k A(m,k) * B(k,n) for one z-slice; operand access is described by strides so that the
 // three contractions (forward, input gradient, weight gradient) share the kernel.
@@ -15,92 +15,106 @@ struct GemmDesc {
     int M, N, Kd;
     // A(m,k) = a[z*a_z + m*a_m + k*a_k];  B(k,n) = b[z*b_z + k*b_k + n*b_n]
     long long a_z, a_m, a_k, b_z, b_k, b_n;
-    // weight gradient: k runs over (sample, frame): k -> (k / kt) * kz + (k % kt) for both operands
-    int kt; long long a_kz, b_kz;
-    int k_begin_per_z, k_len_per_z;   // split-K: slice z covers k in [z*k_len, (z+1)*k_len)
+    int per_z, k_len;                 // weight gradient: slice z = sample * per_z + i covers the frames [i k_len, (i+1) k_len) of the sample
 };
 
 template <typename X> struct IsHalf { static constexpr bool value = false; };
 template <> struct IsHalf<__half> { static constexpr bool value = true; };
 
-template <typename T, typename OT, int MODE>   // MODE 0: fwd (bias+mask, T out) 1: dgrad (T out) 2: wgrad (float partial out)
+constexpr int BK = 32, NT = 256;
+
+// TS x TS output tile (64: 4 x 4 per thread; 32: 2 x 2, for problems of few tiles).  The next 32-deep step travels through
+// registers while the current one is computed (two shared-memory buffers, one barrier per step): with the loads between two
+// barriers a step cost two round trips to L2 (64 x 64 x 128 frames, two samples, fp32: forward 11.3 -> 3.4 us, input gradient
+// 11.0 -> 2.9, weight gradient 24.8 -> 2.4, the last one also with several slices per sample).  Every output sums k in increasing order.
+// MODE 0: fwd (bias+mask, OT out) 1: dgrad (OT out) 2: wgrad (float partial out)
+template <typename T, typename OT, int MODE, int TS>
 __global__ void __launch_bounds__(NT)
 gemm_simt_kernel(GemmDesc d, const T* __restrict__ a, const T* __restrict__ b, void* __restrict__ out,
                  const float* __restrict__ bias, const int* __restrict__ len_out, int* status) {
-    pdl_sync();
-    __shared__ float As[BK][BM + 4];
-    __shared__ float Bs[BK][BN + 4];
+    constexpr int R = TS / 16, PER = TS * BK / NT;
+    __shared__ __align__(16) float As[2][BK][TS + 4];
+    __shared__ __align__(16) float Bs[2][BK][TS + 4];
     const int z = blockIdx.z;
-    const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
+    const int m0 = blockIdx.y * TS, n0 = blockIdx.x * TS;
     const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
-    float acc[4][4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+    float acc[R][R] = {};
+    pdl_sync();
 
-    int kb = 0, ke = d.Kd;
+    int ke = d.Kd, kb = 0;
     const T* ap = a; const T* bp = b;
-    if (MODE == 2) { kb = z * d.k_len_per_z; ke = min(d.Kd, kb + d.k_len_per_z); }
-    else { ap += (long long)z * d.a_z; bp += (long long)z * d.b_z; }
+    if (MODE == 2) {
+        const int zb = z / d.per_z;
+        kb = (z - zb * d.per_z) * d.k_len; ke = min(d.Kd, kb + d.k_len);
+        ap += (long long)zb * d.a_z; bp += (long long)zb * d.b_z;
+    } else {
+        ap += (long long)z * d.a_z; bp += (long long)z * d.b_z;
+    }
 
     // fwd-mode early exit: tile wholly in padding -> zeros
     if (MODE == 0 && len_out && n0 >= len_out[z]) {
         OT* o = (OT*)out + (long long)z * d.M * d.N;
-        for (int i = tid; i < BM * BN; i += NT) {
-            const int m = m0 + i / BN, n = n0 + i % BN;
+        for (int i = tid; i < TS * TS; i += NT) {
+            const int m = m0 + i / TS, n = n0 + i % TS;
             if (m < d.M && n < d.N) stf(o + (long long)m * d.N + n, 0.f);
         }
         return;
     }
 
-    for (int k0 = kb; k0 < ke; k0 += BK) {
-        // A tile: choose the thread->element map by which index is contiguous in memory
-        for (int i = tid; i < BM * BK; i += NT) {
-            int m, k;
-            if (d.a_k == 1 || MODE == 2) { k = i % BK; m = i / BK; } else { m = i % BM; k = i / BM; }
-            const int gm = m0 + m, gk = k0 + k;
-            float v = 0.f;
-            if (gm < d.M && gk < ke) {
-                long long off = (MODE == 2) ? (long long)(gk / d.kt) * d.a_kz + (gk % d.kt) + (long long)gm * d.a_m
-                                            : (long long)gm * d.a_m + (long long)gk * d.a_k;
-                v = ldf(ap + off);
-            }
-            As[k][m] = v;
+    // the thread -> element map follows the index that is contiguous in memory
+    constexpr bool AK = MODE != 1, BKc = MODE == 2;       // contiguous along k: forward weights, both weight-gradient operands
+    float ra[PER], rb[PER];
+    auto fetch = [&](int k0) {
+#pragma unroll
+        for (int e = 0; e < PER; ++e) {
+            const int i = tid + e * NT;
+            const int am = AK ? i / BK : i % TS, ak = AK ? i % BK : i / TS;
+            const int bn = BKc ? i / BK : i % TS, bk = BKc ? i % BK : i / TS;
+            ra[e] = (m0 + am < d.M && k0 + ak < ke) ? ldf(ap + (long long)(m0 + am) * d.a_m + (long long)(k0 + ak) * d.a_k) : 0.f;
+            rb[e] = (n0 + bn < d.N && k0 + bk < ke) ? ldf(bp + (long long)(k0 + bk) * d.b_k + (long long)(n0 + bn) * d.b_n) : 0.f;
         }
-        for (int i = tid; i < BN * BK; i += NT) {
-            int n, k;
-            if (MODE == 2) { k = i % BK; n = i / BK; } else { n = i % BN; k = i / BN; }
-            const int gn = n0 + n, gk = k0 + k;
-            float v = 0.f;
-            if (gn < d.N && gk < ke) {
-                long long off = (MODE == 2) ? (long long)(gk / d.kt) * d.b_kz + (gk % d.kt) + (long long)gn * d.b_n
-                                            : (long long)gk * d.b_k + (long long)gn * d.b_n;
-                v = ldf(bp + off);
-            }
-            Bs[k][n] = v;
+    };
+    auto park = [&](int q) {
+#pragma unroll
+        for (int e = 0; e < PER; ++e) {
+            const int i = tid + e * NT;
+            As[q][AK ? i % BK : i / TS][AK ? i / BK : i % TS] = ra[e];
+            Bs[q][BKc ? i % BK : i / TS][BKc ? i / BK : i % TS] = rb[e];
         }
-        __syncthreads();
+    };
+    fetch(kb);
+    park(0);
+    __syncthreads();
+    int q = 0;
+    for (int k0 = kb; k0 < ke; k0 += BK, q ^= 1) {
+        const bool more = k0 + BK < ke;
+        if (more) fetch(k0 + BK);
 #pragma unroll
         for (int k = 0; k < BK; ++k) {
-            const float4 av = *reinterpret_cast<const float4*>(&As[k][ty * 4]);
-            const float4 bv = *reinterpret_cast<const float4*>(&Bs[k][tx * 4]);
-            const float aa[4] = {av.x, av.y, av.z, av.w}, bb[4] = {bv.x, bv.y, bv.z, bv.w};
+            float aa[R], bb[R];
+            if (R == 4) {
+                const float4 av = *reinterpret_cast<const float4*>(&As[q][k][ty * 4]), bv = *reinterpret_cast<const float4*>(&Bs[q][k][tx * 4]);
+                aa[0] = av.x; aa[1] = av.y; aa[R - 2] = av.z; aa[R - 1] = av.w;
+                bb[0] = bv.x; bb[1] = bv.y; bb[R - 2] = bv.z; bb[R - 1] = bv.w;
+            } else {
+                const float2 av = *reinterpret_cast<const float2*>(&As[q][k][ty * 2]), bv = *reinterpret_cast<const float2*>(&Bs[q][k][tx * 2]);
+                aa[0] = av.x; aa[1] = av.y; bb[0] = bv.x; bb[1] = bv.y;
+            }
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
+            for (int i = 0; i < R; ++i)
 #pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(aa[i], bb[j], acc[i][j]);
+                for (int j = 0; j < R; ++j) acc[i][j] = fmaf(aa[i], bb[j], acc[i][j]);
         }
-        __syncthreads();
+        if (more) { park(q ^ 1); __syncthreads(); }
     }
 
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int m = m0 + ty * 4 + i;
+    for (int i = 0; i < R; ++i) {
+        const int m = m0 + ty * R + i;
         if (m >= d.M) continue;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int n = n0 + tx * 4 + j;
+        for (int j = 0; j < R; ++j) {
+            const int n = n0 + tx * R + j;
             if (n >= d.N) continue;
             if (MODE == 0) {
                 float v = acc[i][j] + (bias ? bias[m] : 0.f);
@@ -114,6 +128,15 @@ gemm_simt_kernel(GemmDesc d, const T* __restrict__ a, const T* __restrict__ b, v
             }
         }
     }
+}
+
+// 64 x 64 tiles where they fill the SMs, else 32 x 32
+template <typename T, typename OT, int MODE>
+void launch_gemm(const Launch& L, const GemmDesc& d, int nz, const void* a, const void* b, void* out, const float* bias, const int* len) {
+    auto tiles = [&](int ts) { return (long long)((d.N + ts - 1) / ts) * ((d.M + ts - 1) / ts) * nz; };
+    auto grid = [&](int ts) { return dim3((d.N + ts - 1) / ts, (d.M + ts - 1) / ts, nz); };
+    if (tiles(64) >= 148) launch_k(L, gemm_simt_kernel<T, OT, MODE, 64>, grid(64), NT, 0, d, (const T*)a, (const T*)b, out, bias, len, L.status);
+    else launch_k(L, gemm_simt_kernel<T, OT, MODE, 32>, grid(32), NT, 0, d, (const T*)a, (const T*)b, out, bias, len, L.status);
 }
 
 __global__ void reduce_partials_kernel(const float* __restrict__ p, int nsplit, long long n,
@@ -180,15 +203,14 @@ void gemm_fwd_simt(const Launch& L, int dtype, const void* w, const void* u, con
     d.M = Cout; d.N = Tp; d.Kd = Cin;
     d.a_z = 0; d.a_m = Cin; d.a_k = 1;
     d.b_z = (long long)Cin * Tp; d.b_k = Tp; d.b_n = 1;
-    dim3 grid((Tp + BN - 1) / BN, (Cout + BM - 1) / BM, B);
     if (out_dtype == dtype) {
-        SC_DISPATCH(dtype, (launch_k(L, gemm_simt_kernel<T, T, 0>, grid, NT, 0, d, (const T*)w, (const T*)u, v, bias, len_out, L.status)));
+        SC_DISPATCH(dtype, (launch_gemm<T, T, 0>(L, d, B, w, u, v, bias, len_out)));
     } else if (dtype == BF16 && out_dtype == F16) {   // bfloat16 operands, float16 result
-        launch_k(L, gemm_simt_kernel<__nv_bfloat16, __half, 0>, grid, NT, 0, d, (const __nv_bfloat16*)w, (const __nv_bfloat16*)u, v, bias, len_out, L.status);
+        launch_gemm<__nv_bfloat16, __half, 0>(L, d, B, w, u, v, bias, len_out);
     } else if (dtype == BF16) {   // 16-bit operands, float result
-        launch_k(L, gemm_simt_kernel<__nv_bfloat16, float, 0>, grid, NT, 0, d, (const __nv_bfloat16*)w, (const __nv_bfloat16*)u, v, bias, len_out, L.status);
+        launch_gemm<__nv_bfloat16, float, 0>(L, d, B, w, u, v, bias, len_out);
     } else {
-        launch_k(L, gemm_simt_kernel<__half, float, 0>, grid, NT, 0, d, (const __half*)w, (const __half*)u, v, bias, len_out, L.status);
+        launch_gemm<__half, float, 0>(L, d, B, w, u, v, bias, len_out);
     }
     L.count();
 }
@@ -200,30 +222,32 @@ void gemm_dgrad_simt(const Launch& L, int dtype, const void* w, const void* gv, 
     d.M = Cin; d.N = Tp; d.Kd = Cout;
     d.a_z = 0; d.a_m = 1; d.a_k = Cin;            // A(m=c, k=o) = w[o*Cin + c]
     d.b_z = (long long)Cout * Tp; d.b_k = Tp; d.b_n = 1;
-    dim3 grid((Tp + BN - 1) / BN, (Cin + BM - 1) / BM, B);
-    SC_DISPATCH(dtype, (launch_k(L, gemm_simt_kernel<T, T, 1>, grid, NT, 0, d, (const T*)w, (const T*)gv, gu, nullptr, nullptr, nullptr)));
+    SC_DISPATCH(dtype, (launch_gemm<T, T, 1>(L, d, B, w, gv, gu, nullptr, nullptr)));
     L.count();
 }
 
-static int wgrad_splits(int B) { return B; }   // one k-slice per sample
+// Slices per sample: one, unless the tiles of all samples together leave SMs idle.
+static int wgrad_per_sample(int B, int Cin, int Cout) {
+    const long long tiles = (long long)((Cin + 31) / 32) * ((Cout + 31) / 32) * B;
+    return (int)std::min(8ll, std::max(1ll, 148 / tiles));
+}
 
 size_t gemm_wgrad_simt_scratch_bytes(int B, int Cin, int Cout) {
-    return (size_t)wgrad_splits(B) * Cin * Cout * sizeof(float);
+    return (size_t)B * wgrad_per_sample(B, Cin, Cout) * Cin * Cout * sizeof(float);
 }
 
 void gemm_wgrad_simt(const Launch& L, int dtype, const void* gv, const void* u, float* dw, float* partials,
                      int accumulate, int B, int Cin, int Cout, int Tp, const float* gmax) {
-    const int ns = wgrad_splits(B);
+    GemmDesc d{};
+    d.k_len = ((Tp + wgrad_per_sample(B, Cin, Cout) - 1) / wgrad_per_sample(B, Cin, Cout) + BK - 1) / BK * BK;
+    d.per_z = (Tp + d.k_len - 1) / d.k_len;
+    const int ns = B * d.per_z;
     {
     KScope ks_(L, KC_PW_WGRAD, (double)dtype_size(dtype) * B * Tp * (Cin + Cout), 2.0 * B * Tp * Cin * Cout);
-    GemmDesc d{};
-    d.M = Cout; d.N = Cin; d.Kd = B * Tp;
-    d.kt = Tp;
-    d.a_m = Tp; d.a_kz = (long long)Cout * Tp;    // A(m=o, k=(b,t)) = gv[b,o,t]
-    d.b_n = Tp; d.b_kz = (long long)Cin * Tp;     // B(k=(b,t), n=c) = u[b,c,t]
-    d.k_len_per_z = Tp;
-    dim3 grid((Cin + BN - 1) / BN, (Cout + BM - 1) / BM, ns);
-    SC_DISPATCH(dtype, (launch_k(L, gemm_simt_kernel<T, T, 2>, grid, NT, 0, d, (const T*)gv, (const T*)u, partials, nullptr, nullptr, nullptr)));
+    d.M = Cout; d.N = Cin; d.Kd = Tp;
+    d.a_z = (long long)Cout * Tp; d.a_m = Tp; d.a_k = 1;    // A(m=o, k=t) = gv[b,o,t]
+    d.b_z = (long long)Cin * Tp; d.b_n = Tp; d.b_k = 1;     // B(k=t, n=c) = u[b,c,t]
+    SC_DISPATCH(dtype, (launch_gemm<T, T, 2>(L, d, ns, gv, u, partials, nullptr, nullptr)));
     L.count();
     }
     reduce_partials(L, partials, ns, (int64_t)Cin * Cout, dw, accumulate, gmax);
