@@ -8,6 +8,7 @@ from __future__ import annotations
 
 import ctypes as C
 import os
+import struct
 from typing import Dict, List, Optional, Sequence
 
 import numpy as np
@@ -62,6 +63,10 @@ class sc_block_grads(C.Structure):
     _fields_ = [(n, C.c_void_p) for n in ("dwd", "dwp", "dgamma", "dbeta", "dbias", "dwr", "dgamma_r", "dbeta_r")]
 
 
+SAVED = tuple(n for n, _ in sc_block_saved._fields_)
+GRADS = tuple(n for n, _ in sc_block_grads._fields_)
+
+
 class sc_encoder_desc(C.Structure):
     _fields_ = [("n_layers", C.c_int32), ("layers", C.POINTER(sc_block_desc)), ("res_from", C.POINTER(C.c_int32))]
 
@@ -97,31 +102,32 @@ def load_library(path: str = LIB_PATH):
     lib.sepconv_set_tile_shape.argtypes = [C.c_void_p, C.c_int]
     lib.sepconv_launch_count.argtypes = [C.c_void_p]
     lib.sepconv_launch_count.restype = C.c_int64
+    # tensor and pointer structs as void pointers: they are passed by reference or as packed bytes (see _tensor)
     lib.sepconv_workspace_bytes.argtypes = [C.POINTER(sc_block_desc), C.POINTER(C.c_size_t), C.POINTER(C.c_size_t)]
-    lib.sepconv_fwd.argtypes = [C.c_void_p, C.POINTER(sc_block_desc), C.POINTER(sc_tensor), C.POINTER(sc_tensor),
-                                C.c_void_p, C.POINTER(sc_block_params), C.POINTER(sc_tensor), C.c_void_p,
-                                C.POINTER(sc_block_saved), C.c_void_p, C.c_void_p, C.c_void_p, C.c_size_t,
+    lib.sepconv_fwd.argtypes = [C.c_void_p, C.POINTER(sc_block_desc), C.c_void_p, C.c_void_p,
+                                C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p,
+                                C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p, C.c_size_t,
                                 C.c_void_p]
-    lib.sepconv_fwd_static.argtypes = [C.c_void_p, C.POINTER(sc_block_desc), C.POINTER(sc_tensor),
-                                       C.POINTER(sc_tensor), C.c_void_p, C.POINTER(sc_block_params),
-                                       C.POINTER(sc_tensor), C.c_void_p, C.POINTER(sc_block_saved), C.c_void_p]
-    lib.sepconv_bwd.argtypes = [C.c_void_p, C.POINTER(sc_block_desc), C.POINTER(sc_tensor), C.POINTER(sc_tensor),
-                                C.POINTER(sc_tensor), C.POINTER(sc_tensor), C.c_void_p,
-                                C.POINTER(sc_block_params), C.POINTER(sc_block_saved), C.POINTER(sc_tensor),
-                                C.POINTER(sc_tensor), C.POINTER(sc_tensor), C.POINTER(sc_block_grads), C.c_int,
+    lib.sepconv_fwd_static.argtypes = [C.c_void_p, C.POINTER(sc_block_desc), C.c_void_p,
+                                       C.c_void_p, C.c_void_p, C.c_void_p,
+                                       C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p]
+    lib.sepconv_bwd.argtypes = [C.c_void_p, C.POINTER(sc_block_desc), C.c_void_p, C.c_void_p,
+                                C.c_void_p, C.c_void_p, C.c_void_p,
+                                C.c_void_p, C.c_void_p, C.c_void_p,
+                                C.c_void_p, C.c_void_p, C.c_void_p, C.c_int,
                                 C.c_void_p, C.c_size_t, C.c_void_p]
     lib.encoder_workspace_bytes.argtypes = [C.POINTER(sc_encoder_desc), C.POINTER(C.c_size_t)]
-    lib.encoder_fwd_bwd.argtypes = [C.c_void_p, C.POINTER(sc_encoder_desc), C.POINTER(sc_tensor), C.c_void_p,
-                                    C.c_void_p, C.POINTER(C.c_int64), C.POINTER(sc_tensor),
-                                    C.POINTER(sc_tensor), C.c_void_p, C.c_void_p, C.POINTER(C.c_int64),
-                                    C.POINTER(sc_tensor), C.c_int, C.c_void_p, C.c_size_t, C.c_void_p]
+    lib.encoder_fwd_bwd.argtypes = [C.c_void_p, C.POINTER(sc_encoder_desc), C.c_void_p, C.c_void_p,
+                                    C.c_void_p, C.POINTER(C.c_int64), C.c_void_p,
+                                    C.c_void_p, C.c_void_p, C.c_void_p, C.POINTER(C.c_int64),
+                                    C.c_void_p, C.c_int, C.c_void_p, C.c_size_t, C.c_void_p]
     lib.sepconv_infer_workspace_bytes.argtypes = [C.POINTER(sc_block_desc), C.POINTER(C.c_size_t)]
-    lib.sepconv_infer.argtypes = [C.c_void_p, C.POINTER(sc_block_desc), C.POINTER(sc_tensor), C.POINTER(sc_tensor),
-                                  C.c_void_p, C.POINTER(sc_block_params), C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p,
-                                  C.POINTER(sc_tensor), C.c_void_p, C.c_void_p, C.c_size_t, C.c_void_p]
+    lib.sepconv_infer.argtypes = [C.c_void_p, C.POINTER(sc_block_desc), C.c_void_p, C.c_void_p,
+                                  C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p,
+                                  C.c_void_p, C.c_void_p, C.c_void_p, C.c_size_t, C.c_void_p]
     lib.encoder_infer_workspace_bytes.argtypes = [C.POINTER(sc_encoder_desc), C.POINTER(C.c_size_t)]
-    lib.encoder_infer.argtypes = [C.c_void_p, C.POINTER(sc_encoder_desc), C.POINTER(sc_tensor), C.c_void_p, C.c_void_p,
-                                  C.POINTER(C.c_int64), C.c_void_p, C.POINTER(C.c_int64), C.POINTER(sc_tensor), C.c_void_p,
+    lib.encoder_infer.argtypes = [C.c_void_p, C.POINTER(sc_encoder_desc), C.c_void_p, C.c_void_p, C.c_void_p,
+                                  C.POINTER(C.c_int64), C.c_void_p, C.POINTER(C.c_int64), C.c_void_p, C.c_void_p,
                                   C.c_void_p, C.c_size_t, C.c_void_p]
     lib.sepconv_profile_begin.argtypes = [C.c_void_p, C.c_int, C.c_int]
     lib.sepconv_profile_end.argtypes = [C.c_void_p, C.c_void_p, C.POINTER(C.c_double), C.POINTER(C.c_int64),
@@ -149,10 +155,15 @@ def _stream_ptr(stream) -> int:
     return int(stream.cuda_stream) if stream is not None else _raw_stream(torch.cuda.current_device())
 
 
-# A call marshals up to eight tensors, and filling an sc_tensor field by field costs about as much as enqueueing a kernel:
-# the descriptor of a dense tensor differs from that of any other of its type and shape in the address alone.
+# A call marshals up to eight tensors and three structs of pointers, and filling a ctypes struct field by field costs about
+# as much as enqueueing a kernel.  They are passed as packed bytes instead (ctypes hands over the address of a bytes
+# object): the descriptor of a dense tensor differs from that of any other of its type and shape in the address alone.
 _DTYPES = {torch.float32: SC_F32, torch.float16: SC_F16, torch.bfloat16: SC_BF16}
-_templates: Dict[tuple, bytes] = {}
+_TAGS = (0, 1, 2)
+_tails: Dict[tuple, bytes] = {}
+_pack1 = struct.Struct("Q").pack
+_pack7 = struct.Struct("7Q").pack
+_pack8 = struct.Struct("8Q").pack
 
 
 def _describe(t: torch.Tensor, tags) -> sc_tensor:
@@ -166,28 +177,38 @@ def _describe(t: torch.Tensor, tags) -> sc_tensor:
     return st
 
 
-def tensor_arg(t: Optional[torch.Tensor], tags=(0, 1, 2)):
+def tensor_arg(t: Optional[torch.Tensor], tags=_TAGS):
     """torch [B,C,T] tensor -> sc_tensor (by reference); None -> NULL."""
     if t is None:
         return None
-    if tags == (0, 1, 2) and t.is_contiguous():
-        key = (t.dtype, t.shape)
-        tmpl = _templates.get(key)
-        if tmpl is None:
-            if len(_templates) >= 1024:
-                _templates.clear()
-            tmpl = _templates[key] = bytes(_describe(t, tags))
-        st = sc_tensor.from_buffer_copy(tmpl)
-    else:
-        st = _describe(t, tags)
+    st = _describe(t, tags)
     st.ptr = t.data_ptr()
     return C.byref(st)
 
 
-def _pointers(struct, tensors: Dict[str, torch.Tensor]):
-    """A struct of device pointers from the tensors of its field names (absent ones null)."""
+def _tensor(t: Optional[torch.Tensor]):
+    """The same as packed bytes, for tensors whose axes are [batch, channel, time]."""
+    if t is None:
+        return None
+    if not t.is_contiguous():
+        return tensor_arg(t)
+    key = (t.dtype, t.shape)
+    tail = _tails.get(key)
+    if tail is None:
+        if len(_tails) >= 1024:
+            _tails.clear()
+        tail = _tails[key] = bytes(_describe(t, _TAGS))[8:]        # what follows the address
+    return _pack1(t.data_ptr()) + tail
+
+
+def _pointers(pack, names, tensors: Dict[str, torch.Tensor]) -> bytes:
+    """A packed struct of device pointers from the tensors of its field names (absent ones null)."""
     get = tensors.get
-    return struct(*[None if (t := get(n)) is None else t.data_ptr() for n, _ in struct._fields_])
+    return pack(*[0 if (t := get(n)) is None else t.data_ptr() for n in names])
+
+
+def _empty(like: torch.Tensor, shape, dtype) -> torch.Tensor:
+    return torch.empty_like(like) if like.dtype == dtype and like.shape == shape else like.new_empty(shape, dtype=dtype)
 
 
 def block_desc(L, B: int, T: int, dtype: str) -> sc_block_desc:
@@ -277,7 +298,7 @@ def _workspace(nbytes: int, device) -> torch.Tensor:
 
 
 def _params_struct(params: Dict[str, torch.Tensor]) -> sc_block_params:
-    return _pointers(sc_block_params, params)
+    return sc_block_params.from_buffer_copy(_pointers(_pack8, PARAM_ORDER, params))
 
 
 def sepconv_fwd(ctx: Context, desc: sc_block_desc, x: torch.Tensor, lengths: torch.Tensor,
@@ -289,27 +310,26 @@ def sepconv_fwd(ctx: Context, desc: sc_block_desc, x: torch.Tensor, lengths: tor
     td = TORCH_DTYPE[desc.io_dtype]
     B, Co, Ci, Tp = desc.B, desc.C_out, desc.C_in, desc.T_out
     if y is None:
-        y = torch.empty((B, Co, Tp), dtype=td, device=dev)
-    out_len = torch.empty((B,), dtype=torch.int32, device=dev)
+        y = _empty(x, (B, Co, Tp), td)
+    out_len = _empty(lengths, (B,), torch.int32)
     if saved is None:
         ut = torch.float16 if (desc.has_dw and desc.has_bn and desc.io_dtype != SC_F32) else td
-        saved = {"u": torch.empty((B, Ci, Tp), dtype=ut, device=dev)}
+        saved = {"u": _empty(x, (B, Ci, Tp), ut)}
         nt = torch.float32 if desc.io_dtype == SC_F32 else torch.float16   # type of the saved pointwise results
-        stats = ()                               # the saved statistics share one allocation
         if desc.has_bn:
-            saved["v"] = torch.empty((B, Co, Tp), dtype=nt, device=dev)
-            stats = ("mean", "invstd")
+            saved["v"] = _empty(y, (B, Co, Tp), nt)
+            g = params.get("gamma")
+            g = x if g is None else g
+            saved["mean"], saved["invstd"] = _empty(g, (Co,), torch.float32), _empty(g, (Co,), torch.float32)
         if desc.residual == 2:
-            saved["vr"] = torch.empty((B, Co, Tp), dtype=nt, device=dev)
-            stats += ("mean_r", "invstd_r")
-        if stats:
-            saved.update(zip(stats, torch.empty((len(stats), Co), dtype=torch.float32, device=dev).unbind()))
-    sv = _pointers(sc_block_saved, saved)
+            saved["vr"] = _empty(y, (B, Co, Tp), nt)
+            saved["mean_r"], saved["invstd_r"] = _empty(x, (Co,), torch.float32), _empty(x, (Co,), torch.float32)
+    sv = _pointers(_pack7, SAVED, saved)
     if workspace is None:
         workspace = _workspace(sepconv_workspace_bytes(desc)[0], dev)
-    p = _params_struct(params)
-    rc = ctx.lib.sepconv_fwd(ctx.h, C.byref(desc), tensor_arg(x), tensor_arg(x_res), lengths.data_ptr(),
-                             C.byref(p), tensor_arg(y), out_len.data_ptr(), C.byref(sv),
+    p = _pointers(_pack8, PARAM_ORDER, params)
+    rc = ctx.lib.sepconv_fwd(ctx.h, C.byref(desc), _tensor(x), _tensor(x_res), lengths.data_ptr(),
+                             p, _tensor(y), out_len.data_ptr(), sv,
                              running_mean.data_ptr() if running_mean is not None else None,
                              running_var.data_ptr() if running_var is not None else None,
                              workspace.data_ptr(), workspace.numel(), _stream_ptr(stream))
@@ -328,10 +348,10 @@ def sepconv_infer(ctx: Context, desc: sc_block_desc, x: torch.Tensor, lengths: t
     n = C.c_size_t()
     _check(ctx.lib.sepconv_infer_workspace_bytes(C.byref(desc), C.byref(n)), "sepconv_infer_workspace_bytes")
     ws = _workspace(int(n.value), dev)
-    p = _params_struct(params)
+    p = _pointers(_pack8, PARAM_ORDER, params)
     ptr = lambda k: running[k].data_ptr() if k in running and running[k] is not None else None
-    rc = ctx.lib.sepconv_infer(ctx.h, C.byref(desc), tensor_arg(x), tensor_arg(x_res), lengths.data_ptr(), C.byref(p),
-                               ptr("mean"), ptr("var"), ptr("mean_r"), ptr("var_r"), tensor_arg(y), out_len.data_ptr(),
+    rc = ctx.lib.sepconv_infer(ctx.h, C.byref(desc), _tensor(x), _tensor(x_res), lengths.data_ptr(), p,
+                               ptr("mean"), ptr("var"), ptr("mean_r"), ptr("var_r"), _tensor(y), out_len.data_ptr(),
                                ws.data_ptr(), ws.numel(), _stream_ptr(stream))
     _check(rc, "sepconv_infer")
     return y, out_len
@@ -345,10 +365,10 @@ def sepconv_fwd_static(ctx: Context, desc: sc_block_desc, x: torch.Tensor, lengt
                        saved: Dict[str, torch.Tensor], x_res: Optional[torch.Tensor] = None, stream=None):
     """sepconv_fwd for callers that cannot allocate: every buffer (y, out_lengths, saved) is passed in
     and the scratch is the library's built-in fixed array.  This wrapper allocates nothing either."""
-    sv = _pointers(sc_block_saved, saved)
-    p = _params_struct(params)
-    rc = ctx.lib.sepconv_fwd_static(ctx.h, C.byref(desc), tensor_arg(x), tensor_arg(x_res), lengths.data_ptr(),
-                                    C.byref(p), tensor_arg(y), out_lengths.data_ptr(), C.byref(sv),
+    sv = _pointers(_pack7, SAVED, saved)
+    p = _pointers(_pack8, PARAM_ORDER, params)
+    rc = ctx.lib.sepconv_fwd_static(ctx.h, C.byref(desc), _tensor(x), _tensor(x_res), lengths.data_ptr(),
+                                    p, _tensor(y), out_lengths.data_ptr(), sv,
                                     _stream_ptr(stream))
     _check(rc, "sepconv_fwd_static")
 
@@ -369,14 +389,14 @@ def sepconv_bwd(ctx: Context, desc: sc_block_desc, dy: torch.Tensor, x: torch.Te
     if grads is None:
         grads = {"d" + n: torch.zeros(params[n].shape, dtype=torch.float32, device=dev)
                  for n in PARAM_ORDER if n in params and params[n] is not None}
-    g = _pointers(sc_block_grads, grads)
-    sv = _pointers(sc_block_saved, saved)
+    g = _pointers(_pack8, GRADS, grads)
+    sv = _pointers(_pack7, SAVED, saved)
     if workspace is None:
         workspace = _workspace(sepconv_workspace_bytes(desc)[1], dev)
-    p = _params_struct(params)
-    rc = ctx.lib.sepconv_bwd(ctx.h, C.byref(desc), tensor_arg(dy), tensor_arg(x), tensor_arg(x_res), tensor_arg(y),
-                             lengths.data_ptr(), C.byref(p), C.byref(sv), tensor_arg(dx), tensor_arg(dx_res),
-                             tensor_arg(dx_add), C.byref(g), int(accumulate), workspace.data_ptr(),
+    p = _pointers(_pack8, PARAM_ORDER, params)
+    rc = ctx.lib.sepconv_bwd(ctx.h, C.byref(desc), _tensor(dy), _tensor(x), _tensor(x_res), _tensor(y),
+                             lengths.data_ptr(), p, sv, _tensor(dx), _tensor(dx_res),
+                             _tensor(dx_add), g, int(accumulate), workspace.data_ptr(),
                              workspace.numel(), _stream_ptr(stream))
     _check(rc, "sepconv_bwd")
     return dx, dx_res, grads
@@ -486,8 +506,8 @@ def encoder_infer(ctx: Context, spec: EncoderSpec, x: torch.Tensor, lengths: tor
         n = C.c_size_t()
         _check(ctx.lib.encoder_infer_workspace_bytes(C.byref(spec.desc), C.byref(n)), "encoder_infer_workspace_bytes")
         workspace = _workspace(int(n.value), dev)
-    rc = ctx.lib.encoder_infer(ctx.h, C.byref(spec.desc), tensor_arg(x), lengths.data_ptr(), params_blob.data_ptr(),
-                               spec.param_offsets, running_blob.data_ptr(), running_offsets, tensor_arg(out),
+    rc = ctx.lib.encoder_infer(ctx.h, C.byref(spec.desc), _tensor(x), lengths.data_ptr(), params_blob.data_ptr(),
+                               spec.param_offsets, running_blob.data_ptr(), running_offsets, _tensor(out),
                                out_len.data_ptr(), workspace.data_ptr(), workspace.numel(), _stream_ptr(stream))
     _check(rc, "encoder_infer")
     return out, out_len
@@ -508,10 +528,10 @@ def encoder_fwd_bwd(ctx: Context, spec: EncoderSpec, x: torch.Tensor, lengths: t
     dx = torch.empty_like(x) if want_dx else None
     if workspace is None:
         workspace = _workspace(encoder_workspace_bytes(spec), dev)
-    rc = ctx.lib.encoder_fwd_bwd(ctx.h, C.byref(spec.desc), tensor_arg(x), lengths.data_ptr(),
-                                 params_blob.data_ptr(), spec.param_offsets, tensor_arg(dlogits),
-                                 tensor_arg(logits), out_len.data_ptr(), grads_blob.data_ptr(),
-                                 spec.grad_offsets, tensor_arg(dx), int(accumulate), workspace.data_ptr(),
+    rc = ctx.lib.encoder_fwd_bwd(ctx.h, C.byref(spec.desc), _tensor(x), lengths.data_ptr(),
+                                 params_blob.data_ptr(), spec.param_offsets, _tensor(dlogits),
+                                 _tensor(logits), out_len.data_ptr(), grads_blob.data_ptr(),
+                                 spec.grad_offsets, _tensor(dx), int(accumulate), workspace.data_ptr(),
                                  workspace.numel(), _stream_ptr(stream))
     _check(rc, "encoder_fwd_bwd")
     return logits, out_len, grads_blob, dx
