@@ -1,8 +1,6 @@
 // Depthwise (per-channel) correlation over time: forward, input gradient, tap gradient.
 //
-// Stride-1 layers (all but the first layer of the encoder) use register-blocked kernels: a thread
-// owns R consecutive outputs, keeps a 2R-wide sliding window of the shared-memory tile and R taps
-// in registers and performs R*R FMAs per 2R shared loads.  The input gradient of a stride-1
+// Stride-1 layers (all but the first layer of the encoder) use register-blocked kernels.  The input gradient of a stride-1
 // correlation is the same correlation with flipped taps, so one kernel serves both.  Any other
 // stride goes through plain tiled kernels.
 #include "common.cuh"
@@ -15,136 +13,117 @@ namespace {
 
 constexpr int R = 8;          // outputs (or taps) per thread
 constexpr int CH = 8;         // channels per CTA in the stride-1 kernel (one warp each)
-constexpr int TT = 32 * R;    // outputs per channel per CTA
 
 // Conflict-free placement for 16-byte shared loads at an 8-float lane pitch.
 __device__ __forceinline__ int phys(int i) { return i + ((i >> 5) << 2); }
 
-// Saturating store for half outputs: a value outside the half range is clamped and reported.
-template <typename TO>
-__device__ __forceinline__ void guard_range(float (&acc)[8], int* status) {
-    if (sizeof(TO) == 2 && !std::is_same<TO, __nv_bfloat16>::value) {
-        bool over = false;
-#pragma unroll
-        for (int r = 0; r < 8; ++r) {
-            if (fabsf(acc[r]) > 65504.f) { over = true; acc[r] = copysignf(65504.f, acc[r]); }
-        }
-        if (over) raise_status(status, kErrRange);
-    }
-}
-
-template <typename TI, typename TW, typename TO>
+// Stride-1 correlation: a thread owns RR consecutive outputs, a 2 RR-wide sliding window of the shared-memory tile and RR
+// taps in registers: RR * RR multiply-adds per RR / 2 16-byte shared loads.  RR = 8 for throughput; RR = 4 where the work
+// is a handful of warps per SM and their serial chain is the kernel's time (a 1.6 s utterance through
+// 26 layers of 256 and 512 channels: 4.2 -> 3.4 us a layer, its whole pass 287 -> 268 us).  The tile starts at t0 - Pa with
+// Pa = P rounded up to 8 and the taps have Pa - P zeros in front, so that staging is whole vectors on both sides.
+template <typename TI, typename TW, typename TO, int RR>
 __global__ void __launch_bounds__(32 * CH)
 dw_corr_s1_kernel(const TI* __restrict__ in, const TW* __restrict__ w, TO* __restrict__ out,
                   const TO* __restrict__ add1, const TO* __restrict__ add2, const float* __restrict__ gmax,
                   const int* __restrict__ len_src, const int* __restrict__ len_dst,
-                  int C, int Tt, int K, int Kpad, int flip, int* status) {
+                  int C, int Tt, int K, int Pa, int Kpad, int flip, int* status) {
     using T = TO;
+    constexpr int TTR = 32 * RR;
     extern __shared__ float smem[];
     const int lane = threadIdx.x, wrp = threadIdx.y;
-    const int b = blockIdx.z, c = blockIdx.y * CH + wrp, t0 = blockIdx.x * TT;
+    const int b = blockIdx.z, c = blockIdx.y * CH + wrp, t0 = blockIdx.x * TTR;
     if (c >= C) return;                       // warps are independent: no CTA-wide barrier below
-    const int P = (K - 1) / 2;
-    const int XW = TT + Kpad;                 // logical tile width
+    const int delta = Pa - (K - 1) / 2;
+    const int XW = TTR + Kpad;                // tile width
     float* xs = smem + (size_t)wrp * (phys(XW) + 4 + Kpad);
     float* ws = xs + phys(XW) + 4;
     // the taps are the caller's parameters: read ahead of the wait (zero padded to Kpad)
-    for (int k = lane; k < Kpad; k += 32)
-        ws[k] = (k < K) ? ldf(w + (size_t)c * K + (flip ? K - 1 - k : k)) : 0.f;
+    for (int i = lane; i < Kpad; i += 32) {
+        const int k = i - delta;
+        ws[i] = (k >= 0 && k < K) ? ldf(w + (size_t)c * K + (flip ? K - 1 - k : k)) : 0.f;
+    }
     pdl_sync();
     const int ls = min(len_src[b], Tt), ld = min(len_dst[b], Tt);
     const size_t row = ((size_t)b * C + c) * Tt;
     T* orow = out + row;
     const bool vec = (Tt % 8 == 0);
-
+    const int t = t0 + lane * RR;
     if (t0 >= ld) {                           // tile lies wholly in padding: zeros
-        float z[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-        const int t = t0 + lane * R;
-        if (vec) { if (t < Tt) st8<T>(orow + t, z); }
-        else { for (int r = 0; r < R; ++r) if (t + r < Tt) stf(orow + t + r, 0.f); }
+        for (int r = 0; r < RR; ++r) if (t + r < Tt) stf(orow + t + r, 0.f);
         return;
     }
-    // input tile: logical index i <-> frame tau = t0 - P + i, zero outside [0, ls)
+    // input tile: index i <-> frame t0 - Pa + i, zero outside [0, ls)
     const TI* irow = in + row;
-    const int tau0 = t0 - P;
     if (vec) {
-        const int a0 = (tau0 >= 0) ? (tau0 & ~7) : -(((-tau0) + 7) & ~7);   // floor to a multiple of 8
-        const int nchunk = (tau0 + XW - a0 + 7) / 8;
-        for (int j = lane; j < nchunk; j += 32) {
-            const int ta = a0 + 8 * j;
-            float f[8];
+        for (int v = lane; 8 * v < XW; v += 32) {
+            const int ta = t0 - Pa + 8 * v;
+            float f[8] = {};
             if (ta >= 0 && ta < Tt) ld8<TI>(irow + ta, f);      // not bounded by ls: the load need not wait for the length
-            else {
 #pragma unroll
-                for (int e = 0; e < 8; ++e) f[e] = 0.f;
-            }
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                const int i = ta + e - tau0;
-                if (i >= 0 && i < XW) xs[phys(i)] = (ta + e < ls) ? f[e] : 0.f;
-            }
+            for (int e = 0; e < 8; ++e) if (ta + e >= ls) f[e] = 0.f;
+            float4* d = reinterpret_cast<float4*>(xs + phys(8 * v));
+            d[0] = make_float4(f[0], f[1], f[2], f[3]);
+            d[1] = make_float4(f[4], f[5], f[6], f[7]);
         }
     } else {
         for (int i = lane; i < XW; i += 32) {
-            const int tau = tau0 + i;
+            const int tau = t0 - Pa + i;
             xs[phys(i)] = (tau >= 0 && tau < ls) ? ldf(irow + tau) : 0.f;
         }
     }
     __syncwarp();
 
-    float acc[R];
+    float acc[RR] = {}, win[2 * RR], wv[RR];
+    const int base = lane * RR;
+    auto ld4 = [](const float* p, float* d) { const float4 q = *reinterpret_cast<const float4*>(p); d[0] = q.x; d[1] = q.y; d[2] = q.z; d[3] = q.w; };
 #pragma unroll
-    for (int r = 0; r < R; ++r) acc[r] = 0.f;
-    float win[2 * R];
-    const int base = lane * R;
-    {
-        const float4 a = *reinterpret_cast<const float4*>(xs + phys(base));
-        const float4 bq = *reinterpret_cast<const float4*>(xs + phys(base + 4));
-        win[0] = a.x; win[1] = a.y; win[2] = a.z; win[3] = a.w;
-        win[4] = bq.x; win[5] = bq.y; win[6] = bq.z; win[7] = bq.w;
-    }
-    for (int kk = 0; kk < Kpad; kk += R) {
-        const float4 a = *reinterpret_cast<const float4*>(xs + phys(base + kk + R));
-        const float4 bq = *reinterpret_cast<const float4*>(xs + phys(base + kk + R + 4));
-        win[8] = a.x; win[9] = a.y; win[10] = a.z; win[11] = a.w;
-        win[12] = bq.x; win[13] = bq.y; win[14] = bq.z; win[15] = bq.w;
-        const float4 w0 = *reinterpret_cast<const float4*>(ws + kk);
-        const float4 w1 = *reinterpret_cast<const float4*>(ws + kk + 4);
-        const float wv[R] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
+    for (int i = 0; i < RR; i += 4) ld4(xs + phys(base + i), win + i);
+    for (int kk = 0; kk < Kpad; kk += RR) {
 #pragma unroll
-        for (int q = 0; q < R; ++q)
+        for (int i = 0; i < RR; i += 4) { ld4(xs + phys(base + kk + RR + i), win + RR + i); ld4(ws + kk + i, wv + i); }
 #pragma unroll
-            for (int r = 0; r < R; ++r) acc[r] = fmaf(wv[q], win[r + q], acc[r]);
+        for (int q = 0; q < RR; ++q)
 #pragma unroll
-        for (int r = 0; r < R; ++r) win[r] = win[r + R];
+            for (int r = 0; r < RR; ++r) acc[r] = fmaf(wv[q], win[r + q], acc[r]);
+#pragma unroll
+        for (int r = 0; r < RR; ++r) win[r] = win[r + RR];
     }
 
-    const int t = t0 + base;
     if (t >= Tt) return;
     if (gmax) {
         const float inv = 1.f / pow2_scale(*gmax);
 #pragma unroll
-        for (int r = 0; r < R; ++r) acc[r] *= inv;
+        for (int r = 0; r < RR; ++r) acc[r] *= inv;
     }
-    guard_range<TO>(acc, status);
-    if (vec) {
-        if (add1) { float f[8]; ld8<T>(add1 + row + t, f);
+    if (std::is_same<TO, __half>::value) {    // a value outside the half range is clamped and reported
+        bool over = false;
 #pragma unroll
-            for (int r = 0; r < R; ++r) acc[r] += f[r]; }
-        if (add2) { float f[8]; ld8<T>(add2 + row + t, f);
+        for (int r = 0; r < RR; ++r) if (fabsf(acc[r]) > 65504.f) { over = true; acc[r] = copysignf(65504.f, acc[r]); }
+        if (over) raise_status(status, kErrRange);
+    }
 #pragma unroll
-            for (int r = 0; r < R; ++r) acc[r] += f[r]; }
-#pragma unroll
-        for (int r = 0; r < R; ++r) if (t + r >= ld) acc[r] = 0.f;
-        st8<T>(orow + t, acc);
-    } else {
-        for (int r = 0; r < R; ++r) {
-            if (t + r >= Tt) break;
-            float q = acc[r];
-            if (add1) q += ldf(add1 + row + t + r);
-            if (add2) q += ldf(add2 + row + t + r);
-            stf(orow + t + r, (t + r < ld) ? q : 0.f);
+    for (int r = 0; r < RR; ++r) {
+        if (t + r < Tt) {
+            if (add1) acc[r] += ldf(add1 + row + t + r);
+            if (add2) acc[r] += ldf(add2 + row + t + r);
+            if (t + r >= ld) acc[r] = 0.f;
         }
+    }
+    if (!vec) {
+        for (int r = 0; r < RR; ++r) if (t + r < Tt) stf(orow + t + r, acc[r]);
+    } else if (RR == 8) {
+        float f[8];
+#pragma unroll
+        for (int r = 0; r < 8; ++r) f[r] = acc[r % RR];
+        st8<T>(orow + t, f);
+    } else if (sizeof(T) == 4) {
+        *reinterpret_cast<float4*>(orow + t) = make_float4(acc[0], acc[1], acc[2], acc[3]);
+    } else {
+        __align__(8) T h[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) stf(h + r, acc[r]);
+        *reinterpret_cast<uint2*>(orow + t) = *reinterpret_cast<const uint2*>(h);
     }
 }
 
@@ -639,11 +618,31 @@ dw_wgrad_reg16_kernel(const TG* __restrict__ gu, const T* __restrict__ x, float*
     }
 }
 
+inline int kpad(int K) { return (K + R - 1) / R * R; }
+inline int host_phys(int i) { return i + ((i >> 5) << 2); }
+
+template <typename TI, typename TW, typename TO, int RR>
+void launch_corr_r(const Launch& L, const TI* in, const TW* w, TO* out, const TO* add1, const TO* add2, const float* gmax, const int* len_src,
+                   const int* len_dst, int B, int C, int Tt, int K, int flip) {
+    const int P = (K - 1) / 2, Pa = (P + 7) / 8 * 8, Kp = (K + Pa - P + 7) / 8 * 8;
+    const size_t smem = (size_t)CH * (host_phys(32 * RR + Kp) + 4 + Kp) * sizeof(float);
+    const dim3 grid((Tt + 32 * RR - 1) / (32 * RR), (C + CH - 1) / CH, B), block(32, CH);
+    launch_k(L, dw_corr_s1_kernel<TI, TW, TO, RR>, grid, block, smem, in, w, out, add1, add2, gmax, len_src, len_dst, C, Tt, K, Pa, Kp, flip,
+             L.status);
+}
+template <typename TI, typename TW, typename TO>
+void launch_corr(const Launch& L, const TI* in, const TW* w, TO* out, const TO* add1, const TO* add2, const float* gmax, const int* len_src,
+                 const int* len_dst, int B, int C, int Tt, int K, int flip) {
+    // at most sixteen of the wide kernel's warps per SM: the narrow one
+    if ((long long)B * C * ((Tt + 255) / 256) <= 16 * 148)
+        launch_corr_r<TI, TW, TO, 4>(L, in, w, out, add1, add2, gmax, len_src, len_dst, B, C, Tt, K, flip);
+    else
+        launch_corr_r<TI, TW, TO, 8>(L, in, w, out, add1, add2, gmax, len_src, len_dst, B, C, Tt, K, flip);
+}
+
 // Below this many multiply-adds the register-blocked kernel is done before a tensor-core CTA has built its Toeplitz blocks.
 inline bool small_corr(int B, int C, int Tt, int K) { return (double)B * C * Tt * K <= 1.0e8; }
 
-inline int kpad(int K) { return (K + R - 1) / R * R; }
-inline int host_phys(int i) { return i + ((i >> 5) << 2); }
 
 }  // namespace
 
@@ -668,12 +667,8 @@ void dw_fwd(const Launch& L, int dtype, int odt, const void* x, const void* wd, 
         return;
     }
     if (s == 1 && plain) {
-        const int Kp = kpad(K);
-        const size_t smem = (size_t)CH * (host_phys(TT + Kp) + 4 + Kp) * sizeof(float);
-        dim3 grid((Tt + TT - 1) / TT, (C + CH - 1) / CH, B), block(32, CH);
-        SC_DISPATCH_IO(dtype, odt, (launch_k(L, dw_corr_s1_kernel<T, T, OT>, grid, block, smem, 
-                                       (const T*)x, (const T*)wd, (OT*)u, nullptr, nullptr, nullptr, len_in, len_out, C, Tt,
-                                       K, Kp, 0, L.status)));
+        SC_DISPATCH_IO(dtype, odt, (launch_corr<T, T, OT>(L, (const T*)x, (const T*)wd, (OT*)u, nullptr, nullptr, nullptr, len_in, len_out,
+                                                          B, C, Tt, K, 0)));
     } else {
         const size_t smem = (size_t)((GT - 1) * s + (K - 1) * dil + 1 + K) * sizeof(float);
         dim3 grid((Tp + GT - 1) / GT, C, B);
@@ -698,12 +693,8 @@ void dw_dgrad(const Launch& L, int dtype, int odt, const void* gu, const void* w
         return;
     }
     if (s == 1 && plain) {
-        const int Kp = kpad(K);
-        const size_t smem = (size_t)CH * (host_phys(TT + Kp) + 4 + Kp) * sizeof(float);
-        dim3 grid((Tt + TT - 1) / TT, (C + CH - 1) / CH, B), block(32, CH);
-        SC_DISPATCH_IO(dtype, odt, (launch_k(L, dw_corr_s1_kernel<OT, T, T>, grid, block, smem, 
-                                       (const OT*)gu, (const T*)wd, (T*)dx, (const T*)add1, (const T*)add2, gmax, len_out,
-                                       len_in, C, Tt, K, Kp, 1, L.status)));
+        SC_DISPATCH_IO(dtype, odt, (launch_corr<OT, T, T>(L, (const OT*)gu, (const T*)wd, (T*)dx, (const T*)add1, (const T*)add2, gmax,
+                                                          len_out, len_in, B, C, Tt, K, 1)));
     } else {
         const size_t smem = (size_t)((GT + (K - 1) * dil + 1) / s + 4 + K) * sizeof(float);
         dim3 grid((Tt + GT - 1) / GT, C, B);
