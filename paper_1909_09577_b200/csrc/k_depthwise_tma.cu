@@ -12,11 +12,9 @@
 // 128-byte swizzle; frames outside [0, T) are zero-filled by the TMA unit, which is the "same" padding.
 // Each input element is read from HBM once (window overlaps hit L2).  Rows of a tile are
 // (time block within a group of 128/BB, sample within a chunk of BB).
-// Warps: 0-7 epilogue (TMEM lane quarter w%4, column half w/4), 8 idle, 10-13 Toeplitz builders, which also
-// mask the input when it may be non-zero beyond a sample's length (they walk the rows that need it, one 16-byte vector per
-// lane, and build the next channel's block after a channel's tiles; with one warp and a row per lane a masked tile took
-// 12 k cycles, several times its loads and MMAs: a ragged fp16 block of 32 x 400 frames 102.2 -> 100.0 us, the projected
-// bf16 one 176.9 -> 171.6), 14 TMA producer (one box per lane),
+// Warps: 0-7 epilogue (TMEM lane quarter w%4, column half w/4), 8 input masking (only when the input
+// may be non-zero beyond a sample's length, and only of the rows whose window crosses it: a tile row wholly in padding
+// needs none, since its outputs are dropped and tile rows do not mix), 10-13 Toeplitz builders, 14 TMA producer (one box per lane),
 // 15 and 9 MMA issuers for the even and odd tiles (a tile costs its issuer about twenty barrier, MMA and
 // commit instructions of a hundred cycles or more each, so two issuers alternate; their tiles use
 // different accumulators and stages).  Accumulators are quadruple-buffered in tensor memory.  In the epilogue a
@@ -106,7 +104,7 @@ dw_tma_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ 
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     if (tid == 0) {
-        for (int s = 0; s < DT_MAX_STAGES; ++s) { ptx::mbar_init(&full[s], 1); ptx::mbar_init(&prep[s], 4); ptx::mbar_init(&empty[s], 1); }
+        for (int s = 0; s < DT_MAX_STAGES; ++s) { ptx::mbar_init(&full[s], 1); ptx::mbar_init(&prep[s], 1); ptx::mbar_init(&empty[s], 1); }
         for (int i = 0; i < DT_NACC; ++i) { ptx::mbar_init(&acc_full[i], 1); ptx::mbar_init(&acc_empty[i], 256); }
         for (int i = 0; i < 2; ++i) { ptx::mbar_init(&b_full[i], 4); ptx::mbar_init(&b_empty[i], 2); }
         ptx::fence_barrier_init();
@@ -194,8 +192,8 @@ dw_tma_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ 
         // index, so rows with an odd base read the copy that is shifted by one element
         const int base = DT_WOFF - j - p.delta;
         const uint32_t* src0 = reinterpret_cast<const uint32_t*>((base & 1) ? (wpadO + base - 1) : (wpadE + base));
-        // `ok` is false once a wait of this warp has run out: it then only meets the named barriers
-        auto build = [&](int c, int ci, bool ok) -> bool {
+        int ci = 0; bool dead = false;
+        for (int c = blockIdx.x; c < p.C && !dead; c += gridDim.x, ++ci) {
             const int bb = ci & 1;
             named_bar(2, 128);                         // everyone is done reading the previous channel's taps
             for (int i = bt; i < DT_WLEN; i += 128) {
@@ -208,8 +206,8 @@ dw_tma_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ 
                 if (i == DT_WLEN - 1) wpadO[i] = 0;
             }
             named_bar(2, 128);
-            if (!ok) return false;
-            if (!ptx::mbar_wait_warp(&b_empty[bb], ((ci >> 1) & 1) ^ 1, 32)) { if (lane == 0) raise_status(p.status, kErrTimeout); return false; }
+            const bool ok = ptx::mbar_wait_warp(&b_empty[bb], ((ci >> 1) & 1) ^ 1, 32);
+            if (!ok) { if (lane == 0) raise_status(p.status, kErrTimeout); dead = true; break; }
             uint4* rowbase = reinterpret_cast<uint4*>(sB + bb * p.b_stride + j * 128);
             for (int v = hv; v < nvec; v += 2) {       // vector v holds j' = 8 v .. 8 v + 7
                 const uint32_t* src = src0 + 4 * v;
@@ -219,33 +217,36 @@ dw_tma_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ 
             ptx::fence_proxy_async();
             __syncwarp();
             if (lane == 0) ptx::mbar_arrive(&b_full[bb]);
-            return true;
-        };
-        const int r0 = 32 * (warp - 10), lb = p.BB == 32 ? 5 : 4;      // masking: this warp's 32 tile rows
-        const int tbl0 = (r0 + lane) >> lb, bi = (r0 + lane) & (p.BB - 1);
-        int ci = 0, s = 0, ph = 0;
-        bool ok = true;
-        for (int c = blockIdx.x; c < p.C; c += gridDim.x, ++ci) {
-            if (!MASK || ci == 0) ok = build(c, ci, ok);
-            if (MASK) {
-                if (ci == 0) pdl_wait();
-                for (int chunk = 0; chunk < p.nchunks && ok; ++chunk) {
+        }
+    } else if (warp == 8) {                            // ---- input masking ----
+        // A row needs it when its window crosses the sample's length and some of its outputs are valid: the last time block
+        // with a valid output, tb1, and perhaps the one before (a window spans at most two blocks behind its first output).
+        // Lanes go over their own samples' rows (BB = 16: half of the lanes over tb1, half over the block before).
+        // Masking every padded row, one vector per lane and row after row, took several times as long as a tile's loads and
+        // MMAs (32 x 512 x 800 with lengths from 300, K = 63: 40.8 us, now 19.3; full lengths 17.5).
+        if (MASK) {
+            const int bi = lane & (p.BB - 1), i0 = p.BB == 32 ? 0 : lane >> 4, i1 = p.BB == 32 ? 2 : i0 + 1;
+            pdl_wait();
+            int s = 0, ph = 0; bool dead = false;
+            for (int c = blockIdx.x; c < p.C && !dead; c += gridDim.x) {
+                for (int chunk = 0; chunk < p.nchunks && !dead; ++chunk) {
                     const int b = chunk * p.BB + bi;
-                    const int len = b < p.B ? min(p.len_src[b], p.T) : 0;               // of this lane's row
-                    for (int g = 0; g < p.ngrp && ok; ++g) {
-                        const int left = len - (128 * (g * p.TBL + tbl0) - p.Pa);       // valid frames from the window's start
-                        uint32_t todo = __ballot_sync(0xffffffffu, left < 64 * p.nxb);
-                        const bool wrote = todo != 0;
-                        ok = ptx::mbar_wait_warp(&full[s], ph);
-                        if (!ok) { if (lane == 0) raise_status(p.status, kErrTimeout); break; }
-                        uint8_t* tile = smem + s * p.stage_bytes + (lane >> 3) * 16384;
-                        for (; todo; todo &= todo - 1) {
-                            const int rr = __ffs(todo) - 1, r = r0 + rr;
-                            const int n = __shfl_sync(0xffffffffu, left, rr) - 8 * lane;   // valid frames of vector `lane`
-                            if (lane < 8 * p.nxb && n < 8) {
-                                uint4* pv = reinterpret_cast<uint4*>(tile + r * 128) + ((lane & 7) ^ (r & 7));
-                                *pv = n <= 0 ? make_uint4(0, 0, 0, 0) : keep_first(*pv, n);
-                            }
+                    const int len = b < p.B ? min(p.len_src[b], p.T) : p.T;     // past T the copy itself has filled in zeros
+                    const int tb1 = (len - 1) >> 7;
+                    for (int g = 0; g < p.ngrp; ++g) {
+                        const bool ok = ptx::mbar_wait_warp(&full[s], ph);
+                        if (!ok) { if (lane == 0) raise_status(p.status, kErrTimeout); dead = true; break; }
+                        bool wrote = false;
+                        for (int i = i0; i < i1; ++i) {
+                            const int tbl = tb1 - i - g * p.TBL, left = len - (128 * (tb1 - i) - p.Pa);   // valid frames of the window
+                            if (len >= p.T || tbl < 0 || tbl >= p.TBL || left >= 64 * p.nxb) continue;
+                            const int r = tbl * p.BB + bi;
+                            uint8_t* row = smem + s * p.stage_bytes + r * 128;
+                            int v = left >> 3;
+                            auto at = [&](int q) { return reinterpret_cast<uint4*>(row + (q >> 3) * 16384) + ((q & 7) ^ (r & 7)); };
+                            if (left & 7) { *at(v) = keep_first(*at(v), left & 7); ++v; }
+                            for (; v < 8 * p.nxb; ++v) *at(v) = make_uint4(0, 0, 0, 0);
+                            wrote = true;
                         }
                         if (wrote) ptx::fence_proxy_async();
                         __syncwarp();
@@ -254,9 +255,8 @@ dw_tma_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ 
                     }
                 }
             }
-            if (MASK && c + gridDim.x < p.C) ok = build(c + gridDim.x, ci + 1, ok);
         }
-    } else if (warp < 8) {                                           // ---- epilogue (warps 0-7) ----
+    } else {                                           // ---- epilogue (warps 0-7) ----
         const int wq = warp & 3, half = warp >> 2;
         uint8_t* stg = stg_all + warp * DT_STG_BYTES;
         pdl_wait();
@@ -353,6 +353,7 @@ dw_tma_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ 
 #pragma unroll 1
                         for (int cc = 0; cc < 2; ++cc) {
                             uint32_t v[32];
+                            __syncwarp();
                             ptx::tmem_ld32(taddr + 32 * cc, v);
                             ptx::tmem_ld_wait();
                             __syncwarp();

@@ -247,23 +247,26 @@ dw_wgrad_tc_kernel(const __grid_constant__ CUtensorMap mapG, const __grid_consta
             const int c = unit / p.S, sp = unit - c * p.S;
             (void)c;
             StepWalk w; w.begin(sp, p.ks_per_split, ks_total, p.ntb, chunk_len);
+            int len_chunk = -1, len0 = 0, len1 = 0;      // lengths of this thread's (at most two) rows, read once per chunk
             for (; w.more(); w.next()) {
                 if (!w.on()) continue;
                 if ((it & 1) == grp) {
+                    if (p.mask && w.chunk != len_chunk) {
+                        const int ba = w.chunk * p.BB + r0, bb = ba + 16;
+                        len0 = ba < p.B ? min(p.len_in[ba], p.T) : 0;
+                        len1 = bb < p.B ? min(p.len_in[bb], p.T) : 0;
+                        len_chunk = w.chunk;
+                    }
                     const bool ok = ptx::mbar_wait_warp(&full[rg.s], rg.ph);
                     if (!ok) { if (lane == 0) raise_status(p.status, kErrTimeout); dead = true; break; }
                     if (p.prep) {
 #pragma unroll 1
                         for (int hb = 0; hb < 2; ++hb) {
                             uint4* sX = reinterpret_cast<uint4*>(smem + rg.s * p.stage_bytes + 2 * g_bytes + hb * x_bytes);
-                            const int tx0 = w.tb * 256 + 128 * hb - p.Pa + toff, b0 = w.chunk * p.BB;
-                            // frames left before the sample's end, for this thread's (at most two) rows
+                            const int tx0 = w.tb * 256 + 128 * hb - p.Pa + toff;
+                            // frames left before the sample's end
                             int left0 = 1 << 30, left1 = 1 << 30;
-                            if (p.mask) {
-                                const int ba = b0 + r0, bb = b0 + r0 + 16;
-                                left0 = (ba < p.B ? min(p.len_in[ba], p.T) : 0) - tx0;
-                                left1 = (bb < p.B ? min(p.len_in[bb], p.T) : 0) - tx0;
-                            }
+                            if (p.mask) { left0 = len0 - tx0; left1 = len1 - tx0; }
                             uint4 raw[8];
 #pragma unroll
                             for (int i = 0; i < 8; ++i) if (i < nvec_t) raw[i] = sX[ctid + 128 * i];
