@@ -157,39 +157,72 @@ template <> __device__ __forceinline__ void st8<__nv_bfloat16>(__nv_bfloat16* p,
     *reinterpret_cast<uint4*>(p) = r;
 }
 
-// Eight consecutive 16-bit elements that start at any element index of a 16-byte aligned dense array: two aligned
-// vectors and a funnel shift.  idx < total; elements at and beyond `total` come back unspecified.  (The second vector
-// is read only when it holds at least one element of the array, so no 16-byte line outside it is touched.)
-__device__ __forceinline__ uint4 ld8_any(const void* base, uint32_t idx, uint32_t total) {
-    const uint4* p = reinterpret_cast<const uint4*>(base) + (idx >> 3);
-    const uint32_t sh = idx & 7;
-    const uint4 lo = p[0];
-    if (sh == 0) return lo;
-    uint4 hi = make_uint4(0, 0, 0, 0);
-    if ((idx | 7u) + 1 < total) hi = p[1];
-    uint32_t w[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
-    if (sh & 4) {
+// Elements of a 16-byte aligned dense 16-bit array that start at any element index.  Fetching and picking are two steps, so
+// that a thread can have the aligned vectors of all its operands in flight before it waits for the first (fetched and
+// shifted one after the other, behind a branch on the alignment, the unaligned batch-norm kernels took 2-3 times as long as
+// the aligned ones).  fetch<N>: the N aligned vectors from the one that holds element idx on; a vector past the array's last
+// is replaced by the last, so no 16-byte line outside it is touched.
+template <int N> struct RawVec { uint4 v[N]; };
+template <int N> __device__ __forceinline__ RawVec<N> fetch(const void* base, uint32_t idx, uint32_t total) {
+    const uint4* p = reinterpret_cast<const uint4*>(base);
+    const uint32_t q = idx >> 3, last = (total - 1) >> 3;
+    RawVec<N> r;
 #pragma unroll
-        for (int i = 0; i < 6; ++i) w[i] = w[i + 2];
-    }
-    if (sh & 2) {
-#pragma unroll
-        for (int i = 0; i < 5; ++i) w[i] = w[i + 1];
-    }
-    if (sh & 1) {
-#pragma unroll
-        for (int i = 0; i < 4; ++i) w[i] = __funnelshift_r(w[i], w[i + 1], 16);
-    }
-    return make_uint4(w[0], w[1], w[2], w[3]);
+    for (int i = 0; i < N; ++i) r.v[i] = p[min(q + i, last)];
+    return r;
 }
-// Eight elements idx, idx + 2, ..., idx + 14 of the same kind of array.
-__device__ __forceinline__ uint4 ld8_even(const void* base, uint32_t idx, uint32_t total) {
-    const uint4 a = ld8_any(base, idx, total);
-    uint4 b = make_uint4(0, 0, 0, 0);
-    if (idx + 8 < total) b = ld8_any(base, idx + 8, total);
-    return make_uint4(__byte_perm(a.x, a.y, 0x5410), __byte_perm(a.z, a.w, 0x5410), __byte_perm(b.x, b.y, 0x5410),
-                      __byte_perm(b.z, b.w, 0x5410));
+// w[0 ..] <- w[off ..], off in 0 .. 3 (the first n words of the result are used)
+template <int M> __device__ __forceinline__ void shift_words(uint32_t (&w)[M], int n, uint32_t off) {
+#pragma unroll
+    for (int i = 0; i < M - 2; ++i) if (i < n + 1) w[i] = (off & 2) ? w[i + 2] : w[i];
+#pragma unroll
+    for (int i = 0; i < M - 3; ++i) if (i < n) w[i] = (off & 1) ? w[i + 1] : w[i];
 }
+// elements idx, idx + 1, ..., idx + 7
+__device__ __forceinline__ uint4 pick8(const RawVec<2>& r, uint32_t idx) {
+    uint32_t w[8] = {r.v[0].x, r.v[0].y, r.v[0].z, r.v[0].w, r.v[1].x, r.v[1].y, r.v[1].z, r.v[1].w};
+    shift_words(w, 5, (idx >> 1) & 3);
+    const uint32_t sh = (idx & 1) * 16;
+    return make_uint4(__funnelshift_r(w[0], w[1], sh), __funnelshift_r(w[1], w[2], sh), __funnelshift_r(w[2], w[3], sh),
+                      __funnelshift_r(w[3], w[4], sh));
+}
+// elements idx, idx + 2, ..., idx + 14
+__device__ __forceinline__ uint4 pick8_even(const RawVec<3>& r, uint32_t idx) {
+    uint32_t w[12] = {r.v[0].x, r.v[0].y, r.v[0].z, r.v[0].w, r.v[1].x, r.v[1].y, r.v[1].z, r.v[1].w, r.v[2].x, r.v[2].y, r.v[2].z, r.v[2].w};
+    shift_words(w, 8, (idx >> 1) & 3);
+    const uint32_t sel = (idx & 1) ? 0x7632u : 0x5410u;
+    return make_uint4(__byte_perm(w[0], w[1], sel), __byte_perm(w[2], w[3], sel), __byte_perm(w[4], w[5], sel), __byte_perm(w[6], w[7], sel));
+}
+__device__ __forceinline__ uint4 ld8_any(const void* base, uint32_t idx, uint32_t total) { return pick8(fetch<2>(base, idx, total), idx); }
+
+// Eight consecutive frames t .. t + 7 of dense row (b, c) from a packed tensor [B D, C, Tq] (kernels.h): for one phase they
+// are contiguous, for two they alternate between the rows of the phases, four from each (aligned when the dense rows are
+// whole vectors).  t may lie up to 7 frames outside the row on either side; what is picked there is unspecified.
+template <int D> struct Packed8 {
+    RawVec<2> r; uint32_t idx;
+    __device__ __forceinline__ Packed8() : r{}, idx(0) {}
+    __device__ __forceinline__ Packed8(const void* src, int b, int c, int C, int Tq, int t, uint32_t total, bool aligned) {
+        if (D == 1) { idx = ((uint32_t)b * C + c) * Tq + t; r = fetch<2>(src, idx, total); return; }
+        const unsigned short* s = reinterpret_cast<const unsigned short*>(src);
+        const uint32_t i0 = ((uint32_t)(b * 2 + (t & 1)) * C + c) * Tq + (t >> 1), i1 = ((uint32_t)(b * 2 + ((t + 1) & 1)) * C + c) * Tq + ((t + 1) >> 1);
+        idx = 0;
+        uint2 a, h;
+        if (aligned) {
+            a = *reinterpret_cast<const uint2*>(s + i0); h = *reinterpret_cast<const uint2*>(s + i1);
+        } else {
+            uint32_t e[8];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) { e[i] = s[min(i0 + i, total - 1)]; e[4 + i] = s[min(i1 + i, total - 1)]; }
+            a = make_uint2(e[0] | (e[1] << 16), e[2] | (e[3] << 16)); h = make_uint2(e[4] | (e[5] << 16), e[6] | (e[7] << 16));
+        }
+        r.v[0] = make_uint4(a.x, a.y, h.x, h.y);
+    }
+    __device__ __forceinline__ uint4 get() const {
+        if (D == 1) return pick8(r, idx);
+        const uint4 q = r.v[0];
+        return make_uint4(__byte_perm(q.x, q.z, 0x5410), __byte_perm(q.x, q.z, 0x7632), __byte_perm(q.y, q.w, 0x5410), __byte_perm(q.y, q.w, 0x7632));
+    }
+};
 // zeroes the elements n, n + 1, ... (n < 8) of a vector of eight 16-bit elements
 __device__ __forceinline__ uint4 keep_first(const uint4& r, int n) {
     uint32_t w[4] = {r.x, r.y, r.z, r.w};
@@ -199,6 +232,25 @@ __device__ __forceinline__ uint4 keep_first(const uint4& r, int n) {
         else if (2 * i + 1 >= n) w[i] &= 0x0000FFFFu;
     }
     return make_uint4(w[0], w[1], w[2], w[3]);
+}
+
+// elements [0, n) of a, the rest of b
+__device__ __forceinline__ uint4 splice(const uint4& a, const uint4& b, int n) {
+    uint32_t x[4] = {a.x, a.y, a.z, a.w};
+    const uint32_t y[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        if (2 * i >= n) x[i] = y[i];
+        else if (2 * i + 1 >= n) x[i] = (x[i] & 0x0000FFFFu) | (y[i] & 0xFFFF0000u);
+    }
+    return make_uint4(x[0], x[1], x[2], x[3]);
+}
+// the first n elements of a 16-byte vector to p (16-byte aligned)
+__device__ __forceinline__ void st8_first(unsigned short* p, const uint4& r, int n) {
+    if (n >= 8) { *reinterpret_cast<uint4*>(p) = r; return; }
+    const uint32_t w[4] = {r.x, r.y, r.z, r.w};
+#pragma unroll
+    for (int i = 0; i < 8; ++i) if (i < n) p[i] = (unsigned short)(w[i >> 1] >> (16 * (i & 1)));
 }
 
 __device__ __forceinline__ float warp_sum(float v) {

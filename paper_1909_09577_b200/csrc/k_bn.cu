@@ -569,13 +569,14 @@ __device__ __forceinline__ void apply_core(T* yp, int n, const uint4& rv, const 
     }
     st8<T>(yp, out);
 }
+template <int RES> __device__ __forceinline__ void fwd_chan(const ApplyArgs& a, int o, FwdChan& c) {
+    c.mu = a.mean[o]; c.is = a.invstd[o]; c.ga = a.gamma[o]; c.be = a.beta[o];
+    if (RES == 2) { c.mur = a.mean_r[o]; c.isr = a.invstd_r[o]; c.gar = a.gamma_r[o]; c.ber = a.beta_r[o]; }
+}
 template <typename T, typename NT, int RES>
 __device__ __forceinline__ void apply_vec(const ApplyArgs& a, int o, int n, size_t off, const uint4& rv, const uint4& rr) {
     FwdChan c{};
-    if (n > 0) {
-        c.mu = a.mean[o]; c.is = a.invstd[o]; c.ga = a.gamma[o]; c.be = a.beta[o];
-        if (RES == 2) { c.mur = a.mean_r[o]; c.isr = a.invstd_r[o]; c.gar = a.gamma_r[o]; c.ber = a.beta_r[o]; }
-    }
+    if (n > 0) fwd_chan<RES>(a, o, c);
     apply_core<T, NT, RES>((T*)a.y + off, n, rv, rr, c);
 }
 
@@ -780,69 +781,81 @@ __global__ void __launch_bounds__(256) bn_apply_fast_kernel(ApplyArgs a, int vpr
 }
 
 // The same step from packed v / vr to dense y: a thread takes V aligned 8-element vectors of the dense tensor and gathers
-// the packed operands (for one phase a vector that starts anywhere in its row; for two, four elements of each phase).
-// A vector that runs over the end of a row is done element by element.  Blocks past the tensor's own copy u out.
+// the packed operands.  A vector that runs over the end of a row (of at least 8 frames) is spliced from this row's last
+// frames and the next row's first; shorter rows are done element by element.  Blocks past the tensor's own copy u out.
 // What it replaces: four extra passes (v, vr, y and u copied to dense form one after the other) and their launches.
-template <int D>
-__device__ __forceinline__ uint32_t packed_index(const ApplyArgs& a, int b, int c, int C, int t) {
-    return D == 1 ? ((uint32_t)b * C + c) * a.Tp + t : (((uint32_t)b * 2 + (t & 1)) * C + c) * a.Tp + (t >> 1);
-}
-template <int D>
-__device__ __forceinline__ uint4 gather_packed(const ApplyArgs& a, const void* src, int b, int c, int C, int t, uint32_t total) {
-    if (D == 1) return ld8_any(src, packed_index<1>(a, b, c, C, t), total);
-    const unsigned short* s = reinterpret_cast<const unsigned short*>(src);
-    const unsigned short* e0 = s + packed_index<2>(a, b, c, C, t);
-    const unsigned short* e1 = s + packed_index<2>(a, b, c, C, t + 1);
-    uint4 r;
-    r.x = e0[0] | ((uint32_t)e1[0] << 16); r.y = e0[1] | ((uint32_t)e1[1] << 16);
-    r.z = e0[2] | ((uint32_t)e1[2] << 16); r.w = e0[3] | ((uint32_t)e1[3] << 16);
-    return r;
-}
 template <typename T, typename NT, int RES, int D>
 __global__ void __launch_bounds__(256) bn_apply_unpack_kernel(ApplyArgs a, uint32_t total, int nblk_apply, uint32_t total_u) {
-    pdl_sync();
     const bool copy = (int)blockIdx.x >= nblk_apply;
-    const int C = copy ? a.Cu : a.C;
+    const int C = copy ? a.Cu : a.C, nrows = a.B * C;
     const uint32_t tot = copy ? total_u : total;
     const uint32_t tot_packed = (uint32_t)a.B * D * C * a.Tp;
-    constexpr int V = 2;
+    const bool aligned = (a.T & 7) == 0, vector_rows = a.T >= 8;
+    // one vector per thread: with two, 30.0 us where this takes 26.1 (bf16, 23 x 384 x 797, projected residual): registers
+    // against warps in flight
+    constexpr int V = 1;
     const uint32_t tid = (blockIdx.x - (copy ? nblk_apply : 0)) * 256u + threadIdx.x;
     const uint32_t base = ((tid >> 5) * (32u * V) + (threadIdx.x & 31)) * 8u;
-    uint4 rv[V], rr[V]; int ch[V], n[V]; bool whole[V];
+    int row[V], t[V], b[V], ch[V], n[V];
 #pragma unroll
     for (int j = 0; j < V; ++j) {
         const uint32_t f = base + 256u * j;
-        whole[j] = false; n[j] = 0; ch[j] = 0;
-        rv[j] = rr[j] = make_uint4(0, 0, 0, 0);
-        if (f >= tot) continue;
-        const int row = (int)a.dT.div(f), t = (int)(f - (uint32_t)row * a.T);
-        const int b = row / C;
-        ch[j] = row - b * C;
-        if (t + 8 > a.T || f + 8 > tot) continue;
-        whole[j] = true;
-        n[j] = min(a.len_out[b], a.T) - t;
-        if (n[j] > 0) {
-            rv[j] = gather_packed<D>(a, copy ? a.u : a.v, b, ch[j], C, t, tot_packed);
-            if (!copy && RES == 1) rr[j] = *reinterpret_cast<const uint4*>((const T*)a.xres + f);
-            if (!copy && RES == 2) rr[j] = gather_packed<D>(a, a.vr, b, ch[j], C, t, tot_packed);
+        row[j] = t[j] = b[j] = ch[j] = n[j] = 0;
+        if (f < tot) {
+            row[j] = (int)a.dT.div(f); t[j] = (int)(f - (uint32_t)row[j] * a.T);
+            b[j] = row[j] / C; ch[j] = row[j] - b[j] * C;
+            n[j] = min(a.len_out[b[j]], a.T) - t[j];
         }
+    }
+    pdl_sync();
+    Packed8<D> rv[V], rr[V]; uint4 rx[V];
+#pragma unroll
+    for (int j = 0; j < V; ++j) {
+        rx[j] = make_uint4(0, 0, 0, 0);
+        if (vector_rows && n[j] > 0) {
+            rv[j] = Packed8<D>(copy ? a.u : a.v, b[j], ch[j], C, a.Tp, t[j], tot_packed, aligned);
+            if (RES == 2 && !copy) rr[j] = Packed8<D>(a.vr, b[j], ch[j], C, a.Tp, t[j], tot_packed, aligned);
+        }
+        // the dense operand is aligned like the result (the last vector may hold less than eight elements)
+        if (RES == 1 && !copy && vector_rows && base + 256u * j < tot) rx[j] = fetch<1>(a.xres, base + 256u * j, tot).v[0];
     }
 #pragma unroll
     for (int j = 0; j < V; ++j) {
         const uint32_t f = base + 256u * j;
         if (f >= tot) continue;
-        if (whole[j]) {
-            if (copy) { *reinterpret_cast<uint4*>((NT*)a.u_out + f) = n[j] >= 8 ? rv[j] : keep_first(rv[j], n[j]); continue; }
-            apply_vec<T, NT, RES>(a, ch[j], n[j], f, rv[j], rr[j]);
-            if (a.v_out) *reinterpret_cast<uint4*>((NT*)a.v_out + f) = rv[j];
-            if (RES == 2 && a.vr_out) *reinterpret_cast<uint4*>((NT*)a.vr_out + f) = rr[j];
+        const int left = (int)min(8u, tot - f);
+        if (vector_rows) {
+            uint4 q = rv[j].get(), qr = RES == 1 ? rx[j] : (RES == 2 ? rr[j].get() : rx[j]), y = make_uint4(0, 0, 0, 0);
+            if (!copy) {
+                FwdChan c{};
+                fwd_chan<RES>(a, ch[j], c);
+                apply_core<T, NT, RES>((T*)&y, n[j], q, qr, c);
+            } else if (n[j] < 8) q = keep_first(q, n[j]);
+            const int k = a.T - t[j];                          // elements of this row
+            if (k < 8 && row[j] + 1 < nrows) {
+                const int b2 = (row[j] + 1) / C, c2 = row[j] + 1 - b2 * C, n2 = min(a.len_out[b2], a.T) + k;
+                uint4 p = Packed8<D>(copy ? a.u : a.v, b2, c2, C, a.Tp, -k, tot_packed, false).get(), pr = rx[j], y2;
+                if (RES == 2 && !copy) pr = Packed8<D>(a.vr, b2, c2, C, a.Tp, -k, tot_packed, false).get();
+                if (!copy) {
+                    FwdChan c{};
+                    fwd_chan<RES>(a, c2, c);
+                    apply_core<T, NT, RES>((T*)&y2, n2, p, pr, c);
+                    y = splice(y, y2, k);
+                } else if (n2 < 8) p = keep_first(p, n2);
+                q = splice(q, p, k);
+                if (RES == 2) qr = splice(qr, pr, k);
+            }
+            if (copy) { st8_first((unsigned short*)a.u_out + f, q, left); continue; }
+            st8_first((unsigned short*)a.y + f, y, left);
+            if (a.v_out) st8_first((unsigned short*)a.v_out + f, q, left);
+            if (RES == 2 && a.vr_out) st8_first((unsigned short*)a.vr_out + f, qr, left);
             continue;
         }
-        for (uint32_t e = f; e < min(f + 8, tot); ++e) {
-            const int row = (int)a.dT.div(e), t = (int)(e - (uint32_t)row * a.T);
-            const int b = row / C, o = row - b * C;
-            const bool in = t < min(a.len_out[b], a.T);
-            const uint32_t q = packed_index<D>(a, b, o, C, t);
+        for (uint32_t e = f; e < f + left; ++e) {
+            const int row_e = (int)a.dT.div(e), te = (int)(e - (uint32_t)row_e * a.T);
+            const int be = row_e / C, o = row_e - be * C;
+            const bool in = te < min(a.len_out[be], a.T);
+            const uint32_t q = D == 1 ? (uint32_t)row_e * a.Tp + te : ((uint32_t)(be * 2 + (te & 1)) * C + o) * a.Tp + (te >> 1);
             if (copy) { ((unsigned short*)a.u_out)[e] = in ? ((const unsigned short*)a.u)[q] : (unsigned short)0; continue; }
             const NT vq = in ? ((const NT*)a.v)[q] : NT(0.f);
             float r = 0.f;
@@ -859,17 +872,23 @@ __global__ void __launch_bounds__(256) bn_apply_unpack_kernel(ApplyArgs a, uint3
     }
 }
 
-// Operand of the backward kernels: eight frames of packed row `row`, position t0 of it, from a tensor that has the same
+// Operand of the backward kernels: eight frames of packed row (b, o), position t0 of it, from a tensor that has the same
 // (packed) layout (G = 0, element offset off) or is dense with one or two phases per sample (G = 1, 2).  n > 0 frames
 // are inside the sample; a dense tensor's frames past them are unspecified and come back as zero (a masked gradient times
 // a NaN would not be zero).
-template <int G>
-__device__ __forceinline__ uint4 bwd_load(const BnBwdArgs& a, const void* src, size_t off, int b, int o, int t0, int n) {
-    if (G == 0) return *reinterpret_cast<const uint4*>(reinterpret_cast<const unsigned short*>(src) + off);
-    const uint4 r = G == 1 ? ld8_any(src, ((uint32_t)b * a.C + o) * a.T + t0, a.total_dense)
-                           : ld8_even(src, ((uint32_t)(b >> 1) * a.C + o) * a.T + 2 * t0 + (b & 1), a.total_dense);
-    return n < 8 ? keep_first(r, n) : r;
-}
+template <int G> struct BwdRaw {
+    RawVec<G + 1> r; uint32_t idx;
+    __device__ __forceinline__ BwdRaw() : r{}, idx(0) {}
+    __device__ __forceinline__ BwdRaw(const BnBwdArgs& a, const void* src, size_t off, int b, int o, int t0) : idx(0) {
+        if (G == 0) { r.v[0] = *reinterpret_cast<const uint4*>(reinterpret_cast<const unsigned short*>(src) + off); return; }
+        idx = G == 1 ? ((uint32_t)b * a.C + o) * a.T + t0 : ((uint32_t)(b >> 1) * a.C + o) * a.T + 2 * t0 + (b & 1);
+        r = fetch<G + 1>(src, idx, a.total_dense);
+    }
+    __device__ __forceinline__ uint4 get(int n) const;
+};
+template <> __device__ __forceinline__ uint4 BwdRaw<0>::get(int) const { return r.v[0]; }
+template <> __device__ __forceinline__ uint4 BwdRaw<1>::get(int n) const { const uint4 q = pick8(r, idx); return n < 8 ? keep_first(q, n) : q; }
+template <> __device__ __forceinline__ uint4 BwdRaw<2>::get(int n) const { const uint4 q = pick8_even(r, idx); return n < 8 ? keep_first(q, n) : q; }
 
 template <typename T, typename NT, typename GT, int RES, int V, int G>
 __global__ void __launch_bounds__(256) bn_bwd_apply_fast_kernel(BnBwdArgs a, int vpr, long long total) {
@@ -877,12 +896,11 @@ __global__ void __launch_bounds__(256) bn_bwd_apply_fast_kernel(BnBwdArgs a, int
     const uint32_t base = (tid >> 5) * (32u * V) + (threadIdx.x & 31), tot = (uint32_t)total;
     const bool fold = !a.gv16 && a.gv_scaled;
     size_t off[V]; int nin[V], ch[V], bs[V], t0s[V];
-    uint4 rg[V], rv[V], rr[V], ry[V];
+    BwdRaw<G> rg[V], rv[V], rr[V], ry[V];
 #pragma unroll
     for (int j = 0; j < V; ++j) {
         const uint32_t idx = base + 32u * j;
         nin[j] = -1; ch[j] = 0; off[j] = 0; bs[j] = 0; t0s[j] = 0;
-        rg[j] = rv[j] = rr[j] = ry[j] = make_uint4(0, 0, 0, 0);
         if (idx < tot) {
             const int row = (int)a.dvpr.div(idx);
             t0s[j] = ((int)idx - row * vpr) * 8;
@@ -898,16 +916,16 @@ __global__ void __launch_bounds__(256) bn_bwd_apply_fast_kernel(BnBwdArgs a, int
     for (int j = 0; j < V; ++j) {
         if (nin[j] > 0) {
             const int b = bs[j], t0 = t0s[j];
-            rg[j] = bwd_load<G>(a, a.g, off[j], b, ch[j], t0, nin[j]);
-            rv[j] = bwd_load<G>(a, a.v, off[j], b, ch[j], t0, nin[j]);
-            if (RES == 2) rr[j] = bwd_load<G>(a, a.vr, off[j], b, ch[j], t0, nin[j]);
-            if (RES != 0) ry[j] = bwd_load<G>(a, a.y, off[j], b, ch[j], t0, nin[j]);
+            rg[j] = BwdRaw<G>(a, a.g, off[j], b, ch[j], t0);
+            rv[j] = BwdRaw<G>(a, a.v, off[j], b, ch[j], t0);
+            if (RES == 2) rr[j] = BwdRaw<G>(a, a.vr, off[j], b, ch[j], t0);
+            if (RES != 0) ry[j] = BwdRaw<G>(a, a.y, off[j], b, ch[j], t0);
         }
     }
 #pragma unroll
     for (int j = 0; j < V; ++j) {
         if (nin[j] < 0) continue;
-        bwd_apply_vec<T, NT, GT, RES>(a, ch[j], nin[j], off[j], sc, fold, rg[j], rv[j], rr[j], ry[j]);
+        bwd_apply_vec<T, NT, GT, RES>(a, ch[j], nin[j], off[j], sc, fold, rg[j].get(nin[j]), rv[j].get(nin[j]), rr[j].get(nin[j]), ry[j].get(nin[j]));
     }
 }
 
@@ -987,11 +1005,12 @@ constexpr int kChThreads = 512;
 // Backward reduction of channel o over every sample, then the channel's coefficients, parameter gradients and its
 // term of the bound on |gv| (what bn_bwd_finalize_kernel does for the row-mapped reduction).
 template <typename T, typename NT, int RES, int G>
-__global__ void __launch_bounds__(kChThreads, 2)
+__global__ void __launch_bounds__(kChThreads, G == 2 && RES == 2 ? 1 : 2)
 bn_bwd_reduce_ch_kernel(BnBwdArgs a, int vpr, const float* gamma_r, float* dgamma, float* dbeta, float* dgamma_r,
                         float* dbeta_r, int accumulate) {
     constexpr int NT_ = kChThreads;
-    constexpr int U = RES == 2 ? 2 : 4;            // 16-byte loads in flight per thread: U * (2 or 4 tensors)
+    // 16-byte loads in flight per thread: U * (2 to 4 tensors) * (1 to 3 vectors)
+    constexpr int U = G == 0 ? (RES == 2 ? 2 : 4) : (G == 1 && RES == 0 ? 2 : 1);
     __shared__ float4 s_sum[NT_ / 32];
     const int o = blockIdx.x, tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     BwdChan c{};
@@ -1003,21 +1022,20 @@ bn_bwd_reduce_ch_kernel(BnBwdArgs a, int vpr, const float* gamma_r, float* dgamm
     float s0 = 0.f, s1 = 0.f, s3 = 0.f, amax = 0.f;
     for (int jb = tid; jb < nvec; jb += U * NT_) {
         int nin[U];
-        uint4 rg[U], rv[U], rr[U], ry[U];
+        BwdRaw<G> rg[U], rv[U], rr[U], ry[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             const int j = jb + u * NT_;
             nin[u] = 0;
-            rg[u] = rv[u] = rr[u] = ry[u] = make_uint4(0, 0, 0, 0);
             if (j < nvec) {
                 const int b = (int)a.dvpr.div((uint32_t)j), t0 = (j - b * vpr) * 8;
                 nin[u] = max(0, min(a.len_out[b], a.Tp) - t0);
                 if (nin[u] > 0) {
                     const size_t off = ((size_t)b * a.C + o) * a.Tp + t0;
-                    rg[u] = bwd_load<G>(a, a.g, off, b, o, t0, nin[u]);
-                    rv[u] = bwd_load<G>(a, a.v, off, b, o, t0, nin[u]);
-                    if (RES == 2) rr[u] = bwd_load<G>(a, a.vr, off, b, o, t0, nin[u]);
-                    if (RES != 0) ry[u] = bwd_load<G>(a, a.y, off, b, o, t0, nin[u]);
+                    rg[u] = BwdRaw<G>(a, a.g, off, b, o, t0);
+                    rv[u] = BwdRaw<G>(a, a.v, off, b, o, t0);
+                    if (RES == 2) rr[u] = BwdRaw<G>(a, a.vr, off, b, o, t0);
+                    if (RES != 0) ry[u] = BwdRaw<G>(a, a.y, off, b, o, t0);
                 }
             }
         }
@@ -1025,7 +1043,7 @@ bn_bwd_reduce_ch_kernel(BnBwdArgs a, int vpr, const float* gamma_r, float* dgamm
         for (int u = 0; u < U; ++u) {
             if (nin[u] <= 0) continue;
             float q0, q1, q3, m;
-            reduce_core<T, NT, RES>(nin[u], rg[u], rv[u], rr[u], ry[u], c, q0, q1, q3, m);
+            reduce_core<T, NT, RES>(nin[u], rg[u].get(nin[u]), rv[u].get(nin[u]), rr[u].get(nin[u]), ry[u].get(nin[u]), c, q0, q1, q3, m);
             s0 += q0; s1 += q1; s3 += q3; amax = fmaxf(amax, m);
         }
     }
@@ -1163,8 +1181,8 @@ void bn_apply(const Launch& L, int dtype, const ApplyArgs& a_in) {
     if (a.phases) {
         a.dT = FastDiv((uint32_t)a.T);
         const uint32_t total = (uint32_t)a.B * a.C * a.T, total_u = a.u_out ? (uint32_t)a.B * a.Cu * a.T : 0;
-        const int nba = (int)fast_grid((total + 7) / 8, 2);
-        const unsigned grid = nba + (a.u_out ? fast_grid((total_u + 7) / 8, 2) : 0);
+        const int nba = (int)fast_grid((total + 7) / 8, 1);
+        const unsigned grid = nba + (a.u_out ? fast_grid((total_u + 7) / 8, 1) : 0);
 #define SC_APPLY_UNPACK(RES)                                                                                                  \
         if (a.phases == 2) { SC_DISPATCH16(dtype, (launch_k(L, bn_apply_unpack_kernel<T, NT, RES, 2>, grid, 256, 0, a, total, nba, total_u))) } \
         else { SC_DISPATCH16(dtype, (launch_k(L, bn_apply_unpack_kernel<T, NT, RES, 1>, grid, 256, 0, a, total, nba, total_u))) }
@@ -1253,11 +1271,11 @@ void bn_bwd_apply(const Launch& L, int dtype, const BnBwdArgs& a_in) {
         const int vpr = a.Tp / 8;
         a.dvpr = FastDiv((uint32_t)vpr); a.dC = FastDiv((uint32_t)a.C);
         const long long total = (long long)a.B * a.C * vpr;
-        const unsigned grid = fast_grid(total, 2);
+        const unsigned grid = fast_grid(total, a.phases ? 1 : 2);
 #define SC_BWD_FAST_G(RES, G)                                                                                        \
         if (dtype == BF16 && a.gv_dtype == F16)                                                                      \
-            launch_k(L, bn_bwd_apply_fast_kernel<__nv_bfloat16, __half, __half, RES, 2, G>, grid, 256, 0, a, vpr, total); \
-        else { SC_DISPATCH16(dtype, (launch_k(L, bn_bwd_apply_fast_kernel<T, NT, T, RES, 2, G>, grid, 256, 0, a, vpr, total))); }
+            launch_k(L, bn_bwd_apply_fast_kernel<__nv_bfloat16, __half, __half, RES, (G ? 1 : 2), G>, grid, 256, 0, a, vpr, total); \
+        else { SC_DISPATCH16(dtype, (launch_k(L, bn_bwd_apply_fast_kernel<T, NT, T, RES, (G ? 1 : 2), G>, grid, 256, 0, a, vpr, total))); }
 #define SC_BWD_FAST(RES) if (a.phases == 2) { SC_BWD_FAST_G(RES, 2) } else if (a.phases == 1) { SC_BWD_FAST_G(RES, 1) } else { SC_BWD_FAST_G(RES, 0) }
         if (a.residual == 0) { SC_BWD_FAST(0) } else if (a.residual == 1) { SC_BWD_FAST(1) } else { SC_BWD_FAST(2) }
 #undef SC_BWD_FAST

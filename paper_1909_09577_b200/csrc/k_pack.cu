@@ -55,36 +55,33 @@ __global__ void __launch_bounds__(256) unpack_kernel(PackArgs p) {
     const int k = blockIdx.y;
     const uint32_t idx = blockIdx.x * 256u + threadIdx.x;
     if (idx >= p.nvec[k]) return;
-    const int C = p.l.C[k];
-    const uint32_t total = (uint32_t)p.B * C * p.T, f = idx * 8;
-    const unsigned short* src = (const unsigned short*)p.l.src[k];
+    const int C = p.l.C[k], nrows = p.B * C;
+    const uint32_t total = (uint32_t)nrows * p.T, f = idx * 8, total_p = (uint32_t)nrows * D * p.Tq;
+    const void* src = p.l.src[k];
     unsigned short* dst = (unsigned short*)p.l.dst[k];
     const uint32_t row = p.dT.div(f);
-    const int t = (int)(f - row * p.T);
-    const int b = (int)(row / C), c = (int)(row - (uint32_t)b * C);
-    if (D == 1 && t + 8 <= p.T && f + 8 <= total) {
-        const int n = (p.l.len[k] ? min(p.l.len[k][b], p.T) : p.T) - t;
-        uint4 r = make_uint4(0, 0, 0, 0);
-        if (n > 0) { r = ld8_any(src, row * p.Tq + t, (uint32_t)p.B * C * p.Tq); if (n < 8) r = keep_first(r, n); }
-        *reinterpret_cast<uint4*>(dst + f) = r;
+    const int t = (int)(f - row * p.T), left = (int)min(8u, total - f);
+    // frames t .. t + 7 of a row, zero past the sample's length
+    auto frames = [&](uint32_t r, int t0, bool aligned) -> uint4 {
+        const int b = (int)(r / C), c = (int)(r - (uint32_t)b * C);
+        const int n = (p.l.len[k] ? min(p.l.len[k][b], p.T) : p.T) - t0;
+        if (n <= 0) return make_uint4(0, 0, 0, 0);
+        const uint4 q = Packed8<D>(src, b, c, C, p.Tq, t0, total_p, aligned).get();
+        return n < 8 ? keep_first(q, n) : q;
+    };
+    if (p.T >= 8) {
+        uint4 q = frames(row, t, (p.T & 7) == 0);
+        const int own = p.T - t;
+        if (own < 8 && (int)row + 1 < nrows) q = splice(q, frames(row + 1, -own, false), own);
+        st8_first(dst + f, q, left);
         return;
     }
-    unsigned short h[8];
-    int bb = b, cc = c, tt = t;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        h[i] = 0;
-        if (f + i < total) {
-            const int len = p.l.len[k] ? min(p.l.len[k][bb], p.T) : p.T;
-            if (tt < len) h[i] = src[((size_t)(bb * D + (D == 2 ? (tt & 1) : 0)) * C + cc) * p.Tq + (D == 2 ? tt >> 1 : tt)];
-            if (++tt == p.T) { tt = 0; if (++cc == C) { cc = 0; ++bb; } }
-        }
-    }
-    if (f + 8 <= total) {
-        *reinterpret_cast<uint4*>(dst + f) = make_uint4(h[0] | ((uint32_t)h[1] << 16), h[2] | ((uint32_t)h[3] << 16),
-                                                        h[4] | ((uint32_t)h[5] << 16), h[6] | ((uint32_t)h[7] << 16));
-    } else {
-        for (int i = 0; i < 8; ++i) if (f + i < total) dst[f + i] = h[i];
+    for (uint32_t e = f; e < f + left; ++e) {
+        const uint32_t r = p.dT.div(e);
+        const int te = (int)(e - r * p.T), b = (int)(r / C), c = (int)(r - (uint32_t)b * C);
+        const int len = p.l.len[k] ? min(p.l.len[k][b], p.T) : p.T;
+        dst[e] = te < len ? ((const unsigned short*)src)[((size_t)(b * D + (D == 2 ? (te & 1) : 0)) * C + c) * p.Tq + (D == 2 ? te >> 1 : te)]
+                          : (unsigned short)0;
     }
 }
 
