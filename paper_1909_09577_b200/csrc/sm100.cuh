@@ -118,7 +118,8 @@ __device__ __forceinline__ void mma_f16(uint32_t d_tmem, uint64_t adesc, uint64_
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
-// 32 lanes x 32 consecutive 32-bit columns -> 32 registers per thread (thread l gets lane base+l).
+// 32 lanes x 32 consecutive 32-bit columns -> 32 registers per thread (thread l gets lane base+l).  The instruction is
+// aligned: a caller that comes to it from lane-dependent code puts a __syncwarp in front.
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x32.b32 "

@@ -884,13 +884,14 @@ tc_gemm_flat_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
             if (MODE == MODE_AFFINE && row < p.M) {
                 mu = p.aff.mean[row]; is = 1.f / sqrtf(p.aff.var[row] + p.aff.eps); ga = p.aff.gamma[row]; be = p.aff.beta[row];
             }
+            int b = flat_find_sample(s_off, p.B, j), len_b = b;
+            int len = min(p.len_out[b], p.Tp);
             if (!ptx::mbar_wait_warp(&acc_full[buf], (jt / NBUF) & 1)) { if (lane == 0) raise_status(p.status, kErrTimeout); dead = true; ++jt; continue; }
             ptx::tc_fence_after();
-            int b = flat_find_sample(s_off, p.B, j);
             for (int i = 0; i < nb; ++i) {
                 while (j + i >= s_off[b + 1]) ++b;
                 const int t0 = (j + i - s_off[b]) * 64;
-                const int len = min(p.len_out[b], p.Tp);
+                if (b != len_b) { len = min(p.len_out[b], p.Tp); len_b = b; }
 #pragma unroll 1
                 for (int h = 0; h < 2; ++h) {
                     if (EPI > 1 && ((2 * i + h) % EPI) != hsel) continue;
@@ -899,6 +900,7 @@ tc_gemm_flat_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
                     float f[32];
                     {
                         uint32_t r[32];
+                        if (MODE == MODE_AFFINE) __syncwarp();          // the addend loads below depend on the lane's row
                         ptx::tmem_ld32(tmem + ((uint32_t)(wq * 32) << 16) + buf * ACC_COLS + mt * (NB * 64) + i * 64 + h * 32, r);
                         ptx::tmem_ld_wait();
 #pragma unroll
