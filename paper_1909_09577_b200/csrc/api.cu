@@ -485,6 +485,8 @@ int block_bwd_impl(sc_ctx* ctx, const Launch& L, const sc_block_desc* d, const D
     // identity residual: its gradient is the gated upstream gradient itself
     a.gres = (d->residual == SC_RES_IDENTITY) ? (io.dx_res ? io.dx_res : s.gres) : nullptr;
     a.phases = io.phases; a.T = io.Td; a.total_dense = io.total_dense;
+    a.skip_padding = tc_ok && !m.full && tc_bwd_blockwise(&ctx->tc, odt, m.B, m.Cin, m.Cout, m.Tp) &&
+                     (d->residual != SC_RES_PROJ || tc_bwd_blockwise(&ctx->tc, dt, m.B, m.Cres, m.Cout, m.Tp));
     bn_bwd_reduce_finalize(L, dt, a, p->gamma, p->gamma_r, g->dgamma, g->dbeta, g->dgamma_r, g->dbeta_r,
                            d->has_bias ? g->dbias : nullptr, acc);
     bn_bwd_apply(L, dt, a);

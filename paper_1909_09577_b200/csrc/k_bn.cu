@@ -906,7 +906,10 @@ __global__ void __launch_bounds__(256) bn_bwd_apply_fast_kernel(BnBwdArgs a, int
             t0s[j] = ((int)idx - row * vpr) * 8;
             bs[j] = (int)a.dC.div((uint32_t)row);
             ch[j] = row - bs[j] * a.C;
-            nin[j] = max(0, min(a.len_out[bs[j]], a.Tp) - t0s[j]);        // frames of this vector inside the sample
+            const int len = min(a.len_out[bs[j]], a.Tp);
+            nin[j] = max(0, len - t0s[j]);                                // frames of this vector inside the sample
+            // with half of a batch in padding the zeros were a quarter of this kernel's traffic
+            if (RES != 1 && a.skip_padding && t0s[j] >= ((len + 63) & ~63)) nin[j] = -1;
             off[j] = (size_t)row * a.Tp + t0s[j];
         }
     }

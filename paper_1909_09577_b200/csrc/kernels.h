@@ -294,6 +294,8 @@ struct BnBwdArgs {
     // bf16 (8 significand bits): multiplied by pow2_scale(*gmax), rounded with error diffusion.
     void* gv16; void* gvr16;
     FastDiv dvpr, dC;                              // by Tp / 8 and by C (set by the launchers)
+    int skip_padding;                              // gv, gvr and their half copies need no zeros past the 64-frame block that a
+                                                   // sample ends in (what reads them never goes beyond it)
     // Packed results (phases > 0): g, y, v and vr are dense [B / phases, C, T] while everything that is written is packed
     // [B, C, Tp] with the lengths len_out [B].
     int phases, T; uint32_t total_dense;

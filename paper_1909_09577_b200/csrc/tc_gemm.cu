@@ -1339,6 +1339,10 @@ void tc_gemm_wgrad(const TcState* st, const Launch& L, int dtype, const void* gv
     reduce_partials(L, partials, w.nsplit, (int64_t)Cin * Cout, dw, accumulate, gmax);
 }
 
+bool tc_bwd_blockwise(const TcState* st, int dtype, int B, int Cin, int Cout, int Tp) {
+    return shape_ok(st, dtype, Cin, Cout, Tp) && st->flat && B <= kFlatMaxB && flat_units_fit(B, Tp, Cin);
+}
+
 // ---- evaluation mode --------------------------------------------------------------------------------
 void tc_gemm_affine(const TcState* st, const Launch& L, int dtype, const void* w, const void* u, void* y, int out_dtype,
                     const AffineTail& aff, const int* len_out, const int* blk_off, int B, int Cin, int Cout, int Tp) {

@@ -40,6 +40,8 @@ size_t tc_stats_bytes(int B, int Cout, int Tp);
 //           U = tiles_m * (number of valid 64-frame blocks) units, M tile major
 struct StatsLayout { int kind = 0, parts_per_b = 1, tile_w = 0, grid = 0, tiles_m = 0, rows_per_tile = 0; };
 
+// Whether the input and weight gradient contractions of these shapes read only the 64-frame blocks of gv that hold a valid frame.
+bool tc_bwd_blockwise(const TcState* st, int dtype, int B, int Cin, int Cout, int Tp);
 bool tc_fwd_supported(const TcState* st, int dtype, int Cin, int Cout, int Tp);
 bool tc_dgrad_supported(const TcState* st, int dtype, int Cin, int Cout, int Tp);
 bool tc_wgrad_supported(const TcState* st, int dtype, int Cin, int Cout, int Tp);
