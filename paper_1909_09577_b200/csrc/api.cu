@@ -174,7 +174,7 @@ void finalize_stats(const Launch& L, const sc_block_desc* d, const Dims& m, Stat
 }
 
 // v = w * u for every sample (stored once, in the type it is kept in for the backward pass), plus masked
-// batch statistics.
+// batch statistics (unless mean is null: the apply step takes them).
 void pointwise_bn(sc_ctx* ctx, const Launch& L, const sc_block_desc* d, const Dims& m, int Cin, int opdt,
                   const void* w, const void* u, void* v, const int* len_out, const int* nvalid, const int* blk_off,
                   float* mean, float* invstd, void* partials, float* rmean, float* rvar) {
@@ -184,7 +184,7 @@ void pointwise_bn(sc_ctx* ctx, const Launch& L, const sc_block_desc* d, const Di
         tc_gemm_fwd(&ctx->tc, L, opdt, w, u, nullptr, v, vdt, len_out, blk_off, m.B, Cin, m.Cout, m.Tp, partials, &sl);
     else
         gemm_fwd_simt(L, opdt, w, u, nullptr, v, vdt, len_out, m.B, Cin, m.Cout, m.Tp);
-    finalize_stats(L, d, m, sl, v, vdt, len_out, nvalid, blk_off, partials, mean, invstd, rmean, rvar);
+    if (mean) finalize_stats(L, d, m, sl, v, vdt, len_out, nvalid, blk_off, partials, mean, invstd, rmean, rvar);
 }
 
 // The launch context of the side stream (same status word, counters and profile), or L itself when overlap is off.
@@ -236,6 +236,7 @@ int block_fwd_impl(sc_ctx* ctx, const Launch& L, const sc_block_desc* d, const D
     const bool fused = inf && d->has_bn && !m.full && !io.phases && ctx->gemm_mode == 0 &&
                        tc_affine_supported(&ctx->tc, odt, m.B, m.Cin, m.Cout, m.Tp) &&
                        (d->residual != SC_RES_PROJ || tc_affine_supported(&ctx->tc, dt, m.B, m.Cres, m.Cout, m.Tp));
+    const bool small = d->has_bn && !inf && bn_small(dt, m.B, m.Tp);     // the apply step takes the main branch's statistics too
     if (d->has_bn && d->residual == SC_RES_PROJ) {
         // the residual projection does not depend on the main branch: its contraction and statistics go to the
         // side stream and are joined just before the apply step
@@ -266,7 +267,8 @@ int block_fwd_impl(sc_ctx* ctx, const Launch& L, const sc_block_desc* d, const D
             conv_fwd_simt(L, dt, p->wp, io.x, bias, v, vdt, io.len_in, io.len_out, m.B, m.Cin, m.Cout, m.T, m.Tp, m.K, m.s, m.dil);
         }
         if (!d->has_bn) return SC_OK;
-        if (stats) finalize_stats(L, d, m, sl, v, vdt, io.len_out, io.nvalid, io.blk_off, f.partials, sv->mean, sv->invstd, rmean, rvar);
+        if (small) {}
+        else if (stats) finalize_stats(L, d, m, sl, v, vdt, io.len_out, io.nvalid, io.blk_off, f.partials, sv->mean, sv->invstd, rmean, rvar);
         else invstd_from_var(L, inf->var, d->bn_eps, sv->invstd, m.Cout);
     }
     const void* u = nullptr;
@@ -309,7 +311,7 @@ int block_fwd_impl(sc_ctx* ctx, const Launch& L, const sc_block_desc* d, const D
     }
     if (m.full) {}
     else if (inf) pointwise_fixed(ctx, L, d, m, m.Cin, odt, wp_op, u, sv->v, io.len_out, io.blk_off, inf->var, sv->invstd);
-    else pointwise_bn(ctx, L, d, m, m.Cin, odt, wp_op, u, sv->v, io.len_out, io.nvalid, io.blk_off, sv->mean, sv->invstd,
+    else pointwise_bn(ctx, L, d, m, m.Cin, odt, wp_op, u, sv->v, io.len_out, io.nvalid, io.blk_off, small ? nullptr : sv->mean, sv->invstd,
                       f.partials, rmean, rvar);
     ApplyArgs a{};
     a.v = sv->v; a.mean = inf ? inf->mean : sv->mean; a.invstd = sv->invstd; a.gamma = p->gamma; a.beta = p->beta;
@@ -324,7 +326,8 @@ int block_fwd_impl(sc_ctx* ctx, const Launch& L, const sc_block_desc* d, const D
         a.phases = io.phases; a.B = m.B / io.phases; a.T = io.Td; a.len_out = io.len_dense;
         a.v_out = io.dense.v; a.vr_out = io.dense.vr; a.u = u; a.u_out = u ? io.dense.u : nullptr; a.Cu = m.Cin;
     }
-    bn_apply(L, dt, a);
+    if (small) bn_small_fwd(L, a, io.nvalid, d->bn_eps, d->bn_momentum, sv->mean, sv->invstd, rmean, rvar);
+    else bn_apply(L, dt, a);
     return SC_OK;
 }
 
@@ -487,9 +490,7 @@ int block_bwd_impl(sc_ctx* ctx, const Launch& L, const sc_block_desc* d, const D
     a.phases = io.phases; a.T = io.Td; a.total_dense = io.total_dense;
     a.skip_padding = tc_ok && !m.full && tc_bwd_blockwise(&ctx->tc, odt, m.B, m.Cin, m.Cout, m.Tp) &&
                      (d->residual != SC_RES_PROJ || tc_bwd_blockwise(&ctx->tc, dt, m.B, m.Cres, m.Cout, m.Tp));
-    bn_bwd_reduce_finalize(L, dt, a, p->gamma, p->gamma_r, g->dgamma, g->dbeta, g->dgamma_r, g->dbeta_r,
-                           d->has_bias ? g->dbias : nullptr, acc);
-    bn_bwd_apply(L, dt, a);
+    bn_bwd(L, dt, a, p->gamma, p->gamma_r, g->dgamma, g->dbeta, g->dgamma_r, g->dbeta_r, d->has_bias ? g->dbias : nullptr, acc);
     const bool conv_tc = tc_ok && conv_on_tc(&ctx->tc, d, m);
     if (conv_tc) to_time_major(L, s.gv, s.gv_tm, io.len_out, m.B, m.Cout, m.T);
 

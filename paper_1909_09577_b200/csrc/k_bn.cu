@@ -273,48 +273,120 @@ bn_finalize_flat_kernel(const float4* __restrict__ partials, int G, int tiles_m,
     }
 }
 
+// Per-channel constants of the forward apply step and of the backward kernels, loaded (or, in the
+// channel-per-CTA kernels, computed) once and passed by value.
+struct FwdChan { float mu, is, ga, be, mur, isr, gar, ber; };
+struct BwdChan { float mu, is, ga, be, mur, isr; float4 cf, cr; };
+
+// Forward apply of eight frames from t0 on of row (b, o): y = [t < len] * act(gamma * vhat + beta, r).
+template <typename T, typename NT>
+__device__ __forceinline__ void apply_chunk(const ApplyArgs& a, size_t off, int t0, int len, bool vec, const FwdChan& c) {
+    const int Tp = a.Tp;
+    float out[8];
+    if (t0 < len) {
+        float f[8], r[8];
+        load_chunk((const NT*)a.v + off, t0, Tp, vec, f);
+        if (a.residual == 1) load_chunk((const T*)a.xres + off, t0, Tp, vec, r);
+        else if (a.residual == 2) {
+            load_chunk((const NT*)a.vr + off, t0, Tp, vec, r);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) r[i] = fmaf(c.gar, bn_norm(r[i], c.mur, c.isr), c.ber);
+        } else {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) r[i] = 0.f;
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            float bn = fmaf(c.ga, bn_norm(f[i], c.mu, c.is), c.be);   // the backward pass recomputes exactly this
+            float q;
+            if (a.res_before_relu) { q = bn + r[i]; if (a.has_relu) q = fmaxf(q, 0.f); }
+            else { q = (a.has_relu ? fmaxf(bn, 0.f) : bn) + r[i]; }
+            out[i] = (t0 + i < len) ? q : 0.f;
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) out[i] = 0.f;
+    }
+    store_chunk((T*)a.y + off, t0, Tp, vec, out);
+}
+
 template <typename T, typename NT>
 __global__ void __launch_bounds__(kRowThreads) bn_apply_kernel(ApplyArgs a) {
     pdl_sync();
     SC_ROW_SETUP(a.B * a.C)
-    const int b = row / a.C, o = row % a.C;
-    const int Tp = a.Tp, len = min(a.len_out[b], Tp);
-    const bool vec = (Tp % 8 == 0);
-    const size_t off = (size_t)row * Tp;
-    const NT* __restrict__ v = (const NT*)a.v + off;
-    const T* __restrict__ xr = a.residual == 1 ? (const T*)a.xres + off : nullptr;
-    const NT* __restrict__ vr = a.residual == 2 ? (const NT*)a.vr + off : nullptr;
-    T* __restrict__ y = (T*)a.y + off;
-    const float mu = a.mean[o], is = a.invstd[o], ga = a.gamma[o], be = a.beta[o];
-    float mur = 0.f, isr = 0.f, gar = 0.f, ber = 0.f;
-    if (a.residual == 2) { mur = a.mean_r[o]; isr = a.invstd_r[o]; gar = a.gamma_r[o]; ber = a.beta_r[o]; }
-    for (int t0 = lane * 8; t0 < Tp; t0 += 256) {
-        float out[8];
-        if (t0 < len) {
-            float f[8], r[8];
-            load_chunk(v, t0, Tp, vec, f);
-            if (a.residual == 1) load_chunk(xr, t0, Tp, vec, r);
-            else if (a.residual == 2) {
-                load_chunk(vr, t0, Tp, vec, r);
+    const int b = row / a.C, o = row % a.C, len = min(a.len_out[b], a.Tp);
+    FwdChan c{a.mean[o], a.invstd[o], a.gamma[o], a.beta[o], 0.f, 0.f, 0.f, 0.f};
+    if (a.residual == 2) { c.mur = a.mean_r[o]; c.isr = a.invstd_r[o]; c.gar = a.gamma_r[o]; c.ber = a.beta_r[o]; }
+    for (int t0 = lane * 8; t0 < a.Tp; t0 += 256) apply_chunk<T, NT>(a, (size_t)row * a.Tp, t0, len, a.Tp % 8 == 0, c);
+}
+
+// ---- one CTA per channel of a small float32 tensor ---------------------------------------------------------
+// A channel of up to kSmallChunks eight-frame chunks: what is left of the three steps (row partials, finalize, apply; in
+// the backward pass too) is the latency of their launches, about 2.2 us each in a chain of dependent kernels.  One CTA
+// sees the whole channel and does all three; the second and third reading of its rows hit the L1 cache.  Above the limit
+// the row-mapped kernels have more CTAs than there are channels and win.  A block forward and backward: 64 channels of
+// 2 x 128 frames 35.9 -> 29.7 us, 128 channels of 7 x 228 frames 75.6 -> 69.7 us.
+constexpr int kSmallChunks = 1024;
+struct ChanRows {            // chunk j of the channel -> sample and frame
+    int cpr, n;
+    __device__ __forceinline__ ChanRows(int B, int Tp) : cpr((Tp + 7) >> 3), n(B * ((Tp + 7) >> 3)) {}
+    __device__ __forceinline__ void at(int j, int& b, int& t0) const { b = j / cpr; t0 = (j - b * cpr) * 8; }
+};
+template <int N>
+__device__ __forceinline__ void cta_sum(float (&v)[N], float* s_red) {      // in every thread, in warp order
+    block_sum(v);
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) {
 #pragma unroll
-                for (int i = 0; i < 8; ++i) r[i] = fmaf(gar, bn_norm(r[i], mur, isr), ber);
-            } else {
+        for (int i = 0; i < N; ++i) s_red[(threadIdx.x >> 5) * N + i] = v[i];
+    }
+    __syncthreads();
 #pragma unroll
-                for (int i = 0; i < 8; ++i) r[i] = 0.f;
-            }
+    for (int i = 0; i < N; ++i) {
+        v[i] = 0.f;
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                float bn = fmaf(ga, bn_norm(f[i], mu, is), be);   // the backward pass recomputes exactly this
-                float q;
-                if (a.res_before_relu) { q = bn + r[i]; if (a.has_relu) q = fmaxf(q, 0.f); }
-                else { q = (a.has_relu ? fmaxf(bn, 0.f) : bn) + r[i]; }
-                out[i] = (t0 + i < len) ? q : 0.f;
-            }
-        } else {
+        for (int w = 0; w < kRowThreads / 32; ++w) v[i] += s_red[w * N + i];
+    }
+}
+
+__global__ void __launch_bounds__(kRowThreads)
+bn_small_fwd_kernel(ApplyArgs a, const int* __restrict__ nvalid, float eps, float momentum, float* mean_out, float* invstd_out,
+                    float* running_mean, float* running_var) {
+    __shared__ float s_red[kRowThreads / 32];
+    const int o = blockIdx.x, tid = threadIdx.x;
+    const ChanRows R(a.B, a.Tp);
+    const bool vec = a.Tp % 8 == 0;
+    const float N = (float)(*nvalid);
+    FwdChan c{0.f, 0.f, a.gamma[o], a.beta[o], 0.f, 0.f, 0.f, 0.f};
+    pdl_sync();              // the parameters and the count above were settled before the previous kernel
+    if (a.residual == 2) { c.mur = a.mean_r[o]; c.isr = a.invstd_r[o]; c.gar = a.gamma_r[o]; c.ber = a.beta_r[o]; }
+    float s[1];
+    for (int pass = 0; pass < 2; ++pass) {      // the sum, then the squares about the mean
+        s[0] = 0.f;
+        for (int j = tid; j < R.n; j += kRowThreads) {
+            int b, t0;
+            R.at(j, b, t0);
+            const int len = min(a.len_out[b], a.Tp);
+            if (t0 >= len) continue;
+            float f[8];
+            load_chunk((const float*)a.v + ((size_t)b * a.C + o) * a.Tp, t0, a.Tp, vec, f);
 #pragma unroll
-            for (int i = 0; i < 8; ++i) out[i] = 0.f;
+            for (int i = 0; i < 8; ++i) if (t0 + i < len) s[0] += pass ? (f[i] - c.mu) * (f[i] - c.mu) : f[i];
         }
-        store_chunk(y, t0, Tp, vec, out);
+        cta_sum(s, s_red);
+        if (!pass) c.mu = N > 0.f ? s[0] / N : 0.f;
+    }
+    const float var = N > 0.f ? s[0] / N : 0.f;
+    c.is = 1.f / sqrtf(var + eps);
+    if (tid == 0) {
+        mean_out[o] = c.mu; invstd_out[o] = c.is;
+        if (running_mean) running_mean[o] = (1.f - momentum) * running_mean[o] + momentum * c.mu;
+        if (running_var) running_var[o] = (1.f - momentum) * running_var[o] + momentum * (N > 1.f ? var * (N / (N - 1.f)) : var);
+    }
+    for (int j = tid; j < R.n; j += kRowThreads) {
+        int b, t0;
+        R.at(j, b, t0);
+        apply_chunk<float, float>(a, ((size_t)b * a.C + o) * a.Tp, t0, min(a.len_out[b], a.Tp), vec, c);
     }
 }
 
@@ -403,13 +475,45 @@ __global__ void __launch_bounds__(kRowThreads) bn_bwd_reduce_kernel(BnBwdArgs a)
     }
 }
 
+// What the sums of channel o over all frames amount to: the coefficients of the apply step (cf, cr), the channel's parameter
+// gradients (one thread writes them) and its term of the bound on |gv|.
+struct BwdGrads { const float *gamma, *gamma_r; float *dgamma, *dbeta, *dgamma_r, *dbeta_r, *dbias; int accumulate; };
+__device__ __forceinline__ void bwd_channel(const BnBwdArgs& a, const BwdGrads& p, int o, bool writes, float d0, float d1, float d2,
+                                            float d3, float amax, float4& cf, float4& cr) {
+    const float N = (float)(*a.nvalid);
+    if (a.gmax && writes) {
+        // |gv| <= |k| (max|ga| + |c1| + max|vhat| |c2|) and max|vhat| <= sqrt(N); a maximum is order-free,
+        // so the integer atomic on the (non-negative) float's bit pattern keeps the result repeatable
+        float bound = amax;
+        if (a.has_bn)
+            bound = fabsf(p.gamma[o] * a.invstd[o]) * (amax + fabsf(d0) / N + sqrtf(N) * fabsf(d1) / N);
+        if (a.residual == 2)     // the residual branch's gradient shares the scale
+            bound = fmaxf(bound, fabsf(p.gamma_r[o] * a.invstd_r[o]) *
+                                     (amax + fabsf(d2) / N + sqrtf(N) * fabsf(d3) / N));
+        if (bound < 3.0e38f) atomicMax(reinterpret_cast<unsigned int*>(a.gmax), __float_as_uint(bound));
+    }
+    auto put = [&](float* dst, float val) {
+        if (dst && writes) dst[o] = p.accumulate ? dst[o] + val : val;
+    };
+    if (a.has_bn) {
+        put(p.dbeta, d0); put(p.dgamma, d1);
+        cf = make_float4(p.gamma[o] * a.invstd[o], d0 / N, d1 / N, 0.f);
+    } else {
+        put(p.dbias, d0);
+        cf = make_float4(1.f, 0.f, 0.f, 0.f);
+    }
+    if (a.residual == 2) {
+        put(p.dbeta_r, d2); put(p.dgamma_r, d3);
+        cr = make_float4(p.gamma_r[o] * a.invstd_r[o], d2 / N, d3 / N, 0.f);
+    }
+}
+
 // Thirty-two channels per CTA, one per lane; warp w takes samples w, w + 32, ... with all their slots (every
 // load issued before the first add) and the thirty-two warp results are combined in warp order
 // (bit-repeatable).
 constexpr int kBwdMaxSlotsUnrolled = 8;
 __global__ void __launch_bounds__(32 * kFinWarps)
-bn_bwd_finalize_kernel(BnBwdArgs a, const float* gamma, const float* gamma_r, float* dgamma, float* dbeta,
-                       float* dgamma_r, float* dbeta_r, float* dbias, int accumulate) {
+bn_bwd_finalize_kernel(BnBwdArgs a, BwdGrads p) {
     pdl_sync();
     __shared__ float4 s_sum[kFinWarps][32];
     __shared__ float s_max[kFinWarps][32];
@@ -453,32 +557,57 @@ bn_bwd_finalize_kernel(BnBwdArgs a, const float* gamma, const float* gamma_r, fl
         d0 += q.x; d1 += q.y; d2 += q.z; d3 += q.w;
         amax = fmaxf(amax, s_max[i][lane]);
     }
-    const float N = (float)(*a.nvalid);
-    if (a.gmax) {
-        // |gv| <= |k| (max|ga| + |c1| + max|vhat| |c2|) and max|vhat| <= sqrt(N); a maximum is order-free,
-        // so the integer atomic on the (non-negative) float's bit pattern keeps the result repeatable
-        float bound = amax;
-        if (a.has_bn)
-            bound = fabsf(gamma[o] * a.invstd[o]) * (amax + fabsf((float)d0) / N + sqrtf(N) * fabsf((float)d1) / N);
-        if (a.residual == 2)     // the residual branch's gradient shares the scale
-            bound = fmaxf(bound, fabsf(gamma_r[o] * a.invstd_r[o]) *
-                                     (amax + fabsf((float)d2) / N + sqrtf(N) * fabsf((float)d3) / N));
-        if (bound < 3.0e38f) atomicMax(reinterpret_cast<unsigned int*>(a.gmax), __float_as_uint(bound));
-    }
-    auto put = [&](float* dst, float val) {
-        if (dst) dst[o] = accumulate ? dst[o] + val : val;
-    };
-    if (a.has_bn) {
-        put(dbeta, d0); put(dgamma, d1);
-        a.coef[o] = make_float4(gamma[o] * a.invstd[o], (float)d0 / N, (float)d1 / N, 0.f);
+    float4 cf, cr = make_float4(0.f, 0.f, 0.f, 0.f);
+    bwd_channel(a, p, o, true, d0, d1, d2, d3, amax, cf, cr);
+    a.coef[o] = cf;
+    if (a.residual == 2) a.coef_r[o] = cr;
+}
+
+// Backward apply of eight frames from t0 on of the row that R describes (cf, cr: the channel's coefficients).
+template <typename T, typename NT, typename GT>
+__device__ __forceinline__ void bwd_apply_chunk(const BnBwdArgs& a, const BwdRow<T, NT>& R, size_t off, int t0, const float4& cf,
+                                                const float4& cr, float sc) {
+    float o1[8], o2[8];
+    if (t0 < R.len) {
+        float ga[8], gr[8], vh[8], vhr[8];
+        R.chunk(a, t0, ga, gr, vh, vhr);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const bool in = (t0 + i < R.len);
+            o1[i] = in ? cf.x * (ga[i] - cf.y - vh[i] * cf.z) : 0.f;
+            if (a.residual == 2) o2[i] = in ? cr.x * (gr[i] - cr.y - vhr[i] * cr.z) : 0.f;
+            else o2[i] = gr[i];
+        }
     } else {
-        put(dbias, d0);
-        a.coef[o] = make_float4(1.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) { o1[i] = 0.f; o2[i] = 0.f; }
     }
-    if (a.residual == 2) {
-        put(dbeta_r, d2); put(dgamma_r, d3);
-        a.coef_r[o] = make_float4(gamma_r[o] * a.invstd_r[o], (float)d2 / N, (float)d3 / N, 0.f);
+    const int nin = R.len - t0;
+    if (a.gv16) {              // half copy for the weight gradient; gv itself keeps plain rounding
+        float h[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) h[i] = o1[i] * sc;
+        diffuse8<__half>(h, nin);
+        store_chunk((__half*)a.gv16 + off, t0, R.Tp, R.vec, h);
+    } else {
+        if (a.gv_scaled) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) o1[i] *= sc;
+        }
+        diffuse8<GT>(o1, nin);
     }
+    if (a.gvr16) {
+        float h[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) h[i] = o2[i] * sc;
+        diffuse8<__half>(h, nin);
+        store_chunk((__half*)a.gvr16 + off, t0, R.Tp, R.vec, h);
+    } else if (a.residual == 2) {
+        diffuse8<T>(o2, nin);
+    }
+    store_chunk((GT*)a.gv + off, t0, R.Tp, R.vec, o1);
+    if (a.residual == 2) store_chunk((T*)a.gvr + off, t0, R.Tp, R.vec, o2);
+    if (a.residual == 1) store_chunk((T*)a.gres + off, t0, R.Tp, R.vec, o2);
 }
 
 template <typename T, typename NT, typename GT>
@@ -490,60 +619,36 @@ __global__ void __launch_bounds__(kRowThreads) bn_bwd_apply_kernel(BnBwdArgs a) 
     const float4 cf = a.coef[o];
     const float sc = a.gmax ? pow2_scale(*a.gmax) : 1.f;      // multiplying by it is exact: a power of two
     const float4 cr = (a.residual == 2) ? a.coef_r[o] : make_float4(0.f, 0.f, 0.f, 0.f);
-    __half* __restrict__ gv16 = a.gv16 ? (__half*)a.gv16 + (size_t)row * R.Tp : nullptr;
-    __half* __restrict__ gvr16 = a.gvr16 ? (__half*)a.gvr16 + (size_t)row * R.Tp : nullptr;
-    GT* __restrict__ gv = (GT*)a.gv + (size_t)row * R.Tp;
-    T* __restrict__ gvr = (a.residual == 2) ? (T*)a.gvr + (size_t)row * R.Tp : nullptr;
-    T* __restrict__ gres = (a.residual == 1) ? (T*)a.gres + (size_t)row * R.Tp : nullptr;
-    for (int t0 = lane * 8; t0 < R.Tp; t0 += 256) {
-        float o1[8], o2[8];
-        if (t0 < R.len) {
-            float ga[8], gr[8], vh[8], vhr[8];
-            R.chunk(a, t0, ga, gr, vh, vhr);
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const bool in = (t0 + i < R.len);
-                o1[i] = in ? cf.x * (ga[i] - cf.y - vh[i] * cf.z) : 0.f;
-                if (a.residual == 2) o2[i] = in ? cr.x * (gr[i] - cr.y - vhr[i] * cr.z) : 0.f;
-                else o2[i] = gr[i];
-            }
-        } else {
-#pragma unroll
-            for (int i = 0; i < 8; ++i) { o1[i] = 0.f; o2[i] = 0.f; }
-        }
-        const int nin = R.len - t0;
-        if (gv16) {              // half copy for the weight gradient; gv itself keeps plain rounding
-            float h[8];
-#pragma unroll
-            for (int i = 0; i < 8; ++i) h[i] = o1[i] * sc;
-            diffuse8<__half>(h, nin);
-            store_chunk(gv16, t0, R.Tp, R.vec, h);
-        } else {
-            if (a.gv_scaled) {
-#pragma unroll
-                for (int i = 0; i < 8; ++i) o1[i] *= sc;
-            }
-            diffuse8<GT>(o1, nin);
-        }
-        if (gvr16) {
-            float h[8];
-#pragma unroll
-            for (int i = 0; i < 8; ++i) h[i] = o2[i] * sc;
-            diffuse8<__half>(h, nin);
-            store_chunk(gvr16, t0, R.Tp, R.vec, h);
-        } else if (a.residual == 2) {
-            diffuse8<T>(o2, nin);
-        }
-        store_chunk(gv, t0, R.Tp, R.vec, o1);
-        if (gvr) store_chunk(gvr, t0, R.Tp, R.vec, o2);
-        if (gres) store_chunk(gres, t0, R.Tp, R.vec, o2);
-    }
+    for (int t0 = lane * 8; t0 < R.Tp; t0 += 256) bwd_apply_chunk<T, NT, GT>(a, R, (size_t)row * R.Tp, t0, cf, cr, sc);
 }
 
-// Per-channel constants of the forward apply step and of the backward kernels, loaded (or, in the
-// channel-per-CTA kernels, computed) once and passed by value.
-struct FwdChan { float mu, is, ga, be, mur, isr, gar, ber; };
-struct BwdChan { float mu, is, ga, be, mur, isr; float4 cf, cr; };
+// The backward counterpart of bn_small_fwd_kernel.
+__global__ void __launch_bounds__(kRowThreads) bn_small_bwd_kernel(BnBwdArgs a, BwdGrads p) {
+    pdl_sync();
+    __shared__ float s_red[4 * kRowThreads / 32];
+    const int o = blockIdx.x, tid = threadIdx.x;
+    const ChanRows C(a.B, a.Tp);
+    float s[4] = {0.f, 0.f, 0.f, 0.f};
+    for (int j = tid; j < C.n; j += kRowThreads) {
+        int b, t0;
+        C.at(j, b, t0);
+        const BwdRow<float, float> R(a, b * a.C + o, b, o);
+        if (t0 >= R.len) continue;
+        float ga[8], gr[8], vh[8], vhr[8];
+        R.chunk(a, t0, ga, gr, vh, vhr);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) { s[0] += ga[i]; s[1] += ga[i] * vh[i]; s[2] += gr[i]; s[3] += gr[i] * vhr[i]; }
+    }
+    cta_sum(s, s_red);
+    float4 cf, cr = make_float4(0.f, 0.f, 0.f, 0.f);
+    bwd_channel(a, p, o, tid == 0, s[0], s[1], s[2], s[3], 0.f, cf, cr);
+    for (int j = tid; j < C.n; j += kRowThreads) {
+        int b, t0;
+        C.at(j, b, t0);
+        const int row = b * a.C + o;
+        bwd_apply_chunk<float, float, float>(a, BwdRow<float, float>(a, row, b, o), (size_t)row * a.Tp, t0, cf, cr, 1.f);
+    }
+}
 
 // One 8-frame vector of the forward apply step: y = [t < len] * relu(gamma * vhat + beta (+ r)); n = frames of the
 // vector inside the sample (0: wholly padding), rv / rr = the raw 16 bytes of v and of the residual operand.
@@ -1168,6 +1273,15 @@ void bn_finalize_flat(const Launch& L, const float4* partials, int grid, int til
     L.count();
 }
 
+bool bn_small(int dtype, int B, int Tp) { return dtype == F32 && (long long)B * ((Tp + 7) / 8) <= kSmallChunks; }
+
+void bn_small_fwd(const Launch& L, const ApplyArgs& a, const int* nvalid, float eps, float momentum, float* mean, float* invstd,
+                  float* running_mean, float* running_var) {
+    KScope ks_(L, KC_BN_APPLY, 4.0 * a.B * a.C * a.Tp * (a.residual ? 3 : 2), 0.0);
+    launch_k(L, bn_small_fwd_kernel, (unsigned)a.C, kRowThreads, 0, a, nvalid, eps, momentum, mean, invstd, running_mean, running_var);
+    L.count();
+}
+
 // the flattened kernels index with 32 bits
 static bool fits32(int B, int C, int Tp) { return (long long)B * C * (Tp / 8) < (1ll << 31) && (long long)B * C * Tp < (1ll << 31); }
 static unsigned fast_grid(long long total, int V) { return (unsigned)((total + 256ll * V - 1) / (256ll * V)); }
@@ -1238,12 +1352,11 @@ void bn_bwd_finalize(const Launch& L, const BnBwdArgs& a, const float* gamma, co
                      float* dgamma, float* dbeta, float* dgamma_r, float* dbeta_r, float* dbias,
                      int accumulate) {
     KScope ks_(L, KC_BN_BWD_FINALIZE, 16.0 * a.B * a.C * a.nslots, 0.0);
-    launch_k(L, bn_bwd_finalize_kernel, (a.C + 31) / 32, 32 * kFinWarps, 0, a, gamma, gamma_r, dgamma, dbeta, dgamma_r,
-                                                                          dbeta_r, dbias, accumulate);
+    launch_k(L, bn_bwd_finalize_kernel, (a.C + 31) / 32, 32 * kFinWarps, 0, a, BwdGrads{gamma, gamma_r, dgamma, dbeta, dgamma_r, dbeta_r, dbias, accumulate});
     L.count();
 }
 
-void bn_bwd_reduce_finalize(const Launch& L, int dtype, BnBwdArgs& a, const float* gamma, const float* gamma_r,
+static void bn_bwd_reduce_finalize(const Launch& L, int dtype, BnBwdArgs& a, const float* gamma, const float* gamma_r,
                             float* dgamma, float* dbeta, float* dgamma_r, float* dbeta_r, float* dbias, int accumulate) {
     const bool fast = dtype != F32 && a.Tp % 8 == 0 && a.has_bn && a.has_relu && a.res_before_relu && fits32(a.B, a.C, a.Tp);
     if (a.phases || (fast && channel_mapped(a.B, a.C, a.Tp))) {
@@ -1265,7 +1378,7 @@ void bn_bwd_reduce_finalize(const Launch& L, int dtype, BnBwdArgs& a, const floa
     bn_bwd_finalize(L, a, gamma, gamma_r, dgamma, dbeta, dgamma_r, dbeta_r, dbias, accumulate);
 }
 
-void bn_bwd_apply(const Launch& L, int dtype, const BnBwdArgs& a_in) {
+static void bn_bwd_apply(const Launch& L, int dtype, const BnBwdArgs& a_in) {
     BnBwdArgs a = a_in;
     const bool fast_apply = dtype != F32 && a.Tp % 8 == 0 && a.has_bn && a.has_relu && a.res_before_relu && fits32(a.B, a.C, a.Tp);
     const double e = (double)dtype_size(dtype), en = (double)dtype_size(ntype_of(dtype));
@@ -1291,6 +1404,18 @@ void bn_bwd_apply(const Launch& L, int dtype, const BnBwdArgs& a_in) {
     else
         SC_DISPATCH3(dtype, (launch_k(L, bn_bwd_apply_kernel<T, NT, T>, (a.B * a.C + kRowsPerCta - 1) / kRowsPerCta, kRowThreads, 0, a)));
     L.count();
+}
+
+void bn_bwd(const Launch& L, int dtype, BnBwdArgs& a, const float* gamma, const float* gamma_r, float* dgamma, float* dbeta,
+            float* dgamma_r, float* dbeta_r, float* dbias, int accumulate) {
+    if (bn_small(dtype, a.B, a.Tp)) {
+        KScope ks_(L, KC_BN_BWD_APPLY, 4.0 * a.B * a.C * a.Tp * (a.residual ? 5 : 4), 0.0);
+        launch_k(L, bn_small_bwd_kernel, (unsigned)a.C, kRowThreads, 0, a, BwdGrads{gamma, gamma_r, dgamma, dbeta, dgamma_r, dbeta_r, dbias, accumulate});
+        L.count();
+        return;
+    }
+    bn_bwd_reduce_finalize(L, dtype, a, gamma, gamma_r, dgamma, dbeta, dgamma_r, dbeta_r, dbias, accumulate);
+    bn_bwd_apply(L, dtype, a);
 }
 
 void ew_add_masked(const Launch& L, int dtype, void* out, const void* a, const void* b, const void* c,

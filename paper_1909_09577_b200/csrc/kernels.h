@@ -273,6 +273,10 @@ struct ApplyArgs {
     FastDiv dT;
 };
 void bn_apply(const Launch& L, int dtype, const ApplyArgs& a);
+// Statistics of v and the apply step in one kernel, for the float32 tensors that bn_small accepts.
+bool bn_small(int dtype, int B, int Tp);
+void bn_small_fwd(const Launch& L, const ApplyArgs& a, const int* nvalid, float eps, float momentum, float* mean, float* invstd,
+                  float* running_mean, float* running_var);
 
 struct BnBwdArgs {
     const void* g; const void* y; const void* v; const void* vr;          // v, vr in NT
@@ -300,17 +304,11 @@ struct BnBwdArgs {
     // [B, C, Tp] with the lengths len_out [B].
     int phases, T; uint32_t total_dense;
 };
-void bn_bwd_reduce(const Launch& L, int dtype, BnBwdArgs& a);
 // partial slots per row that bn_bwd_reduce may use for rows of Tp frames (for scratch sizing)
 inline int bn_bwd_max_slots(int Tp) { return Tp / 256 + 2; }
-void bn_bwd_finalize(const Launch& L, const BnBwdArgs& a, const float* gamma, const float* gamma_r,
-                     float* dgamma, float* dbeta, float* dgamma_r, float* dbeta_r, float* dbias,
-                     int accumulate);
-// bn_bwd_reduce followed by bn_bwd_finalize, or -- for the encoder's block shape -- one kernel with a CTA per
-// channel that does both.
-void bn_bwd_reduce_finalize(const Launch& L, int dtype, BnBwdArgs& a, const float* gamma, const float* gamma_r,
-                            float* dgamma, float* dbeta, float* dgamma_r, float* dbeta_r, float* dbias, int accumulate);
-void bn_bwd_apply(const Launch& L, int dtype, const BnBwdArgs& a);
+// Reduction over the frames, parameter gradients and gv / gvr / gres: two or three kernels, or one for a small float32 tensor.
+void bn_bwd(const Launch& L, int dtype, BnBwdArgs& a, const float* gamma, const float* gamma_r, float* dgamma, float* dbeta,
+            float* dgamma_r, float* dbeta_r, float* dbias, int accumulate);
 
 // ---- decoder tail / evaluation mode ---------------------------------------------------------------
 // y[b,:,t] = [t < len_out[b]] * (z[b,:,t] - log(sum_c exp(z[b,c,t]))), z in float32
