@@ -173,18 +173,25 @@ void finalize_stats(const Launch& L, const sc_block_desc* d, const Dims& m, Stat
                 mean, invstd, rmean, rvar);
 }
 
+bool apply_takes_stats(int dt, const ApplyArgs& a, const StatsLayout& sl) {
+    return sl.kind == 2 ? bn_apply_takes_stats(dt, a) : sl.kind == 0 && bn_small(dt, a.B, a.Tp);
+}
+
 // v = w * u for every sample (stored once, in the type it is kept in for the backward pass), plus masked
-// batch statistics (unless mean is null: the apply step takes them).
+// batch statistics, unless the apply step takes them (apply: its arguments, null when it must not): then *left is what the
+// contraction left behind.
 void pointwise_bn(sc_ctx* ctx, const Launch& L, const sc_block_desc* d, const Dims& m, int Cin, int opdt,
                   const void* w, const void* u, void* v, const int* len_out, const int* nvalid, const int* blk_off,
-                  float* mean, float* invstd, void* partials, float* rmean, float* rvar) {
+                  float* mean, float* invstd, void* partials, float* rmean, float* rvar, const ApplyArgs* apply = nullptr,
+                  StatsLayout* left = nullptr) {
     const int vdt = ntype_of(d->io_dtype);
     StatsLayout sl;
     if (ctx->gemm_mode == 0 && tc_fwd_supported(&ctx->tc, opdt, Cin, m.Cout, m.Tp))
         tc_gemm_fwd(&ctx->tc, L, opdt, w, u, nullptr, v, vdt, len_out, blk_off, m.B, Cin, m.Cout, m.Tp, partials, &sl);
     else
         gemm_fwd_simt(L, opdt, w, u, nullptr, v, vdt, len_out, m.B, Cin, m.Cout, m.Tp);
-    if (mean) finalize_stats(L, d, m, sl, v, vdt, len_out, nvalid, blk_off, partials, mean, invstd, rmean, rvar);
+    if (apply && apply_takes_stats(d->io_dtype, *apply, sl)) *left = sl;
+    else finalize_stats(L, d, m, sl, v, vdt, len_out, nvalid, blk_off, partials, mean, invstd, rmean, rvar);
 }
 
 // The launch context of the side stream (same status word, counters and profile), or L itself when overlap is off.
@@ -236,7 +243,20 @@ int block_fwd_impl(sc_ctx* ctx, const Launch& L, const sc_block_desc* d, const D
     const bool fused = inf && d->has_bn && !m.full && !io.phases && ctx->gemm_mode == 0 &&
                        tc_affine_supported(&ctx->tc, odt, m.B, m.Cin, m.Cout, m.Tp) &&
                        (d->residual != SC_RES_PROJ || tc_affine_supported(&ctx->tc, dt, m.B, m.Cres, m.Cout, m.Tp));
-    const bool small = d->has_bn && !inf && bn_small(dt, m.B, m.Tp);     // the apply step takes the main branch's statistics too
+    ApplyArgs a{};
+    a.v = sv->v; a.mean = inf ? inf->mean : sv->mean; a.invstd = sv->invstd; a.gamma = p->gamma; a.beta = p->beta;
+    a.residual = d->residual; a.y = io.y; a.len_out = io.len_out;
+    a.B = m.B; a.C = m.Cout; a.Tp = m.Tp; a.has_relu = d->has_relu; a.res_before_relu = d->res_before_relu;
+    if (d->residual == SC_RES_IDENTITY) a.xres = io.xres;
+    if (d->residual == SC_RES_PROJ) {
+        a.vr = sv->vr; a.mean_r = inf ? inf->mean_r : sv->mean_r; a.invstd_r = sv->invstd_r; a.gamma_r = p->gamma_r; a.beta_r = p->beta_r;
+    }
+    if (io.phases) {
+        a.phases = io.phases; a.B = m.B / io.phases; a.T = io.Td; a.len_out = io.len_dense;
+        a.v_out = io.dense.v; a.vr_out = io.dense.vr; a.Cu = m.Cin;
+    }
+    StatsLayout left;              // statistics of the main branch that the apply step takes
+    left.kind = -1;
     if (d->has_bn && d->residual == SC_RES_PROJ) {
         // the residual projection does not depend on the main branch: its contraction and statistics go to the
         // side stream and are joined just before the apply step
@@ -267,7 +287,7 @@ int block_fwd_impl(sc_ctx* ctx, const Launch& L, const sc_block_desc* d, const D
             conv_fwd_simt(L, dt, p->wp, io.x, bias, v, vdt, io.len_in, io.len_out, m.B, m.Cin, m.Cout, m.T, m.Tp, m.K, m.s, m.dil);
         }
         if (!d->has_bn) return SC_OK;
-        if (small) {}
+        if (stats && apply_takes_stats(dt, a, sl)) left = sl;
         else if (stats) finalize_stats(L, d, m, sl, v, vdt, io.len_out, io.nvalid, io.blk_off, f.partials, sv->mean, sv->invstd, rmean, rvar);
         else invstd_from_var(L, inf->var, d->bn_eps, sv->invstd, m.Cout);
     }
@@ -311,22 +331,14 @@ int block_fwd_impl(sc_ctx* ctx, const Launch& L, const sc_block_desc* d, const D
     }
     if (m.full) {}
     else if (inf) pointwise_fixed(ctx, L, d, m, m.Cin, odt, wp_op, u, sv->v, io.len_out, io.blk_off, inf->var, sv->invstd);
-    else pointwise_bn(ctx, L, d, m, m.Cin, odt, wp_op, u, sv->v, io.len_out, io.nvalid, io.blk_off, small ? nullptr : sv->mean, sv->invstd,
-                      f.partials, rmean, rvar);
-    ApplyArgs a{};
-    a.v = sv->v; a.mean = inf ? inf->mean : sv->mean; a.invstd = sv->invstd; a.gamma = p->gamma; a.beta = p->beta;
-    a.residual = d->residual; a.y = io.y; a.len_out = io.len_out;
-    a.B = m.B; a.C = m.Cout; a.Tp = m.Tp; a.has_relu = d->has_relu; a.res_before_relu = d->res_before_relu;
-    if (d->residual == SC_RES_IDENTITY) a.xres = io.xres;
-    if (d->residual == SC_RES_PROJ) {
-        a.vr = sv->vr; a.mean_r = inf ? inf->mean_r : sv->mean_r; a.invstd_r = sv->invstd_r; a.gamma_r = p->gamma_r; a.beta_r = p->beta_r;
-        wait_side(ctx, L, ctx->ev[5]);      // the projection branch (enqueued above on the side stream) is complete
-    }
-    if (io.phases) {
-        a.phases = io.phases; a.B = m.B / io.phases; a.T = io.Td; a.len_out = io.len_dense;
-        a.v_out = io.dense.v; a.vr_out = io.dense.vr; a.u = u; a.u_out = u ? io.dense.u : nullptr; a.Cu = m.Cin;
-    }
-    if (small) bn_small_fwd(L, a, io.nvalid, d->bn_eps, d->bn_momentum, sv->mean, sv->invstd, rmean, rvar);
+    else pointwise_bn(ctx, L, d, m, m.Cin, odt, wp_op, u, sv->v, io.len_out, io.nvalid, io.blk_off, sv->mean, sv->invstd,
+                      f.partials, rmean, rvar, &a, &left);
+    if (d->residual == SC_RES_PROJ) wait_side(ctx, L, ctx->ev[5]);      // the projection branch (enqueued above on the side stream) is complete
+    if (io.phases) { a.u = u; a.u_out = u ? io.dense.u : nullptr; }
+    if (left.kind == 2)
+        bn_apply_flat(L, dt, a, FlatStats{(const float4*)f.partials, left.grid, left.tiles_m, left.rows_per_tile, io.blk_off, io.nvalid,
+                                          d->bn_eps, d->bn_momentum, sv->mean, sv->invstd, rmean, rvar});
+    else if (left.kind == 0) bn_small_fwd(L, a, io.nvalid, d->bn_eps, d->bn_momentum, sv->mean, sv->invstd, rmean, rvar);
     else bn_apply(L, dt, a);
     return SC_OK;
 }

@@ -206,6 +206,37 @@ bn_finalize_kernel(const float2* __restrict__ partials, int parts_per_b, int til
 // The same merge for the per-(CTA, channel) partials (count, sum, M2) of the flattened-block contraction.
 // CTA c of the contraction contributed to M tile m iff its unit range [c U / G, (c+1) U / G) meets
 // [m nblk, (m+1) nblk); the pivot is the mean of the first contributing CTA's partial.
+// Unit x belongs to CTA ((x + 1) G - 1) / U, so the contributors are the CTAs between the owners of the tile's first and last
+// unit, without those that have no unit at all (only when U < G).  Two divisions; testing every CTA's range took twenty.
+struct FlatShare {
+    int first, last, G; uint32_t U; bool sparse;
+    __device__ __forceinline__ FlatShare(int nblk, int tiles_m, int G_, int m) : G(G_) {
+        const long long u = (long long)tiles_m * nblk, lo = (long long)m * nblk, hi = lo + nblk;
+        first = 0; last = -1; U = (uint32_t)u; sparse = u < G;
+        if (u <= 0) return;
+        if (u * (G + 1) < (1ll << 31)) {               // the same quotients in 32-bit arithmetic
+            first = (int)((((uint32_t)lo + 1u) * (uint32_t)G - 1u) / U); last = (int)(((uint32_t)hi * (uint32_t)G - 1u) / U);
+        } else {
+            first = (int)(((lo + 1) * G - 1) / u); last = (int)((hi * G - 1) / u);
+        }
+    }
+    __device__ __forceinline__ bool takes_part(int c) const {
+        return c >= first && c <= last && (!sparse || (uint32_t)c * U / (uint32_t)G != ((uint32_t)c + 1u) * U / (uint32_t)G);
+    }
+};
+// sum t and M2 about the pivot -> mean and variance
+__device__ __forceinline__ void merged_stats(float N, float t, float m2, float pivot, float& mean, float& var) {
+    mean = N > 0.f ? t / N : 0.f;
+    const float dm = mean - pivot;
+    var = fmaxf(N > 0.f ? (m2 - N * dm * dm) / N : 0.f, 0.f);
+}
+__device__ __forceinline__ void put_stats(int o, float mean, float invstd, float var, float N, float momentum, float* mean_out, float* invstd_out,
+                                          float* running_mean, float* running_var) {
+    mean_out[o] = mean;
+    invstd_out[o] = invstd;
+    if (running_mean) running_mean[o] = (1.f - momentum) * running_mean[o] + momentum * mean;
+    if (running_var) running_var[o] = (1.f - momentum) * running_var[o] + momentum * (N > 1.f ? var * (N / (N - 1.f)) : var);
+}
 constexpr int kFlatParts = 10;        // partials per lane: the contraction has at most 320 CTAs
 __global__ void __launch_bounds__(32 * kFinWarps)
 bn_finalize_flat_kernel(const float4* __restrict__ partials, int G, int tiles_m, int rows_per_tile,
@@ -216,31 +247,19 @@ bn_finalize_flat_kernel(const float4* __restrict__ partials, int G, int tiles_m,
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int o = blockIdx.x * 32 + lane;
     const bool act = o < C;
-    const long long nblk = blk_off[B];
-    const long long U = (long long)tiles_m * nblk;
-    const int m = min(o, C - 1) / rows_per_tile;
-    const long long lo = m * nblk, hi = lo + nblk;
-    const bool small = U * (G + 1) < (1ll << 31);      // the same quotients in 32-bit arithmetic (no 64-bit divisions)
-    auto takes_part = [&](int c) -> bool {
-        long long b0, b1;
-        if (small) { b0 = (uint32_t)U * (uint32_t)c / (uint32_t)G; b1 = (uint32_t)U * (uint32_t)(c + 1) / (uint32_t)G; }
-        else { b0 = U * c / G; b1 = U * (c + 1) / G; }
-        return max(b0, lo) < min(b1, hi);
-    };
-    int c_first = U > 0 ? (small ? (int)((uint32_t)lo * (uint32_t)G / (uint32_t)U) : (int)(lo * G / U)) : 0;
-    while (c_first < G - 1 && !takes_part(c_first)) ++c_first;
+    const FlatShare F(blk_off[B], tiles_m, G, min(o, C - 1) / rows_per_tile);
     // everything above works on the lengths alone and runs ahead of the wait for the contraction; after it the pivot and
     // the partials are one round of independent loads
     uint32_t part = 0;
 #pragma unroll
     for (int i = 0; i < kFlatParts; ++i) {
         const int c = w + i * kFinWarps;
-        if (act && U > 0 && c < G && takes_part(c)) part |= 1u << i;
+        if (act && F.takes_part(c)) part |= 1u << i;
     }
     const float N = (float)(*nvalid);
     pdl_sync();
     float4 pv = make_float4(0.f, 0.f, 0.f, 0.f), v[kFlatParts];
-    if (act && U > 0) pv = partials[(size_t)c_first * C + o];
+    if (act && F.last >= 0) pv = partials[(size_t)F.first * C + o];
 #pragma unroll
     for (int i = 0; i < kFlatParts; ++i)
         v[i] = (part >> i) & 1 ? partials[(size_t)(w + i * kFinWarps) * C + o] : make_float4(0.f, 0.f, 0.f, 0.f);
@@ -260,17 +279,9 @@ bn_finalize_flat_kernel(const float4* __restrict__ partials, int G, int tiles_m,
     float t = 0.f, m2 = 0.f;
 #pragma unroll
     for (int i = 0; i < kFinWarps; ++i) { t += s_red[i][lane].x; m2 += s_red[i][lane].y; }
-    const float mean = N > 0.f ? t / N : 0.f;
-    const float dm = mean - pivot;
-    float var = N > 0.f ? (m2 - N * dm * dm) / N : 0.f;
-    var = fmaxf(var, 0.f);
-    mean_out[o] = mean;
-    invstd_out[o] = 1.f / sqrtf(var + eps);
-    if (running_mean) running_mean[o] = (1.f - momentum) * running_mean[o] + momentum * mean;
-    if (running_var) {
-        const float unb = N > 1.f ? var * (N / (N - 1.f)) : var;
-        running_var[o] = (1.f - momentum) * running_var[o] + momentum * unb;
-    }
+    float mean, var;
+    merged_stats(N, t, m2, pivot, mean, var);
+    put_stats(o, mean, 1.f / sqrtf(var + eps), var, N, momentum, mean_out, invstd_out, running_mean, running_var);
 }
 
 // Per-channel constants of the forward apply step and of the backward kernels, loaded (or, in the
@@ -1109,6 +1120,69 @@ __global__ void __launch_bounds__(256) bn_bwd_reduce_fast_kernel(BnBwdArgs a, in
 // the 32 rows of a channel streams about 10 % slower than one that walks the tensor in address order, and a forward
 // apply that merges the contraction's statistics partials in its prologue pays that merge once per CTA.)
 constexpr int kChThreads = 512;
+// One round of two vectors per thread and one wave of two CTAs per SM (148 of them): with more of either the flattened kernel
+// streams faster by more than the launch costs (800 vectors in 512 channels: 94.5 us with two kernels, 95.2 with one).
+constexpr int kApplyChVectors = 2 * kChThreads, kApplyChChannels = 2 * 148;
+
+// Merge of the contraction's statistics partials and the apply step, one CTA per channel: one launch instead of two.  A thread
+// takes one of the partials (there are at most 320) while its vectors are on their way; the sums are taken in the order of
+// bn_finalize_flat_kernel, so the statistics do not depend on which of the two a block takes.  Latency-bound like the chain it
+// belongs to.  Blocks forward and backward: 256 channels, 2 x 160 frames 39.9 -> 37.9 us; the same with 8 x 400 57.0 -> 55.4.
+template <typename T, typename NT, int RES>
+__global__ void __launch_bounds__(kChThreads, 2) bn_apply_ch_kernel(ApplyArgs a, FlatStats f, int vpr) {
+    constexpr int NT_ = kChThreads, U = 2;
+    __shared__ float2 s_part[kFlatParts * kFinWarps], s_red[kFinWarps];
+    const int o = blockIdx.x, tid = threadIdx.x;
+    const FlatShare F(f.blk_off[a.B], f.tiles_m, f.G, o / f.rows_per_tile);
+    const bool part = F.takes_part(tid);
+    const float N = (float)(*f.nvalid);
+    FwdChan c{0.f, 0.f, a.gamma[o], a.beta[o], 0.f, 0.f, 0.f, 0.f};
+    const int nvec = a.B * vpr;      // at most U * NT_
+    int nin[U]; size_t off[U]; uint4 rv[U], rr[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        const int j = tid + u * NT_;
+        nin[u] = -1; off[u] = 0;
+        if (j < nvec) {
+            const int b = (int)a.dvpr.div((uint32_t)j), t0 = (j - b * vpr) * 8;
+            nin[u] = max(0, min(a.len_out[b], a.Tp) - t0);
+            off[u] = ((size_t)b * a.C + o) * a.Tp + t0;
+        }
+    }
+    pdl_sync();              // lengths, offsets and parameters (read above) were settled well before the contraction
+    const float4 pv = F.last >= 0 ? f.partials[(size_t)F.first * a.C + o] : make_float4(0.f, 0.f, 0.f, 0.f);
+    const float4 v = part ? f.partials[(size_t)tid * a.C + o] : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        if (nin[u] <= 0) continue;
+        rv[u] = *reinterpret_cast<const uint4*>((const NT*)a.v + off[u]);
+        if (RES == 1) rr[u] = *reinterpret_cast<const uint4*>((const T*)a.xres + off[u]);
+        if (RES == 2) rr[u] = *reinterpret_cast<const uint4*>((const NT*)a.vr + off[u]);
+    }
+    if (RES == 2) { c.mur = a.mean_r[o]; c.isr = a.invstd_r[o]; c.gar = a.gamma_r[o]; c.ber = a.beta_r[o]; }
+    const float pivot = pv.x > 0.f ? pv.y / pv.x : 0.f;
+    if (tid < kFlatParts * kFinWarps) {
+        const float d = v.x > 0.f ? v.y / v.x - pivot : 0.f;
+        s_part[tid] = make_float2(v.x > 0.f ? v.y : 0.f, v.x > 0.f ? fmaf(v.x * d, d, v.z) : 0.f);
+    }
+    __syncthreads();
+    if (tid < kFinWarps) {
+        float s1 = 0.f, q = 0.f;
+#pragma unroll
+        for (int i = 0; i < kFlatParts; ++i) { s1 += s_part[tid + i * kFinWarps].x; q += s_part[tid + i * kFinWarps].y; }
+        s_red[tid] = make_float2(s1, q);
+    }
+    __syncthreads();
+    float t = 0.f, m2 = 0.f, var;
+#pragma unroll
+    for (int i = 0; i < kFinWarps; ++i) { t += s_red[i].x; m2 += s_red[i].y; }
+    merged_stats(N, t, m2, pivot, c.mu, var);
+    c.is = 1.f / sqrtf(var + f.eps);
+    if (tid == 0) put_stats(o, c.mu, c.is, var, N, f.momentum, f.mean, f.invstd, f.running_mean, f.running_var);
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+        if (nin[u] >= 0) apply_core<T, NT, RES>((T*)a.y + off[u], nin[u], rv[u], rr[u], c);
+}
 
 // Backward reduction of channel o over every sample, then the channel's coefficients, parameter gradients and its
 // term of the bound on |gv| (what bn_bwd_finalize_kernel does for the row-mapped reduction).
@@ -1320,6 +1394,22 @@ void bn_apply(const Launch& L, int dtype, const ApplyArgs& a_in) {
         return;
     }
     SC_DISPATCH3(dtype, (launch_k(L, bn_apply_kernel<T, NT>, (a.B * a.C + kRowsPerCta - 1) / kRowsPerCta, kRowThreads, 0, a)));
+    L.count();
+}
+
+bool bn_apply_takes_stats(int dtype, const ApplyArgs& a) {
+    return dtype != F32 && !a.phases && a.Tp % 8 == 0 && a.has_relu && a.res_before_relu && fits32(a.B, a.C, a.Tp) &&
+           (long long)a.B * (a.Tp / 8) <= kApplyChVectors && a.C <= kApplyChChannels;
+}
+void bn_apply_flat(const Launch& L, int dtype, const ApplyArgs& a_in, const FlatStats& f) {
+    ApplyArgs a = a_in;
+    const double e = (double)dtype_size(dtype), en = (double)dtype_size(ntype_of(dtype));
+    KScope ks_(L, KC_BN_APPLY, (double)a.B * a.C * a.Tp * (en + e + (a.residual == 1 ? e : 0) + (a.residual == 2 ? en : 0)), 0.0);
+    const int vpr = a.Tp / 8;
+    a.dvpr = FastDiv((uint32_t)vpr);
+    if (a.residual == 0) { SC_DISPATCH16(dtype, (launch_k(L, bn_apply_ch_kernel<T, NT, 0>, (unsigned)a.C, kChThreads, 0, a, f, vpr))); }
+    else if (a.residual == 1) { SC_DISPATCH16(dtype, (launch_k(L, bn_apply_ch_kernel<T, NT, 1>, (unsigned)a.C, kChThreads, 0, a, f, vpr))); }
+    else { SC_DISPATCH16(dtype, (launch_k(L, bn_apply_ch_kernel<T, NT, 2>, (unsigned)a.C, kChThreads, 0, a, f, vpr))); }
     L.count();
 }
 

@@ -273,6 +273,15 @@ struct ApplyArgs {
     FastDiv dT;
 };
 void bn_apply(const Launch& L, int dtype, const ApplyArgs& a);
+// The same with the merge of the contraction's per-(CTA, channel) statistics partials in front (see bn_finalize_flat), where
+// bn_apply_takes_stats says so.
+struct FlatStats {
+    const float4* partials; int G, tiles_m, rows_per_tile;
+    const int *blk_off, *nvalid;
+    float eps, momentum; float *mean, *invstd, *running_mean, *running_var;
+};
+bool bn_apply_takes_stats(int dtype, const ApplyArgs& a);
+void bn_apply_flat(const Launch& L, int dtype, const ApplyArgs& a, const FlatStats& f);
 // Statistics of v and the apply step in one kernel, for the float32 tensors that bn_small accepts.
 bool bn_small(int dtype, int B, int Tp);
 void bn_small_fwd(const Launch& L, const ApplyArgs& a, const int* nvalid, float eps, float momentum, float* mean, float* invstd,
