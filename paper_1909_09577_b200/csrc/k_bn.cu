@@ -1361,9 +1361,10 @@ static bool fits32(int B, int C, int Tp) { return (long long)B * C * (Tp / 8) < 
 static unsigned fast_grid(long long total, int V) { return (unsigned)((total + 256ll * V - 1) / (256ll * V)); }
 
 // Algorithmic bytes per element of the batch-norm kernels: every tensor they must read or write, once.
-// The channel-per-CTA reduction pays off once a channel holds a few vectors per thread; below that (or with few
-// channels) the row-mapped kernel and its separate finalize step are used.
-static bool channel_mapped(int B, int C, int Tp) { return C >= 32 && (long long)B * (Tp / 8) >= 1024; }
+// The channel-per-CTA reduction: one launch instead of two, so small tensors take it at any width (a block forward and
+// backward with 40 to 2000 vectors per channel: 2.5-7 % faster than with the row-mapped kernel and its finalize step); longer
+// channels only where there are enough of them to fill the SMs.
+static bool channel_mapped(int B, int C, int Tp) { return C >= 32 || (long long)B * (Tp / 8) <= 1024; }
 
 void bn_apply(const Launch& L, int dtype, const ApplyArgs& a_in) {
     ApplyArgs a = a_in;
