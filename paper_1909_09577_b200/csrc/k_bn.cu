@@ -1414,7 +1414,7 @@ void bn_apply_flat(const Launch& L, int dtype, const ApplyArgs& a_in, const Flat
     L.count();
 }
 
-void bn_bwd_reduce(const Launch& L, int dtype, BnBwdArgs& a) {
+static void bn_bwd_reduce(const Launch& L, int dtype, BnBwdArgs& a) {
     a.nslots = 1; a.vpw = 32; a.vpw_shift = 5;
     const double e = (double)dtype_size(dtype), en = (double)dtype_size(ntype_of(dtype));
     if (dtype != F32 && a.Tp % 8 == 0 && a.Tp >= 256 && a.has_bn && a.has_relu && a.res_before_relu && fits32(a.B, a.C, a.Tp)) {
@@ -1439,7 +1439,7 @@ void bn_bwd_reduce(const Launch& L, int dtype, BnBwdArgs& a) {
     L.count();
 }
 
-void bn_bwd_finalize(const Launch& L, const BnBwdArgs& a, const float* gamma, const float* gamma_r,
+static void bn_bwd_finalize(const Launch& L, const BnBwdArgs& a, const float* gamma, const float* gamma_r,
                      float* dgamma, float* dbeta, float* dgamma_r, float* dbeta_r, float* dbias,
                      int accumulate) {
     KScope ks_(L, KC_BN_BWD_FINALIZE, 16.0 * a.B * a.C * a.nslots, 0.0);
