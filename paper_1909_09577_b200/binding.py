@@ -157,7 +157,8 @@ def _stream_ptr(stream) -> int:
 
 # A call marshals up to eight tensors and three structs of pointers, and filling a ctypes struct field by field costs about
 # as much as enqueueing a kernel.  They are passed as packed bytes instead (ctypes hands over the address of a bytes
-# object): the descriptor of a dense tensor differs from that of any other of its type and shape in the address alone.
+# object): the descriptor of a contiguous tensor differs from that of any other of its type and shape in the address alone,
+# unless an axis has size 1, whose stride may be anything.
 _DTYPES = {torch.float32: SC_F32, torch.float16: SC_F16, torch.bfloat16: SC_BF16}
 _TAGS = (0, 1, 2)
 _tails: Dict[tuple, bytes] = {}
@@ -194,6 +195,9 @@ def _tensor(t: Optional[torch.Tensor]):
         return tensor_arg(t)
     key = (t.dtype, t.shape)
     tail = _tails.get(key)
+    if tail is None and 1 in t.shape:
+        key += t.stride()
+        tail = _tails.get(key)
     if tail is None:
         if len(_tails) >= 1024:
             _tails.clear()

@@ -5,6 +5,7 @@ import os
 import re
 
 import pytest
+import torch
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
@@ -85,6 +86,21 @@ def test_residual_spans_may_overlap_but_not_point_forward(api):
     with pytest.raises(api.SepconvError) as e:
         bytes_of([plain, res(2), plain])
     assert e.value.code == -6
+
+
+def test_descriptor_strides_are_the_tensors_own(api):
+    """The stride of an axis of size 1 is arbitrary in a contiguous tensor: it reaches the library as it is, and describing
+    such a tensor does not change how later tensors of its shape are described."""
+    b = api.binding
+    def strides(t):
+        return list(b.sc_tensor.from_buffer_copy(bytes(b._tensor(t))).stride)
+    plain = lambda: torch.zeros((1, 64, 160), dtype=torch.float16)
+    odd = torch.zeros((64, 1, 160), dtype=torch.float16).transpose(0, 1)
+    assert odd.is_contiguous() and odd.shape == plain().shape and odd.stride() == (160, 160, 1)
+    for first, second in ((odd, plain()), (plain(), odd)):
+        b._tails.clear()
+        for t in (first, second, first):
+            assert strides(t) == list(t.stride())
 
 
 def test_missing_library_fails_loudly(api, tmp_path):
