@@ -247,11 +247,13 @@ int  sepconv_infer(sc_ctx* ctx, const sc_block_desc* desc,
  * has nowhere to get the scratch that sepconv_fwd asks for.
  *
  * The scratch is a fixed array of SEPCONV_STATIC_SCRATCH_BYTES inside the library image: every GPU on
- * which the library is loaded sets that much memory aside until the process exits.  A block whose
- * forward scratch (sepconv_workspace_bytes) exceeds it is refused with SC_ERR_WORKSPACE and a message
- * on stderr; nothing is enqueued.  Arguments and results are exactly those of sepconv_fwd (running
- * statistics are not updated).  The call itself uses no cudaMalloc/cudaFree or other allocating
- * routine.
+ * which the library is loaded sets that much memory aside until the process exits.  A block that
+ * sepconv_fwd would run on copies of its operands (rows that are no multiple of 8 frames, dilation 2, the
+ * non-separable convolution) does so here only when they fit; otherwise it runs on the dense tensors with
+ * the kernels that take these, slower and with sums in another order.  A block whose scratch exceeds the
+ * array even so is refused with SC_ERR_WORKSPACE and a message on stderr; nothing is enqueued.  Arguments
+ * and results are otherwise those of sepconv_fwd (running statistics are not updated).  The call itself
+ * uses no cudaMalloc/cudaFree or other allocating routine.
  *
  * The first call on each device looks up the array's device address; with CUDA's lazy module loading
  * that is also the moment the device sets the array aside, so this first call can still fail with

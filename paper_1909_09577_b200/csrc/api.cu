@@ -146,7 +146,9 @@ bool conv_on_tc(const TcState* tc, const sc_block_desc* d, const Dims& m) {
     return m.full && tc_conv_supported(tc, d->io_dtype, m.B, m.Cin, m.Cout, m.T, m.s);
 }
 
-void plan_fwd(const sc_block_desc* d, const Dims& m, Bump& ws, FwdScratch* f, const TcState* tc) {
+// copies: whether the non-separable convolution may take the operand copies of its tensor-core form; without them it runs on
+// the dense tensors
+void plan_fwd(const sc_block_desc* d, const Dims& m, Bump& ws, FwdScratch* f, const TcState* tc, bool copies = true) {
     f->len_out = (int*)ws.take(sizeof(int) * m.B);
     f->nvalid = (int*)ws.take(sizeof(int));
     f->blk_off = (int*)ws.take(sizeof(int) * (m.B + 1));
@@ -154,7 +156,7 @@ void plan_fwd(const sc_block_desc* d, const Dims& m, Bump& ws, FwdScratch* f, co
     f->partials_r = (d->residual == SC_RES_PROJ) ? ws.take(tc_stats_bytes(m.B, m.Cout, m.Tp)) : nullptr;
     f->zf32 = d->log_softmax ? (float*)ws.take(sizeof(float) * m.B * m.Cout * m.Tp) : nullptr;
     f->xr = (d->residual == SC_RES_PROJ) ? ws.take(esize(d->io_dtype) * m.B * m.Cres * m.Tp) : nullptr;
-    const bool conv = conv_on_tc(tc, d, m);
+    const bool conv = copies && conv_on_tc(tc, d, m);
     f->x_tm = conv ? ws.take((size_t)2 * m.B * m.Cin * m.T) : nullptr;
     f->taps = conv ? ws.take((size_t)2 * m.Cin * m.Cout * m.K) : nullptr;
     f->w16 = (op_dtype(d) != d->io_dtype) ? ws.take((size_t)2 * m.Cout * m.Cin) : nullptr;
@@ -278,7 +280,7 @@ int block_fwd_impl(sc_ctx* ctx, const Launch& L, const sc_block_desc* d, const D
         const float* bias = !d->has_bn && d->has_bias ? p->bias : nullptr;
         const bool stats = d->has_bn && !inf;
         StatsLayout sl;
-        if (ctx->gemm_mode == 0 && conv_on_tc(&ctx->tc, d, m)) {
+        if (ctx->gemm_mode == 0 && f.x_tm) {
             to_time_major(L, io.x, f.x_tm, io.len_in, m.B, m.Cin, m.T);
             split_taps(L, p->wp, f.taps, m.Cout, m.Cin, m.K, 0);
             tc_conv_fwd(&ctx->tc, L, dt, f.taps, f.x_tm, bias, v, vdt, io.len_out, io.blk_off, m.B, m.Cin, m.Cout, m.T, m.K, m.dil,
@@ -817,7 +819,8 @@ int sepconv_workspace_bytes(const sc_block_desc* desc, size_t* fwd, size_t* bwd)
 namespace {
 int fwd_call(sc_ctx* ctx, const Launch& L, const sc_block_desc* desc, const sc_tensor* x, const sc_tensor* x_res,
              const int32_t* lengths_dev, const sc_block_params* params, sc_tensor* y, int32_t* out_lengths_dev,
-             sc_block_saved* saved, float* running_mean, float* running_var, void* workspace, size_t workspace_bytes) {
+             sc_block_saved* saved, float* running_mean, float* running_var, void* workspace, size_t workspace_bytes,
+             bool dense_if_short) {
     Dims m;
     SC_TRY(desc_dims(desc, &m));
     const int dt = desc->io_dtype;
@@ -832,10 +835,15 @@ int fwd_call(sc_ctx* ctx, const Launch& L, const sc_block_desc* desc, const sc_t
     if (!workspace) return SC_ERR_WORKSPACE;
     Packed pk;
     if (ctx->gemm_mode == 0) pk = plan_packed(desc, m);
-    Bump ws(workspace, workspace_bytes);
     FwdScratch f; FwdPack fp;
+    Bump ws(workspace, workspace_bytes);
     plan_fwd(desc, pk.phases ? pk.m : m, ws, &f, &ctx->tc);
     if (pk.phases) plan_fwd_pack(desc, pk, ws, &fp);
+    if (!ws.ok() && dense_if_short) {
+        pk = Packed();
+        ws = Bump(workspace, workspace_bytes);
+        plan_fwd(desc, m, ws, &f, &ctx->tc, false);
+    }
     if (!ws.ok()) return SC_ERR_WORKSPACE;
     BlockIO io{};
     io.x = x->ptr; io.xres = desc->residual != SC_RES_NONE ? (x_res ? x_res->ptr : x->ptr) : nullptr;
@@ -860,7 +868,7 @@ int sepconv_fwd(sc_ctx* ctx, const sc_block_desc* desc, const sc_tensor* x, cons
     key_tensor(k, y); k.val(out_lengths_dev); k.add(saved, sizeof(*saved)); k.val(running_mean); k.val(running_var);
     return run_call(ctx, cuda_stream, [&](const Launch& L) {
         return fwd_call(ctx, L, desc, x, x_res, lengths_dev, params, y, out_lengths_dev, saved, running_mean, running_var, workspace,
-                        workspace_bytes);
+                        workspace_bytes, false);
     });
 }
 
@@ -1445,5 +1453,13 @@ int sc::fwd_direct(sc_ctx* ctx, const sc_block_desc* desc, const sc_tensor* x, c
                    size_t workspace_bytes, void* cuda_stream) {
     if (!ctx || !lengths_dev) return SC_ERR_NULL;
     return fwd_call(ctx, Launch{(cudaStream_t)cuda_stream, ctx->status_dev, &ctx->launches, &ctx->prof, ctx->gemm_mode, ctx->pdl}, desc, x,
-                    x_res, lengths_dev, params, y, out_lengths_dev, saved, nullptr, nullptr, workspace, workspace_bytes);
+                    x_res, lengths_dev, params, y, out_lengths_dev, saved, nullptr, nullptr, workspace, workspace_bytes, true);
+}
+
+int sc::fwd_dense_bytes(const sc_block_desc* desc, size_t* bytes) {
+    Dims m;
+    SC_TRY(desc_dims(desc, &m));
+    Bump b(nullptr, 0); FwdScratch f; plan_fwd(desc, m, b, &f, nullptr, false);
+    *bytes = b.off + 256;
+    return SC_OK;
 }

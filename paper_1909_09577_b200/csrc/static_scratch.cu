@@ -24,10 +24,10 @@ extern "C" int sepconv_fwd_static(sc_ctx* ctx, const sc_block_desc* desc, const 
                                   sc_block_saved* saved, void* cuda_stream) {
     if (!ctx || !desc) return SC_ERR_NULL;
     size_t need = 0;
-    int rc = sepconv_workspace_bytes(desc, &need, nullptr);
+    int rc = sc::fwd_dense_bytes(desc, &need);
     if (rc != SC_OK) return rc;
     if (need > (size_t)SEPCONV_STATIC_SCRATCH_BYTES) {
-        fprintf(stderr, "sepconv_fwd_static: this block needs %zu bytes of scratch, the built-in buffer holds %zu; "
+        fprintf(stderr, "sepconv_fwd_static: this block needs at least %zu bytes of scratch, the built-in buffer holds %zu; "
                         "use sepconv_fwd with a caller-owned workspace\n",
                 need, (size_t)SEPCONV_STATIC_SCRATCH_BYTES);
         return SC_ERR_WORKSPACE;

@@ -7,6 +7,7 @@ import pytest
 import torch
 
 import synth_inputs as si
+from oracle import sepconv_oracle as O
 from tests import parity_util as U
 
 pytestmark = pytest.mark.gpu
@@ -73,3 +74,44 @@ def test_static_scratch_rejects_large_blocks():
         assert e.value.code == -7
     finally:
         ctx.close()
+
+
+DENSE = [
+    # blocks whose operand copies exceed the built-in array while the scratch of the dense form does not
+    (dict(C_in=256, C_out=256, K=33), 32, 397, "bf16"),
+    (dict(C_in=512, C_out=512, K=33, dilation=2), 8, 400, "bf16"),
+    (dict(C_in=256, C_out=256, K=11, has_dw=False, full_conv=True), 32, 800, "f16"),
+    (dict(C_in=64, C_out=64, K=33), 32, 797, "f16"),
+]
+
+
+@pytest.mark.parametrize("case", range(len(DENSE)))
+def test_static_scratch_without_room_for_copies(case):
+    import paper_1909_09577_b200 as api
+    kw, B, T, dtype = DENSE[case]
+    L = si.LayerCfg(**kw)
+    d = si.draw(si.Workload("static", dtype, B, T, [L], 40 + case, len_lo=T // 3, len_hi=T, affine="random"))
+    desc = api.block_desc(L, B, T, dtype)
+    assert api.sepconv_workspace_bytes(desc)[0] > api.binding.STATIC_SCRATCH_BYTES
+    new = lambda shape, dt: torch.full(shape, float("nan"), dtype=dt, device="cuda")
+    y, out_len = new((B, L.C_out, T), U.TD[dtype]), torch.zeros(B, dtype=torch.int32, device="cuda")
+    saved = {"u": new((B, L.C_in, T), torch.float16), "v": new((B, L.C_out, T), torch.float16),
+             "mean": new((L.C_out,), torch.float32), "invstd": new((L.C_out,), torch.float32)}
+    ctx = api.Context(0)
+    try:
+        api.sepconv_fwd_static(ctx, desc, U.dev(d.x, dtype), torch.from_numpy(d.lengths).cuda(), U.params_dev(d.params[0], dtype),
+                               y, out_len, saved)
+        assert ctx.last_status() == 0
+    finally:
+        ctx.close()
+    S = O.block_fwd(L, d.x, d.lengths, d.params[0])
+    vm = S["valid"]
+    rep = U.Report(dtype)
+    if L.has_dw:
+        rep.add("u", U.host(saved["u"]), S["u"], vm)
+    rep.add("v", U.masked(saved["v"], vm), np.where(vm, S["v"], 0.0), vm)
+    rep.add("mean", U.host(saved["mean"]), S["mean"])
+    rep.add("invstd", U.host(saved["invstd"]), S["invstd"])
+    rep.add("y", U.host(y), S["y"], vm, stored=True)
+    rep.check()
+    np.testing.assert_array_equal(out_len.cpu().numpy(), S["out_len"])
