@@ -1196,10 +1196,11 @@ bn_bwd_reduce_ch_kernel(BnBwdArgs a, int vpr, const float* gamma_r, float* dgamm
     __shared__ float4 s_sum[NT_ / 32];
     const int o = blockIdx.x, tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     BwdChan c{};
+    if (RES == 0) { c.ga = a.gamma[o]; c.be = a.beta[o]; }       // the caller's parameters
+    pdl_sync();
+    // the statistics may come from the kernel just before this one: the last layer's bn_apply_ch_kernel writes them itself
     c.mu = a.mean[o]; c.is = a.invstd[o];
-    if (RES == 0) { c.ga = a.gamma[o]; c.be = a.beta[o]; }
     if (RES == 2) { c.mur = a.mean_r[o]; c.isr = a.invstd_r[o]; }
-    pdl_sync();              // the coefficients above come from the forward pass and the caller's parameters
     const int nvec = a.B * vpr;
     float s0 = 0.f, s1 = 0.f, s3 = 0.f, amax = 0.f;
     for (int jb = tid; jb < nvec; jb += U * NT_) {

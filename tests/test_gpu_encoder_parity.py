@@ -165,6 +165,29 @@ def test_encoder_with_overlapping_residual_spans(api, ctx, dtype):
         assert rep.worst()[1] <= E2E_GRAD_LIMIT, rep.worst()
 
 
+@pytest.mark.parametrize("residual", ["none", "identity", "proj"])
+@pytest.mark.parametrize("dtype", ["bf16", "f16"])
+def test_encoder_ending_in_batch_norm(api, ctx, dtype, residual):
+    """No decoder behind the last block: its apply step, which merges the statistics itself, is followed directly by its own
+    backward reduction.  The workspace starts as zeros every time, so that statistics read too early show (a scale of zero);
+    direct calls and replays, each bit-equal to the chain of block calls."""
+    layers = [si.LayerCfg(16, 32, K=5, stride=2), si.LayerCfg(32, 64, K=7), si.LayerCfg(64, 64, K=9, residual=residual)]
+    w = si.Workload("tiny_encoder_bn_end", dtype, 8, 512, layers, 29, len_lo=128, len_hi=512, affine="random")
+    d = si.draw(w)
+    reports, chain = U.run_chain(ctx, api, w, d)
+    spec = api.EncoderSpec(w.layers, w.B, w.T, w.dtype)
+    blob, xd, gd = spec.pack_params(d.params, "cuda"), U.dev(d.x, w.dtype), U.dev(d.g, w.dtype)
+    ld = torch.from_numpy(d.lengths).cuda()
+    ws = torch.empty(api.encoder_workspace_bytes(spec), dtype=torch.uint8, device="cuda")
+    grads = torch.zeros(spec.grad_bytes, dtype=torch.uint8, device="cuda")
+    for call in range(4):
+        ws.zero_()
+        logits, out_len, gblob, dx = api.encoder_fwd_bwd(ctx, spec, xd, ld, blob, gd, grads_blob=grads, want_dx=True, workspace=ws)
+        assert ctx.last_status() == 0
+        assert_encoder_equals_chain(w, d, spec, logits, out_len, gblob, dx, chain)
+        del logits, out_len, dx                  # so that the next call gets the same buffers: the third is captured
+
+
 def test_encoder_without_dx_and_accumulate(api, ctx):
     w = si.tiny_encoder(dtype="bf16", B=2, T=64, ragged=True, width=32)
     d = si.draw(w)
