@@ -1361,6 +1361,8 @@ int encoder_call(sc_ctx* ctx, const Launch& L, const sc_encoder_desc* e, const s
     }
     const void *x_in = x->ptr, *dl = dlogits->ptr;
     void *lg = logits->ptr, *dx_out = dx ? dx->ptr : nullptr;
+    // ahead of the copies: the first layer's contraction reads the block offsets before it waits, so a kernel has to lie between
+    encoder_prologue(L, e, P, lengths_dev, out_lengths_dev, params_blob, param_offsets, true);
     if (P.T_pad) {
         copy_frames(L, true, x->ptr, P.x_pad, m0.Cin, lengths_dev, m0.B, T_in, m0.T);
         copy_frames(L, true, dlogits->ptr, P.dlogits_pad, ml.Cout, nullptr, ml.B, T_out, ml.Tp);
@@ -1370,7 +1372,6 @@ int encoder_call(sc_ctx* ctx, const Launch& L, const sc_encoder_desc* e, const s
     auto len_in_of = [&](int i) -> const int* { return i == 0 ? lengths_dev : P.L[i - 1].len_out; };
     auto res_src = [&](int i) -> int { return (e->res_from && e->res_from[i] >= 0) ? e->res_from[i] : i; };
 
-    encoder_prologue(L, e, P, lengths_dev, out_lengths_dev, params_blob, param_offsets, true);
     // forward
     for (int i = 0; i < n; ++i) {
         LayerPlan& lp = P.L[i];

@@ -50,6 +50,20 @@ def test_packed_blocks(api, ctx, dtype, case):
     rep.check()
 
 
+def compare_with_chain(spec, w, d, logits, out_len, grads, dx, chain):
+    """Every result of a padded encoder against the chain of packed block calls.  The two differ where a layer without batch
+    norm takes another kernel (its sums in another order), which moves an element of its bf16 input gradient by at most one
+    unit, 2^-8 of it; that difference re-rounds once in every layer before it."""
+    got = {"logits": (logits, chain["logits"]), "dx": (dx, chain["dx"])}
+    for i in range(len(w.layers)):
+        for name in d.params[i]:
+            got[f"{i}.{name}"] = (spec.grad_view(grads, i, name), chain["grads"][i]["d" + name])
+    err = {k: ((a.float() - b.float()).norm() / b.float().norm()).item() for k, (a, b) in got.items()}
+    print("\npadded encoder against the chain:", {k: f"{e:.1e}" for k, e in err.items()})
+    assert (out_len.cpu().numpy() == chain["out_len"]).all()
+    assert max(err.values()) <= 2.0 ** -8 * len(w.layers) ** 0.5, err
+
+
 @pytest.mark.parametrize("T", [497, 500])
 def test_padded_encoder_equals_chain(api, ctx, T):
     """A whole encoder on rows that are no multiple of 8 frames against the chain of (packed) block calls."""
@@ -66,6 +80,24 @@ def test_padded_encoder_equals_chain(api, ctx, T):
     assert (logits.float() - chain["logits"].float()).abs().max() <= 0.1 * scale
     assert logits.shape[2] == spec.T_out and (out_len.cpu().numpy() == chain["out_len"]).all()
     assert (dx.float() - chain["dx"].float()).norm() <= 0.05 * chain["dx"].float().norm()
+
+
+def test_padded_encoder_starting_without_depthwise(api, ctx):
+    """Padded rows into a first layer whose contraction follows the copies directly: its block offsets must be settled.  The
+    workspace starts as zeros (an empty block list: nothing out of range is reachable, and the results would be zero)."""
+    layers = [si.LayerCfg(16, 32, K=1, has_dw=False), si.LayerCfg(32, 32, K=7, stride=2),
+              si.LayerCfg(32, 29, K=1, has_dw=False, has_bn=False, has_relu=False, has_bias=True)]
+    w = si.Workload("padded_pointwise_first", "bf16", 18, 497, layers, 31, len_lo=120, len_hi=497, affine="random")
+    d = si.draw(w)
+    reports, chain = U.run_chain(ctx, api, w, d)
+    spec = api.EncoderSpec(layers, w.B, w.T, w.dtype)
+    blob, x, g = spec.pack_params(d.params, "cuda"), U.dev(d.x, w.dtype), U.dev(d.g, w.dtype)
+    lens, ws = torch.from_numpy(d.lengths).cuda(), torch.empty(api.encoder_workspace_bytes(spec), dtype=torch.uint8, device="cuda")
+    for call in range(2):
+        ws.zero_()
+        logits, out_len, grads, dx = api.encoder_fwd_bwd(ctx, spec, x, lens, blob, g, want_dx=True, workspace=ws)
+        assert ctx.last_status() == 0
+        compare_with_chain(spec, w, d, logits, out_len, grads, dx, chain)
 
 
 @pytest.mark.parametrize("K,B,T", [(1, 3, 16), (3, 2, 1040), (7, 9, 528), (35, 4, 512), (87, 2, 4112), (95, 5, 304)])
