@@ -29,6 +29,7 @@ struct sc_ctx {
     cudaEvent_t ev[8] = {};     // backward fork (and the tap gradients' of a block call), done[0], done[1], forward fork, forward join, done[2], (unused)
     int overlap = 1;
     int pdl = 1;          // launch kernels with programmatic stream serialization
+    bool fresh[2] = {};   // see launch_early in kernels.h
     GraphCache graphs;
     CallKey key;
 };
@@ -199,7 +200,7 @@ void pointwise_bn(sc_ctx* ctx, const Launch& L, const sc_block_desc* d, const Di
 // The launch context of the side stream (same status word, counters and profile), or L itself when overlap is off.
 Launch side_launch(sc_ctx* ctx, const Launch& L) {
     Launch s = L;
-    if (ctx->overlap && ctx->side) s.stream = ctx->side;
+    if (ctx->overlap && ctx->side) { s.stream = ctx->side; s.lane = 1; }
     return s;
 }
 // side stream waits for everything enqueued on L.stream so far
@@ -664,7 +665,7 @@ void key_begin(sc_ctx* ctx, CallTag tag, void* ws, size_t ws_bytes) {
 // timed launch by launch are never replayed.
 template <typename F> int run_call(sc_ctx* ctx, void* stream, F&& body) {
     auto go = [&](cudaStream_t s) -> int {
-        return body(Launch{s, ctx->status_dev, &ctx->launches, &ctx->prof, ctx->gemm_mode, ctx->pdl});
+        return body(Launch{s, ctx->status_dev, &ctx->launches, &ctx->prof, ctx->gemm_mode, ctx->pdl, ctx->fresh});
     };
     if (ctx->prof.filter != -2) return go((cudaStream_t)stream);
     return ctx->graphs.run(ctx->key, (cudaStream_t)stream, &ctx->launches, SC_ERR_CUDA, go);
@@ -1453,7 +1454,7 @@ int sc::fwd_direct(sc_ctx* ctx, const sc_block_desc* desc, const sc_tensor* x, c
                    const sc_block_params* params, sc_tensor* y, int32_t* out_lengths_dev, sc_block_saved* saved, void* workspace,
                    size_t workspace_bytes, void* cuda_stream) {
     if (!ctx || !lengths_dev) return SC_ERR_NULL;
-    return fwd_call(ctx, Launch{(cudaStream_t)cuda_stream, ctx->status_dev, &ctx->launches, &ctx->prof, ctx->gemm_mode, ctx->pdl}, desc, x,
+    return fwd_call(ctx, Launch{(cudaStream_t)cuda_stream, ctx->status_dev, &ctx->launches, &ctx->prof, ctx->gemm_mode, ctx->pdl, ctx->fresh}, desc, x,
                     x_res, lengths_dev, params, y, out_lengths_dev, saved, nullptr, nullptr, workspace, workspace_bytes, true);
 }
 

@@ -275,8 +275,8 @@ __device__ __forceinline__ void chan_merge(float& n, float& mean, float& m2, flo
 // be launched.  Work placed before pdl_wait() (barrier set-up, tensor-memory allocation, descriptor prefetch) overlaps the
 // previous kernel.  Because the trigger comes after the wait, a kernel starts only once everything up to the kernel before
 // the previous one has completed; so it may also read, ahead of its wait, what was settled that early: the caller's
-// parameters (from the second kernel of a call on) and the lengths and weight copies (when another kernel lies between it
-// and the prologue that wrote them).  Both are no-ops in a kernel launched without the attribute.
+// parameters (from the second kernel of a call on) and what the prologue wrote (such kernels go through launch_early in
+// kernels.h, where the rules stand).  Both are no-ops in a kernel launched without the attribute.
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_sync() { pdl_wait(); pdl_launch_dependents(); }

@@ -369,7 +369,7 @@ bn_small_fwd_kernel(ApplyArgs a, const int* __restrict__ nvalid, float eps, floa
     const bool vec = a.Tp % 8 == 0;
     const float N = (float)(*nvalid);
     FwdChan c{0.f, 0.f, a.gamma[o], a.beta[o], 0.f, 0.f, 0.f, 0.f};
-    pdl_sync();              // the parameters and the count above were settled before the previous kernel
+    pdl_sync();              // launch_early: the parameters and the count above were settled before the previous kernel
     if (a.residual == 2) { c.mur = a.mean_r[o]; c.isr = a.invstd_r[o]; c.gar = a.gamma_r[o]; c.ber = a.beta_r[o]; }
     float s[1];
     for (int pass = 0; pass < 2; ++pass) {      // the sum, then the squares about the mean
@@ -880,7 +880,7 @@ __global__ void __launch_bounds__(256) bn_apply_fast_kernel(ApplyArgs a, int vpr
             off[j] = (size_t)row * a.Tp + t0;
         }
     }
-    pdl_sync();              // indices and lengths (settled well before the previous kernel) are worked out ahead of the wait
+    pdl_sync();              // indices and lengths are worked out ahead of the wait (launch_early)
 #pragma unroll
     for (int j = 0; j < V; ++j) {
         if (nin[j] > 0) {
@@ -1149,7 +1149,7 @@ __global__ void __launch_bounds__(kChThreads, 2) bn_apply_ch_kernel(ApplyArgs a,
             off[u] = ((size_t)b * a.C + o) * a.Tp + t0;
         }
     }
-    pdl_sync();              // lengths, offsets and parameters (read above) were settled well before the contraction
+    pdl_sync();              // launch_early: lengths, offsets and parameters (read above) were settled before the contraction
     const float4 pv = F.last >= 0 ? f.partials[(size_t)F.first * a.C + o] : make_float4(0.f, 0.f, 0.f, 0.f);
     const float4 v = part ? f.partials[(size_t)tid * a.C + o] : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
@@ -1319,6 +1319,7 @@ void prologue(const Launch& L, Prologue& p) {
     }
     KScope ks_(L, KC_LENGTHS, bytes, 0.0);
     launch_k(L, prologue_kernel, 1 + blocks, kLenThreads, 0, p, L.status);
+    if (L.fresh) L.fresh[0] = L.fresh[1] = true;
     L.count();
 }
 
@@ -1343,7 +1344,7 @@ void bn_finalize_flat(const Launch& L, const float4* partials, int grid, int til
                       const int* blk_off, const int* nvalid, int B, int C, float eps, float momentum, float* mean,
                       float* invstd, float* running_mean, float* running_var) {
     KScope ks_(L, KC_BN_FINALIZE, 16.0 * grid * C / std::max(1, tiles_m), 0.0);
-    launch_k(L, bn_finalize_flat_kernel, (C + 31) / 32, 32 * kFinWarps, 0, partials, grid, tiles_m, rows_per_tile, blk_off, nvalid, B,
+    launch_early(L, bn_finalize_flat_kernel, (C + 31) / 32, 32 * kFinWarps, 0, partials, grid, tiles_m, rows_per_tile, blk_off, nvalid, B,
                                                                           C, eps, momentum, mean, invstd, running_mean, running_var);
     L.count();
 }
@@ -1353,7 +1354,7 @@ bool bn_small(int dtype, int B, int Tp) { return dtype == F32 && (long long)B * 
 void bn_small_fwd(const Launch& L, const ApplyArgs& a, const int* nvalid, float eps, float momentum, float* mean, float* invstd,
                   float* running_mean, float* running_var) {
     KScope ks_(L, KC_BN_APPLY, 4.0 * a.B * a.C * a.Tp * (a.residual ? 3 : 2), 0.0);
-    launch_k(L, bn_small_fwd_kernel, (unsigned)a.C, kRowThreads, 0, a, nvalid, eps, momentum, mean, invstd, running_mean, running_var);
+    launch_early(L, bn_small_fwd_kernel, (unsigned)a.C, kRowThreads, 0, a, nvalid, eps, momentum, mean, invstd, running_mean, running_var);
     L.count();
 }
 
@@ -1377,8 +1378,8 @@ void bn_apply(const Launch& L, int dtype, const ApplyArgs& a_in) {
         const int nba = (int)fast_grid((total + 7) / 8, 1);
         const unsigned grid = nba + (a.u_out ? fast_grid((total_u + 7) / 8, 1) : 0);
 #define SC_APPLY_UNPACK(RES)                                                                                                  \
-        if (a.phases == 2) { SC_DISPATCH16(dtype, (launch_k(L, bn_apply_unpack_kernel<T, NT, RES, 2>, grid, 256, 0, a, total, nba, total_u))) } \
-        else { SC_DISPATCH16(dtype, (launch_k(L, bn_apply_unpack_kernel<T, NT, RES, 1>, grid, 256, 0, a, total, nba, total_u))) }
+        if (a.phases == 2) { SC_DISPATCH16(dtype, (launch_early(L, bn_apply_unpack_kernel<T, NT, RES, 2>, grid, 256, 0, a, total, nba, total_u))) } \
+        else { SC_DISPATCH16(dtype, (launch_early(L, bn_apply_unpack_kernel<T, NT, RES, 1>, grid, 256, 0, a, total, nba, total_u))) }
         if (a.residual == 0) { SC_APPLY_UNPACK(0) } else if (a.residual == 1) { SC_APPLY_UNPACK(1) } else { SC_APPLY_UNPACK(2) }
 #undef SC_APPLY_UNPACK
         L.count();
@@ -1389,7 +1390,7 @@ void bn_apply(const Launch& L, int dtype, const ApplyArgs& a_in) {
         a.dvpr = FastDiv((uint32_t)vpr); a.dC = FastDiv((uint32_t)a.C);
         const long long total = (long long)a.B * a.C * vpr;
         const unsigned grid = fast_grid(total, 2);
-#define SC_APPLY_FAST(RES) SC_DISPATCH16(dtype, (launch_k(L, bn_apply_fast_kernel<T, NT, RES, 2>, grid, 256, 0, a, vpr, total)))
+#define SC_APPLY_FAST(RES) SC_DISPATCH16(dtype, (launch_early(L, bn_apply_fast_kernel<T, NT, RES, 2>, grid, 256, 0, a, vpr, total)))
         if (a.residual == 0) { SC_APPLY_FAST(0); } else if (a.residual == 1) { SC_APPLY_FAST(1); } else { SC_APPLY_FAST(2); }
 #undef SC_APPLY_FAST
         L.count();
@@ -1409,9 +1410,9 @@ void bn_apply_flat(const Launch& L, int dtype, const ApplyArgs& a_in, const Flat
     KScope ks_(L, KC_BN_APPLY, (double)a.B * a.C * a.Tp * (en + e + (a.residual == 1 ? e : 0) + (a.residual == 2 ? en : 0)), 0.0);
     const int vpr = a.Tp / 8;
     a.dvpr = FastDiv((uint32_t)vpr);
-    if (a.residual == 0) { SC_DISPATCH16(dtype, (launch_k(L, bn_apply_ch_kernel<T, NT, 0>, (unsigned)a.C, kChThreads, 0, a, f, vpr))); }
-    else if (a.residual == 1) { SC_DISPATCH16(dtype, (launch_k(L, bn_apply_ch_kernel<T, NT, 1>, (unsigned)a.C, kChThreads, 0, a, f, vpr))); }
-    else { SC_DISPATCH16(dtype, (launch_k(L, bn_apply_ch_kernel<T, NT, 2>, (unsigned)a.C, kChThreads, 0, a, f, vpr))); }
+    if (a.residual == 0) { SC_DISPATCH16(dtype, (launch_early(L, bn_apply_ch_kernel<T, NT, 0>, (unsigned)a.C, kChThreads, 0, a, f, vpr))); }
+    else if (a.residual == 1) { SC_DISPATCH16(dtype, (launch_early(L, bn_apply_ch_kernel<T, NT, 1>, (unsigned)a.C, kChThreads, 0, a, f, vpr))); }
+    else { SC_DISPATCH16(dtype, (launch_early(L, bn_apply_ch_kernel<T, NT, 2>, (unsigned)a.C, kChThreads, 0, a, f, vpr))); }
     L.count();
 }
 
@@ -1482,8 +1483,8 @@ static void bn_bwd_apply(const Launch& L, int dtype, const BnBwdArgs& a_in) {
         const unsigned grid = fast_grid(total, a.phases ? 1 : 2);
 #define SC_BWD_FAST_G(RES, G)                                                                                        \
         if (dtype == BF16 && a.gv_dtype == F16)                                                                      \
-            launch_k(L, bn_bwd_apply_fast_kernel<__nv_bfloat16, __half, __half, RES, (G ? 1 : 2), G>, grid, 256, 0, a, vpr, total); \
-        else { SC_DISPATCH16(dtype, (launch_k(L, bn_bwd_apply_fast_kernel<T, NT, T, RES, (G ? 1 : 2), G>, grid, 256, 0, a, vpr, total))); }
+            launch_early(L, bn_bwd_apply_fast_kernel<__nv_bfloat16, __half, __half, RES, (G ? 1 : 2), G>, grid, 256, 0, a, vpr, total); \
+        else { SC_DISPATCH16(dtype, (launch_early(L, bn_bwd_apply_fast_kernel<T, NT, T, RES, (G ? 1 : 2), G>, grid, 256, 0, a, vpr, total))); }
 #define SC_BWD_FAST(RES) if (a.phases == 2) { SC_BWD_FAST_G(RES, 2) } else if (a.phases == 1) { SC_BWD_FAST_G(RES, 1) } else { SC_BWD_FAST_G(RES, 0) }
         if (a.residual == 0) { SC_BWD_FAST(0) } else if (a.residual == 1) { SC_BWD_FAST(1) } else { SC_BWD_FAST(2) }
 #undef SC_BWD_FAST

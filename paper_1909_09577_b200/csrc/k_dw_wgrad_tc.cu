@@ -143,7 +143,7 @@ dw_wgrad_tc_kernel(const __grid_constant__ CUtensorMap mapG, const __grid_consta
         ptx::prefetch_tensormap(&mapG);
         ptx::prefetch_tensormap(&mapX);
     }
-    // the set-up below reads the lengths only, which were settled well before the previous kernel; the roles that read or
+    // the set-up below reads the lengths only (launch_early: settled before the previous kernel); the roles that read or
     // write the tensors wait for it themselves
     // longest output length in every sample chunk: time blocks past it hold only zeros of gu
     for (int ch = tid; ch < p.nchunks && ch < WT_MAX_CHUNKS; ch += WT_THREADS) {
@@ -369,7 +369,7 @@ template <typename TG, typename TX>
 void launch_wt(const Launch& L, int grid, const CUtensorMap& mg, const CUtensorMap& mx, const WtParams& p) {
     auto kern = dw_wgrad_tc_kernel<TG, TX>;
     set_max_smem_once<dw_wgrad_tc_kernel<TG, TX>>(kWtSmem);
-    launch_k(L, kern, grid, WT_THREADS, kWtSmem, mg, mx, p);
+    launch_early(L, kern, grid, WT_THREADS, kWtSmem, mg, mx, p);
     L.count();
 }
 

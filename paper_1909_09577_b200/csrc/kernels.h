@@ -33,20 +33,39 @@ struct Launch {
     Prof* prof = nullptr;
     int simt_only = 0;    // 1: never take a tensor-core kernel (used by tests)
     int pdl = 1;          // 1: launch with programmatic stream serialization (see pdl_sync in common.cuh)
+    bool* fresh = nullptr;   // per lane: no kernel has been launched there since the prologue (see launch_early)
+    int lane = 0;            // 0: the caller's stream, 1: the context's second stream
     void count(int n = 1) const { if (counter) *counter += n; }
 };
 
 // Launches `kern` on L.stream; with L.pdl the launch carries the programmatic-stream-serialization attribute, so
 // the kernel may begin (up to its pdl_wait()) before the previous kernel on the stream has completed.
-template <typename K, typename... Args>
-inline void launch_k(const Launch& L, K kern, dim3 grid, dim3 block, size_t smem, Args&&... args) {
+template <bool EARLY, typename K, typename... Args>
+inline void launch_as(const Launch& L, K kern, dim3 grid, dim3 block, size_t smem, Args&&... args) {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = L.stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr; cfg.numAttrs = L.pdl ? 1 : 0;
+    const bool behind_prologue = L.fresh && L.fresh[L.lane];
+    if (L.fresh) L.fresh[L.lane] = false;
+    cfg.attrs = attr; cfg.numAttrs = L.pdl && !(EARLY && behind_prologue) ? 1 : 0;
     cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
+}
+template <typename K, typename... Args>
+inline void launch_k(const Launch& L, K kern, dim3 grid, dim3 block, size_t smem, Args&&... args) {
+    launch_as<false>(L, kern, grid, block, smem, std::forward<Args>(args)...);
+}
+// For kernels that read what the prologue wrote (lengths, block offsets, frame count, float16 weight copies) ahead of their
+// pdl_wait().  When such a kernel starts, everything up to the kernel before the previous one is complete (common.cuh), so the
+// read is safe exactly when another kernel lies between it and the prologue.  The launch sequences are arranged so that one
+// does (the depthwise step, a masked or packed copy of the input, the backward reduction); a launch that finds the prologue
+// directly ahead of it goes without the attribute and waits for it to complete.  Two further rules have no such guard:
+//   - the caller's parameters may be read early, because every call begins with the prologue;
+//   - whatever any other kernel of the call wrote (statistics, coefficients, activations) is read after the wait only.
+template <typename K, typename... Args>
+inline void launch_early(const Launch& L, K kern, dim3 grid, dim3 block, size_t smem, Args&&... args) {
+    launch_as<true>(L, kern, grid, block, smem, std::forward<Args>(args)...);
 }
 
 // Brackets the launches of one launcher call.  bytes/flops are the algorithmic figures of the call.

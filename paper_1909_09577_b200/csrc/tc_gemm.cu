@@ -675,7 +675,7 @@ tc_gemm_flat_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
         if (p.tma_out) ptx::prefetch_tensormap(&mapO);
     }
     if (warp == 0) { ptx::tmem_alloc(tmem_slot, TMEM_COLS); ptx::tmem_relinquish(); }
-    // Ahead of the wait for the previous kernel: the block offsets (the lengths were settled at least two kernels ago), and
+    // Ahead of the wait for the previous kernel: the block offsets (launch_early: the prologue is at least two kernels back), and
     // in the producer the first stages' weights.  Both latencies then overlap that kernel's last wave.
     for (int i = tid; i <= p.B; i += blockDim.x) s_off[i] = p.blk_off[i];
     ptx::tc_fence_before();
@@ -1103,7 +1103,7 @@ void launch(const Launch& L, dim3 grid, const CUtensorMap& a, const CUtensorMap&
     constexpr int smem = STAGES * (MT * 16384 + BN * 128) + 1024 + 256 + 4 * kStgFloatsPerWarp * 4;
     auto kern = tc_gemm_kernel<T, MODE, MT, BN, STAGES>;
     set_max_smem_once<tc_gemm_kernel<T, MODE, MT, BN, STAGES>>(smem);
-    launch_k(L, kern, grid, kThreads, smem, a, b, p);
+    launch_early(L, kern, grid, kThreads, smem, a, b, p);
     L.count();
 }
 
@@ -1203,7 +1203,7 @@ void launch_flat(const Launch& L, int sm_count, const CUtensorMap& a, const CUte
     set_max_smem_once<tc_gemm_flat_kernel<T, MODE, MT, NB, NBUF, OCC, EPI>>(OCC == 1 ? kSmemMax : Cfg::smem_bytes(Cfg::MAXB));
     const long long units = (long long)p.tiles_m * p.B * p.nbT;
     const int grid = (int)std::max(1ll, std::min<long long>(std::min(sm_count * OCC, kFlatMaxGrid), units));
-    launch_k(L, kern, grid, 32 * (4 * MT * EPI + 2), smem, a, b, o, p);
+    launch_early(L, kern, grid, 32 * (4 * MT * EPI + 2), smem, a, b, o, p);
     L.count();
     if (grid_out) *grid_out = grid;
 }
