@@ -208,6 +208,7 @@ void fork_to_side(sc_ctx* ctx, const Launch& L, cudaEvent_t ev) {
     if (!(ctx->overlap && ctx->side)) return;
     cudaEventRecord(ev, L.stream);
     cudaStreamWaitEvent(ctx->side, ev, 0);
+    ctx->fresh[1] = ctx->fresh[0];      // what is launched there next follows the last kernel of the caller's stream
 }
 void record_side(sc_ctx* ctx, cudaEvent_t ev) { if (ctx->overlap && ctx->side) cudaEventRecord(ev, ctx->side); }
 void wait_side(sc_ctx* ctx, const Launch& L, cudaEvent_t ev) { if (ctx->overlap && ctx->side) cudaStreamWaitEvent(L.stream, ev, 0); }

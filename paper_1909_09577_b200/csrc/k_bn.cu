@@ -1319,7 +1319,7 @@ void prologue(const Launch& L, Prologue& p) {
     }
     KScope ks_(L, KC_LENGTHS, bytes, 0.0);
     launch_k(L, prologue_kernel, 1 + blocks, kLenThreads, 0, p, L.status);
-    if (L.fresh) L.fresh[0] = L.fresh[1] = true;
+    if (L.fresh) L.fresh[L.lane] = true;
     L.count();
 }
 

@@ -33,7 +33,7 @@ struct Launch {
     Prof* prof = nullptr;
     int simt_only = 0;    // 1: never take a tensor-core kernel (used by tests)
     int pdl = 1;          // 1: launch with programmatic stream serialization (see pdl_sync in common.cuh)
-    bool* fresh = nullptr;   // per lane: no kernel has been launched there since the prologue (see launch_early)
+    bool* fresh = nullptr;   // per lane: the kernel that the next launch follows is the prologue (see launch_early)
     int lane = 0;            // 0: the caller's stream, 1: the context's second stream
     void count(int n = 1) const { if (counter) *counter += n; }
 };
