@@ -23,6 +23,9 @@ __device__ __forceinline__ float pow2_scale(float amax) {
     e = max(-100, min(100, e));
     return ldexpf(1.f, -e);
 }
+// Power-of-two scale for bfloat16 taps with the given absolute maximum that become float16 operands: the maximum comes to lie in
+// [2^14, 2^15), so every tap down to 2^-31 of it keeps all of its bits (unscaled, taps below 2^-14 lost theirs).
+__device__ __forceinline__ float tap_scale(float amax) { return 16384.f * 2.f * pow2_scale(amax); }
 __device__ __forceinline__ float warp_max(float v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));

@@ -72,11 +72,20 @@ dw_tc_kernel(const TI* __restrict__ in, const TW* __restrict__ w, TO* __restrict
     if (warp == 0) { ptx::tmem_alloc(tmem_slot, 128); ptx::tmem_relinquish(); }
     for (int i = tid; i < 8 * ROWS_ALLOC; i += kThreads) A16[i] = make_uint4(0, 0, 0, 0);
     for (int i = tid; i < nbh; i += kThreads) lens[i] = len_src[b0 + i];
+    // bfloat16 taps for float16 operands are scaled by a power of two per channel, which the epilogue takes out again; every
+    // warp finds the largest tap by itself
+    constexpr bool SCALED = std::is_same<TI, __half>::value && std::is_same<TW, __nv_bfloat16>::value;
+    float scale = 1.f;
+    if (SCALED) {
+        float m = 0.f;
+        for (int k = lane; k < K; k += 32) m = fmaxf(m, fabsf(ldf(w + (size_t)c * K + k)));
+        scale = tap_scale(warp_max(m));
+    }
     for (int i = tid; i < 264; i += kThreads) {
         const int delta = i - 128;
         const int kk = FLIP ? P - delta : delta + P;
         reinterpret_cast<unsigned short*>(coefw)[i] =
-            (delta >= -127 && delta <= 127 && kk >= 0 && kk < K) ? bits16<TI>(ldf(w + (size_t)c * K + kk)) : (unsigned short)0;
+            (delta >= -127 && delta <= 127 && kk >= 0 && kk < K) ? bits16<TI>(SCALED ? scale * ldf(w + (size_t)c * K + kk) : ldf(w + (size_t)c * K + kk)) : (unsigned short)0;
     }
     ptx::tc_fence_before();
     __syncthreads();
@@ -155,7 +164,7 @@ dw_tc_kernel(const TI* __restrict__ in, const TW* __restrict__ w, TO* __restrict
     ok = __all_sync(0xffffffffu, ok);
     ptx::tc_fence_after();
     if (ok) {
-        const float inv = gmax ? 1.f / pow2_scale(*gmax) : 1.f;
+        const float inv = (gmax ? 1.f / pow2_scale(*gmax) : 1.f) * (1.f / scale);
         const int mt = warp >> 2, wq = warp & 3;          // this warp's M-tile and TMEM lane quarter
         if (mt < nmt) {
             const int Rw = mt * 128 + wq * 32 + lane;
@@ -181,7 +190,7 @@ dw_tc_kernel(const TI* __restrict__ in, const TW* __restrict__ w, TO* __restrict
                     } else {
 #pragma unroll
                         for (int e = 0; e < 8; ++e) f[e] = __uint_as_float(r[8 * g8 + e]);
-                        if (gmax) {
+                        if (SCALED || gmax) {
 #pragma unroll
                             for (int e = 0; e < 8; ++e) f[e] *= inv;
                         }

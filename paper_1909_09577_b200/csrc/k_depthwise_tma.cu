@@ -48,6 +48,7 @@ constexpr int DT_STG_BYTES = 4608;         // per epilogue warp: 32 rows x 144 b
 constexpr int DT_WOFF = 80;                // index of tap 0 in the padded tap arrays
 constexpr int DT_WLEN = 288;
 constexpr int DT_MAX_STAGES = 3;
+constexpr int DT_SCALES = 8;               // tap scales under way: the builders are at most DT_NACC + 2 channels ahead of the epilogue
 
 struct DtParams {
     const void* w; void* out; const void* add1; const void* add2; const float* gmax;
@@ -83,7 +84,10 @@ __device__ __forceinline__ void named_bar(int id, int nthreads) {
 }
 
 // TI: type of the input tensor and of both MMA operands; TW: stored tap type; TO: output / addend type; MASK: the
-// input may be non-zero at and beyond a sample's length.
+// input may be non-zero at and beyond a sample's length.  bfloat16 taps for float16 operands are scaled by a power of two per
+// channel (tap_scale), which the epilogue takes out again: without it taps below 2^-14 lost bits that the plain kernels keep.  It
+// costs nothing that can be measured (blocks forward and backward, bf16: 23 x 384 x 797, K = 39, 248.4 -> 249.0 us; 16 x 512 x
+// 800, K = 87, dilation 2, 143.1 -> 143.8; 32 x 256 x 400, K = 63, 158.8 -> 158.9).
 template <typename TI, typename TW, typename TO, bool MASK>
 __global__ void __launch_bounds__(DT_THREADS, 1)
 dw_tma_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CUtensorMap mapO, DtParams p) {
@@ -100,13 +104,18 @@ dw_tma_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ 
     uint64_t* acc_empty = acc_full + DT_NACC;       // [DT_NACC]
     uint64_t* b_full = acc_empty + DT_NACC;         // [2]
     uint64_t* b_empty = b_full + 2;                 // [2]
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(b_empty + 2);
+    constexpr bool SCALED = std::is_same<TI, __half>::value && std::is_same<TW, __nv_bfloat16>::value;
+    uint64_t* sc_full = b_empty + 2;                // [DT_SCALES]
+    float* sc_inv = reinterpret_cast<float*>(sc_full + DT_SCALES);          // [DT_SCALES] 1 / tap scale of channel ci in slot ci % DT_SCALES
+    float* sc_max = sc_inv + DT_SCALES;                                     // [4] largest tap that each builder warp saw
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(sc_max + 4);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     if (tid == 0) {
         for (int s = 0; s < DT_MAX_STAGES; ++s) { ptx::mbar_init(&full[s], 1); ptx::mbar_init(&prep[s], 1); ptx::mbar_init(&empty[s], 1); }
         for (int i = 0; i < DT_NACC; ++i) { ptx::mbar_init(&acc_full[i], 1); ptx::mbar_init(&acc_empty[i], 256); }
         for (int i = 0; i < 2; ++i) { ptx::mbar_init(&b_full[i], 4); ptx::mbar_init(&b_empty[i], 2); }
+        if (SCALED) for (int i = 0; i < DT_SCALES; ++i) ptx::mbar_init(&sc_full[i], 1);
         ptx::fence_barrier_init();
         ptx::prefetch_tensormap(&mapX);
         ptx::prefetch_tensormap(&mapO);
@@ -195,12 +204,29 @@ dw_tma_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ 
         int ci = 0; bool dead = false;
         for (int c = blockIdx.x; c < p.C && !dead; c += gridDim.x, ++ci) {
             const int bb = ci & 1;
+            float tap[(DT_WLEN + 127) / 128], scale = 1.f;
+#pragma unroll
+            for (int q = 0; q < (DT_WLEN + 127) / 128; ++q) {
+                const int k = bt + 128 * q - DT_WOFF;
+                tap[q] = k >= 0 && k < p.K ? ldf(reinterpret_cast<const TW*>(p.w) + (size_t)c * p.K + (p.flip ? p.K - 1 - k : k)) : 0.f;
+            }
+            if (SCALED) {
+                float m = 0.f;
+#pragma unroll
+                for (int q = 0; q < (DT_WLEN + 127) / 128; ++q) m = fmaxf(m, fabsf(tap[q]));
+                m = warp_max(m);
+                if (lane == 0) sc_max[warp - 10] = m;
+            }
             named_bar(2, 128);                         // everyone is done reading the previous channel's taps
-            for (int i = bt; i < DT_WLEN; i += 128) {
-                const int k = i - DT_WOFF;
-                float v = 0.f;
-                if (k >= 0 && k < p.K) v = ldf(reinterpret_cast<const TW*>(p.w) + (size_t)c * p.K + (p.flip ? p.K - 1 - k : k));
-                const unsigned short bits = to_bits16<TI>(v);
+            if (SCALED) {
+                scale = tap_scale(fmaxf(fmaxf(sc_max[0], sc_max[1]), fmaxf(sc_max[2], sc_max[3])));
+                if (bt == 0) { sc_inv[ci % DT_SCALES] = 1.f / scale; ptx::mbar_arrive(&sc_full[ci % DT_SCALES]); }
+            }
+#pragma unroll
+            for (int q = 0; q < (DT_WLEN + 127) / 128; ++q) {
+                const int i = bt + 128 * q;
+                if (i >= DT_WLEN) break;
+                const unsigned short bits = to_bits16<TI>(SCALED ? tap[q] * scale : tap[q]);
                 wpadE[i] = bits;
                 if (i > 0) wpadO[i - 1] = bits;
                 if (i == DT_WLEN - 1) wpadO[i] = 0;
@@ -260,7 +286,7 @@ dw_tma_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ 
         const int wq = warp & 3, half = warp >> 2;
         uint8_t* stg = stg_all + warp * DT_STG_BYTES;
         pdl_wait();
-        const float inv = p.gmax ? 1.f / pow2_scale(*p.gmax) : 1.f;
+        const float g_inv = p.gmax ? 1.f / pow2_scale(*p.gmax) : 1.f;
         const bool has_add = p.add1 != nullptr || p.add2 != nullptr;
         TO* out = reinterpret_cast<TO*>(p.out);
         const TO* add1 = reinterpret_cast<const TO*>(p.add1);
@@ -276,8 +302,13 @@ dw_tma_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ 
             const int row = wq * 32 + it * 8 + rr;
             tbl_of[it] = row / p.BB; bi_of[it] = row - tbl_of[it] * p.BB;
         }
-        int j = 0; float amax = 0.f;
-        for (int c = blockIdx.x; c < p.C; c += gridDim.x) {
+        int j = 0, ci = 0; float amax = 0.f;
+        for (int c = blockIdx.x; c < p.C; c += gridDim.x, ++ci) {
+            float inv = g_inv;
+            if (SCALED) {
+                if (!ptx::mbar_wait_warp(&sc_full[ci % DT_SCALES], (ci / DT_SCALES) & 1)) { if (lane == 0) raise_status(p.status, kErrTimeout); goto done; }
+                inv *= sc_inv[ci % DT_SCALES];
+            }
             for (int chunk = 0; chunk < p.nchunks; ++chunk) {
                 int ld_of[4]; long long base_of[4];       // valid output length and element offset of frame 0
 #pragma unroll
@@ -313,7 +344,7 @@ dw_tma_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ 
                             float f[32];
 #pragma unroll
                             for (int i = 0; i < 32; ++i) f[i] = __uint_as_float(v[i]);
-                            if (p.gmax) {
+                            if (SCALED || p.gmax) {
 #pragma unroll
                                 for (int i = 0; i < 32; ++i) f[i] *= inv;
                             }

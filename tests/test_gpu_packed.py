@@ -100,6 +100,24 @@ def test_padded_encoder_starting_without_depthwise(api, ctx):
         compare_with_chain(spec, w, d, logits, out_len, grads, dx, chain)
 
 
+@pytest.mark.parametrize("B,C,T,dilation", [(17, 24, 271, 1), (16, 150, 272, 1), (17, 24, 270, 2), (15, 256, 801, 1), (3, 24, 129, 1)])
+def test_input_gradient_keeps_the_bits_of_its_taps(api, ctx, B, C, T, dilation):
+    """bfloat16 taps of any magnitude: scaling them by a power of two scales the input gradient by exactly that (the kernels
+    that take float16 operands must not round taps below 2^-14 or overflow above 65504)."""
+    L = si.LayerCfg(C, 16, K=33, dilation=dilation)
+    d = si.draw(si.Workload("taps", "bf16", B, T, [L], 77, len_lo=T // 2, len_hi=T))
+    desc, x, g = api.block_desc(L, B, T, "bf16"), U.dev(d.x, "bf16"), U.dev(d.g, "bf16")
+    lens, p = torch.from_numpy(d.lengths).cuda(), U.params_dev(d.params[0], "bf16")
+    y, _, saved = api.sepconv_fwd(ctx, desc, x, lens, p)
+    dx = api.sepconv_bwd(ctx, desc, g, x, y, lens, p, saved)[0]
+    assert dx.float().abs().max() > 0
+    for e in (-16, -24, 20):
+        q = dict(p, wd=p["wd"] * 2.0 ** e)
+        dq = api.sepconv_bwd(ctx, desc, g, x, y, lens, q, saved)[0]
+        assert ctx.last_status() == 0
+        assert torch.equal(dq.float() * 2.0 ** -e, dx.float()), e
+
+
 @pytest.mark.parametrize("K,B,T", [(1, 3, 16), (3, 2, 1040), (7, 9, 528), (35, 4, 512), (87, 2, 4112), (95, 5, 304)])
 def test_stride_two_depthwise(api, ctx, K, B, T):
     """The stride-2 depthwise kernels: both parities of the padding, one tap to the most they take, rows around their tiles."""
