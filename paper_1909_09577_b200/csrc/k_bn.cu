@@ -523,6 +523,7 @@ __device__ __forceinline__ void bwd_channel(const BnBwdArgs& a, const BwdGrads& 
 // load issued before the first add) and the thirty-two warp results are combined in warp order
 // (bit-repeatable).
 constexpr int kBwdMaxSlotsUnrolled = 8;
+constexpr int kRedV = 2, kRedVectors = 32 * kRedV;       // vectors per lane and per warp of the flattened reduction
 __global__ void __launch_bounds__(32 * kFinWarps)
 bn_bwd_finalize_kernel(BnBwdArgs a, BwdGrads p) {
     pdl_sync();
@@ -538,7 +539,7 @@ bn_bwd_finalize_kernel(BnBwdArgs a, BwdGrads p) {
             int used = 1;
             if (a.nslots > 1) {      // slots in use for this row (see bn_bwd_reduce_fast_kernel); r * vpr < 2^31
                 const uint32_t r = (uint32_t)b * (uint32_t)a.C + (uint32_t)o;
-                used = (int)((((r + 1u) * vpr - 1u) >> a.vpw_shift) - ((r * vpr) >> a.vpw_shift)) + 1;
+                used = (int)(((r + 1u) * vpr - 1u) / kRedVectors - (r * vpr) / kRedVectors) + 1;
             }
             for (int sl0 = 0; sl0 < used; sl0 += kBwdMaxSlotsUnrolled) {
                 float4 pv[kBwdMaxSlotsUnrolled]; float am[kBwdMaxSlotsUnrolled];
@@ -1048,13 +1049,14 @@ __global__ void __launch_bounds__(256) bn_bwd_apply_fast_kernel(BnBwdArgs a, int
     }
 }
 
-// Flattened reduce: a warp's 32 * V consecutive vectors belong to at most two rows (vpr >= 32 * V), so two
+// Flattened reduce: a warp's kRedVectors consecutive vectors belong to at most two rows (vpr >= kRedVectors), so two
 // masked warp reductions give one partial per (row, warp) pair.  Row r's partials sit in slots
-// [0, last_warp(r) - first_warp(r)] with first_warp(r) = (r * vpr) / (32 * V): a static assignment,
+// [0, last_warp(r) - first_warp(r)] with first_warp(r) = (r * vpr) / kRedVectors: a static assignment,
 // summed later in slot order.
-template <typename T, typename NT, int RES, int V>
+template <typename T, typename NT, int RES>
 __global__ void __launch_bounds__(256) bn_bwd_reduce_fast_kernel(BnBwdArgs a, int vpr, long long total) {
     pdl_sync();
+    constexpr int V = kRedV;
     const uint32_t tid = blockIdx.x * 256u + threadIdx.x;        // the launcher guarantees total < 2^31
     const int lane = threadIdx.x & 31;
     const uint32_t wg = tid >> 5;                                // global warp index
@@ -1363,10 +1365,19 @@ static bool fits32(int B, int C, int Tp) { return (long long)B * C * (Tp / 8) < 
 static unsigned fast_grid(long long total, int V) { return (unsigned)((total + 256ll * V - 1) / (256ll * V)); }
 
 // Algorithmic bytes per element of the batch-norm kernels: every tensor they must read or write, once.
-// The channel-per-CTA reduction: one launch instead of two, so small tensors take it at any width (a block forward and
-// backward with 40 to 2000 vectors per channel: 2.5-7 % faster than with the row-mapped kernel and its finalize step); longer
-// channels only where there are enough of them to fill the SMs.
-static bool channel_mapped(int B, int C, int Tp) { return C >= 32 || (long long)B * (Tp / 8) <= 1024; }
+// The channel-per-CTA reduction: one launch instead of two, which wins unless the tensor is large and its channels are too few
+// for their CTAs (two per SM) to stream as fast as the flattened kernel does on all SMs.  Blocks forward and backward without a
+// depthwise step, bf16: time with the flattened kernel and its finalize step over time with this one,
+//   at any width up to 4096 vectors per channel                          1.00-1.08 (identity residual, rows of 1600: 0.97-1.03)
+//   rows of 2048 frames and more: 8 to 24 channels, 8192 / 32768 vectors 0.96-0.98 / 0.90-0.94
+//                                 32 channels                            0.99 / 0.95      (identity, 8192: 0.92)
+//                                 64 channels                            1.01 / 0.99      (identity, 8192: 0.94)
+//                                 96 channels and more                   1.03-1.09        (identity, rows of 1600: 0.97-1.02)
+//   16 to 48 channels, 8192 and 16384 vectors: rows of 512 frames        1.04-1.09
+//                                              rows of 1024              0.98-1.04
+//   rows of 128 and 256 frames, 2048 to 16384 vectors                    0.97-1.21, below 1 only in 8 channels of 128 frames
+static bool channel_mapped(int B, int C, int Tp) { return C >= 64 || Tp < 2048 || (long long)B * (Tp / 8) <= 4096; }
+static_assert(2048 / 8 >= kRedVectors, "a warp of the flattened reduction meets at most two rows");
 
 void bn_apply(const Launch& L, int dtype, const ApplyArgs& a_in) {
     ApplyArgs a = a_in;
@@ -1417,20 +1428,16 @@ void bn_apply_flat(const Launch& L, int dtype, const ApplyArgs& a_in, const Flat
 }
 
 static void bn_bwd_reduce(const Launch& L, int dtype, BnBwdArgs& a) {
-    a.nslots = 1; a.vpw = 32; a.vpw_shift = 5;
+    a.nslots = 1;
     const double e = (double)dtype_size(dtype), en = (double)dtype_size(ntype_of(dtype));
-    if (dtype != F32 && a.Tp % 8 == 0 && a.Tp >= 256 && a.has_bn && a.has_relu && a.res_before_relu && fits32(a.B, a.C, a.Tp)) {
+    if (dtype != F32 && a.Tp % 8 == 0 && a.has_bn && a.has_relu && a.res_before_relu && fits32(a.B, a.C, a.Tp)) {
         a.dvpr = FastDiv((uint32_t)(a.Tp / 8)); a.dC = FastDiv((uint32_t)a.C);
         KScope ks2_(L, KC_BN_BWD_REDUCE, (double)a.B * a.C * a.Tp * (e * (a.residual == 0 ? 1 : 2) + en * (a.residual == 2 ? 2 : 1)), 0.0);
         const int vpr = a.Tp / 8;
         a.nslots = bn_bwd_max_slots(a.Tp);
         const long long total = (long long)a.B * a.C * vpr;
-        const int V = vpr >= 64 ? 2 : 1;
-        a.vpw = 32 * V; a.vpw_shift = V == 2 ? 6 : 5;
-        const unsigned grid = fast_grid(total, V);
-#define SC_RED_FAST(RES)                                                                                                   \
-        if (V == 2) { SC_DISPATCH16(dtype, (launch_k(L, bn_bwd_reduce_fast_kernel<T, NT, RES, 2>, grid, 256, 0, a, vpr, total))); } \
-        else { SC_DISPATCH16(dtype, (launch_k(L, bn_bwd_reduce_fast_kernel<T, NT, RES, 1>, grid, 256, 0, a, vpr, total))); }
+        const unsigned grid = fast_grid(total, kRedV);
+#define SC_RED_FAST(RES) SC_DISPATCH16(dtype, (launch_k(L, bn_bwd_reduce_fast_kernel<T, NT, RES>, grid, 256, 0, a, vpr, total)))
         if (a.residual == 2) { SC_RED_FAST(2); } else if (a.residual == 1) { SC_RED_FAST(1); } else { SC_RED_FAST(0); }
 #undef SC_RED_FAST
         L.count();
@@ -1453,7 +1460,7 @@ static void bn_bwd_reduce_finalize(const Launch& L, int dtype, BnBwdArgs& a, con
                             float* dgamma, float* dbeta, float* dgamma_r, float* dbeta_r, float* dbias, int accumulate) {
     const bool fast = dtype != F32 && a.Tp % 8 == 0 && a.has_bn && a.has_relu && a.res_before_relu && fits32(a.B, a.C, a.Tp);
     if (a.phases || (fast && channel_mapped(a.B, a.C, a.Tp))) {
-        a.nslots = 1; a.vpw = 32; a.vpw_shift = 5;
+        a.nslots = 1;
         const double e = (double)dtype_size(dtype), en = (double)dtype_size(ntype_of(dtype));
         KScope ks_(L, KC_BN_BWD_REDUCE, (double)a.B * a.C * a.Tp * (e * (a.residual == 0 ? 1 : 2) + en * (a.residual == 2 ? 2 : 1)), 0.0);
         const int vpr = a.Tp / 8;

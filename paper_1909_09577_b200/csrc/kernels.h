@@ -316,7 +316,6 @@ struct BnBwdArgs {
     float4* partials;                              // [B*C*nslots]
     float* amax_part;                              // [B*C*nslots] max |gated gradient| (only with gmax)
     int nslots;                                    // partial slots per (sample, channel) row; set by bn_bwd_reduce
-    int vpw, vpw_shift;                            // 8-frame vectors per warp of the flattened reduce (a power of two) and its log2; set by bn_bwd_reduce
     float* gmax;                                   // device scalar: bound on |gv| over the tensor (nullable)
     int gv_dtype;                                  // storage type of gv (OT)
     float4* coef; float4* coef_r;                  // [C]: (k, c1, c2, unused)

@@ -15,6 +15,12 @@ CASES = [
     (dict(C_in=16, C_out=304, K=9, residual="proj"), 4, 264, 1),                  # too many channels
     (dict(C_in=16, C_out=24, K=11), 5, 1640, 300),                                # 1025 vectors
     (dict(C_in=64, C_out=136, K=5, has_dw=False, full_conv=True), 3, 264, 20),
+    # the row-mapped reduction: few channels with more than 4096 vectors, in its shortest rows and in rows that end inside a warp
+    (dict(C_in=8, C_out=16, K=5), 17, 2048, 100),
+    (dict(C_in=16, C_out=63, K=5, residual="proj"), 16, 2056, 900),
+    (dict(C_in=24, C_out=24, K=5, residual="identity"), 9, 3648, 1200),
+    (dict(C_in=8, C_out=8, K=3), 16, 2048, 700),                                  # 4096 vectors: not yet
+    (dict(C_in=8, C_out=8, K=3), 17, 2040, 100),                                  # rows too short for it
 ]
 
 
