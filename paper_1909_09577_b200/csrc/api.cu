@@ -177,7 +177,7 @@ void finalize_stats(const Launch& L, const sc_block_desc* d, const Dims& m, Stat
 }
 
 bool apply_takes_stats(int dt, const ApplyArgs& a, const StatsLayout& sl) {
-    return sl.kind == 2 ? bn_apply_takes_stats(dt, a) : sl.kind == 0 && bn_small(dt, a.B, a.Tp);
+    return sl.kind == 2 ? bn_apply_takes_stats(dt, a) : sl.kind == 0 && bn_small(dt, a.B, a.C, a.Tp);
 }
 
 // v = w * u for every sample (stored once, in the type it is kept in for the backward pass), plus masked

@@ -332,12 +332,23 @@ __global__ void __launch_bounds__(kRowThreads) bn_apply_kernel(ApplyArgs a) {
 }
 
 // ---- one CTA per channel of a small float32 tensor ---------------------------------------------------------
-// A channel of up to kSmallChunks eight-frame chunks: what is left of the three steps (row partials, finalize, apply; in
-// the backward pass too) is the latency of their launches, about 2.2 us each in a chain of dependent kernels.  One CTA
-// sees the whole channel and does all three; the second and third reading of its rows hit the L1 cache.  Above the limit
-// the row-mapped kernels have more CTAs than there are channels and win.  A block forward and backward: 64 channels of
-// 2 x 128 frames 35.9 -> 29.7 us, 128 channels of 7 x 228 frames 75.6 -> 69.7 us.
-constexpr int kSmallChunks = 1024;
+// In a channel of few eight-frame chunks, what is left of the three steps (row partials, finalize, apply; in the backward
+// pass too) is the latency of their launches, about 2.2 us each in a chain of dependent kernels.  One CTA sees the whole
+// channel and does all three; the second and third reading of its rows hit the L1 cache.  A block forward and backward:
+// 64 channels of 2 x 128 frames 35.9 -> 29.7 us, 128 channels of 7 x 228 frames 75.6 -> 69.7 us.  Against it stand the three
+// passes of one CTA where the row-mapped kernels give every (sample, channel) row a warp, and rows that are no whole number
+// of chunks, whose elements are loaded one by one in each pass.  Time with the row-mapped kernels over time with this one, 32 to
+// 512 channels (blocks without a depthwise step):
+//                   chunks   64-256       512          1024         2048
+//   whole chunks,  2 samples 1.15-1.44    1.18-1.58    1.14-1.65    1.26-1.70     (256 channels, identity residual: 0.90-1.08)
+//                  8 samples 0.95-1.28    1.03-1.19    1.02-1.12    1.01-1.03
+//                 32 samples 1.11-1.57    1.04-1.22    0.99-1.05    0.91-1.00
+//   other rows (up to 256 channels),
+//                  4 samples 0.93-1.41    1.03-1.32    1.04-1.38    1.05-1.40
+//                  8 samples 0.97-1.36    1.00-1.19    0.94-1.10    0.96-0.99     (512 channels, 64 / 128 / 256 chunks: 1.23 / 1.02 / 0.87)
+//                 16 samples 0.98-1.36    0.89-1.01    0.85-0.98    0.83-0.98     (512 channels: 1.40 / 0.88 / 0.83)
+//                 32 samples 1.00-1.33    0.86-1.05    0.84-0.97    0.77-0.88     (512 channels: 1.30 / 1.15 / 1.12)
+constexpr int kSmallChunks = 1024, kSmallOddChunks = 256, kSmallOddWork = 256 * 256, kSmallOddSamples = 4;
 struct ChanRows {            // chunk j of the channel -> sample and frame
     int cpr, n;
     __device__ __forceinline__ ChanRows(int B, int Tp) : cpr((Tp + 7) >> 3), n(B * ((Tp + 7) >> 3)) {}
@@ -1351,7 +1362,11 @@ void bn_finalize_flat(const Launch& L, const float4* partials, int grid, int til
     L.count();
 }
 
-bool bn_small(int dtype, int B, int Tp) { return dtype == F32 && (long long)B * ((Tp + 7) / 8) <= kSmallChunks; }
+bool bn_small(int dtype, int B, int C, int Tp) {
+    const long long chunks = (long long)B * ((Tp + 7) / 8);
+    return dtype == F32 && chunks <= kSmallChunks &&
+           (Tp % 8 == 0 || B <= kSmallOddSamples || (chunks <= kSmallOddChunks && chunks * C <= kSmallOddWork));
+}
 
 void bn_small_fwd(const Launch& L, const ApplyArgs& a, const int* nvalid, float eps, float momentum, float* mean, float* invstd,
                   float* running_mean, float* running_var) {
@@ -1508,7 +1523,7 @@ static void bn_bwd_apply(const Launch& L, int dtype, const BnBwdArgs& a_in) {
 
 void bn_bwd(const Launch& L, int dtype, BnBwdArgs& a, const float* gamma, const float* gamma_r, float* dgamma, float* dbeta,
             float* dgamma_r, float* dbeta_r, float* dbias, int accumulate) {
-    if (bn_small(dtype, a.B, a.Tp)) {
+    if (bn_small(dtype, a.B, a.C, a.Tp)) {
         KScope ks_(L, KC_BN_BWD_APPLY, 4.0 * a.B * a.C * a.Tp * (a.residual ? 5 : 4), 0.0);
         launch_k(L, bn_small_bwd_kernel, (unsigned)a.C, kRowThreads, 0, a, BwdGrads{gamma, gamma_r, dgamma, dbeta, dgamma_r, dbeta_r, dbias, accumulate});
         L.count();

@@ -302,7 +302,7 @@ struct FlatStats {
 bool bn_apply_takes_stats(int dtype, const ApplyArgs& a);
 void bn_apply_flat(const Launch& L, int dtype, const ApplyArgs& a, const FlatStats& f);
 // Statistics of v and the apply step in one kernel, for the float32 tensors that bn_small accepts.
-bool bn_small(int dtype, int B, int Tp);
+bool bn_small(int dtype, int B, int C, int Tp);
 void bn_small_fwd(const Launch& L, const ApplyArgs& a, const int* nvalid, float eps, float momentum, float* mean, float* invstd,
                   float* running_mean, float* running_var);
 
