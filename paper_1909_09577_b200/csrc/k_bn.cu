@@ -908,8 +908,9 @@ __global__ void __launch_bounds__(256) bn_apply_fast_kernel(ApplyArgs a, int vpr
     }
 }
 
-// The same step from packed v / vr to dense y: a thread takes V aligned 8-element vectors of the dense tensor and gathers
-// the packed operands.  A vector that runs over the end of a row (of at least 8 frames) is spliced from this row's last
+// The same step from packed v / vr to dense y: a thread takes one aligned 8-element vector of the dense tensor and gathers the
+// packed operands (two vectors per thread took 30.0 us where one takes 26.1, bf16, 23 x 384 x 797, projected residual: registers
+// against warps in flight).  A vector that runs over the end of a row (of at least 8 frames) is spliced from this row's last
 // frames and the next row's first; shorter rows are done element by element.  Blocks past the tensor's own copy u out.
 // What it replaces: four extra passes (v, vr, y and u copied to dense form one after the other) and their launches.
 template <typename T, typename NT, int RES, int D>
@@ -919,84 +920,67 @@ __global__ void __launch_bounds__(256) bn_apply_unpack_kernel(ApplyArgs a, uint3
     const uint32_t tot = copy ? total_u : total;
     const uint32_t tot_packed = (uint32_t)a.B * D * C * a.Tp;
     const bool aligned = (a.T & 7) == 0, vector_rows = a.T >= 8;
-    // one vector per thread: with two, 30.0 us where this takes 26.1 (bf16, 23 x 384 x 797, projected residual): registers
-    // against warps in flight
-    constexpr int V = 1;
-    const uint32_t tid = (blockIdx.x - (copy ? nblk_apply : 0)) * 256u + threadIdx.x;
-    const uint32_t base = ((tid >> 5) * (32u * V) + (threadIdx.x & 31)) * 8u;
-    int row[V], t[V], b[V], ch[V], n[V];
-#pragma unroll
-    for (int j = 0; j < V; ++j) {
-        const uint32_t f = base + 256u * j;
-        row[j] = t[j] = b[j] = ch[j] = n[j] = 0;
-        if (f < tot) {
-            row[j] = (int)a.dT.div(f); t[j] = (int)(f - (uint32_t)row[j] * a.T);
-            b[j] = row[j] / C; ch[j] = row[j] - b[j] * C;
-            n[j] = min(a.len_out[b[j]], a.T) - t[j];
-        }
+    const uint32_t f = ((blockIdx.x - (copy ? nblk_apply : 0)) * 256u + threadIdx.x) * 8u;      // first element
+    int row = 0, t = 0, b = 0, ch = 0, n = 0;
+    if (f < tot) {
+        row = (int)a.dT.div(f); t = (int)(f - (uint32_t)row * a.T);
+        b = row / C; ch = row - b * C;
+        n = min(a.len_out[b], a.T) - t;
     }
-    pdl_sync();
-    Packed8<D> rv[V], rr[V]; uint4 rx[V];
-#pragma unroll
-    for (int j = 0; j < V; ++j) {
-        rx[j] = make_uint4(0, 0, 0, 0);
-        if (vector_rows && n[j] > 0) {
-            rv[j] = Packed8<D>(copy ? a.u : a.v, b[j], ch[j], C, a.Tp, t[j], tot_packed, aligned);
-            if (RES == 2 && !copy) rr[j] = Packed8<D>(a.vr, b[j], ch[j], C, a.Tp, t[j], tot_packed, aligned);
+    pdl_sync();              // the lengths above: launch_early
+    if (f >= tot) return;
+    const int left = (int)min(8u, tot - f);
+    if (vector_rows) {
+        Packed8<D> rv, rr; uint4 rx = make_uint4(0, 0, 0, 0);
+        if (n > 0) {
+            rv = Packed8<D>(copy ? a.u : a.v, b, ch, C, a.Tp, t, tot_packed, aligned);
+            if (RES == 2 && !copy) rr = Packed8<D>(a.vr, b, ch, C, a.Tp, t, tot_packed, aligned);
         }
         // the dense operand is aligned like the result (the last vector may hold less than eight elements)
-        if (RES == 1 && !copy && vector_rows && base + 256u * j < tot) rx[j] = fetch<1>(a.xres, base + 256u * j, tot).v[0];
-    }
-#pragma unroll
-    for (int j = 0; j < V; ++j) {
-        const uint32_t f = base + 256u * j;
-        if (f >= tot) continue;
-        const int left = (int)min(8u, tot - f);
-        if (vector_rows) {
-            uint4 q = rv[j].get(), qr = RES == 1 ? rx[j] : (RES == 2 ? rr[j].get() : rx[j]), y = make_uint4(0, 0, 0, 0);
+        if (RES == 1 && !copy) rx = fetch<1>(a.xres, f, tot).v[0];
+        uint4 q = rv.get(), qr = RES == 2 ? rr.get() : rx, y = make_uint4(0, 0, 0, 0);
+        if (!copy) {
+            FwdChan c{};
+            fwd_chan<RES>(a, ch, c);
+            apply_core<T, NT, RES>((T*)&y, n, q, qr, c);
+        } else if (n < 8) q = keep_first(q, n);
+        const int k = a.T - t;                                 // elements of this row
+        if (k < 8 && row + 1 < nrows) {
+            const int b2 = (row + 1) / C, c2 = row + 1 - b2 * C, n2 = min(a.len_out[b2], a.T) + k;
+            uint4 p = Packed8<D>(copy ? a.u : a.v, b2, c2, C, a.Tp, -k, tot_packed, false).get(), pr = rx, y2;
+            if (RES == 2 && !copy) pr = Packed8<D>(a.vr, b2, c2, C, a.Tp, -k, tot_packed, false).get();
             if (!copy) {
                 FwdChan c{};
-                fwd_chan<RES>(a, ch[j], c);
-                apply_core<T, NT, RES>((T*)&y, n[j], q, qr, c);
-            } else if (n[j] < 8) q = keep_first(q, n[j]);
-            const int k = a.T - t[j];                          // elements of this row
-            if (k < 8 && row[j] + 1 < nrows) {
-                const int b2 = (row[j] + 1) / C, c2 = row[j] + 1 - b2 * C, n2 = min(a.len_out[b2], a.T) + k;
-                uint4 p = Packed8<D>(copy ? a.u : a.v, b2, c2, C, a.Tp, -k, tot_packed, false).get(), pr = rx[j], y2;
-                if (RES == 2 && !copy) pr = Packed8<D>(a.vr, b2, c2, C, a.Tp, -k, tot_packed, false).get();
-                if (!copy) {
-                    FwdChan c{};
-                    fwd_chan<RES>(a, c2, c);
-                    apply_core<T, NT, RES>((T*)&y2, n2, p, pr, c);
-                    y = splice(y, y2, k);
-                } else if (n2 < 8) p = keep_first(p, n2);
-                q = splice(q, p, k);
-                if (RES == 2) qr = splice(qr, pr, k);
-            }
-            if (copy) { st8_first((unsigned short*)a.u_out + f, q, left); continue; }
-            st8_first((unsigned short*)a.y + f, y, left);
-            if (a.v_out) st8_first((unsigned short*)a.v_out + f, q, left);
-            if (RES == 2 && a.vr_out) st8_first((unsigned short*)a.vr_out + f, qr, left);
-            continue;
+                fwd_chan<RES>(a, c2, c);
+                apply_core<T, NT, RES>((T*)&y2, n2, p, pr, c);
+                y = splice(y, y2, k);
+            } else if (n2 < 8) p = keep_first(p, n2);
+            q = splice(q, p, k);
+            if (RES == 2) qr = splice(qr, pr, k);
         }
-        for (uint32_t e = f; e < f + left; ++e) {
-            const int row_e = (int)a.dT.div(e), te = (int)(e - (uint32_t)row_e * a.T);
-            const int be = row_e / C, o = row_e - be * C;
-            const bool in = te < min(a.len_out[be], a.T);
-            const uint32_t q = D == 1 ? (uint32_t)row_e * a.Tp + te : ((uint32_t)(be * 2 + (te & 1)) * C + o) * a.Tp + (te >> 1);
-            if (copy) { ((unsigned short*)a.u_out)[e] = in ? ((const unsigned short*)a.u)[q] : (unsigned short)0; continue; }
-            const NT vq = in ? ((const NT*)a.v)[q] : NT(0.f);
-            float r = 0.f;
-            if (RES == 1 && in) r = ldf((const T*)a.xres + e);
-            if (RES == 2) {
-                const NT vrq = in ? ((const NT*)a.vr)[q] : NT(0.f);
-                r = fmaf(a.gamma_r[o], bn_norm(ldf(&vrq), a.mean_r[o], a.invstd_r[o]), a.beta_r[o]);
-                if (a.vr_out) ((NT*)a.vr_out)[e] = vrq;
-            }
-            const float y = fmaxf(fmaf(a.gamma[o], bn_norm(ldf(&vq), a.mean[o], a.invstd[o]), a.beta[o]) + r, 0.f);
-            stf((T*)a.y + e, in ? y : 0.f);
-            if (a.v_out) ((NT*)a.v_out)[e] = vq;
+        if (copy) { st8_first((unsigned short*)a.u_out + f, q, left); return; }
+        st8_first((unsigned short*)a.y + f, y, left);
+        if (a.v_out) st8_first((unsigned short*)a.v_out + f, q, left);
+        if (RES == 2 && a.vr_out) st8_first((unsigned short*)a.vr_out + f, qr, left);
+        return;
+    }
+    for (uint32_t e = f; e < f + left; ++e) {
+        const int row_e = (int)a.dT.div(e), te = (int)(e - (uint32_t)row_e * a.T);
+        const int be = row_e / C, o = row_e - be * C;
+        const bool in = te < min(a.len_out[be], a.T);
+        const uint32_t q = D == 1 ? (uint32_t)row_e * a.Tp + te : ((uint32_t)(be * 2 + (te & 1)) * C + o) * a.Tp + (te >> 1);
+        if (copy) { ((unsigned short*)a.u_out)[e] = in ? ((const unsigned short*)a.u)[q] : (unsigned short)0; continue; }
+        const NT vq = in ? ((const NT*)a.v)[q] : NT(0.f);
+        float r = 0.f;
+        if (RES == 1 && in) r = ldf((const T*)a.xres + e);
+        if (RES == 2) {
+            const NT vrq = in ? ((const NT*)a.vr)[q] : NT(0.f);
+            r = fmaf(a.gamma_r[o], bn_norm(ldf(&vrq), a.mean_r[o], a.invstd_r[o]), a.beta_r[o]);
+            if (a.vr_out) ((NT*)a.vr_out)[e] = vrq;
         }
+        const float y = fmaxf(fmaf(a.gamma[o], bn_norm(ldf(&vq), a.mean[o], a.invstd[o]), a.beta[o]) + r, 0.f);
+        stf((T*)a.y + e, in ? y : 0.f);
+        if (a.v_out) ((NT*)a.v_out)[e] = vq;
     }
 }
 
