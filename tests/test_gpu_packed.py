@@ -80,6 +80,7 @@ def test_padded_encoder_equals_chain(api, ctx, T):
     assert (logits.float() - chain["logits"].float()).abs().max() <= 0.1 * scale
     assert logits.shape[2] == spec.T_out and (out_len.cpu().numpy() == chain["out_len"]).all()
     assert (dx.float() - chain["dx"].float()).norm() <= 0.05 * chain["dx"].float().norm()
+    compare_with_chain(spec, w, d, logits, out_len, grads, dx, chain)
 
 
 def test_padded_encoder_starting_without_depthwise(api, ctx):
