@@ -72,13 +72,14 @@ typedef enum {
     SC_ERR_DIM_INCOMPATIBLE = -3,  /* an axis size disagrees with the descriptor                   */
     SC_ERR_TRANSPOSED = -4,        /* right sizes, wrong axis order (e.g. [B,T,C]) or not dense    */
     SC_ERR_ALIGNMENT = -5,         /* base pointer not 16-byte aligned                             */
-    SC_ERR_UNSUPPORTED = -6,       /* even K, stride not 1|2, illegal residual, ...                */
+    SC_ERR_UNSUPPORTED = -6,       /* K < 1, stride not 1|2, illegal residual, ...                 */
     SC_ERR_WORKSPACE = -7,         /* workspace too small or null                                  */
     SC_ERR_LENGTHS = -8,           /* (device) some length is outside [1, T_in]                    */
     SC_ERR_DEVICE_TIMEOUT = -9,    /* (device) a bounded wait inside a kernel ran out              */
     SC_ERR_ARCH = -10,             /* the device is not compute capability 10.x                    */
     SC_ERR_CUDA = -11,             /* a CUDA runtime/driver call failed                            */
-    SC_ERR_RANGE = -12             /* (device) a depthwise or pointwise result exceeded the float16 range */
+    SC_ERR_RANGE = -12             /* (device) a value that the library keeps in float16 left its range: a  */
+                                   /* depthwise or pointwise result, or a bf16 input of a weight gradient */
 } sc_status;
 
 /* A typed tensor argument: size/stride in elements, tag[i] names axis i. */
@@ -93,9 +94,10 @@ typedef struct {
 
 typedef struct {
     int32_t B, C_in, C_out, T_in;
-    int32_t K, stride;          /* K >= 1; stride 1 or 2 (ignored when has_dw = 0).  Odd K with adjacent */
-                                /* taps takes the tensor-core depthwise kernels; even K or dilation > 1  */
-                                /* takes plain kernels                                                   */
+    int32_t K, stride;          /* K >= 1; stride 1 or 2 (ignored when has_dw = 0).  16-bit types: odd K  */
+                                /* with stride 1 and dilation 1 or 2 can take the tensor-core depthwise  */
+                                /* kernels, odd K with stride 2 register-blocked ones; even K, larger    */
+                                /* dilations and float32 take plain kernels                              */
     int32_t io_dtype;           /* sc_dtype of activations and conv weights                        */
     int32_t residual;           /* sc_residual                                                     */
     int32_t C_res;              /* channels of the residual source (0: same as C_in)               */
@@ -110,7 +112,8 @@ typedef struct {
                                 /* depthwise + pointwise (the convolution of the original Jasper block,   */
                                 /* section 4.1.1): params.wp is [C_out, C_in, K]; K, stride and dilation   */
                                 /* apply to it with the depthwise step's conventions; has_dw must be 0 and */
-                                /* log_softmax 0; saved.u is not used.  Plain (non-tensor-core) kernels    */
+                                /* log_softmax 0; saved.u is not used.  16-bit types with stride 1 and     */
+                                /* channels in multiples of 8 can take the tensor cores, others plain kernels */
 } sc_block_desc;
 
 typedef struct {          /* device pointers; absent parts may be null                             */
@@ -153,7 +156,9 @@ typedef struct {
 /* ---- context ------------------------------------------------------------------------------ */
 
 /* Creates a context on CUDA device `device` (which must be compute capability 10.x) and allocates
- * the 64-byte device status word -- the only device allocation the library ever makes.
+ * the 64-byte device status word -- the only device memory the library itself ever allocates (the runtime
+ * sets some aside for the second stream, the events and the graphs that the context holds; all of it goes
+ * with the context).
  * Returns SC_ERR_ARCH on any other architecture.  (The paper's modules are created once by a factory
  * and then only executed, section 3.1; the context is that create-once state: device, status word,
  * resolved driver entry points.) */
@@ -182,8 +187,9 @@ int  sepconv_selftest_bounded_wait(sc_ctx* ctx, void* cuda_stream);
 /* Bytes of scratch the two block calls need for this descriptor (host-only computation).  The block
  * descriptor is the module's constructor arguments as a plain struct: the paper keeps a module's
  * structure in data, not in code (section 3).  Returns SC_ERR_UNSUPPORTED for a descriptor the
- * library does not implement (even K, stride other than 1 or 2, identity residual across a channel
- * change, ...). */
+ * library does not implement (K < 1, stride other than 1 or 2, identity residual across a channel
+ * change, ...).  Blocks that run on copies of their operands (rows that are no multiple of 8 frames, dilation 2, the
+ * non-separable convolution) need room for those: the size is that of the fastest form. */
 int  sepconv_workspace_bytes(const sc_block_desc* desc, size_t* fwd_bytes, size_t* bwd_bytes);
 
 /* Forward of one block (definition at the top of this file): the body of the encoder module of section
