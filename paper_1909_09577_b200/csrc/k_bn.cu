@@ -348,7 +348,7 @@ __global__ void __launch_bounds__(kRowThreads) bn_apply_kernel(ApplyArgs a) {
 //                  8 samples 0.97-1.36    1.00-1.19    0.94-1.10    0.96-0.99     (512 channels, 64 / 128 / 256 chunks: 1.23 / 1.02 / 0.87)
 //                 16 samples 0.98-1.36    0.89-1.01    0.85-0.98    0.83-0.98     (512 channels: 1.40 / 0.88 / 0.83)
 //                 32 samples 1.00-1.33    0.86-1.05    0.84-0.97    0.77-0.88     (512 channels: 1.30 / 1.15 / 1.12)
-constexpr int kSmallChunks = 1024, kSmallOddChunks = 256, kSmallOddWork = 256 * 256, kSmallOddSamples = 4;
+constexpr int kSmallChunks = 1024, kSmallOddChunks = 256, kSmallOddWork = 256 * 256, kSmallOddSamples = 8;
 struct ChanRows {            // chunk j of the channel -> sample and frame
     int cpr, n;
     __device__ __forceinline__ ChanRows(int B, int Tp) : cpr((Tp + 7) >> 3), n(B * ((Tp + 7) >> 3)) {}

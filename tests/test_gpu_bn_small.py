@@ -17,10 +17,11 @@ CASES = [
     (dict(C_in=24, C_out=24, K=7, residual="identity", res_before_relu=False), 3, 130, 64),
     (dict(C_in=16, C_out=8, K=1, has_dw=False, has_bn=False, has_bias=True, has_relu=False), 4, 50, 9),
     (dict(C_in=16, C_out=12, K=5, has_dw=False, full_conv=True), 3, 77, 20),
-    # rows that are no whole number of chunks: at the limit for four samples, at that for more and one sample past it
-    (dict(C_in=24, C_out=24, K=5, residual="identity"), 4, 2043, 700),
-    (dict(C_in=16, C_out=24, K=5), 8, 253, 90),
+    # rows that are no whole number of chunks: at the limit for eight samples, at that for more and past it
+    (dict(C_in=24, C_out=24, K=5, residual="identity"), 8, 1021, 300),
+    (dict(C_in=16, C_out=24, K=5), 9, 221, 90),
     (dict(C_in=16, C_out=24, K=5, residual="proj"), 9, 253, 90),
+    (dict(C_in=8, C_out=264, K=3), 16, 125, 60),
 ]
 
 
